@@ -5,16 +5,13 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <string>
 #include <vector>
 
 #include "lbm_internal.cuh"
 #include "lbm_trace.h"
-
-namespace lbm {
-size_t meas_partial_bytes(int nblocks);
-}
 
 namespace {
 
@@ -184,17 +181,19 @@ void free_all(lbm_ctx* c) {
     cudaFree(c->dlt);
     c->dlt = nullptr;
     cudaFree(c->red_partials);
-    cudaFree(c->red_out);
     cudaFree(c->meas_partials);
-    cudaFree(c->meas_out);
+    cudaFree(c->aux);
+    cudaFree(c->band);
+    if (c->host_out) cudaFreeHost(c->host_out);
     cudaFree(c->vel);
     cudaFree(c->stage);
     c->stage = nullptr;
     c->muw = c->vel = c->meas_partials = nullptr;
     c->flags = c->linkmask = nullptr;
     c->red_partials = nullptr;
-    c->red_out = nullptr;
-    c->meas_out = nullptr;
+    c->aux = nullptr;
+    c->band = nullptr;
+    c->host_out = c->host_out_dev = nullptr;
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     c->stream = nullptr;
 }
@@ -352,7 +351,13 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
     c->mu_sat = co[3];
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    c->red_blocks = 2 * sms;
+    c->sms = sms;
+    // one block per row up to a single wave of eight 256-thread blocks per SM
+    c->red_blocks = std::min(p->ny, 8 * sms);
+    // the wall band: an annulus clipped to the lattice is at most as long as the lattice's
+    // perimeter (a convex curve inside a convex box) and about six nodes wide
+    c->band_cap = 16 * (p->nx + p->ny) + 256;
+    c->meas_blocks = std::min(2 * sms, (c->band_cap + 511) / 512);
 
     auto cleanup = [&](const std::string& msg) {
         cudaGetLastError();
@@ -376,10 +381,11 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
     if (e == cudaSuccess) e = cudaMalloc(&c->muw, c->plane * esz);
     if (e == cudaSuccess) e = cudaMalloc((void**)&c->flags, c->plane);
     if (e == cudaSuccess) e = cudaMalloc((void**)&c->linkmask, c->plane);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&c->red_partials, sizeof(double) * 8 * c->red_blocks);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&c->red_out, sizeof(lbm::ReduceOut));
-    if (e == cudaSuccess) e = cudaMalloc(&c->meas_partials, lbm::meas_partial_bytes(c->red_blocks));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&c->meas_out, 2 * sizeof(lbm_angle));
+    if (e == cudaSuccess) e = cudaMalloc(&c->red_partials, lbm::reduce_partial_bytes(c->red_blocks));
+    if (e == cudaSuccess) e = cudaMalloc(&c->meas_partials, lbm::meas_partial_bytes(c->meas_blocks));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&c->band, sizeof(int) * c->band_cap);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&c->aux, sizeof(lbm::DevScratch));
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->aux, 0, sizeof(lbm::DevScratch), c->stream);
     if (e == cudaSuccess) e = lbm::step_configure(c);
     if (e != cudaSuccess) return cleanup(std::string("lbm_create: ") + cudaGetErrorString(e));
     *out = c;
@@ -590,10 +596,10 @@ lbm_status lbm_measure_contact_angle(lbm_ctx* c, lbm_angle out[2]) {
     if (!out) return fail(c, LBM_ERR_ARG, "lbm_measure_contact_angle: out is NULL");
     if (!c->has_geometry) return fail(c, LBM_ERR_STATE, "lbm_measure_contact_angle: no geometry");
     DeviceGuard dg(c->device);
+    LBM_CUDA(c, lbm::ensure_host_out(c));
     LBM_CUDA(c, lbm::launch_measure(c));
-    LBM_CUDA(c, cudaMemcpyAsync(out, c->meas_out, 2 * sizeof(lbm_angle), cudaMemcpyDeviceToHost,
-                                c->stream));
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+    memcpy(out, c->host_out->angle, 2 * sizeof(lbm_angle));
     if (out[0].status != LBM_OK || out[1].status != LBM_OK)
         return fail(c, LBM_ERR_NO_CONTACT, "lbm_measure_contact_angle: a side has no contact");
     return LBM_OK;
@@ -605,10 +611,10 @@ lbm_status lbm_mass(lbm_ctx* c, double out[4]) {
     if (!out) return fail(c, LBM_ERR_ARG, "lbm_mass: out is NULL");
     if (!c->has_geometry) return fail(c, LBM_ERR_STATE, "lbm_mass: no geometry");
     DeviceGuard dg(c->device);
-    lbm::ReduceOut r{};
-    LBM_CUDA(c, lbm::launch_reduce(c));
-    LBM_CUDA(c, cudaMemcpyAsync(&r, c->red_out, sizeof r, cudaMemcpyDeviceToHost, c->stream));
+    LBM_CUDA(c, lbm::ensure_host_out(c));
+    LBM_CUDA(c, lbm::launch_reduce(c, true));
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+    const lbm::ReduceOut r = c->host_out->red;
     out[0] = r.mass;
     out[1] = r.n_liquid;
     out[2] = r.sx;

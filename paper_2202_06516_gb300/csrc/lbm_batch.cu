@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "lbm_step_body.cuh"
+#include "lbm_sum.cuh"
 #include "lbm_trace.h"
 
 namespace lbm {
@@ -40,6 +41,8 @@ struct lbm_batch {
     int* d_ntiles = nullptr;
     int* d_active = nullptr;      // running instance ids (residual kernel)
     double* d_res = nullptr;      // per instance: residual sum, mass
+    double* d_part = nullptr;     // per instance and slice: the same two sums
+    unsigned* d_ticket = nullptr; // per instance: finished slices
     float* snap = nullptr;        // one density snapshot plane per instance
     std::vector<size_t> snap_off;
     int max_tiles = 0;
@@ -105,42 +108,66 @@ __global__ void __launch_bounds__(NTB, MINB)
     }
 }
 
-// One block per running instance: sum |rho - snapshot| and sum rho over fluid nodes in a fixed
-// order, then refresh the snapshot. res[2 i] = sum |drho|, res[2 i + 1] = sum rho.
-__global__ void k_batch_residual(const BatchInst* inst, const int* active, int parity, double* res,
-                                 int refresh) {
+// Sum |rho - snapshot| and sum rho over the fluid nodes of every running instance in a fixed
+// order, then refresh the snapshot: res[2 i] = sum |drho|, res[2 i + 1] = sum rho. kResSlices blocks
+// per instance, each a strided set of rows, eight nodes per access; the instance's last block adds
+// the slices in order. (One block per instance and FP64 arithmetic on every node took 1.0 ms on
+// the 64-instance sweep; the FP64 pipe, two lanes per cycle and SM, was the bound.)
+constexpr int kResSlices = 32;
+__global__ void __launch_bounds__(NTB)
+    k_batch_residual(const BatchInst* inst, const int* active, int parity, double* part,
+                     unsigned* tickets, double* res, int refresh) {
     const int id = active[blockIdx.x];
     const BatchInst& I = inst[id];
     const float* rho = I.rho[parity];
-    double dsum = 0, msum = 0;
-    const int n = I.nx * I.ny;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const int j = k / I.nx, i = k - j * I.nx;
-        const int o = lidx(I.P, i, j);
-        if (I.flags[o] != kFluid) continue;
-        const float r = rho[o];
-        dsum += fabs((double)r - (double)I.snap[o]);
-        msum += (double)r;
-        if (refresh) I.snap[o] = r;
-    }
-    __shared__ double s[2][NTB / 32];
-    for (int o = 16; o > 0; o >>= 1) {
-        dsum += __shfl_down_sync(0xffffffffu, dsum, o);
-        msum += __shfl_down_sync(0xffffffffu, msum, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        s[0][threadIdx.x >> 5] = dsum;
-        s[1][threadIdx.x >> 5] = msum;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0, b = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            a += s[0][w];
-            b += s[1][w];
+    FixSum dsum, msum;
+    const int groups = (I.nx + 7) / 8;
+    for (int j = blockIdx.y; j < I.ny; j += kResSlices) {
+        const int row = lidx(I.P, 0, j);
+        for (int g = threadIdx.x; g < groups; g += NTB) {
+            const int o = row + 8 * g;
+            float r[8], w[8];
+            load8(rho + o, r);  // columns past nx lie in the row's pad
+            load8(I.snap + o, w);
+            const uint2 f = __ldg(reinterpret_cast<const uint2*>(I.flags + o));
+            if (refresh) {
+                reinterpret_cast<float4*>(I.snap + o)[0] = make_float4(r[0], r[1], r[2], r[3]);
+                reinterpret_cast<float4*>(I.snap + o)[1] = make_float4(r[4], r[5], r[6], r[7]);
+            }
+            dsum.make_room(16);  // a difference's halves are twice as large
+            msum.make_room(8);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const unsigned fk = ((k < 4 ? f.x : f.y) >> (8 * (k & 3))) & 0xFFu;
+                if (fk != kFluid || 8 * g + k >= I.nx) continue;
+                if (fix_ok(r[k]) && fix_ok(w[k])) {
+                    const Fix x = to_fix(r[k]), y = to_fix(w[k]);
+                    msum.add(x);
+                    dsum.add(r[k] >= w[k] ? Fix{x.hi - y.hi, x.lo - y.lo}
+                                          : Fix{y.hi - x.hi, y.lo - x.lo});
+                } else {
+                    msum.acc += (double)r[k];
+                    dsum.acc += fabs((double)r[k] - (double)w[k]);
+                }
+            }
         }
-        res[2 * id] = a;
-        res[2 * id + 1] = b;
+    }
+    __shared__ double s_acc[NTB / 32];
+    __shared__ long long s_fix[NTB / 32];
+    __shared__ int s_last;
+    const double d = block_sum(dsum, s_fix, s_acc);
+    __syncthreads();  // thread 0 may still read the first sum's warps
+    const double m = block_sum(msum, s_fix, s_acc);
+    double* p = part + 2 * (size_t)id * kResSlices;
+    if (threadIdx.x == 0) {
+        p[2 * blockIdx.y] = d;
+        p[2 * blockIdx.y + 1] = m;
+    }
+    if (!last_block(tickets + id, kResSlices, &s_last)) return;
+    if (threadIdx.x < 2) {
+        double t = 0;
+        for (int k = 0; k < kResSlices; ++k) t += __ldcg(p + 2 * k + threadIdx.x);
+        res[2 * id + threadIdx.x] = t;
     }
 }
 
@@ -276,6 +303,12 @@ cudaError_t launch_batch_step(lbm_batch* b, int parity) {
     return cudaErrorInvalidValue;
 }
 
+cudaError_t launch_residual(lbm_batch* b, int nact, int parity) {
+    k_batch_residual<<<dim3(nact, kResSlices), NTB, 0, b->stream>>>(
+        (const BatchInst*)b->d_desc, b->d_active, parity, b->d_part, b->d_ticket, b->d_res, 1);
+    return cudaGetLastError();
+}
+
 lbm_status capture(lbm_batch* b, int chunk, int parity) {
     if (b->graph) cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
@@ -330,6 +363,8 @@ lbm_status lbm_batch_create(const lbm_params* model, int32_t n, const int32_t* n
         cudaFree(b->d_ntiles);
         cudaFree(b->d_active);
         cudaFree(b->d_res);
+        cudaFree(b->d_part);
+        cudaFree(b->d_ticket);
         cudaFree(b->snap);
         if (b->stream) cudaStreamDestroy(b->stream);
         delete b;
@@ -377,6 +412,9 @@ lbm_status lbm_batch_create(const lbm_params* model, int32_t n, const int32_t* n
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_ntiles, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_active, sizeof(int) * n);
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_res, sizeof(double) * 2 * n);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_part, sizeof(double) * 2 * kResSlices * n);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_ticket, sizeof(unsigned) * n);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_ticket, 0, sizeof(unsigned) * n, b->stream);
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->snap, sizeof(float) * snap_total);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->snap, 0, sizeof(float) * snap_total, b->stream);
     if (e == cudaSuccess) e = configure_variant(b, kBatchDefaultVariant);
@@ -459,9 +497,7 @@ lbm_status lbm_batch_run(lbm_batch* b, int64_t max_steps, int32_t check_every, d
     lbm_status st = upload_tiles(b, parity, &ntiles, &act);
     if (st != LBM_OK) return st;
     if (!act.empty()) {
-        k_batch_residual<<<(int)act.size(), NTB, 0, b->stream>>>((const BatchInst*)b->d_desc,
-                                                                 b->d_active, parity, b->d_res, 1);
-        BCUDA(b, cudaGetLastError());
+        BCUDA(b, launch_residual(b, (int)act.size(), parity));
     }
     while (done < max_steps && !act.empty()) {
         const int chunk = (int)std::min<int64_t>(check_every, max_steps - done);
@@ -482,9 +518,7 @@ lbm_status lbm_batch_run(lbm_batch* b, int64_t max_steps, int32_t check_every, d
             b->steps[i] += chunk;
             b->cur[i] = parity;
         }
-        k_batch_residual<<<(int)act.size(), NTB, 0, b->stream>>>((const BatchInst*)b->d_desc,
-                                                                 b->d_active, parity, b->d_res, 1);
-        BCUDA(b, cudaGetLastError());
+        BCUDA(b, launch_residual(b, (int)act.size(), parity));
         std::vector<double> res(2 * b->n);
         BCUDA(b, cudaMemcpyAsync(res.data(), b->d_res, sizeof(double) * 2 * b->n,
                                  cudaMemcpyDeviceToHost, b->stream));
@@ -656,6 +690,8 @@ void lbm_batch_destroy(lbm_batch* b) {
     cudaFree(b->d_ntiles);
     cudaFree(b->d_active);
     cudaFree(b->d_res);
+    cudaFree(b->d_part);
+    cudaFree(b->d_ticket);
     cudaFree(b->snap);
     if (b->stream) cudaStreamDestroy(b->stream);
     delete b;

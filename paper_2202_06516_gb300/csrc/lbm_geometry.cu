@@ -87,9 +87,14 @@ __global__ void k_muw(const uint8_t* flags, T* muw, GeomArgs g) {
     }
 }
 
-// bit (q-1) set when fluid node x has a solid node at x + e_q; counts fluid nodes
+// Bit (q-1) set when fluid node x has a solid node at x + e_q; counts fluid nodes; and lists
+// (when band_n) the fluid nodes that can start a link with an Eq. 15 point in the measurement's
+// band 0.5 <= d <= 2.5 from the wall surface: a point lies within sqrt(2) of its link's node, so
+// those have -0.92 <= d <= 3.92; the list takes -1.5 <= d <= 4.5 in FP32 (coordinates and radii up
+// to 10^6 err by less than 0.2), in no particular order. The measurement then reads this list
+// instead of every node; entries past cap are counted but not stored.
 __global__ void k_linkmask(const uint8_t* flags, uint8_t* mask, unsigned long long* n_fluid,
-                           GeomArgs g) {
+                           int* band, int* band_n, int cap, GeomArgs g) {
     unsigned long long local = 0;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < (long long)g.ny * g.nx;
          n += (long long)gridDim.x * blockDim.x) {
@@ -101,6 +106,19 @@ __global__ void k_linkmask(const uint8_t* flags, uint8_t* mask, unsigned long lo
             for (int q = 1; q < 9; ++q)
                 if (flags[lidx(g.P, wrap(i + qx(q), g.nx), j + qy(q))] != kFluid)
                     m |= (uint8_t)(1u << (q - 1));
+            if (band_n) {
+                float d = (float)j + 0.5f;
+                if (g.has_circle) {
+                    const float dx = (float)i - (float)g.cx, dy = (float)j - (float)g.cy;
+                    const float Rs = (float)(g.R + 0.5);
+                    d = sqrtf(dx * dx + dy * dy) - Rs;
+                    if (g.concave) d = -d;
+                }
+                if (d >= -1.5f && d <= 4.5f) {
+                    const int k = atomicAdd(band_n, 1);
+                    if (k < cap) band[k] = (int)n;
+                }
+            }
         }
         mask[lidx(g.P, i, j)] = m;
     }
@@ -255,10 +273,16 @@ cudaError_t launch_geometry(lbm_ctx* c, const GeomArgs& g) {
     else
         k_fill_pads<double><<<grid_for(rows * 2 * kPadX), kThreads, 0, c->stream>>>(
             (double*)c->muw, c->nx, c->P, rows);
-    unsigned long long* d_nf = (unsigned long long*)c->red_out;  // scratch, overwritten later
+    unsigned long long* d_nf = &c->aux->n_fluid;
+    const bool listed = !g.has_circle ||
+                        (fabs(g.cx) <= 1e6 && fabs(g.cy) <= 1e6 && g.R <= 1e6);
     cudaError_t e = cudaMemsetAsync(d_nf, 0, sizeof(unsigned long long), c->stream);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(&c->aux->band_n, listed ? 0 : 0xFF, sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
-    k_linkmask<<<grid_for(nf), kThreads, 0, c->stream>>>(c->flags, c->linkmask, d_nf, g);
+    k_linkmask<<<grid_for(nf), kThreads, 0, c->stream>>>(c->flags, c->linkmask, d_nf, c->band,
+                                                         listed ? &c->aux->band_n : nullptr,
+                                                         c->band_cap, g);
     unsigned long long nfl = 0;
     e = cudaMemcpyAsync(&nfl, d_nf, sizeof nfl, cudaMemcpyDeviceToHost, c->stream);
     if (e != cudaSuccess) return e;

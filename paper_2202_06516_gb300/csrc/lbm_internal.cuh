@@ -85,6 +85,20 @@ struct ReduceOut {
     double mass, n_liquid, sx, sy, bad, pad0, pad1, pad2;
 };
 
+// Per-lattice device scratch besides the planes. The tickets count finished blocks of the
+// reduction and of the measurement; the last block resets its ticket.
+struct DevScratch {
+    ReduceOut red;
+    unsigned long long n_fluid;
+    int band_n;           // entries of lbm_ctx::band; negative or above band_cap: not usable
+    unsigned ticket[2];
+};
+
+struct HostOut {
+    ReduceOut red;
+    lbm_angle angle[2];
+};
+
 struct Substrate {
     int circle;       // 1: circle (cx, cy, Rs), 0: flat bottom wall at y = -1/2
     int concave;      // circle only: 1 = the fluid lies inside the circle
@@ -95,7 +109,7 @@ struct Substrate {
 
 struct lbm_ctx {
     lbm_params p;
-    int device = 0;
+    int device = 0, sms = 152;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int nx = 0, ny = 0, P = 0;
@@ -117,11 +131,14 @@ struct lbm_ctx {
     lbm_geometry geom{};
     lbm::Substrate sub{};
     // reduction / measurement scratch
-    double* red_partials = nullptr;
-    lbm::ReduceOut* red_out = nullptr;
-    void* meas_partials = nullptr;
-    lbm_angle* meas_out = nullptr;
-    int red_blocks = 0;
+    void* red_partials = nullptr;  // per-block partial sums (reduce_partial_bytes)
+    void* meas_partials = nullptr; // per-block best links (meas_partial_bytes)
+    lbm::DevScratch* aux = nullptr;
+    lbm::HostOut* host_out = nullptr;      // mapped host memory the kernels write results to
+    lbm::HostOut* host_out_dev = nullptr;  // its device address (both set at the first use)
+    int* band = nullptr;           // fluid nodes near the wall surface, aux->band_n of them
+    int band_cap = 0;
+    int red_blocks = 0, meas_blocks = 0;
     // velocity scratch for lbm_read_fields
     void* vel = nullptr;
     // nx * ny doubles staging host transfers (initial density in, fields out), kept between calls
@@ -155,8 +172,12 @@ struct StepVariant {
 void step_variants(size_t esz, std::vector<StepVariant>* out);
 bool step_has_ibb(size_t esz, int tile_x, int tile_y, int min_blocks);
 cudaError_t step_configure(lbm_ctx* c);
-cudaError_t launch_reduce(lbm_ctx* c);
+// sums into aux->red, and into host_out (to_host)
+cudaError_t launch_reduce(lbm_ctx* c, bool to_host);
 cudaError_t launch_measure(lbm_ctx* c);
+size_t reduce_partial_bytes(int nblocks);
+size_t meas_partial_bytes(int nblocks);
+cudaError_t ensure_host_out(lbm_ctx* c);
 cudaError_t launch_candidates(lbm_ctx* c, uint8_t* d_mark, double* d_pxyd);
 cudaError_t launch_to_double(lbm_ctx* c, const void* src, double* dst, int src_is_rho_plane);
 cudaError_t launch_fill_pads(lbm_ctx* c, void* plane, size_t esz);

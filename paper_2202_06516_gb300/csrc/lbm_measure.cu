@@ -1,19 +1,24 @@
 // FP64 reductions and the on-device contact-angle measurement (Sec. 3.2, Eq. 15, Fig. 1-2).
 //
-// Reductions (mass, liquid-node count and centroid) are two-pass and deterministic: every block
-// writes FP64 partial sums to scratch, one block adds them in a fixed order.
+// Reductions (mass, liquid-node count and centroid): one kernel, deterministic. Every block writes
+// its partial sums to scratch, and the block that finishes last adds them in a fixed order.
 //
-// Measurement: every thread scans nodes for liquid/gas links (one end rho > rho_m, the other not)
-// in the four undirected link directions, places the Eq. 15 point on the link, measures its
-// distance d to the substrate and keeps, per side, the links nearest to d = 1 and d = 2 within
+// Measurement: the threads scan the nodes near the wall surface (a list made with the geometry)
+// for liquid/gas links (one end rho > rho_m, the other not)
+// in the four undirected link directions, place the Eq. 15 point on the link, measure its
+// distance d to the substrate and keep, per side, the links nearest to d = 1 and d = 2 within
 // the band 0.5 <= d <= 2.5 (ordered by |d - target|, then link id). Blocks reduce with warp
-// shuffles into per-block partials; a final single-block kernel picks the winners and builds the
+// shuffles into per-block partials; the last block to finish picks the winners and builds the
 // line, the contact point and the angle. The point and distance arithmetic uses explicitly
 // rounded FP64 operations (no contraction), so the candidate set and the chosen links are
 // reproducible bit for bit by any IEEE implementation that evaluates the same operations.
+//
+// Both kernels write their results straight into mapped host memory, so a call is one or two
+// launches and one stream synchronisation.
 #include <math.h>
 
 #include "lbm_internal.cuh"
+#include "lbm_sum.cuh"
 
 namespace lbm {
 namespace {
@@ -24,8 +29,11 @@ struct Best {
     double px, py, d;
 };
 
+// keys are non-negative, so their order is that of their bit patterns (integer comparisons: the FP64
+// pipe takes two lanes per cycle and SM)
 __device__ __forceinline__ bool better(double k1, long long i1, double k2, long long i2) {
-    return k1 < k2 || (k1 == k2 && i1 < i2);
+    const long long a = __double_as_longlong(k1), b = __double_as_longlong(k2);
+    return a < b || (a == b && i1 < i2);
 }
 
 __device__ __forceinline__ void shfl_best(Best& b, int o) {
@@ -42,67 +50,158 @@ __device__ __forceinline__ void shfl_best(Best& b, int o) {
 __device__ __forceinline__ int slot_x(int sl) { return sl == 1 ? 0 : (sl == 3 ? -1 : 1); }
 __device__ __forceinline__ int slot_y(int sl) { return sl == 0 ? 0 : 1; }
 
-template <typename T>
-__global__ void k_reduce(const T* rho, const uint8_t* flags, int nx, int ny, int P, double rho_m,
-                         double* partials) {
-    double acc[5] = {0, 0, 0, 0, 0};  // mass, n_liquid, sx, sy, bad
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < (long long)nx * ny;
-         n += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(n / nx), i = (int)(n % nx);
-        if (flags[lidx(P, i, j)] != kFluid) continue;
-        const double r = (double)rho[lidx(P, i, j)];
-        acc[0] += r;
-        if (!(r > 0.0) || !isfinite(r)) acc[4] += 1.0;
-        if (r > rho_m) {
-            acc[1] += 1.0;
-            acc[2] += (double)i;
-            acc[3] += (double)j;
-        }
-    }
-    __shared__ double s[kRedThreads / 32][5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        double v = acc[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 5) {
-        double v = 0;
-        for (int w = 0; w < kRedThreads / 32; ++w) v += s[w][threadIdx.x];
-        partials[(size_t)blockIdx.x * 8 + threadIdx.x] = v;
+// Sums of one block, one plane per quantity: mass[nb], then n_liquid, sx, sy, bad [nb] as integers.
+struct Partials {
+    double* mass;
+    unsigned long long* cnt;  // 4 planes
+};
+
+// one node's density into the sums; a density that is not a positive finite number is counted
+__device__ __forceinline__ void add_node(FixSum& m, unsigned& nbad, float v) {
+    if (fix_ok(v)) {
+        m.add(to_fix(v));
+    } else {
+        m.acc += (double)v;
+        if (!(v > 0.f) || !isfinite(v)) ++nbad;
     }
 }
+__device__ __forceinline__ void add_node(FixSum& m, unsigned& nbad, double v) {
+    m.acc += v;
+    if (!(v > 0.0) || !isfinite(v)) ++nbad;
+}
 
-__global__ void k_reduce_final(const double* partials, int nblocks, ReduceOut* out) {
-    __shared__ double s[5];
-    if (threadIdx.x < 5) {
-        double v = 0;
-        for (int b = 0; b < nblocks; ++b) v += partials[(size_t)b * 8 + threadIdx.x];
-        s[threadIdx.x] = v;
+// Mass, liquid count, liquid centroid and the count of non-finite or non-positive densities over
+// the fluid nodes, one block per row (then striding), eight nodes per thread and access. Bound by
+// the 5 bytes per node it reads and, with few rows, by latency: the mass is summed in exact
+// fixed point (lbm_sum.cuh), counts and coordinate sums are integers (the same values the FP64
+// sums of whole numbers had), and the comparison with rho_m is made against the largest T not
+// above it (the same truth value for every T), so that FP32 lattices use the FP64 pipe only
+// for the blocks' totals. 4096 x 1024: 82 us and 26 us for a serial last pass
+// (every operation in FP64) became 20 us; 200 x 120: 7 + 26 us became 8.
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads)
+    k_reduce(const T* rho, const uint8_t* flags, int nx, int ny, int P, T thr, Partials part,
+             unsigned* ticket, ReduceOut* out, ReduceOut* host_out) {
+    FixSum mass;
+    unsigned long long cnt[4] = {0, 0, 0, 0};  // n_liquid, sx, sy, bad
+    const int groups = (nx + 7) / 8;
+    for (int j = blockIdx.x; j < ny; j += gridDim.x) {
+        const int row = lidx(P, 0, j);
+        unsigned nl = 0, nbad = 0;
+        unsigned long long sx = 0;
+        for (int g = threadIdx.x; g < groups; g += kRedThreads) {
+            const int i0 = 8 * g;
+            T v[8];
+            load8(rho + row + i0, v);  // columns past nx lie in the row's pad
+            const uint2 f = __ldg(reinterpret_cast<const uint2*>(flags + row + i0));
+            mass.make_room(8);
+            unsigned top = 0;  // FP32: the largest fix_key of the eight
+            if constexpr (sizeof(T) == 4) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) top = max(top, fix_key(v[k]));
+            }
+            if (sizeof(T) == 4 && (f.x | f.y) == 0 && i0 + 8 <= nx && top < kFixRange) {
+                // eight ordinary fluid nodes
+                if constexpr (sizeof(T) == 4) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) mass.add(to_fix(v[k]));
+                    if (__uint_as_float(top + kFixLo) > thr) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (v[k] > thr) {
+                                ++nl;
+                                sx += (unsigned)(i0 + k);
+                            }
+                    }
+                }
+                continue;
+            }
+#pragma unroll 1
+            for (int k = 0; k < 8; ++k) {
+                const unsigned fk = ((k < 4 ? f.x : f.y) >> (8 * (k & 3))) & 0xFFu;
+                if (fk != kFluid || i0 + k >= nx) continue;
+                T x = v[0];
+#pragma unroll
+                for (int m = 1; m < 8; ++m) x = k == m ? v[m] : x;
+                add_node(mass, nbad, x);
+                if (x > thr) {
+                    ++nl;
+                    sx += (unsigned)(i0 + k);
+                }
+            }
+        }
+        cnt[0] += nl;
+        cnt[1] += sx;
+        cnt[2] += (unsigned long long)nl * (unsigned)j;
+        cnt[3] += nbad;
+    }
+    __shared__ double s_acc[kRedThreads / 32];
+    __shared__ long long s_fix[kRedThreads / 32];
+    __shared__ unsigned long long s_cnt[4][kRedThreads / 32];
+    __shared__ int s_last;
+    const int nb = gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // a block without liquid or bad nodes (most of them) has four zero counts
+    const int has_cnt = __syncthreads_or(cnt[0] != 0 || cnt[3] != 0);
+    if (has_cnt)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long u = warp_sum(cnt[k]);
+            if (lane == 0) s_cnt[k][warp] = u;
+        }
+    const double m = block_sum(mass, s_fix, s_acc);
+    if (threadIdx.x == 0) part.mass[blockIdx.x] = m;
+    if (threadIdx.x < 4) {
+        unsigned long long u = 0;
+        if (has_cnt)
+            for (int w = 0; w < kRedThreads / 32; ++w) u += s_cnt[threadIdx.x][w];
+        part.cnt[(size_t)threadIdx.x * nb + blockIdx.x] = u;
+    }
+    if (!last_block(ticket, gridDim.x, &s_last)) return;
+    double md = 0;
+    unsigned long long c[4] = {0, 0, 0, 0};
+    for (int b = threadIdx.x; b < nb; b += kRedThreads) {
+        md += __ldcg(part.mass + b);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) c[k] += __ldcg(part.cnt + (size_t)k * nb + b);
+    }
+    md = warp_sum(md);
+    if (lane == 0) s_acc[warp] = md;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const unsigned long long u = warp_sum(c[k]);
+        if (lane == 0) s_cnt[k][warp] = u;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        out->mass = s[0];
-        out->n_liquid = s[1];
-        out->sx = s[1] > 0 ? s[2] / s[1] : 0.0;
-        out->sy = s[1] > 0 ? s[3] / s[1] : 0.0;
-        out->bad = s[4];
+        md = 0;
+        for (int w = 0; w < kRedThreads / 32; ++w) md += s_acc[w];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            c[k] = 0;
+            for (int w = 0; w < kRedThreads / 32; ++w) c[k] += s_cnt[k][w];
+        }
+        ReduceOut r{};
+        const double n = (double)c[0];
+        r.mass = md;
+        r.n_liquid = n;
+        r.sx = c[0] ? (double)c[1] / n : 0.0;
+        r.sy = c[0] ? (double)c[2] / n : 0.0;
+        r.bad = (double)c[3];
+        *out = r;
+        if (host_out) *host_out = r;
     }
 }
 
-// Eq. 15 point of the link from node (i, j) along slot sl, if it joins liquid and gas.
+// Eq. 15 point of the link from node (i, j) with density va along slot sl to a fluid node with
+// density vb, if it joins liquid and gas. thr: the largest T not above rho_m (rho > rho_m exactly
+// when rho > thr).
 template <typename T>
-__device__ __forceinline__ bool link_point(const T* rho, const uint8_t* flags, int nx, int ny,
-                                           int P, double rho_m, int i, int j, int sl, double& px,
-                                           double& py) {
-    const int ti = i + slot_x(sl), tj = j + slot_y(sl);
-    if (tj >= ny) return false;
-    const int wi = ti < 0 ? ti + nx : (ti >= nx ? ti - nx : ti);
-    if (flags[lidx(P, wi, tj)] != kFluid) return false;
-    const double ra = (double)rho[lidx(P, i, j)], rb = (double)rho[lidx(P, wi, tj)];
-    const bool la = ra > rho_m, lb = rb > rho_m;
+__device__ __forceinline__ bool link_point(T va, T vb, double rho_m, T thr, int i, int j, int sl,
+                                           double& px, double& py) {
+    const bool la = va > thr, lb = vb > thr;
     if (la == lb) return false;
+    const double ra = (double)va, rb = (double)vb;
+    const int ti = i + slot_x(sl), tj = j + slot_y(sl);
     double xg, yg, rg, rl, ex, ey;
     if (la) {
         xg = ti; yg = tj; rg = rb; rl = ra; ex = -slot_x(sl); ey = -slot_y(sl);
@@ -115,6 +214,23 @@ __device__ __forceinline__ bool link_point(const T* rho, const uint8_t* flags, i
     return true;
 }
 
+// Densities at the other ends of node (i, j)'s four links; bit sl of the result: that end exists
+// and is fluid
+template <typename T>
+__device__ __forceinline__ unsigned link_ends(const T* rho, const uint8_t* flags, int nx, int ny,
+                                              int P, int i, int j, T (&vb)[4]) {
+    unsigned ok = 0;
+#pragma unroll
+    for (int sl = 0; sl < 4; ++sl) {
+        const int ti = i + slot_x(sl), tj = j + slot_y(sl);
+        const int wi = ti < 0 ? ti + nx : (ti >= nx ? ti - nx : ti);
+        const int e = lidx(P, wi, tj);  // row ny is a pad row of the planes
+        vb[sl] = rho[e];
+        if (tj < ny && flags[e] == kFluid) ok |= 1u << sl;
+    }
+    return ok;
+}
+
 // distance from the wall surface into the fluid
 __device__ __forceinline__ double substrate_dist(const Substrate& s, double px, double py) {
     if (s.circle) {
@@ -125,64 +241,67 @@ __device__ __forceinline__ double substrate_dist(const Substrate& s, double px, 
     return __dsub_rn(py, -0.5);
 }
 
-template <typename T>
-__global__ void k_meas_cand(const T* rho, const uint8_t* flags, int nx, int ny, int P,
-                            double rho_m, Substrate sub, const ReduceOut* red, Best* partials) {
-    const double qxc = red->sx, qyc = red->sy;
-    Best b[4];
+// Candidate links of node n (fluid) into the four running bests (side * 2 + target). PRE: points
+// whose FP32 distance is more than a quarter outside the band are dropped before the FP64
+// construction (coordinates and radii up to 10^6: the FP32 distance errs by less than 0.2).
+template <typename T, bool PRE>
+__device__ __forceinline__ bool scan_node(const T* rho, const uint8_t* flags, int nx, int ny, int P,
+                                          double rho_m, T thr, const Substrate& sub, double qxc,
+                                          double qyc, long long n, Best (&b)[4]) {
+    const int j = (int)n / nx, i = (int)n - j * nx;  // fewer than 2^31 nodes
+    T vb[4];
+    const T va = rho[lidx(P, i, j)];
+    const unsigned ok = link_ends<T>(rho, flags, nx, ny, P, i, j, vb);
+    bool any = false;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) b[k] = Best{INFINITY, 0x7fffffffffffffffLL, 0, 0, 0};
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < (long long)nx * ny;
-         n += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(n / nx), i = (int)(n % nx);
-        if (flags[lidx(P, i, j)] != kFluid) continue;
-        for (int sl = 0; sl < 4; ++sl) {
-            double px, py;
-            if (!link_point<T>(rho, flags, nx, ny, P, rho_m, i, j, sl, px, py)) continue;
-            const double d = substrate_dist(sub, px, py);
-            if (!(d >= 0.5 && d <= 2.5)) continue;
-            int side;
+    for (int sl = 0; sl < 4; ++sl) {
+        if (!(ok >> sl & 1) || (va > thr) == (vb[sl] > thr)) continue;
+        if (PRE) {
+            const float a = (float)va, fr = __fdividef((float)rho_m - a, (float)vb[sl] - a);
+            const float x = i + fr * slot_x(sl), y = j + fr * slot_y(sl);
+            float d = y + 0.5f;
             if (sub.circle) {
-                const double ax = __dsub_rn(qxc, sub.cx), ay = __dsub_rn(qyc, sub.cy);
-                const double bx = __dsub_rn(px, sub.cx), by = __dsub_rn(py, sub.cy);
-                const double cr = __dsub_rn(__dmul_rn(ax, by), __dmul_rn(ay, bx));
-                // the wall normal into the fluid at the centroid is (ax, ay) on the convex
-                // circle and -(ax, ay) on the concave one
-                side = (sub.concave ? cr < 0.0 : cr > 0.0) ? 0 : 1;
-            } else {
-                side = px < qxc ? 0 : 1;
+                const float dx = x - (float)sub.cx, dy = y - (float)sub.cy;
+                d = sqrtf(dx * dx + dy * dy) - (float)sub.Rs;
+                if (sub.concave) d = -d;
             }
-            const long long id = n * 4 + sl;
+            if (d < 0.25f || d > 2.75f) continue;
+        }
+        double px, py;
+        if (!link_point<T>(va, vb[sl], rho_m, thr, i, j, sl, px, py)) continue;
+        const double d = substrate_dist(sub, px, py);
+        if (!(d >= 0.5 && d <= 2.5)) continue;
+        any = true;
+        int side;
+        if (sub.circle) {
+            const double ax = __dsub_rn(qxc, sub.cx), ay = __dsub_rn(qyc, sub.cy);
+            const double bx = __dsub_rn(px, sub.cx), by = __dsub_rn(py, sub.cy);
+            const double cr = __dsub_rn(__dmul_rn(ax, by), __dmul_rn(ay, bx));
+            // the wall normal into the fluid at the centroid is (ax, ay) on the convex
+            // circle and -(ax, ay) on the concave one
+            side = (sub.concave ? cr < 0.0 : cr > 0.0) ? 0 : 1;
+        } else {
+            side = px < qxc ? 0 : 1;
+        }
+        const long long id = n * 4 + sl;
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                const double key = fabs(__dsub_rn(d, (double)(t + 1)));
-                Best& bb = b[side * 2 + t];
-                if (better(key, id, bb.key, bb.id)) bb = Best{key, id, px, py, d};
-            }
+        for (int k = 0; k < 4; ++k) {
+            if ((k >> 1) != side) continue;
+            const double key = fabs(__dsub_rn(d, (double)((k & 1) + 1)));
+            if (better(key, id, b[k].key, b[k].id)) b[k] = Best{key, id, px, py, d};
         }
     }
-    __shared__ Best s[kRedThreads / 32][4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        for (int o = 16; o > 0; o >>= 1) shfl_best(b[k], o);
-        if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5][k] = b[k];
-    }
-    __syncthreads();
-    if (threadIdx.x < 4) {
-        Best r = s[0][threadIdx.x];
-        for (int w = 1; w < kRedThreads / 32; ++w)
-            if (better(s[w][threadIdx.x].key, s[w][threadIdx.x].id, r.key, r.id)) r = s[w][threadIdx.x];
-        partials[(size_t)blockIdx.x * 4 + threadIdx.x] = r;
-    }
+    return any;
 }
 
-// Contact point, tangent and angle for one side (Fig. 1, Fig. 2).
-__device__ void finish_side(const Best& b1, const Best& b2, const Substrate& sub, int side,
-                            lbm_angle* o) {
+// The line of one side through its two points, its contact point and the wall tangent toward the
+// liquid (Fig. 1, Fig. 2); false (and the status set) where the side has none.
+__device__ bool side_line(const Best& b1, const Best& b2, const Substrate& sub, int side,
+                          lbm_angle* o, double& ct, double& at) {
     o->status = LBM_OK;
     if (!(b1.key < INFINITY) || !(b2.key < INFINITY) || b1.id == b2.id) {
         o->status = LBM_ERR_NO_CONTACT;
-        return;
+        return false;
     }
     o->p1_x = b1.px; o->p1_y = b1.py; o->d1 = b1.d; o->link1 = b1.id;
     o->p2_x = b2.px; o->p2_y = b2.py; o->d2 = b2.d; o->link2 = b2.id;
@@ -197,7 +316,7 @@ __device__ void finish_side(const Best& b1, const Best& b2, const Substrate& sub
         const double disc = wv * wv - (wx * wx + wy * wy - sub.Rs * sub.Rs);
         if (disc < 0) {
             o->status = LBM_ERR_NO_CONTACT;
-            return;
+            return false;
         }
         const double sq = sqrt(disc);
         const double s1 = -wv - sq, s2 = -wv + sq;
@@ -223,7 +342,7 @@ __device__ void finish_side(const Best& b1, const Best& b2, const Substrate& sub
     } else {
         if (vy == 0) {
             o->status = LBM_ERR_NO_CONTACT;
-            return;
+            return false;
         }
         const double sc = (-0.5 - b1.py) / vy;
         Cx = b1.px + sc * vx;
@@ -231,58 +350,117 @@ __device__ void finish_side(const Best& b1, const Best& b2, const Substrate& sub
         tx = side == 0 ? 1.0 : -1.0;
         ty = 0.0;
     }
-    const double ct = fmin(1.0, fmax(-1.0, tx * vx + ty * vy));
-    o->theta_deg = acos(ct) * (180.0 / M_PI);
-    o->alpha_deg = acos(fmin(1.0, fabs(tx))) * (180.0 / M_PI);
-    o->beta_deg = !sub.circle ? o->theta_deg
-                  : (sub.concave ? o->theta_deg - o->alpha_deg : o->theta_deg + o->alpha_deg);
+    ct = fmin(1.0, fmax(-1.0, tx * vx + ty * vy));
+    at = fmin(1.0, fabs(tx));
     o->contact_x = Cx;
     o->contact_y = Cy;
+    return true;
 }
 
-__global__ void k_meas_final(const Best* partials, int nblocks, Substrate sub, lbm_angle* out) {
-    __shared__ Best s[kRedThreads / 32][4];
+// Both contact angles. The nodes scanned are the listed ones (a few thousand on the wall, against
+// millions in the lattice: the whole-lattice scan it replaces took 152 us on 4096 x 1024 and 18 us on
+// 200 x 120) or, where the list could not be made (band_n negative or above cap), every fluid
+// node. The order of the list does not matter: the winners are minima by (key, link id). The
+// block that finishes last builds the angles, one warp per (side, angle), because chains of
+// dependent FP64 operations are what this part costs.
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads)
+    k_measure(const T* rho, const uint8_t* flags, int nx, int ny, int P, double rho_m, T thr,
+              Substrate sub, const DevScratch* aux, const int* band, int cap, Best* partials,
+              unsigned* ticket, lbm_angle* out) {
+    const double qxc = aux->red.sx, qyc = aux->red.sy;
+    const int nband = aux->band_n;
     Best b[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) b[k] = Best{INFINITY, 0x7fffffffffffffffLL, 0, 0, 0};
-    for (int blk = threadIdx.x; blk < nblocks; blk += blockDim.x)
+    bool any = false;
+    const int stride = gridDim.x * kRedThreads, t0 = blockIdx.x * kRedThreads + threadIdx.x;
+    if (nband >= 0 && nband <= cap) {
+        for (int t = t0; t < nband; t += stride)
+            any |= scan_node<T, true>(rho, flags, nx, ny, P, rho_m, thr, sub, qxc, qyc, band[t], b);
+    } else {
+        for (long long n = t0; n < (long long)nx * ny; n += stride) {
+            const int j = (int)(n / nx), i = (int)(n - (long long)j * nx);
+            if (flags[lidx(P, i, j)] == kFluid)
+                any |= scan_node<T, false>(rho, flags, nx, ny, P, rho_m, thr, sub, qxc, qyc, n, b);
+        }
+    }
+    __shared__ Best s[kRedThreads / 32][4];
+    __shared__ int s_last;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (__syncthreads_or(any)) {
+        const bool warp_any = __any_sync(0xffffffffu, any);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const Best& c = partials[(size_t)blk * 4 + k];
-            if (better(c.key, c.id, b[k].key, b[k].id)) b[k] = c;
+            if (warp_any)
+                for (int o = 16; o > 0; o >>= 1) shfl_best(b[k], o);
+            if (lane == 0) s[warp][k] = b[k];
         }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        for (int o = 16; o > 0; o >>= 1) shfl_best(b[k], o);
-        if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5][k] = b[k];
+        __syncthreads();
+        if (threadIdx.x < 4) {
+            Best r = s[0][threadIdx.x];
+            for (int w = 1; w < kRedThreads / 32; ++w)
+                if (better(s[w][threadIdx.x].key, s[w][threadIdx.x].id, r.key, r.id))
+                    r = s[w][threadIdx.x];
+            partials[(size_t)blockIdx.x * 4 + threadIdx.x] = r;
+        }
+    } else if (threadIdx.x < 4) {
+        partials[(size_t)blockIdx.x * 4 + threadIdx.x] =
+            Best{INFINITY, 0x7fffffffffffffffLL, 0, 0, 0};
+    }
+    if (!last_block(ticket, gridDim.x, &s_last)) return;
+    __shared__ Best win[4];
+    if (warp < 4) {
+        Best r = Best{INFINITY, 0x7fffffffffffffffLL, 0, 0, 0};
+        for (int blk = lane; blk < (int)gridDim.x; blk += 32) {
+            const Best* c = partials + (size_t)blk * 4 + warp;
+            const double key = __ldcg(&c->key);
+            if (!(key < INFINITY)) continue;
+            const long long id = __ldcg(&c->id);
+            if (better(key, id, r.key, r.id))
+                r = Best{key, id, __ldcg(&c->px), __ldcg(&c->py), __ldcg(&c->d)};
+        }
+        for (int o = 16; o > 0; o >>= 1) shfl_best(r, o);
+        if (lane == 0) win[warp] = r;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        Best w[4];
-        for (int k = 0; k < 4; ++k) {
-            w[k] = s[0][k];
-            for (int v = 1; v < kRedThreads / 32; ++v)
-                if (better(s[v][k].key, s[v][k].id, w[k].key, w[k].id)) w[k] = s[v][k];
+    __shared__ double s_alpha[2];
+    const int side = warp & 1;
+    lbm_angle o{};
+    bool ok = false;
+    if (warp < 4 && lane == 0) {
+        double ct = 0, at = 0;
+        ok = side_line(win[side * 2], win[side * 2 + 1], sub, side, &o, ct, at);
+        if (ok && warp < 2) o.theta_deg = acos(ct) * (180.0 / M_PI);
+        if (ok && warp >= 2) s_alpha[side] = acos(at) * (180.0 / M_PI);
+    }
+    __syncthreads();
+    if (warp < 2 && lane == 0) {
+        if (ok) {
+            o.alpha_deg = s_alpha[side];
+            o.beta_deg = !sub.circle ? o.theta_deg
+                         : (sub.concave ? o.theta_deg - o.alpha_deg : o.theta_deg + o.alpha_deg);
         }
-        for (int side = 0; side < 2; ++side) {
-            lbm_angle o{};
-            finish_side(w[side * 2], w[side * 2 + 1], sub, side, &o);
-            out[side] = o;
-        }
+        out[side] = o;
     }
 }
 
 // dense per-(node, slot) candidate marks and points, for parity checks
 template <typename T>
 __global__ void k_cand_dense(const T* rho, const uint8_t* flags, int nx, int ny, int P,
-                             double rho_m, Substrate sub, uint8_t* mark, double* pxyd) {
+                             double rho_m, T thr, Substrate sub, uint8_t* mark, double* pxyd) {
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < (long long)nx * ny;
          n += (long long)gridDim.x * blockDim.x) {
         const int j = (int)(n / nx), i = (int)(n % nx);
         const bool fl = flags[lidx(P, i, j)] == kFluid;
+        const T va = rho[lidx(P, i, j)];
+        T vb[4];
+        const unsigned ends = link_ends<T>(rho, flags, nx, ny, P, i, j, vb);
+#pragma unroll
         for (int sl = 0; sl < 4; ++sl) {
             double px = 0, py = 0;
-            const bool ok = fl && link_point<T>(rho, flags, nx, ny, P, rho_m, i, j, sl, px, py);
+            const bool ok = fl && (ends >> sl & 1) &&
+                            link_point<T>(va, vb[sl], rho_m, thr, i, j, sl, px, py);
             mark[n * 4 + sl] = ok ? 1 : 0;
             if (ok) {
                 pxyd[(n * 4 + sl) * 3 + 0] = px;
@@ -293,69 +471,116 @@ __global__ void k_cand_dense(const T* rho, const uint8_t* flags, int nx, int ny,
     }
 }
 
+// Field out as doubles (0 at solid nodes): one block per row and 1024 columns, so that the index
+// needs no division; four nodes per thread when the rows of the destination allow it.
 template <typename T>
-__global__ void k_to_double(const T* src, const uint8_t* flags, int nx, int ny, int P,
-                            double* dst) {
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < (long long)nx * ny;
-         n += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(n / nx), i = (int)(n % nx);
-        dst[n] = flags[lidx(P, i, j)] == kFluid ? (double)src[lidx(P, i, j)] : 0.0;
+__global__ void __launch_bounds__(kRedThreads)
+    k_to_double(const T* src, const uint8_t* flags, int nx, int P, double* dst) {
+    const int j = blockIdx.x, i0 = (blockIdx.y * kRedThreads + threadIdx.x) * 4;
+    if (i0 >= nx) return;
+    const int e = lidx(P, i0, j);
+    const uint32_t f = __ldg(reinterpret_cast<const unsigned*>(flags + e));
+    T r[4];
+    load4(src + e, r);
+    double v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = ((f >> (8 * k)) & 0xFFu) == kFluid ? (double)r[k] : 0.0;
+    double* o = dst + (size_t)j * nx + i0;
+    if (i0 + 4 <= nx && ((uintptr_t)o & 15) == 0) {
+        reinterpret_cast<double2*>(o)[0] = make_double2(v[0], v[1]);
+        reinterpret_cast<double2*>(o)[1] = make_double2(v[2], v[3]);
+    } else {
+        for (int k = 0; k < 4 && i0 + k < nx; ++k) o[k] = v[k];
     }
 }
 
 }  // namespace
 
-cudaError_t launch_reduce(lbm_ctx* c) {
+size_t reduce_partial_bytes(int nblocks) { return 5 * sizeof(double) * (size_t)nblocks; }
+size_t meas_partial_bytes(int nblocks) { return sizeof(Best) * 4 * (size_t)nblocks; }
+
+// mapped host memory for the results, made at the first call that needs it
+cudaError_t ensure_host_out(lbm_ctx* c) {
+    if (c->host_out_dev) return cudaSuccess;
+    if (!c->host_out) {
+        void* h = nullptr;
+        const cudaError_t e = cudaHostAlloc(&h, sizeof(HostOut), cudaHostAllocMapped);
+        if (e != cudaSuccess) return e;
+        c->host_out = (HostOut*)h;
+    }
+    void* d = nullptr;
+    const cudaError_t e = cudaHostGetDevicePointer(&d, c->host_out, 0);
+    if (e == cudaSuccess) c->host_out_dev = (HostOut*)d;
+    return e;
+}
+
+namespace {
+
+// the largest T that is not above x
+float floor_to(double x, float) {
+    const float f = (float)x;
+    return (double)f > x ? nextafterf(f, -INFINITY) : f;
+}
+double floor_to(double x, double) { return x; }
+
+template <typename T>
+cudaError_t reduce_t(lbm_ctx* c, ReduceOut* host) {
     const double rho_m = 0.5 * (c->rho_g + c->rho_l);
-    if (c->esz == 4)
-        k_reduce<float><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-            (const float*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m, c->red_partials);
-    else
-        k_reduce<double><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-            (const double*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m, c->red_partials);
-    k_reduce_final<<<1, 32, 0, c->stream>>>(c->red_partials, c->red_blocks, c->red_out);
+    Partials p;
+    p.mass = (double*)c->red_partials;
+    p.cnt = (unsigned long long*)(p.mass + c->red_blocks);
+    k_reduce<T><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
+        (const T*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, floor_to(rho_m, T()), p,
+        &c->aux->ticket[0], &c->aux->red, host);
     return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t measure_t(lbm_ctx* c) {
+    const double rho_m = 0.5 * (c->rho_g + c->rho_l);
+    k_measure<T><<<c->meas_blocks, kRedThreads, 0, c->stream>>>(
+        (const T*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m, floor_to(rho_m, T()), c->sub,
+        c->aux, c->band,
+        c->band_cap, (Best*)c->meas_partials, &c->aux->ticket[1], c->host_out_dev->angle);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_reduce(lbm_ctx* c, bool to_host) {
+    ReduceOut* host = to_host ? &c->host_out_dev->red : nullptr;
+    return c->esz == 4 ? reduce_t<float>(c, host) : reduce_t<double>(c, host);
 }
 
 cudaError_t launch_measure(lbm_ctx* c) {
-    cudaError_t e = launch_reduce(c);
+    const cudaError_t e = launch_reduce(c, false);
     if (e != cudaSuccess) return e;
-    const double rho_m = 0.5 * (c->rho_g + c->rho_l);
-    Best* part = (Best*)c->meas_partials;
-    if (c->esz == 4)
-        k_meas_cand<float><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-            (const float*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m, c->sub, c->red_out,
-            part);
-    else
-        k_meas_cand<double><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-            (const double*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m, c->sub, c->red_out,
-            part);
-    k_meas_final<<<1, kRedThreads, 0, c->stream>>>(part, c->red_blocks, c->sub, c->meas_out);
-    return cudaGetLastError();
+    return c->esz == 4 ? measure_t<float>(c) : measure_t<double>(c);
 }
-
-size_t meas_partial_bytes(int nblocks) { return sizeof(Best) * 4 * (size_t)nblocks; }
 
 cudaError_t launch_candidates(lbm_ctx* c, uint8_t* d_mark, double* d_pxyd) {
     const double rho_m = 0.5 * (c->rho_g + c->rho_l);
     if (c->esz == 4)
         k_cand_dense<float><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-            (const float*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m, c->sub, d_mark,
+            (const float*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m,
+            floor_to(rho_m, 0.f), c->sub, d_mark,
             d_pxyd);
     else
         k_cand_dense<double><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-            (const double*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m, c->sub, d_mark,
+            (const double*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m, rho_m, c->sub, d_mark,
             d_pxyd);
     return cudaGetLastError();
 }
 
 cudaError_t launch_to_double(lbm_ctx* c, const void* src, double* dst, int) {
+    // rows along x (2^20 of them at most), column blocks along y
+    const dim3 grid(c->ny, (c->nx + 4 * kRedThreads - 1) / (4 * kRedThreads));
     if (c->esz == 4)
-        k_to_double<float><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-            (const float*)src, c->flags, c->nx, c->ny, c->P, dst);
+        k_to_double<float><<<grid, kRedThreads, 0, c->stream>>>((const float*)src, c->flags, c->nx,
+                                                                c->P, dst);
     else
-        k_to_double<double><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-            (const double*)src, c->flags, c->nx, c->ny, c->P, dst);
+        k_to_double<double><<<grid, kRedThreads, 0, c->stream>>>((const double*)src, c->flags, c->nx,
+                                                                 c->P, dst);
     return cudaGetLastError();
 }
 
