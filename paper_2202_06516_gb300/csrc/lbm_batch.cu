@@ -65,11 +65,13 @@ using namespace stepdev;
 
 constexpr int NTB = 256;
 
-// Compiled tile variants of the persistent kernel: tile (TX, TY) and the CTAs per SM its
-// register budget is fitted to. Variant 1 (32 x 16, 5 CTAs/SM) is the default; the autotuner
-// times all of them on the batch's own tile table.
-#define LBM_BATCH_VARIANTS(X) X(32, 8, 5) X(32, 16, 5) X(64, 16, 3) X(32, 32, 3)
-constexpr int kBatchDefaultVariant = 1;
+// Compiled tile variants of the batched kernel: tile (TX, TY), the CTAs per SM its register budget
+// is fitted to, and threads. Variant 1 (32 x 16, 5 CTAs/SM) is the default; the autotuner times
+// the first four on the batch's own tile table. The others are the small-lattice forms of the
+// default (see lbm_step.cu), taken where all instances together have few tiles.
+#define LBM_BATCH_VARIANTS(X) X(32, 8, 5, 256) X(32, 16, 5, 256) X(64, 16, 3, 256) X(32, 32, 3, 256)
+#define LBM_BATCH_SMALL(X) X(16, 8, 3, 320) X(32, 8, 3, 384)
+constexpr int kBatchDefaultVariant = 1, kBatchSmall0 = 4, kBatchSmall1 = 5;
 
 struct BatchInst {
     float* h[2];
@@ -81,11 +83,12 @@ struct BatchInst {
     float rho_mid;
 };
 
-template <int TX, int TY, int MINB>
-__global__ void __launch_bounds__(NTB, MINB)
+template <int TX, int TY, int MINB, int NT>
+__global__ void __launch_bounds__(NT, MINB)
     k_batch_step(const StepArgs<float> model, const BatchInst* inst, const int2* tiles,
                  const int* n_tiles, int parity) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_launch_next();
     const int nt = *n_tiles;
     for (int t = blockIdx.x; t < nt; t += gridDim.x) {
         const int2 e = tiles[t];
@@ -103,7 +106,7 @@ __global__ void __launch_bounds__(NTB, MINB)
         a.plane = I.plane;
         const int tiles_x = (I.nx + TX - 1) / TX;
         const int ty = e.y / tiles_x, tx = e.y - ty * tiles_x;
-        step_tile<float, TX, TY, NTB, false, false>(a, I.rho_mid, smem_raw, tx * TX, ty * TY);
+        step_tile<float, TX, TY, NT, false, false>(a, I.rho_mid, smem_raw, tx * TX, ty * TY);
         __syncthreads();  // the next tile reuses shared memory
     }
 }
@@ -193,7 +196,7 @@ int tiles_of(const lbm_batch* b, const lbm_ctx* c) { return tiles_of(c, b->tx, b
 
 int num_variants() {
     int n = 0;
-#define X(A, B, M) ++n;
+#define X(A, B, M, N) ++n;
     LBM_BATCH_VARIANTS(X)
 #undef X
     return n;
@@ -204,18 +207,20 @@ int num_variants() {
 cudaError_t configure_variant(lbm_batch* b, int v) {
     int i = 0, per_sm = 0, sms = 0, dev = 0;
     cudaError_t e = cudaErrorInvalidValue;
-#define X(A, B, M)                                                                           \
+#define X(A, B, M, N)                                                                        \
     if (v == i++) {                                                                          \
         const int bytes = (int)Layout<float, A, B>::bytes;                                   \
-        e = cudaFuncSetAttribute(k_batch_step<A, B, M>,                                      \
+        e = cudaFuncSetAttribute(k_batch_step<A, B, M, N>,                                   \
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);        \
         if (e == cudaSuccess)                                                                \
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_step<A, B, M>, \
-                                                              NTB, bytes);                   \
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm,                       \
+                                                              k_batch_step<A, B, M, N>, N,   \
+                                                              bytes);                        \
         b->tx = A;                                                                           \
         b->ty = B;                                                                           \
     }
     LBM_BATCH_VARIANTS(X)
+    LBM_BATCH_SMALL(X)
 #undef X
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -227,13 +232,14 @@ cudaError_t configure_variant(lbm_batch* b, int v) {
 
 void variant_shape(int v, int* tx, int* ty, int* minb) {
     int i = 0;
-#define X(A, B, M)  \
-    if (v == i++) { \
-        *tx = A;    \
-        *ty = B;    \
-        *minb = M;  \
+#define X(A, B, M, N) \
+    if (v == i++) {   \
+        *tx = A;      \
+        *ty = B;      \
+        *minb = M;    \
     }
     LBM_BATCH_VARIANTS(X)
+    LBM_BATCH_SMALL(X)
 #undef X
 }
 
@@ -292,13 +298,24 @@ cudaError_t launch_batch_step(lbm_batch* b, int parity) {
         for (const lbm_ctx* c : b->inst) all += tiles_of(b, c);
         grid = (int)std::max<long long>(1, all);
     }
-#define X(A, B, M)                                                                           \
+#define X(A, B, M, N)                                                                        \
     if (b->variant == i++) {                                                                 \
-        k_batch_step<A, B, M><<<grid, NTB, Layout<float, A, B>::bytes, b->stream>>>(         \
-            b->model, (const BatchInst*)b->d_desc, b->d_tiles, b->d_ntiles, parity);         \
-        return cudaGetLastError();                                                           \
+        cudaLaunchAttribute at{};  /* as for k_step: overlap with the previous step's tail */ \
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;                          \
+        at.val.programmaticStreamSerializationAllowed = 1;                                   \
+        cudaLaunchConfig_t cfg{};                                                            \
+        cfg.gridDim = dim3(grid);                                                            \
+        cfg.blockDim = dim3(N);                                                              \
+        cfg.dynamicSmemBytes = Layout<float, A, B>::bytes;                                   \
+        cfg.stream = b->stream;                                                              \
+        cfg.attrs = &at;                                                                     \
+        cfg.numAttrs = 1;                                                                    \
+        return cudaLaunchKernelEx(&cfg, k_batch_step<A, B, M, N>, (const StepArgs<float>)b->model, \
+                                  (const BatchInst*)b->d_desc, (const int2*)b->d_tiles,      \
+                                  (const int*)b->d_ntiles, parity);                          \
     }
     LBM_BATCH_VARIANTS(X)
+    LBM_BATCH_SMALL(X)
 #undef X
     return cudaErrorInvalidValue;
 }
@@ -396,7 +413,7 @@ lbm_status lbm_batch_create(const lbm_params* model, int32_t n, const int32_t* n
         b->snap_off.push_back(snap_total);
         snap_total += c->plane;
         int most = 0;
-        for (int v = 0; v < num_variants(); ++v) {
+        for (int v = 0; v <= kBatchSmall1; ++v) {
             int vx = 0, vy = 0, vm = 0;
             variant_shape(v, &vx, &vy, &vm);
             most = std::max(most, tiles_of(c, vx, vy));
@@ -417,7 +434,18 @@ lbm_status lbm_batch_create(const lbm_params* model, int32_t n, const int32_t* n
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_ticket, 0, sizeof(unsigned) * n, b->stream);
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->snap, sizeof(float) * snap_total);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->snap, 0, sizeof(float) * snap_total, b->stream);
-    if (e == cudaSuccess) e = configure_variant(b, kBatchDefaultVariant);
+    if (e == cudaSuccess) {
+        // the rule of small_form (lbm_step.cu) on the tiles of all instances together
+        long long t16 = 0, t32 = 0;
+        for (const lbm_ctx* c : b->inst) {
+            t16 += tiles_of(c, 16, 8);
+            t32 += tiles_of(c, 32, 8);
+        }
+        const long long sms = b->inst[0]->sms;
+        e = configure_variant(b, 2 * t16 <= 3 * sms ? kBatchSmall0
+                                 : t32 <= 6 * sms   ? kBatchSmall1
+                                                    : kBatchDefaultVariant);
+    }
     if (e != cudaSuccess)
         return cleanup(LBM_ERR_CUDA, std::string("lbm_batch_create: ") + cudaGetErrorString(e));
     b->autotune_pending = model->tile_x == LBM_TILE_AUTO;

@@ -28,52 +28,94 @@ namespace {
 using namespace stepdev;
 
 // the interpolated bounce-back kernels exist for the default variants only (32 x 16 tiles,
-// 5 CTAs per SM in FP32, unconstrained in FP64)
+// 5 CTAs per SM in FP32, unconstrained in FP64) and the small-lattice forms of the FP32 one
 template <typename T, int TX, int TY, int MINB>
 constexpr bool has_ibb() {
     return TX == 32 && TY == 16 && MINB == (sizeof(T) == 4 ? 5 : 1);
 }
 
+// Launch with programmatic stream serialization: a step's launch, block placement and class staging
+// overlap the previous step's tail (k_step waits before it reads what that step wrote).
+template <typename T, int TX, int TY, int NT, int MINB, bool MACRO, bool IBB>
+cudaError_t launch_k(lbm_ctx* c, const StepArgs<T>& a) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((c->nx + TX - 1) / TX, (c->ny + TY - 1) / TY);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = Layout<T, TX, TY>::bytes;
+    cfg.stream = c->stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_step<T, TX, TY, NT, MACRO, MINB, IBB>, a,
+                              (T)(0.5 * (c->rho_g + c->rho_l)));
+}
+
+template <typename T, int TX, int TY, int NT, int MINB, bool MACRO, bool IBB>
+cudaError_t allow_smem() {
+    return cudaFuncSetAttribute(k_step<T, TX, TY, NT, MACRO, MINB, IBB>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)Layout<T, TX, TY>::bytes);
+}
+
+// Small-lattice forms of the default FP32 variant. A step of a small lattice is one chain of
+// latencies (launch, staging, wetting layers, chemical potential, gathers, streaming, each with its
+// barrier) on a chip that is mostly idle, so these forms give a tile so many threads that
+// every stage is one round, or spread the lattice over more, smaller tiles; on large lattices the
+// recomputed halo and the fewer resident tiles make them slower. Chosen by the number of tiles
+// against the number of SMs. Measured, us per step, 32x16 tiles of 256 threads / forms 1 / 2 / 3:
+// 128x96 7.4 / 4.3 / 5.1 / 4.8; 200x120 8.0 / 4.6 / 5.1 / 5.2; 256x256 8.0 / 6.0 / 5.2 / 5.6;
+// 520x190 10.2 / 6.8 / 7.2 / 6.1; 512x384 11.6 / 10.8 / 10.5 / 8.5; 768x512 12.1 / 17 / 17 / 13.3.
+#define LBM_SMALL_FORMS(X) X(1, 16, 8, 320, 3) X(2, 32, 16, 640, 1) X(3, 32, 8, 384, 3)
+int small_form(const lbm_ctx* c) {
+    const long long nx = c->nx, ny = c->ny, sms = c->sms;
+    auto tiles = [&](long long tx, long long ty) {
+        return ((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
+    };
+    if (2 * tiles(16, 8) <= 3 * sms) return 1;
+    if (tiles(32, 16) <= sms) return 2;
+    if (tiles(32, 8) <= 6 * sms) return 3;
+    return 0;
+}
+
 template <typename T, int TX, int TY, int MINB>
 cudaError_t configure_one() {
-    using L = Layout<T, TX, TY>;
-    cudaError_t e = cudaFuncSetAttribute(k_step<T, TX, TY, 256, false, MINB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_step<T, TX, TY, 256, true, MINB>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
+    cudaError_t e = allow_smem<T, TX, TY, 256, MINB, false, false>();
+    if (e == cudaSuccess) e = allow_smem<T, TX, TY, 256, MINB, true, false>();
     if constexpr (has_ibb<T, TX, TY, MINB>()) {
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_step<T, TX, TY, 256, false, MINB, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_step<T, TX, TY, 256, true, MINB, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
+        if (e == cudaSuccess) e = allow_smem<T, TX, TY, 256, MINB, false, true>();
+        if (e == cudaSuccess) e = allow_smem<T, TX, TY, 256, MINB, true, true>();
+    }
+    if constexpr (sizeof(T) == 4 && TX == 32 && TY == 16 && MINB == 5) {
+#define X(F, A, B, N, M)                                                       \
+    if (e == cudaSuccess) e = allow_smem<float, A, B, N, M, false, false>();   \
+    if (e == cudaSuccess) e = allow_smem<float, A, B, N, M, false, true>();
+        LBM_SMALL_FORMS(X)
+#undef X
     }
     return e;
 }
 
 template <typename T, int TX, int TY, int MINB>
 cudaError_t launch_one(lbm_ctx* c, const StepArgs<T>& a, bool macro) {
-    using L = Layout<T, TX, TY>;
-    dim3 grid((c->nx + TX - 1) / TX, (c->ny + TY - 1) / TY);
-    const T rho_mid = (T)(0.5 * (c->rho_g + c->rho_l));
+    if constexpr (sizeof(T) == 4 && TX == 32 && TY == 16 && MINB == 5) {
+        const int form = macro ? 0 : small_form(c);
+#define X(F, A, B, N, M)                                                       \
+    if (form == F)                                                             \
+        return c->ibb ? launch_k<float, A, B, N, M, false, true>(c, a)         \
+                      : launch_k<float, A, B, N, M, false, false>(c, a);
+        LBM_SMALL_FORMS(X)
+#undef X
+    }
     if (c->ibb) {
-        if constexpr (has_ibb<T, TX, TY, MINB>()) {
-            if (macro)
-                k_step<T, TX, TY, 256, true, MINB, true><<<grid, 256, L::bytes, c->stream>>>(a, rho_mid);
-            else
-                k_step<T, TX, TY, 256, false, MINB, true><<<grid, 256, L::bytes, c->stream>>>(a,
-                                                                                         rho_mid);
-            return cudaGetLastError();
-        }
+        if constexpr (has_ibb<T, TX, TY, MINB>())
+            return macro ? launch_k<T, TX, TY, 256, MINB, true, true>(c, a)
+                         : launch_k<T, TX, TY, 256, MINB, false, true>(c, a);
         return cudaErrorInvalidValue;
     }
-    if (macro)
-        k_step<T, TX, TY, 256, true, MINB><<<grid, 256, L::bytes, c->stream>>>(a, rho_mid);
-    else
-        k_step<T, TX, TY, 256, false, MINB><<<grid, 256, L::bytes, c->stream>>>(a, rho_mid);
-    return cudaGetLastError();
+    return macro ? launch_k<T, TX, TY, 256, MINB, true, false>(c, a)
+                 : launch_k<T, TX, TY, 256, MINB, false, false>(c, a);
 }
 
 template <typename T>

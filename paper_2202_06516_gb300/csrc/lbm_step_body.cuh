@@ -169,14 +169,29 @@ struct Layout {
         sizeof(T) * ((size_t)RW * RH + (size_t)MW * MH + 10 * (size_t)CW * CH) + (size_t)RW * RH;
 };
 
-// four consecutive elements, global (aligned to 4 elements) to shared
-__device__ __forceinline__ void load4(const float* g, float* s) {
-    *reinterpret_cast<float4*>(s) = __ldg(reinterpret_cast<const float4*>(g));
-}
-__device__ __forceinline__ void load4(const double* g, double* s) {
-    *reinterpret_cast<double2*>(s) = __ldg(reinterpret_cast<const double2*>(g));
-    *reinterpret_cast<double2*>(s + 2) = __ldg(reinterpret_cast<const double2*>(g + 2));
-}
+// four consecutive elements (aligned to four elements)
+template <typename T>
+struct V4;
+template <>
+struct V4<float> {
+    float4 v;
+    __device__ __forceinline__ void load(const float* g) {
+        v = *reinterpret_cast<const float4*>(g);
+    }
+    __device__ __forceinline__ void store(float* s) const { *reinterpret_cast<float4*>(s) = v; }
+};
+template <>
+struct V4<double> {
+    double2 v, w;
+    __device__ __forceinline__ void load(const double* g) {
+        v = *reinterpret_cast<const double2*>(g);
+        w = *reinterpret_cast<const double2*>(g + 2);
+    }
+    __device__ __forceinline__ void store(double* s) const {
+        *reinterpret_cast<double2*>(s) = v;
+        *reinterpret_cast<double2*>(s + 2) = w;
+    }
+};
 
 template <typename T, int RW>
 __device__ __forceinline__ T mu_fluid(const T* s_rho, int o, const StepArgs<T>& a) {
@@ -195,24 +210,49 @@ __device__ __forceinline__ T mu_fluid(const T* s_rho, int o, const StepArgs<T>& 
 //   D < 1/2: 2D f*_qbar(x) + (1 - 2D) f*_qbar(x + e_q)   (the half-way value if x + e_q is not
 //            fluid), i.e. 2D out + (1 - 2D) (h_qbar(x + e_q) + w_q (rho(x + e_q) - rho(x)));
 //   D >= 1/2: f*_qbar(x) / 2D + (1 - 1/2D) f*_q(x), i.e. out / 2D + (1 - 1/2D) h_q(x).
-// The caller adds out minus the returned value to the rest population (mass correction).
-template <typename T, int RW, bool PP>
-__device__ __forceinline__ T ibb_return(const StepArgs<T>& a, int q, unsigned us, int o, T rho,
-                                        T out, const T* s_rho, const uint8_t* s_flag) {
-    const T D = a.dlt[(unsigned)(q - 1) * (unsigned)a.plane + us];
+// The caller adds out minus the returned value to the rest population (mass correction) and passes
+// alt = h_qbar(x + e_q) (D < 1/2, and only where x + e_q is fluid) or h_q(x).
+template <typename T, int RW>
+__device__ __forceinline__ T ibb_return(int q, int o, T rho, T out, T D, T alt, const T* s_rho,
+                                        const uint8_t* s_flag) {
     const T D2 = add_rn(D, D);
     if (D < (T)0.5) {
         const int ob = o + qy(q) * RW + qx(q);
         if (s_flag[ob] != kFluid) return out;
-        const unsigned ub = us + (unsigned)(qy(q) * a.P + qx(q));
-        const T hbh = PP ? __ldg(a.hq_in[qopp(q)] + ub)
-                         : __ldg(a.h_in + (unsigned)qopp(q) * (unsigned)a.plane + ub);
-        const T behind = fma_rn(qw<T>(q), sub_rn(s_rho[ob], rho), hbh);
+        const T behind = fma_rn(qw<T>(q), sub_rn(s_rho[ob], rho), alt);
         return fma_rn(D2, out, mul_rn(sub_rn((T)1, D2), behind));
     }
-    const T hq = PP ? __ldg(a.hq_in[q] + us) : __ldg(a.h_in + (unsigned)q * (unsigned)a.plane + us);
     const T c = recip(D2);
-    return fma_rn(c, out, mul_rn(sub_rn((T)1, c), hq));  // exactly out at D = 1/2
+    return fma_rn(c, out, mul_rn(sub_rn((T)1, c), alt));  // exactly out at D = 1/2
+}
+
+// The link fractions and the further populations that ibb_return needs, of all cut links of a
+// node: first every fraction is loaded, then every population, so that a node with several cut
+// links waits for two memory latencies and not for two per link (that chain was most of the
+// interpolated step's time on small lattices: 17.5 us per step against 8.9 half-way on 520 x 190).
+template <typename T, int RW, bool PP>
+__device__ __forceinline__ void ibb_gather(const StepArgs<T>& a, unsigned us, int o,
+                                           const uint8_t* s_flag, T (&D)[9], T (&alt)[9]) {
+    const unsigned upl = (unsigned)a.plane;
+#pragma unroll
+    for (int q = 1; q < 9; ++q) {
+        D[q] = (T)0.5;
+        if (s_flag[o - qy(q) * RW - qx(q)] != kFluid) D[q] = __ldg(a.dlt + (unsigned)(q - 1) * upl + us);
+    }
+#pragma unroll
+    for (int q = 1; q < 9; ++q) {
+        alt[q] = (T)0;
+        if (s_flag[o - qy(q) * RW - qx(q)] == kFluid) continue;
+        if (D[q] < (T)0.5) {
+            if (s_flag[o + qy(q) * RW + qx(q)] == kFluid) {
+                const unsigned ub = us + (unsigned)(qy(q) * a.P + qx(q));
+                alt[q] = PP ? a.hq_in[qopp(q)][ub]
+                            : a.h_in[(unsigned)qopp(q) * upl + ub];
+            }
+        } else {
+            alt[q] = PP ? a.hq_in[q][us] : a.h_in[(unsigned)q * upl + us];
+        }
+    }
 }
 
 // (6) of the step: new density rho(t+1) = sum_q f*_q(x - e_q) (half-way bounce-back where the
@@ -376,8 +416,9 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid,
         const T* hb = a.h_in + us;
         // PP: rows of the sources with e_q,y = 0, +1, -1
         const unsigned r0 = us, rdn = us - uP, rup = us + uP;
-        T g[9];
-        g[0] = PP ? __ldg(a.hq_in[0] + r0) : __ldg(hb);
+        T g[9], D[9], alt[9];
+        if (MIXED && IBB) ibb_gather<T, RW, PP>(a, us, o, s_flag, D, alt);
+        g[0] = PP ? a.hq_in[0][r0] : *hb;
         T A = mul_rn(qw<T>(0), rho);  // sum_q w_q rho(x - e_q); bounce-back sources take rho(x)
         T dm = (T)0;                  // interpolated bounce-back: mass returned to the rest population
 #pragma unroll
@@ -385,16 +426,16 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid,
             const int os = o - qy(q) * RW - qx(q);
             if (!MIXED || s_flag[os] == kFluid) {
                 const T rs = s_rho[os];
-                const T h = PP ? __ldg(a.hq_in[q] + (int)((qy(q) > 0 ? rdn : qy(q) < 0 ? rup : r0) -
-                                                          qx(q)))
-                               : __ldg(hb + (int)QSRC(q));
+                const T h = PP ? *(a.hq_in[q] + (int)((qy(q) > 0 ? rdn : qy(q) < 0 ? rup : r0) -
+                                                      qx(q)))
+                               : *(hb + (int)QSRC(q));
                 g[q] = fma_rn(qw<T>(q), sub_rn(rs, rho), h);
                 A = fma_rn(qw<T>(q), rs, A);
             } else {
-                const T out = PP ? __ldg(a.hq_in[qopp(q)] + r0) : __ldg(hb + (int)QPL(qopp(q)));
+                const T out = PP ? a.hq_in[qopp(q)][r0] : *(hb + (int)QPL(qopp(q)));
                 g[q] = out;
                 if (MIXED && IBB) {
-                    g[q] = ibb_return<T, RW, PP>(a, q, us, o, rho, out, s_rho, s_flag);
+                    g[q] = ibb_return<T, RW>(q, o, rho, out, D[q], alt[q], s_rho, s_flag);
                     dm = add_rn(dm, sub_rn(out, g[q]));
                 }
                 A = fma_rn(qw<T>(q), rho, A);
@@ -427,33 +468,57 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid,
 #undef QSRC
 }
 
-// (1) density and flags on x0-8 .. x0+TX+7, y0-7 .. y0+TY+6, four nodes per access; the pads
-// supply periodic images and wall rows, positions past the padded plane read as solid. Returns,
-// in the thread's bits: 1 if it saw a non-fluid node, 2 if it saw a fluid node of the tile.
+// Programmatic dependent launch (no effect without its launch attribute): the next step's blocks
+// may be placed while this grid drains, and wait for it here before they touch what it writes.
+// What the previous step wrote (density, populations) is read with plain loads: a read-only load
+// (__ldg) promises that the data does not change during the kernel, and the compiler may then move it
+// above the wait.
+__device__ __forceinline__ void pdl_launch_next() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// (1) node classes and density on x0-8 .. x0+TX+7, y0-7 .. y0+TY+6, four nodes per access; the
+// pads supply periodic images and wall rows, positions past the padded plane read as solid.
+// Every load of a thread is issued before its first store, so the tile waits for one memory
+// latency; the classes do not change between steps and are loaded before the wait for the
+// previous step. Returns, in the thread's bits: 1 if it saw a non-fluid node, 2 if it saw a
+// fluid node of the tile.
 template <typename T, int TX, int TY, int NT>
 __device__ __forceinline__ int stage_load(const StepArgs<T>& a, T* s_rho, uint8_t* s_flag, int x0,
                                           int y0) {
     using L = Layout<T, TX, TY>;
-    constexpr int RW = L::RW, RH = L::RH;
-    constexpr int NV = RW / 4;
-    int any = 0;
-    for (int v = threadIdx.x; v < NV * RH; v += NT) {
-        const int r = v / NV, c4 = v - r * NV;
+    constexpr int RW = L::RW, RH = L::RH, NV = RW / 4, K = (NV * RH + NT - 1) / NT;
+    int e[K];  // element of the first node, -1 outside the plane
+    uint32_t fl[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int v = threadIdx.x + k * NT, r = v / NV, c4 = v - r * NV;
         const int gy = y0 - 7 + r, gx = x0 - 8 + 4 * c4;
-        T* sr = s_rho + r * RW + 4 * c4;
-        uint32_t fl = 0x03030303u;
-        if (gy >= -kPadY && gy < a.ny + kPadY && gx < a.nx + kPadX) {
-            const int e = lidx(a.P, gx, gy);
-            load4(a.rho_in + e, sr);
-            fl = __ldg(reinterpret_cast<const unsigned int*>(a.flags + e));
-        } else {
-            sr[0] = sr[1] = sr[2] = sr[3] = (T)0;
-        }
-        *reinterpret_cast<uint32_t*>(s_flag + r * RW + 4 * c4) = fl;
-        any |= fl != 0u ? 1 : 0;
+        const bool in = r < RH && gy >= -kPadY && gy < a.ny + kPadY && gx < a.nx + kPadX;
+        e[k] = in ? lidx(a.P, gx, gy) : -1;
+        fl[k] = in ? __ldg(reinterpret_cast<const unsigned int*>(a.flags + e[k])) : 0x03030303u;
+    }
+    pdl_wait_previous();
+    V4<T> d[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        d[k] = V4<T>{};
+        if (e[k] >= 0) d[k].load(a.rho_in + e[k]);
+    }
+    int any = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int v = threadIdx.x + k * NT, r = v / NV, c4 = v - r * NV;
+        if (r >= RH) continue;
+        d[k].store(s_rho + r * RW + 4 * c4);
+        *reinterpret_cast<uint32_t*>(s_flag + r * RW + 4 * c4) = fl[k];
+        any |= fl[k] != 0u ? 1 : 0;
         // a zero byte (fluid) among the four, inside the tile proper
         const bool inside = r >= 7 && r < 7 + TY && c4 >= 2 && c4 < 2 + TX / 4;
-        if (inside && ((fl - 0x01010101u) & ~fl & 0x80808080u)) any |= 2;
+        if (inside && ((fl[k] - 0x01010101u) & ~fl[k] & 0x80808080u)) any |= 2;
     }
     return any;
 }
@@ -483,6 +548,7 @@ __device__ __forceinline__ void step_tile(const StepArgs<T>& a, const T rho_mid,
 template <typename T, int TX, int TY, int NT, bool MACRO, int MINB, bool IBB = false>
 __global__ void __launch_bounds__(NT, MINB) k_step(const StepArgs<T> a, const T rho_mid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_launch_next();
     step_tile<T, TX, TY, NT, MACRO, true, IBB>(a, rho_mid, smem_raw, blockIdx.x * TX,
                                                blockIdx.y * TY);
 }
