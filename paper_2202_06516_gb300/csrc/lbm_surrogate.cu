@@ -103,20 +103,53 @@ __global__ void k_im2col(const bf16* x1, int C1, int up1, const bf16* x2, int C2
     }
 }
 
-__global__ void k_avgpool(const bf16* x, bf16* y, int B, int H, int W, int C) {
-    const int h = H / 2, w = W / 2;
-    const long long total = (long long)B * h * w * C;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
+// 2 x 2 average pool, eight channels per thread (16-byte accesses; C / 8 = 2^lc8). Bound by its 10
+// bytes per output element of traffic; one channel per thread with 64-bit index divisions took 36 us
+// on the 32-channel 256 x 256 x 8 map (42 MB).
+__global__ void __launch_bounds__(kT)
+    k_avgpool(const bf16* x, bf16* y, long long n8, int H, int W, int lc8) {
+    const int h = H / 2, w = W / 2, C = 8 << lc8;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n8;
          t += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(t % C);
-        const long long q = t / C;
-        const int X = (int)(q % w), Y = (int)((q / w) % h), n = (int)(q / ((long long)w * h));
-        const size_t b = (((size_t)n * H + 2 * Y) * W + 2 * X) * C + c;
-        const float s = __bfloat162float(x[b]) + __bfloat162float(x[b + C]) +
-                        __bfloat162float(x[b + (size_t)W * C]) +
-                        __bfloat162float(x[b + (size_t)W * C + C]);
-        y[t] = __float2bfloat16_rn(0.25f * s);
+        const int c = (int)(t & ((1 << lc8) - 1)) * 8;
+        const int q = (int)(t >> lc8), X = q % w, r = q / w, Y = r % h, n = r / h;
+        const bf16* src = x + (((size_t)n * H + 2 * Y) * W + 2 * X) * C + c;
+        const uint4 v[4] = {__ldg(reinterpret_cast<const uint4*>(src)),
+                            __ldg(reinterpret_cast<const uint4*>(src + C)),
+                            __ldg(reinterpret_cast<const uint4*>(src + (size_t)W * C)),
+                            __ldg(reinterpret_cast<const uint4*>(src + (size_t)W * C + C))};
+        uint4 out;
+        __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(&out);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float2 f = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&v[k])[i]);
+                s.x = k ? s.x + f.x : f.x;
+                s.y = k ? s.y + f.y : f.y;
+            }
+            o[i] = __floats2bfloat162_rn(0.25f * s.x, 0.25f * s.y);
+        }
+        reinterpret_cast<uint4*>(y)[t] = out;
     }
+}
+
+// Number of non-zero bytes of the loss mask, added to *cnt (integer atomics: exact)
+__global__ void __launch_bounds__(kT) k_mask_count(const uint8_t* mask, long long n, int* cnt) {
+    int c = 0;
+    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    const long long n16 = ((uintptr_t)mask & 15) == 0 ? n / 16 : 0;
+    for (long long t = t0; t < n16; t += stride) {
+        const uint4 v = reinterpret_cast<const uint4*>(mask)[t];
+        c += __popc(__vcmpne4(v.x, 0u)) + __popc(__vcmpne4(v.y, 0u)) + __popc(__vcmpne4(v.z, 0u)) +
+             __popc(__vcmpne4(v.w, 0u));
+    }
+    c /= 8;
+    for (long long t = 16 * n16 + t0; t < n; t += stride) c += mask[t] != 0;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(cnt, c);
 }
 
 // The leaky-ReLU adjoint of one convolution's output fused with what feeds it and what reads
@@ -124,20 +157,33 @@ __global__ void k_avgpool(const bf16* x, bf16* y, int B, int H, int W, int C) {
 // (POOL) is the gradient of the 2 x 2 average pool taken of this output, whose adjoint gives a
 // quarter to each of the four source pixels (added after the other consumers' contributions,
 // as a separate pass would); and the per-block column sums of the stored g (the bias gradient's
-// partials). Thread t always covers the eight channels 8 t mod C (8 x threads per block is a
+// partials). MODE 2: dy is the head's, the product of the pixel's dz and the head weight hw[c], formed
+// here instead of being written and read as a tensor. Thread t always covers the eight channels 8 t mod C (8 x threads per block is a
 // multiple of C), so each block adds its threads' sums per channel in thread order into
 // part[c][block] (deterministic). H, W: the output resolution (even when POOL).
-template <bool POOL>
-__global__ void k_relu_bias(const float* dy, const float* dyp, const bf16* y, bf16* g,
-                            long long n8, int C, int H, int W, float* part) {
+// MODE 0: dy alone, 1: with the pool's gradient (POOL), 2: dy[p] hw[c].
+template <int MODE>
+__global__ void k_relu_bias(const float* dy, const float* dyp, const float* hw, const bf16* y,
+                            bf16* g, long long n8, int C, int H, int W, float* part) {
+    constexpr bool POOL = MODE == 1;
     __shared__ float sred[kT * 8];
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n8;
          t += (long long)gridDim.x * blockDim.x) {
         const uint4 yv = reinterpret_cast<const uint4*>(y)[t];
-        const float4 a = reinterpret_cast<const float4*>(dy)[2 * t];
-        const float4 b = reinterpret_cast<const float4*>(dy)[2 * t + 1];
-        float d[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        float d[8];
+        if (MODE == 2) {
+            const long long e = 8 * t, p = e / C;
+            const int c = (int)(e - p * C);
+            const float dz = dy[p];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) d[j] = dz * __ldg(hw + c + j);
+        } else {
+            const float4 a = reinterpret_cast<const float4*>(dy)[2 * t];
+            const float4 b = reinterpret_cast<const float4*>(dy)[2 * t + 1];
+            d[0] = a.x, d[1] = a.y, d[2] = a.z, d[3] = a.w;
+            d[4] = b.x, d[5] = b.y, d[6] = b.z, d[7] = b.w;
+        }
         if (POOL) {
             const long long e = 8 * t, p = e / C;
             const int c = (int)(e - p * C);
@@ -195,17 +241,20 @@ __global__ void k_colsum_final(const float* part, int nb, int C, float* out, int
 }
 
 // head: phi = sigmoid(sum_c x[p][c] w[c] + b); with targets, also the loss terms and the
-// gradient: dz = 2 m (phi - t) phi (1 - phi) / n_mask, dx[p][c] = dz w[c]; per-block partial sums
-// of loss, dz * x[p][c] (weight gradient) and dz (bias gradient) for a deterministic reduction.
+// gradient: dz = 2 m (phi - t) phi (1 - phi) / n_mask (the input's gradient is dz w[c], formed by
+// the pass that reads it); per-block partial sums of loss, dz * x[p][c] (weight gradient) and dz
+// (bias gradient) for a deterministic reduction. n_mask: the device's count of loss pixels.
 template <int C>
 __global__ void k_head(const bf16* x, const float* w, const float* bptr, float* phi, long long P,
-                       const float* target, const uint8_t* mask, float inv_n, float* dx,
+                       const float* target, const uint8_t* mask, const int* n_mask, float* dzp,
                        float* part /* per block: C + 2 */) {
     __shared__ float sw[C];
     __shared__ float red[kT / 32][C + 2];
     for (int c = threadIdx.x; c < C; c += blockDim.x) sw[c] = w[c];
     __syncthreads();
     const float b = *bptr;
+    const int cnt = target ? *n_mask : 0;
+    const float inv_n = cnt > 0 ? 1.f / (float)cnt : 0.f;
     float acc[C + 2];
 #pragma unroll
     for (int c = 0; c < C + 2; ++c) acc[c] = 0.f;
@@ -237,10 +286,7 @@ __global__ void k_head(const bf16* x, const float* w, const float* bptr, float* 
             acc[C + 1] += dz;
 #pragma unroll
             for (int c = 0; c < C; ++c) acc[c] += dz * xv[c];
-#pragma unroll
-            for (int c = 0; c < C; c += 4)
-                reinterpret_cast<float4*>(dx + p * C)[c / 4] =
-                    make_float4(dz * sw[c], dz * sw[c + 1], dz * sw[c + 2], dz * sw[c + 3]);
+            dzp[p] = dz;
         }
     }
     if (!target) return;
@@ -369,10 +415,13 @@ struct lbm_surrogate {
     float* part = nullptr;  // reduction partials
     float* phi = nullptr;   // head output
     float* hpart = nullptr;
+    float* dz = nullptr;      // head: gradient with respect to the pre-sigmoid value, per pixel
+    int* n_mask = nullptr;    // loss pixels of the current step
+    float* host_loss = nullptr;  // pinned
     float* bpart = nullptr;   // per-block column sums of the bias gradients
     float* splitk = nullptr;  // split-K partials of the weight gradient
     size_t splitk_elems = 0;
-    int part_blocks = 256;
+    int part_blocks = 608;  // head: two resident waves of two blocks per SM
     ConvTable tab{};  // convolution weight shapes for the BF16 copies
     long long adam_t = 0;
     std::string err;
@@ -893,8 +942,9 @@ lbm_status forward(lbm_surrogate* s, const bf16* x, int B) {
         for (const auto& pl : s->pools)
             if (pl.first == c.out) {
                 const Tensor& src = s->t[pl.first];
-                k_avgpool<<<blocks_for((long long)B * src.H * src.W * src.C / 4), kT, 0,
-                            s->stream>>>(src.y, s->t[pl.second].y, B, src.H, src.W, src.C);
+                const long long n8 = (long long)B * src.H * src.W / 4 * (src.C / 8);
+                k_avgpool<<<blocks_for(n8), kT, 0, s->stream>>>(src.y, s->t[pl.second].y, n8, src.H,
+                                                                src.W, ilog2_exact(src.C / 8));
             }
     }
     return LBM_OK;
@@ -1049,6 +1099,9 @@ lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->gmask, s->act_elems * sizeof(bf16));
     if (e == cudaSuccess)
         e = cudaMalloc((void**)&s->part, (size_t)s->part_blocks * 8 * base * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->dz, (size_t)max_batch * H * W * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->n_mask, sizeof(int));
+    if (e == cudaSuccess) e = cudaHostAlloc((void**)&s->host_loss, sizeof(float), cudaHostAllocDefault);
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->phi, (size_t)max_batch * H * W * sizeof(float));
     if (e == cudaSuccess)
         e = cudaMalloc((void**)&s->hpart, (size_t)s->part_blocks * (base + 2) * sizeof(float));
@@ -1105,15 +1158,15 @@ lbm_status lbm_surrogate_forward(lbm_surrogate* s, const void* x, int32_t B, flo
     const int nb = std::min(s->part_blocks, blocks_for(P));
     if (s->base == 32)
         k_head<32><<<nb, kT, 0, s->stream>>>(s->t[s->head_in].y, s->w + s->head_w,
-                                             s->w + s->head_b, phi_out, P, nullptr, nullptr, 0.f,
+                                             s->w + s->head_b, phi_out, P, nullptr, nullptr, nullptr,
                                              nullptr, nullptr);
     else if (s->base == 8)
         k_head<8><<<nb, kT, 0, s->stream>>>(s->t[s->head_in].y, s->w + s->head_w,
-                                            s->w + s->head_b, phi_out, P, nullptr, nullptr, 0.f,
+                                            s->w + s->head_b, phi_out, P, nullptr, nullptr, nullptr,
                                             nullptr, nullptr);
     else if (s->base == 16)
         k_head<16><<<nb, kT, 0, s->stream>>>(s->t[s->head_in].y, s->w + s->head_w,
-                                             s->w + s->head_b, phi_out, P, nullptr, nullptr, 0.f,
+                                             s->w + s->head_b, phi_out, P, nullptr, nullptr, nullptr,
                                              nullptr, nullptr);
     else
         return sfail(s, LBM_ERR_ARG, "lbm_surrogate_forward: base must be 8, 16 or 32");
@@ -1134,35 +1187,24 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
     lbm_status st = forward(s, (const bf16*)xin, B);
     if (st != LBM_OK) return st;
     const long long P = (long long)B * s->H * s->W;
-    std::vector<uint8_t> hm;
-    // zero all activation gradients (they accumulate from several consumers)
-    for (size_t k = 1; k < s->t.size(); ++k) {
-        const Tensor& x = s->t[k];
-        SCUDA(s, cudaMemsetAsync(x.dy, 0, (size_t)B * x.H * x.W * x.C * sizeof(float), s->stream));
-    }
-    SCUDA(s, cudaMemsetAsync(s->g, 0, s->nparams * sizeof(float), s->stream));
-    float inv_n = 1.f / (float)P;
-    {
-        // number of loss pixels: the mask (B*H*W bytes) is counted on the host once per step
-        hm.resize((size_t)P);
-        SCUDA(s, cudaMemcpyAsync(hm.data(), mask, (size_t)P, cudaMemcpyDeviceToHost, s->stream));
-        SCUDA(s, cudaStreamSynchronize(s->stream));
-        long long cnt = 0;
-        for (uint8_t b : hm) cnt += b != 0;
-        inv_n = cnt > 0 ? 1.f / (float)cnt : 0.f;
-    }
+    // Everything below is queued without waiting for the device. Activation gradients need no
+    // zero fill: the first consumer's data gradient stores, a further one would accumulate.
+    SCUDA(s, cudaMemsetAsync(s->n_mask, 0, sizeof(int), s->stream));
+    k_mask_count<<<(int)std::min<long long>(152, blocks_for(P / 16 + 1)), kT, 0, s->stream>>>(
+        mask, P, s->n_mask);
+    std::vector<char> written(s->t.size(), 0);
     const int C = s->base;
     const int nb = std::min(s->part_blocks, blocks_for(P));
-    Tensor& hin = s->t[s->head_in];
+    const Tensor& hin = s->t[s->head_in];
     if (C == 32)
         k_head<32><<<nb, kT, 0, s->stream>>>(hin.y, s->w + s->head_w, s->w + s->head_b, s->phi, P,
-                                             target, mask, inv_n, hin.dy, s->hpart);
+                                             target, mask, s->n_mask, s->dz, s->hpart);
     else if (C == 16)
         k_head<16><<<nb, kT, 0, s->stream>>>(hin.y, s->w + s->head_w, s->w + s->head_b, s->phi, P,
-                                             target, mask, inv_n, hin.dy, s->hpart);
+                                             target, mask, s->n_mask, s->dz, s->hpart);
     else if (C == 8)
         k_head<8><<<nb, kT, 0, s->stream>>>(hin.y, s->w + s->head_w, s->w + s->head_b, s->phi, P,
-                                            target, mask, inv_n, hin.dy, s->hpart);
+                                            target, mask, s->n_mask, s->dz, s->hpart);
     else
         return sfail(s, LBM_ERR_ARG, "lbm_surrogate_train_step: base must be 8, 16 or 32");
     SCUDA(s, cudaGetLastError());
@@ -1172,8 +1214,8 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
                              cudaMemcpyDeviceToDevice, s->stream));
     SCUDA(s, cudaMemcpyAsync(s->g + s->head_b, s->part + C + 1, sizeof(float),
                              cudaMemcpyDeviceToDevice, s->stream));
-    float hl = 0.f;
-    SCUDA(s, cudaMemcpyAsync(&hl, s->part + C, sizeof(float), cudaMemcpyDeviceToHost, s->stream));
+    SCUDA(s, cudaMemcpyAsync(s->host_loss, s->part + C, sizeof(float), cudaMemcpyDeviceToHost,
+                             s->stream));
     // backward through the convolutions (reverse order), pools interleaved
     for (int ci = (int)s->convs.size() - 1; ci >= 0; --ci) {
         const Conv& c = s->convs[ci];
@@ -1188,12 +1230,15 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         const long long n_out = Pc * c.Cout;
         // leaky-ReLU adjoint (with the pool's), BF16 copy and the bias gradient's partial sums
         const int rb = (int)std::min<long long>(kReluBlocks, (n_out / 8 + kT - 1) / kT);
-        if (dyp)
-            k_relu_bias<true><<<rb, kT, 0, s->stream>>>(o.dy, dyp, o.y, s->gmask, n_out / 8,
-                                                        c.Cout, c.H, c.W, s->bpart);
+        if (c.out == s->head_in)
+            k_relu_bias<2><<<rb, kT, 0, s->stream>>>(s->dz, nullptr, s->w + s->head_w, o.y, s->gmask,
+                                                     n_out / 8, c.Cout, c.H, c.W, s->bpart);
+        else if (dyp)
+            k_relu_bias<1><<<rb, kT, 0, s->stream>>>(o.dy, dyp, nullptr, o.y, s->gmask, n_out / 8,
+                                                     c.Cout, c.H, c.W, s->bpart);
         else
-            k_relu_bias<false><<<rb, kT, 0, s->stream>>>(o.dy, nullptr, o.y, s->gmask, n_out / 8,
-                                                         c.Cout, c.H, c.W, s->bpart);
+            k_relu_bias<0><<<rb, kT, 0, s->stream>>>(o.dy, nullptr, nullptr, o.y, s->gmask,
+                                                     n_out / 8, c.Cout, c.H, c.W, s->bpart);
         k_colsum_final<<<c.Cout, kT, 0, s->stream>>>(s->bpart, rb, c.Cout, s->g + c.b_off, 1);
         // weight gradient: dW[co][k] = sum_p g[p][co] col[p][k], the im2col columns gathered by
         // the GEMM's loader when the resolution allows (powers of two), else from a buffer
@@ -1239,7 +1284,15 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         gd.K = (c.up1 ? 36 : 9) * c.Cout;
         gd.Cf = s->t[c.src1].dy;
         gd.ldc = c.C1;
-        gd.accumulate = 1;
+        if (c.C2 > 0 && written[c.src1] != written[c.src2]) {
+            const int fresh = written[c.src1] ? c.src2 : c.src1;
+            const Tensor& x = s->t[fresh];
+            SCUDA(s, cudaMemsetAsync(x.dy, 0, (size_t)B * x.H * x.W * x.C * sizeof(float), s->stream));
+            written[fresh] = 1;
+        }
+        gd.accumulate = written[c.src1];
+        written[c.src1] = 1;
+        if (c.src2 >= 0) written[c.src2] = 1;
         if (c.C2 > 0) {
             gd.Cf2 = s->t[c.src2].dy;
             gd.ldc2 = c.C2;
@@ -1264,7 +1317,7 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
     SCUDA(s, cudaStreamSynchronize(s->stream));
     if (tc_timed_out())
         return sfail(s, LBM_ERR_TIMEOUT, "lbm_surrogate_train_step: a tensor-core wait timed out");
-    if (loss) *loss = hl;
+    if (loss) *loss = *s->host_loss;
     return LBM_OK;
 }
 
@@ -1344,6 +1397,9 @@ void lbm_surrogate_destroy(lbm_surrogate* s) {
     cudaFree(s->part);
     cudaFree(s->phi);
     cudaFree(s->hpart);
+    cudaFree(s->dz);
+    cudaFree(s->n_mask);
+    if (s->host_loss) cudaFreeHost(s->host_loss);
     cudaFree(s->splitk);
     cudaFree(s->bpart);
     if (s->stream) cudaStreamDestroy(s->stream);
