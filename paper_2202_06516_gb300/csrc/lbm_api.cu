@@ -179,7 +179,8 @@ void free_all(lbm_ctx* c) {
     cudaFree(c->flags);
     cudaFree(c->linkmask);
     cudaFree(c->dlt);
-    c->dlt = nullptr;
+    cudaFree(c->scratch64);
+    c->dlt = c->scratch64 = nullptr;
     cudaFree(c->red_partials);
     cudaFree(c->meas_partials);
     cudaFree(c->aux);
@@ -380,6 +381,7 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
     }
     if (e == cudaSuccess) e = cudaMalloc(&c->muw, c->plane * esz);
     if (e == cudaSuccess) e = cudaMalloc((void**)&c->flags, c->plane);
+    if (e == cudaSuccess && esz == 8) e = cudaMalloc(&c->scratch64, lbm::step64_scratch_bytes(c->plane));
     if (e == cudaSuccess) e = cudaMalloc((void**)&c->linkmask, c->plane);
     if (e == cudaSuccess) e = cudaMalloc(&c->red_partials, lbm::reduce_partial_bytes(c->red_blocks));
     if (e == cudaSuccess) e = cudaMalloc(&c->meas_partials, lbm::meas_partial_bytes(c->meas_blocks));

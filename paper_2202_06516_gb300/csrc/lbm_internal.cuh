@@ -122,6 +122,7 @@ struct lbm_ctx {
     uint8_t* linkmask = nullptr;   // per node, bit q-1 set when fluid x has a solid x + e_q
     void* dlt = nullptr;           // 8 planes of link fractions (interpolated bounce-back)
     bool ibb = false;
+    void* scratch64 = nullptr;     // FP64 lattices: scratch planes of the step
     int cur = 0;
     bool has_geometry = false;
     int64_t steps = 0;
@@ -164,6 +165,8 @@ cudaError_t launch_geometry(lbm_ctx* c, const GeomArgs& g);
 cudaError_t launch_link_fractions(lbm_ctx* c, const GeomArgs& g);
 cudaError_t launch_init_state(lbm_ctx* c, const lbm_geometry& g, const double* d_rho0);
 cudaError_t launch_step(lbm_ctx* c, int src, bool macro);
+cudaError_t launch_step64(lbm_ctx* c, const StepArgs<double>& a, bool macro);
+size_t step64_scratch_bytes(size_t plane);
 size_t step_smem_bytes(int tile_x, int tile_y, size_t esz, int min_blocks);
 struct StepVariant {
     int tile_x, tile_y, min_blocks;

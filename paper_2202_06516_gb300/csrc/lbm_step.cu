@@ -27,11 +27,11 @@ namespace {
 
 using namespace stepdev;
 
-// the interpolated bounce-back kernels exist for the default variants only (32 x 16 tiles,
-// 5 CTAs per SM in FP32, unconstrained in FP64) and the small-lattice forms of the FP32 one
+// the interpolated bounce-back kernels exist for the default variant (32 x 16 tiles, 5 CTAs per SM)
+// and its small-lattice forms
 template <typename T, int TX, int TY, int MINB>
 constexpr bool has_ibb() {
-    return TX == 32 && TY == 16 && MINB == (sizeof(T) == 4 ? 5 : 1);
+    return TX == 32 && TY == 16 && MINB == 5;
 }
 
 // Launch with programmatic stream serialization: a step's launch, block placement and class staging
@@ -87,7 +87,7 @@ cudaError_t configure_one() {
         if (e == cudaSuccess) e = allow_smem<T, TX, TY, 256, MINB, false, true>();
         if (e == cudaSuccess) e = allow_smem<T, TX, TY, 256, MINB, true, true>();
     }
-    if constexpr (sizeof(T) == 4 && TX == 32 && TY == 16 && MINB == 5) {
+    if constexpr (has_ibb<T, TX, TY, MINB>()) {
 #define X(F, A, B, N, M)                                                       \
     if (e == cudaSuccess) e = allow_smem<float, A, B, N, M, false, false>();   \
     if (e == cudaSuccess) e = allow_smem<float, A, B, N, M, false, true>();
@@ -99,7 +99,7 @@ cudaError_t configure_one() {
 
 template <typename T, int TX, int TY, int MINB>
 cudaError_t launch_one(lbm_ctx* c, const StepArgs<T>& a, bool macro) {
-    if constexpr (sizeof(T) == 4 && TX == 32 && TY == 16 && MINB == 5) {
+    if constexpr (has_ibb<T, TX, TY, MINB>()) {
         const int form = macro ? 0 : small_form(c);
 #define X(F, A, B, N, M)                                                       \
     if (form == F)                                                             \
@@ -160,7 +160,8 @@ StepArgs<T> make_args(lbm_ctx* c, int src) {
 }  // namespace
 
 // Supported step-kernel variants: tile (TX, TY) and the minimum resident CTAs per SM the
-// compiler is asked to fit (register budget); min_blocks 0 = no constraint.
+// compiler is asked to fit (register budget); min_blocks 0 = no constraint. FP64 lattices step
+// with the kernels of lbm_step64.cu, which have no tiles: both names select them.
 #define LBM_STEP_VARIANTS(X)                                     \
     X(float, 32, 8, 1) X(float, 32, 8, 6) X(float, 32, 16, 1)    \
     X(float, 32, 16, 5) X(float, 32, 16, 6) X(float, 64, 16, 1)  \
@@ -190,32 +191,25 @@ void step_variants(size_t esz, std::vector<StepVariant>* out) {
 }
 
 cudaError_t step_configure(lbm_ctx* c) {
-#define X(T, A, B, M) \
-    if (c->esz == sizeof(T) && c->tile_x == A && c->tile_y == B && minb_of(c) == M) \
-        return configure_one<T, A, B, M>();
+#define X(T, A, B, M)                                                                       \
+    if (c->esz == sizeof(T) && c->tile_x == A && c->tile_y == B && minb_of(c) == M) {       \
+        if constexpr (sizeof(T) == 4) return configure_one<T, A, B, M>();                   \
+        return cudaSuccess;                                                                 \
+    }
     LBM_STEP_VARIANTS(X)
 #undef X
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_step(lbm_ctx* c, int src, bool macro) {
-    if (c->esz == 4) {
-        const StepArgs<float> a = make_args<float>(c, src);
+    if (c->esz == 8) return launch_step64(c, make_args<double>(c, src), macro);
+    const StepArgs<float> a = make_args<float>(c, src);
 #define X(T, A, B, M)                                                                 \
     if constexpr (sizeof(T) == 4)                                                     \
         if (c->tile_x == A && c->tile_y == B && minb_of(c) == M)                      \
             return launch_one<float, A, B, M>(c, a, macro);
-        LBM_STEP_VARIANTS(X)
+    LBM_STEP_VARIANTS(X)
 #undef X
-    } else {
-        const StepArgs<double> a = make_args<double>(c, src);
-#define X(T, A, B, M)                                                                 \
-    if constexpr (sizeof(T) == 8)                                                     \
-        if (c->tile_x == A && c->tile_y == B && minb_of(c) == M)                      \
-            return launch_one<double, A, B, M>(c, a, macro);
-        LBM_STEP_VARIANTS(X)
-#undef X
-    }
     return cudaErrorInvalidValue;
 }
 

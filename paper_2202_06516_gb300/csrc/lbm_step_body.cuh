@@ -1,6 +1,6 @@
 // Device code of the fused multiphase LBM time step, shared by the single-lattice kernel
-// (lbm_step.cu) and the batched multi-lattice kernel (lbm_batch.cu). See lbm_step.cu for the
-// storage scheme and the stage structure.
+// (lbm_step.cu) and the batched multi-lattice kernel (lbm_batch.cu); the collision also serves the
+// FP64 step (lbm_step64.cu). See lbm_step.cu for the storage scheme and the stage structure.
 #pragma once
 
 #include <math.h>
@@ -25,7 +25,7 @@ __device__ __forceinline__ double fma_rn(double x, double y, double z) { return 
 // Bulk chemical potential psi'(rho) at k = 1: Eq. 11 without the gradient term (PR), or the CS
 // counterpart from Eq. 9 with the ideal-gas antiderivative. The FP32 path uses the hardware
 // logarithm and approximate division (relative error ~1e-6 on psi', far below the FP32 noise
-// of the force); the FP64 path keeps correctly rounded operations.
+// of the force).
 template <typename T>
 __device__ __forceinline__ T psi_prime(T rho, const StepArgs<T>& a);
 
@@ -52,23 +52,6 @@ __device__ __forceinline__ float psi_prime<float>(float rho, const StepArgs<floa
     const float num = mul_rn(n, fma_rn(fma_rn(3.0f, n, -9.0f), n, 8.0f));  // 8n - 9n^2 + 3n^3
     return fma_rn(a.RT, add_rn(__logf(rho), __fdividef(num, mul_rn(mul_rn(om, om), om))),
                   mul_rn(-2.0f * a.aal, rho));
-}
-
-template <>
-__device__ __forceinline__ double psi_prime<double>(double rho, const StepArgs<double>& a) {
-    if (a.eos == LBM_EOS_PR) {
-        const double br = a.b * rho;
-        const double s2 = 1.4142135623730951;
-        const double t1 = a.RT * log(rho / (1.0 - br));
-        const double t2 = a.aal / (2.0 * s2 * a.b) * log((s2 - 1.0 + br) / (s2 + 1.0 - br));
-        const double t3 = a.RT / (1.0 - br);
-        const double t4 = a.aal * rho / (1.0 + 2.0 * br - br * br);
-        return t1 - t2 + t3 - t4;
-    }
-    const double n = a.b * rho * 0.25;
-    const double om = 1.0 - n;
-    return a.RT * (log(rho) + (8.0 * n - 9.0 * n * n + 3.0 * n * n * n) / (om * om * om)) -
-           2.0 * a.aal * rho;
 }
 
 // correctly rounded reciprocal (hardware approximation plus refinement in FP32)
@@ -180,19 +163,6 @@ struct V4<float> {
     }
     __device__ __forceinline__ void store(float* s) const { *reinterpret_cast<float4*>(s) = v; }
 };
-template <>
-struct V4<double> {
-    double2 v, w;
-    __device__ __forceinline__ void load(const double* g) {
-        v = *reinterpret_cast<const double2*>(g);
-        w = *reinterpret_cast<const double2*>(g + 2);
-    }
-    __device__ __forceinline__ void store(double* s) const {
-        *reinterpret_cast<double2*>(s) = v;
-        *reinterpret_cast<double2*>(s + 2) = w;
-    }
-};
-
 template <typename T, int RW>
 __device__ __forceinline__ T mu_fluid(const T* s_rho, int o, const StepArgs<T>& a) {
     const T c0 = s_rho[o];
