@@ -77,6 +77,8 @@ __device__ __forceinline__ void pix_split(int p, const PixDims& d, int& n, int& 
 template <bool P2>
 __global__ void k_im2col(const bf16* x1, int C1, int up1, const bf16* x2, int C2, PixDims d,
                          int P, int lc8, bf16* col) {
+    pdl_next();
+    pdl_wait();
     const int C8 = 1 << lc8;
     const long long total = (long long)P * 9 * C8;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
@@ -108,16 +110,18 @@ __global__ void k_im2col(const bf16* x1, int C1, int up1, const bf16* x2, int C2
 // on the 32-channel 256 x 256 x 8 map (42 MB).
 __global__ void __launch_bounds__(kT)
     k_avgpool(const bf16* x, bf16* y, long long n8, int H, int W, int lc8) {
+    pdl_next();
+    pdl_wait();
     const int h = H / 2, w = W / 2, C = 8 << lc8;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n8;
          t += (long long)gridDim.x * blockDim.x) {
         const int c = (int)(t & ((1 << lc8) - 1)) * 8;
         const int q = (int)(t >> lc8), X = q % w, r = q / w, Y = r % h, n = r / h;
         const bf16* src = x + (((size_t)n * H + 2 * Y) * W + 2 * X) * C + c;
-        const uint4 v[4] = {__ldg(reinterpret_cast<const uint4*>(src)),
-                            __ldg(reinterpret_cast<const uint4*>(src + C)),
-                            __ldg(reinterpret_cast<const uint4*>(src + (size_t)W * C)),
-                            __ldg(reinterpret_cast<const uint4*>(src + (size_t)W * C + C))};
+        const uint4 v[4] = {*reinterpret_cast<const uint4*>(src),
+                            *reinterpret_cast<const uint4*>(src + C),
+                            *reinterpret_cast<const uint4*>(src + (size_t)W * C),
+                            *reinterpret_cast<const uint4*>(src + (size_t)W * C + C)};
         uint4 out;
         __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(&out);
 #pragma unroll
@@ -137,6 +141,8 @@ __global__ void __launch_bounds__(kT)
 
 // Number of non-zero bytes of the loss mask, added to *cnt (integer atomics: exact)
 __global__ void __launch_bounds__(kT) k_mask_count(const uint8_t* mask, long long n, int* cnt) {
+    pdl_next();
+    pdl_wait();
     int c = 0;
     const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -165,6 +171,8 @@ __global__ void __launch_bounds__(kT) k_mask_count(const uint8_t* mask, long lon
 template <int MODE>
 __global__ void k_relu_bias(const float* dy, const float* dyp, const float* hw, const bf16* y,
                             bf16* g, long long n8, int C, int H, int W, float* part) {
+    pdl_next();
+    pdl_wait();
     constexpr bool POOL = MODE == 1;
     __shared__ float sred[kT * 8];
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -177,7 +185,7 @@ __global__ void k_relu_bias(const float* dy, const float* dyp, const float* hw, 
             const int c = (int)(e - p * C);
             const float dz = dy[p];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) d[j] = dz * __ldg(hw + c + j);
+            for (int j = 0; j < 8; ++j) d[j] = dz * hw[c + j];
         } else {
             const float4 a = reinterpret_cast<const float4*>(dy)[2 * t];
             const float4 b = reinterpret_cast<const float4*>(dy)[2 * t + 1];
@@ -224,8 +232,13 @@ __global__ void k_relu_bias(const float* dy, const float* dyp, const float* hw, 
 }
 
 // out[c] = sum over b of the partials of column c: part[b * C + c], or part[c * nb + b] when
-// transposed; one block per column, a fixed-shape tree in shared memory (deterministic)
-__global__ void k_colsum_final(const float* part, int nb, int C, float* out, int transposed = 0) {
+// transposed; one block per column, a fixed-shape tree in shared memory (deterministic). loss (the
+// head's sums: weights, loss, bias): the last but one column goes to *loss and the last takes its
+// place in out.
+__global__ void k_colsum_final(const float* part, int nb, int C, float* out, int transposed,
+                               float* loss) {
+    pdl_next();
+    pdl_wait();
     __shared__ float sm[kT];
     const int c = blockIdx.x;
     float s = 0.f;
@@ -237,7 +250,11 @@ __global__ void k_colsum_final(const float* part, int nb, int C, float* out, int
         if (threadIdx.x < h) sm[threadIdx.x] += sm[threadIdx.x + h];
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[c] = sm[0];
+    if (threadIdx.x != 0) return;
+    if (loss && c == C - 2)
+        *loss = sm[0];
+    else
+        out[loss && c == C - 1 ? c - 1 : c] = sm[0];
 }
 
 // head: phi = sigmoid(sum_c x[p][c] w[c] + b); with targets, also the loss terms and the
@@ -248,6 +265,8 @@ template <int C>
 __global__ void k_head(const bf16* x, const float* w, const float* bptr, float* phi, long long P,
                        const float* target, const uint8_t* mask, const int* n_mask, float* dzp,
                        float* part /* per block: C + 2 */) {
+    pdl_next();
+    pdl_wait();
     __shared__ float sw[C];
     __shared__ float red[kT / 32][C + 2];
     for (int c = threadIdx.x; c < C; c += blockDim.x) sw[c] = w[c];
@@ -337,6 +356,8 @@ __device__ __forceinline__ void store_bf16_copies(long long t, float x, bf16* wb
 __global__ void k_adam(float* w, const float* g, float* m, float* v, long long n, float lr,
                        float b1, float b2, float eps, float c1, float c2, bf16* wb, bf16* wd,
                        const ConvTable tab) {
+    pdl_next();
+    pdl_wait();
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
          t += (long long)gridDim.x * blockDim.x) {
         const float gi = g[t];
@@ -384,6 +405,11 @@ struct Conv {
     // source 2 likewise, and the weights as 32 x N-tile blocks
     int fw_cb = 0, fw_bn = 0, dw_cb = 0, dw_bn = 0;
     CUtensorMap fwmap[3] = {}, dwmap[3] = {};
+    // training: gradient with respect to the pre-activation (BF16), the bias gradient's per-block
+    // sums, and the event after which the side stream may read them
+    bf16* g = nullptr;
+    float* bpart = nullptr;
+    cudaEvent_t ready = nullptr;
 };
 
 struct Tensor {
@@ -400,7 +426,10 @@ using namespace lbm::sg;
 
 struct lbm_surrogate {
     int H = 0, W = 0, base = 0, maxB = 0, device = 0;
-    cudaStream_t stream = nullptr;
+    // main stream, and a side stream for the weight and bias gradients of the backward pass, which
+    // nothing in the chain of data gradients waits for
+    cudaStream_t stream = nullptr, side = nullptr;
+    cudaEvent_t head_ready = nullptr, side_done = nullptr;
     std::vector<Tensor> t;      // 0: input (8 channels)
     std::vector<Conv> convs;
     std::vector<std::pair<int, int>> pools;  // (from, to)
@@ -410,16 +439,14 @@ struct lbm_surrogate {
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     bf16* wb = nullptr;
     bf16* wbd = nullptr;        // per convolution [C_in][tap][C_out] (data-gradient operand)
-    bf16 *col = nullptr, *gmask = nullptr;
-    size_t col_elems = 0, act_elems = 0;
-    float* part = nullptr;  // reduction partials
+    bf16* col = nullptr;
+    size_t col_elems = 0;
     float* phi = nullptr;   // head output
     float* hpart = nullptr;
     float* dz = nullptr;      // head: gradient with respect to the pre-sigmoid value, per pixel
     int* n_mask = nullptr;    // loss pixels of the current step
-    float* host_loss = nullptr;  // pinned
-    float* bpart = nullptr;   // per-block column sums of the bias gradients
-    float* splitk = nullptr;  // split-K partials of the weight gradient
+    float *host_loss = nullptr, *host_loss_dev = nullptr;  // mapped host memory
+    float *splitk = nullptr, *splitk_side = nullptr;  // split-K partials, one per stream
     size_t splitk_elems = 0;
     int part_blocks = 608;  // head: two resident waves of two blocks per SM
     ConvTable tab{};  // convolution weight shapes for the BF16 copies
@@ -507,9 +534,8 @@ cudaError_t launch_tc(cudaStream_t st, const GemmArgs& a, int splits,
     dim3 grid((a.N + BN - 1) / BN, (a.M + lbm::sgtc::BM - 1) / lbm::sgtc::BM, splits);
     static const CUtensorMap none[3] = {};
     const CUtensorMap* m = maps ? maps : none;
-    lbm::sgtc::k_gemm_tc<BN, STAGES, AMN, BMN, GA, GD, GAM, TMA>
-        <<<grid, lbm::sgtc::TC_THREADS, TS::SMEM_BYTES, st>>>(a, flag, m[0], m[1], m[2]);
-    return cudaGetLastError();
+    return launch_pdl(lbm::sgtc::k_gemm_tc<BN, STAGES, AMN, BMN, GA, GD, GAM, TMA>, grid,
+                      lbm::sgtc::TC_THREADS, TS::SMEM_BYTES, st, a, flag, m[0], m[1], m[2]);
 }
 
 // C = A B on the tcgen05 tensor cores, each operand K-major or MN-major (AMN, BMN). The N tile
@@ -654,10 +680,9 @@ cudaError_t gemm_tc_split(cudaStream_t st, const GemmArgs& a, float* scratch,
     cudaError_t e = ks ? gemm_tc_tma<GA, GD>(st, p, nsp, maps, ks)
                        : gemm_tc<false, false, GA, GD>(st, p, nsp);
     if (e != cudaSuccess) return e;
-    k_splitk_finish<<<blocks_for((long long)a.M * a.N / 4), kT, 0, st>>>(
-        scratch, nsp, a.M, a.N, a.bias, a.relu, a.Cb, a.Cf, a.ldc, a.Cf2, a.ldc2, a.nsplit,
-        a.accumulate);
-    return cudaGetLastError();
+    return launch_pdl(k_splitk_finish, dim3(blocks_for((long long)a.M * a.N / 4)), kT, 0, st, scratch,
+                      nsp, a.M, a.N, a.bias, a.relu, a.Cb, a.Cf, a.ldc, a.Cf2, a.ldc2, a.nsplit,
+                      a.accumulate);
 }
 
 // AK / BK: operand stored K-major (else MN-major)
@@ -705,8 +730,8 @@ cudaError_t launch_wwin(cudaStream_t st, const GemmArgs& a, int splits, const CU
     }
     int* flag = tc_flag().dev;
     if (!flag) return cudaErrorMemoryAllocation;
-    kern<<<splits, lbm::sgtc::TC_THREADS, SMEM, st>>>(a, flag, maps[0], maps[1], maps[2]);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(splits), lbm::sgtc::TC_THREADS, SMEM, st, a, flag, maps[0], maps[1],
+                      maps[2]);
 }
 
 // Launch of k_gemm_fwin: one CTA per tile of 128 pixels x BN columns.
@@ -729,8 +754,8 @@ cudaError_t launch_fwin(cudaStream_t st, const GemmArgs& a, const CUtensorMap* m
     int* flag = tc_flag().dev;
     if (!flag) return cudaErrorMemoryAllocation;
     dim3 grid(a.N / BN, a.M / lbm::sgtc::BM);
-    kern<<<grid, lbm::sgtc::TC_THREADS, SMEM, st>>>(a, flag, maps[0], maps[1], maps[2]);
-    return cudaGetLastError();
+    return launch_pdl(kern, grid, lbm::sgtc::TC_THREADS, SMEM, st, a, flag, maps[0], maps[1],
+                      maps[2]);
 }
 
 // The window-fed forward (GD false) or data gradient of a convolution that qualifies (see
@@ -741,6 +766,15 @@ cudaError_t gemm_fwin(cudaStream_t st, const GemmArgs& a, int cb, int bn, const 
     if (cb == 1 && bn == 32) return launch_fwin<32, 1, GD>(st, a, maps);
     if (cb == 1 && bn == 64) return launch_fwin<64, 1, GD>(st, a, maps);
     return cudaErrorInvalidValue;
+}
+
+// out = the sum of `splits` FP32 partials of `stride` values each, in split order
+cudaError_t sum_splits(cudaStream_t st, const float* part, int splits, long long stride, float* out) {
+    if (stride % 4 == 0 && ((uintptr_t)out & 15) == 0)
+        return launch_pdl(k_splitk_sum4, dim3((unsigned)((stride / 4 + 31) / 32)), 256, 0, st, part,
+                          splits, stride, stride, out);
+    return launch_pdl(k_splitk_sum, dim3(blocks_for(stride)), kT, 0, st, part, splits, stride, stride,
+                      out);
 }
 
 // The weight gradient through k_gemm_wwin (a: the transposed, gathered form of gemm_wgrad):
@@ -762,12 +796,7 @@ cudaError_t gemm_wgrad_window(cudaStream_t st, GemmArgs a, float* scratch, size_
     if (a.N == 64 && cb == 1) e = launch_wwin<64, 1>(st, a, splits, maps);
     if (a.N == 64 && cb == 2) e = launch_wwin<64, 2>(st, a, splits, maps);
     if (e != cudaSuccess || splits == 1) return e;
-    if (stride % 4 == 0 && ((uintptr_t)out & 15) == 0)
-        k_splitk_sum4<<<(unsigned)((stride / 4 + 31) / 32), 256, 0, st>>>(scratch, splits, stride,
-                                                                          stride, out);
-    else
-        k_splitk_sum<<<blocks_for(stride), kT, 0, st>>>(scratch, splits, stride, stride, out);
-    return cudaGetLastError();
+    return sum_splits(st, scratch, splits, stride, out);
 }
 
 cudaError_t gemm_wgrad(cudaStream_t st, GemmArgs a, float* scratch, size_t scratch_elems,
@@ -809,12 +838,7 @@ cudaError_t gemm_wgrad(cudaStream_t st, GemmArgs a, float* scratch, size_t scrat
                     : gather ? gemm_tc<true, true, false, false, true>(st, a, splits)
                              : gemm_tc<true, true>(st, a, splits);
     if (e != cudaSuccess) return e;
-    if (stride % 4 == 0 && ((uintptr_t)out & 15) == 0)
-        k_splitk_sum4<<<(unsigned)((stride / 4 + 31) / 32), 256, 0, st>>>(scratch, splits, stride,
-                                                                          stride, out);
-    else
-        k_splitk_sum<<<blocks_for(stride), kT, 0, st>>>(scratch, splits, stride, stride, out);
-    return cudaGetLastError();
+    return sum_splits(st, scratch, splits, stride, out);
 }
 
 // BF16 copies of the weights (after the FP32 masters changed): W for the forward pass and the
@@ -834,20 +858,15 @@ int ilog2_exact(int v) {
 PixDims pix_dims(int H, int W) { return PixDims{H, W, ilog2_exact(H), ilog2_exact(W)}; }
 
 // im2col of convolution c (channel groups of 8, a power of two, checked at creation)
-cudaError_t launch_im2col(lbm_surrogate* s, const Conv& c, int B) {
+cudaError_t launch_im2col(lbm_surrogate* s, cudaStream_t st, const Conv& c, int B) {
     const bf16* x1 = s->t[c.src1].y;
     const bf16* x2 = c.src2 >= 0 ? s->t[c.src2].y : nullptr;
     const PixDims d = pix_dims(c.H, c.W);
     const int P = B * c.H * c.W;
     const int lc8 = ilog2_exact((c.C1 + c.C2) / 8);
     const long long total = (long long)P * 9 * ((c.C1 + c.C2) / 8);
-    if (d.lh >= 0 && d.lw >= 0)
-        k_im2col<true><<<blocks_for(total), kT, 0, s->stream>>>(x1, c.C1, c.up1, x2, c.C2, d, P,
-                                                                lc8, s->col);
-    else
-        k_im2col<false><<<blocks_for(total), kT, 0, s->stream>>>(x1, c.C1, c.up1, x2, c.C2, d, P,
-                                                                 lc8, s->col);
-    return cudaGetLastError();
+    return launch_pdl(d.lh >= 0 && d.lw >= 0 ? k_im2col<true> : k_im2col<false>,
+                      dim3(blocks_for(total)), kT, 0, st, x1, c.C1, c.up1, x2, c.C2, d, P, lc8, s->col);
 }
 
 int add_tensor(lbm_surrogate* s, int H, int W, int C) {
@@ -904,6 +923,14 @@ void build(lbm_surrogate* s) {
     s->nparams += 1;
 }
 
+// the head on the last activation; with a target (training) also its loss terms and gradients
+cudaError_t launch_head(lbm_surrogate* s, int blocks, float* phi, long long P, const float* target,
+                        const uint8_t* mask) {
+    auto* k = s->base == 32 ? k_head<32> : s->base == 16 ? k_head<16> : k_head<8>;
+    return launch_pdl(k, dim3(blocks), kT, 0, s->stream, s->t[s->head_in].y, s->w + s->head_w,
+                      s->w + s->head_b, phi, P, target, mask, s->n_mask, s->dz, s->hpart);
+}
+
 lbm_status forward(lbm_surrogate* s, const bf16* x, int B) {
     s->t[0].y = const_cast<bf16*>(x);
     // convolutions run in production order; a pool runs right after the conv that feeds it
@@ -943,8 +970,8 @@ lbm_status forward(lbm_surrogate* s, const bf16* x, int B) {
             if (pl.first == c.out) {
                 const Tensor& src = s->t[pl.first];
                 const long long n8 = (long long)B * src.H * src.W / 4 * (src.C / 8);
-                k_avgpool<<<blocks_for(n8), kT, 0, s->stream>>>(src.y, s->t[pl.second].y, n8, src.H,
-                                                                src.W, ilog2_exact(src.C / 8));
+                SCUDA(s, launch_pdl(k_avgpool, dim3(blocks_for(n8)), kT, 0, s->stream, src.y,
+                                    s->t[pl.second].y, n8, src.H, src.W, ilog2_exact(src.C / 8)));
             }
     }
     return LBM_OK;
@@ -977,7 +1004,7 @@ void make_tensor_maps(lbm_surrogate* s) {
             if ((Ws % 128 == 0 || 128 % Ws == 0) && (Hs * Ws) % 128 == 0 && dk &&
                 (9 * c.Cout) % dk == 0 && tma_width(pick_bn(cin))) {
                 const int bw = std::min(Ws, 128), bh = 128 / bw;
-                if (map_nhwc(&c.dmap[0], s->gmask, c.Cout, W, H, s->maxB, bw, bh, dk, 2) &&
+                if (map_nhwc(&c.dmap[0], c.g, c.Cout, W, H, s->maxB, bw, bh, dk, 2) &&
                     map_rows(&c.dmap[2], s->wbd + c.w_off, 9 * c.Cout, cin, pick_bn(cin), dk))
                     c.d_ks = dk;
             }
@@ -986,7 +1013,7 @@ void make_tensor_maps(lbm_surrogate* s) {
             if (W % 64 == 0 && c.C2 == 0 && c.C1 % 32 == 0 && c.Cout % 32 == 0 &&
                 tma_width(pick_bn(c.Cout)))
                 c.w_tma = map_nhwc(&c.wmap[0], s->t[c.src1].y, c.C1, Ws, Hs, s->maxB, 32, 1, 32) &&
-                          map_nhwc(&c.wmap[2], s->gmask, c.Cout, W, H, s->maxB, 32, 1, 32, 2);
+                          map_nhwc(&c.wmap[2], c.g, c.Cout, W, H, s->maxB, 32, 1, 32, 2);
             continue;
         }
         if (!((W % 128 == 0 || 128 % W == 0) && (H * W) % 128 == 0) || c.src1 == 0)
@@ -1011,7 +1038,7 @@ void make_tensor_maps(lbm_surrogate* s) {
                 c.fw_bn = c.Cout;
             }
             if (c.Cout == 32 && c.C1 % 32 == 0 && c.C2 % 32 == 0 && (cin == 32 || cin == 64) &&
-                map_nhwc(&c.dwmap[0], s->gmask, c.Cout, W, H, s->maxB, 136, 3, 32) &&
+                map_nhwc(&c.dwmap[0], c.g, c.Cout, W, H, s->maxB, 136, 3, 32) &&
                 map_rows(&c.dwmap[2], s->wbd + c.w_off, 9 * c.Cout, cin, cin, 32)) {
                 c.dw_cb = 1;
                 c.dw_bn = cin;
@@ -1023,7 +1050,7 @@ void make_tensor_maps(lbm_surrogate* s) {
             if (map_nhwc(&c.wwmap[0], s->t[c.src1].y, c.C1, W, H, s->maxB, 72, 3, 32) &&
                 (c.src2 < 0 ||
                  map_nhwc(&c.wwmap[1], s->t[c.src2].y, c.C2, W, H, s->maxB, 72, 3, 32)) &&
-                map_nhwc(&c.wwmap[2], s->gmask, c.Cout, W, H, s->maxB, 64, 1, 32))
+                map_nhwc(&c.wwmap[2], c.g, c.Cout, W, H, s->maxB, 64, 1, 32))
                 c.ww_cb = wc;
         }
         if (W % 64 == 0 || 64 % W == 0) {
@@ -1033,10 +1060,10 @@ void make_tensor_maps(lbm_surrogate* s) {
                       map_nhwc(&c.wmap[0], s->t[c.src1].y, c.C1, W, H, s->maxB, ww, wh, 32) &&
                       (c.src2 < 0 ||
                        map_nhwc(&c.wmap[1], s->t[c.src2].y, c.C2, W, H, s->maxB, ww, wh, 32)) &&
-                      map_nhwc(&c.wmap[2], s->gmask, c.Cout, W, H, s->maxB, ww, wh, 32);
+                      map_nhwc(&c.wmap[2], c.g, c.Cout, W, H, s->maxB, ww, wh, 32);
         }
         if (dk && tma_width(pick_bn(cin)) &&
-            map_nhwc(&c.dmap[0], s->gmask, c.Cout, W, H, s->maxB, bw, bh, dk) &&
+            map_nhwc(&c.dmap[0], c.g, c.Cout, W, H, s->maxB, bw, bh, dk) &&
             map_rows(&c.dmap[2], s->wbd + c.w_off, 9 * c.Cout, cin, pick_bn(cin), dk))
             c.d_ks = dk;
     }
@@ -1076,6 +1103,7 @@ lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_
         return sfail(nullptr, LBM_ERR_CUDA, std::string("lbm_surrogate_create: ") + e);
     };
     cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cleanup(cudaGetErrorString(e));
     size_t colmax = 0;
     for (const Conv& c : s->convs)
@@ -1086,7 +1114,6 @@ lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_
         const size_t n = (size_t)max_batch * x.H * x.W * x.C;
         e = cudaMalloc((void**)&x.y, n * sizeof(bf16));
         if (e == cudaSuccess) e = cudaMalloc((void**)&x.dy, n * sizeof(float));
-        s->act_elems = std::max(s->act_elems, n);
     }
     const size_t np = s->nparams;
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->w, np * sizeof(float));
@@ -1096,21 +1123,27 @@ lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->wb, np * sizeof(bf16));
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->wbd, np * sizeof(bf16));
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->col, colmax * sizeof(bf16));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->gmask, s->act_elems * sizeof(bf16));
-    if (e == cudaSuccess)
-        e = cudaMalloc((void**)&s->part, (size_t)s->part_blocks * 8 * base * sizeof(float));
+    for (Conv& c : s->convs) {
+        if (e == cudaSuccess)
+            e = cudaMalloc((void**)&c.g, (size_t)max_batch * c.H * c.W * c.Cout * sizeof(bf16));
+        if (e == cudaSuccess)
+            e = cudaMalloc((void**)&c.bpart, (size_t)kReluBlocks * c.Cout * sizeof(float));
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.ready, cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->head_ready, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->side_done, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->dz, (size_t)max_batch * H * W * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->n_mask, sizeof(int));
-    if (e == cudaSuccess) e = cudaHostAlloc((void**)&s->host_loss, sizeof(float), cudaHostAllocDefault);
+    if (e == cudaSuccess) e = cudaHostAlloc((void**)&s->host_loss, sizeof(float), cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&s->host_loss_dev, s->host_loss, 0);
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->phi, (size_t)max_batch * H * W * sizeof(float));
     if (e == cudaSuccess)
         e = cudaMalloc((void**)&s->hpart, (size_t)s->part_blocks * (base + 2) * sizeof(float));
-    if (e == cudaSuccess)
-        e = cudaMalloc((void**)&s->bpart, (size_t)kReluBlocks * 8 * base * sizeof(float));
     size_t wmax = 0;
     for (const Conv& c : s->convs) wmax = std::max(wmax, (size_t)c.Cout * 9 * (c.C1 + c.C2));
     s->splitk_elems = std::min<size_t>(wmax * 128, (size_t)64 << 20);
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->splitk, s->splitk_elems * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->splitk_side, s->splitk_elems * sizeof(float));
     if (e == cudaSuccess) e = cudaMemsetAsync(s->w, 0, np * sizeof(float), s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->m, 0, np * sizeof(float), s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->v, 0, np * sizeof(float), s->stream);
@@ -1156,21 +1189,7 @@ lbm_status lbm_surrogate_forward(lbm_surrogate* s, const void* x, int32_t B, flo
     if (st != LBM_OK) return st;
     const long long P = (long long)B * s->H * s->W;
     const int nb = std::min(s->part_blocks, blocks_for(P));
-    if (s->base == 32)
-        k_head<32><<<nb, kT, 0, s->stream>>>(s->t[s->head_in].y, s->w + s->head_w,
-                                             s->w + s->head_b, phi_out, P, nullptr, nullptr, nullptr,
-                                             nullptr, nullptr);
-    else if (s->base == 8)
-        k_head<8><<<nb, kT, 0, s->stream>>>(s->t[s->head_in].y, s->w + s->head_w,
-                                            s->w + s->head_b, phi_out, P, nullptr, nullptr, nullptr,
-                                            nullptr, nullptr);
-    else if (s->base == 16)
-        k_head<16><<<nb, kT, 0, s->stream>>>(s->t[s->head_in].y, s->w + s->head_w,
-                                             s->w + s->head_b, phi_out, P, nullptr, nullptr, nullptr,
-                                             nullptr, nullptr);
-    else
-        return sfail(s, LBM_ERR_ARG, "lbm_surrogate_forward: base must be 8, 16 or 32");
-    SCUDA(s, cudaGetLastError());
+    SCUDA(s, launch_head(s, nb, phi_out, P, nullptr, nullptr));
     SCUDA(s, cudaStreamSynchronize(s->stream));
     if (tc_timed_out())
         return sfail(s, LBM_ERR_TIMEOUT, "lbm_surrogate_forward: a tensor-core wait timed out");
@@ -1190,32 +1209,17 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
     // Everything below is queued without waiting for the device. Activation gradients need no
     // zero fill: the first consumer's data gradient stores, a further one would accumulate.
     SCUDA(s, cudaMemsetAsync(s->n_mask, 0, sizeof(int), s->stream));
-    k_mask_count<<<(int)std::min<long long>(152, blocks_for(P / 16 + 1)), kT, 0, s->stream>>>(
-        mask, P, s->n_mask);
+    SCUDA(s, launch_pdl(k_mask_count, dim3((unsigned)std::min<long long>(152, blocks_for(P / 16 + 1))),
+                        kT, 0, s->stream, mask, P, s->n_mask));
     std::vector<char> written(s->t.size(), 0);
     const int C = s->base;
     const int nb = std::min(s->part_blocks, blocks_for(P));
-    const Tensor& hin = s->t[s->head_in];
-    if (C == 32)
-        k_head<32><<<nb, kT, 0, s->stream>>>(hin.y, s->w + s->head_w, s->w + s->head_b, s->phi, P,
-                                             target, mask, s->n_mask, s->dz, s->hpart);
-    else if (C == 16)
-        k_head<16><<<nb, kT, 0, s->stream>>>(hin.y, s->w + s->head_w, s->w + s->head_b, s->phi, P,
-                                             target, mask, s->n_mask, s->dz, s->hpart);
-    else if (C == 8)
-        k_head<8><<<nb, kT, 0, s->stream>>>(hin.y, s->w + s->head_w, s->w + s->head_b, s->phi, P,
-                                            target, mask, s->n_mask, s->dz, s->hpart);
-    else
-        return sfail(s, LBM_ERR_ARG, "lbm_surrogate_train_step: base must be 8, 16 or 32");
-    SCUDA(s, cudaGetLastError());
-    // head gradients: sum the per-block partials (C weights, loss, bias)
-    k_colsum_final<<<C + 2, kT, 0, s->stream>>>(s->hpart, nb, C + 2, s->part);
-    SCUDA(s, cudaMemcpyAsync(s->g + s->head_w, s->part, C * sizeof(float),
-                             cudaMemcpyDeviceToDevice, s->stream));
-    SCUDA(s, cudaMemcpyAsync(s->g + s->head_b, s->part + C + 1, sizeof(float),
-                             cudaMemcpyDeviceToDevice, s->stream));
-    SCUDA(s, cudaMemcpyAsync(s->host_loss, s->part + C, sizeof(float), cudaMemcpyDeviceToHost,
-                             s->stream));
+    SCUDA(s, launch_head(s, nb, s->phi, P, target, mask));
+    // head gradients and loss: sums of the per-block partials (C weights, loss, bias)
+    SCUDA(s, cudaEventRecord(s->head_ready, s->stream));
+    SCUDA(s, cudaStreamWaitEvent(s->side, s->head_ready, 0));
+    SCUDA(s, launch_pdl(k_colsum_final, dim3(C + 2), kT, 0, s->side, s->hpart, nb, C + 2,
+                        s->g + s->head_w, 0, s->host_loss_dev));
     // backward through the convolutions (reverse order), pools interleaved
     for (int ci = (int)s->convs.size() - 1; ci >= 0; --ci) {
         const Conv& c = s->convs[ci];
@@ -1231,15 +1235,16 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         // leaky-ReLU adjoint (with the pool's), BF16 copy and the bias gradient's partial sums
         const int rb = (int)std::min<long long>(kReluBlocks, (n_out / 8 + kT - 1) / kT);
         if (c.out == s->head_in)
-            k_relu_bias<2><<<rb, kT, 0, s->stream>>>(s->dz, nullptr, s->w + s->head_w, o.y, s->gmask,
-                                                     n_out / 8, c.Cout, c.H, c.W, s->bpart);
-        else if (dyp)
-            k_relu_bias<1><<<rb, kT, 0, s->stream>>>(o.dy, dyp, nullptr, o.y, s->gmask, n_out / 8,
-                                                     c.Cout, c.H, c.W, s->bpart);
+            SCUDA(s, launch_pdl(k_relu_bias<2>, dim3(rb), kT, 0, s->stream, s->dz, nullptr,
+                                s->w + s->head_w, o.y, c.g, n_out / 8, c.Cout, c.H, c.W, c.bpart));
         else
-            k_relu_bias<0><<<rb, kT, 0, s->stream>>>(o.dy, nullptr, nullptr, o.y, s->gmask,
-                                                     n_out / 8, c.Cout, c.H, c.W, s->bpart);
-        k_colsum_final<<<c.Cout, kT, 0, s->stream>>>(s->bpart, rb, c.Cout, s->g + c.b_off, 1);
+            SCUDA(s, launch_pdl(dyp ? k_relu_bias<1> : k_relu_bias<0>, dim3(rb), kT, 0, s->stream,
+                                o.dy, dyp, nullptr, o.y, c.g, n_out / 8, c.Cout, c.H, c.W, c.bpart));
+        // the side stream takes the bias and weight gradients from here
+        SCUDA(s, cudaEventRecord(c.ready, s->stream));
+        SCUDA(s, cudaStreamWaitEvent(s->side, c.ready, 0));
+        SCUDA(s, launch_pdl(k_colsum_final, dim3(c.Cout), kT, 0, s->side, c.bpart, rb, c.Cout,
+                            s->g + c.b_off, 1, nullptr));
         // weight gradient: dW[co][k] = sum_p g[p][co] col[p][k], the im2col columns gathered by
         // the GEMM's loader when the resolution allows (powers of two), else from a buffer
         GemmArgs gw{};
@@ -1254,8 +1259,8 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         gw.conv.lh = ilog2_exact(c.H);
         gw.conv.lw = ilog2_exact(c.W);
         const bool gather = gw.conv.lh >= 0 && gw.conv.lw >= 0;
-        if (!gather) SCUDA(s, launch_im2col(s, c, B));
-        gw.A = s->gmask;
+        if (!gather) SCUDA(s, launch_im2col(s, s->side, c, B));
+        gw.A = c.g;
         gw.B = s->col;
         gw.M = c.Cout;
         gw.N = 9 * Cin;
@@ -1263,7 +1268,7 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         gw.lda = c.Cout;
         gw.ldb = 9 * Cin;
         gw.ldc = 9 * Cin;
-        SCUDA(s, gemm_wgrad(s->stream, gw, s->splitk, s->splitk_elems, s->g + c.w_off, gather,
+        SCUDA(s, gemm_wgrad(s->side, gw, s->splitk_side, s->splitk_elems, s->g + c.w_off, gather,
                             gather && c.w_tma ? c.wmap : nullptr, gather ? c.ww_cb : 0, c.wwmap));
         // data gradient (not needed for the input tensor)
         if (c.src1 == 0) continue;
@@ -1271,7 +1276,7 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         // of dY gathered around q times the rearranged weights (no column buffer)
         if (c.up1 && c.C2 > 0) return sfail(s, LBM_ERR_STATE, "surrogate: upsampled cat source");
         GemmArgs gd{};
-        gd.dg.dy = s->gmask;
+        gd.dg.dy = c.g;
         gd.dg.H = c.H;
         gd.dg.W = c.W;
         gd.dg.lco = ilog2_exact(c.Cout);
@@ -1304,16 +1309,17 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
             SCUDA(s, (gemm_tc_split<false, true>(s->stream, gd, s->splitk, s->splitk_elems,
                                                   c.dmap, c.d_ks)));
     }
+    SCUDA(s, cudaEventRecord(s->side_done, s->side));
+    SCUDA(s, cudaStreamWaitEvent(s->stream, s->side_done, 0));
     if (lr > 0.f) {
         ++s->adam_t;
         const float b1 = 0.9f, b2 = 0.999f;
         const float c1 = 1.f / (1.f - powf(b1, (float)s->adam_t));
         const float c2 = 1.f / (1.f - powf(b2, (float)s->adam_t));
-        k_adam<<<blocks_for((long long)s->nparams), kT, 0, s->stream>>>(
-            s->w, s->g, s->m, s->v, (long long)s->nparams, lr, b1, b2, 1e-8f, c1, c2, s->wb, s->wbd,
-            s->tab);
+        SCUDA(s, launch_pdl(k_adam, dim3(blocks_for((long long)s->nparams)), kT, 0, s->stream, s->w,
+                            s->g, s->m, s->v, (long long)s->nparams, lr, b1, b2, 1e-8f, c1, c2, s->wb,
+                            s->wbd, s->tab));
     }
-    SCUDA(s, cudaGetLastError());
     SCUDA(s, cudaStreamSynchronize(s->stream));
     if (tc_timed_out())
         return sfail(s, LBM_ERR_TIMEOUT, "lbm_surrogate_train_step: a tensor-core wait timed out");
@@ -1382,6 +1388,14 @@ lbm_status lbm_sg_inject_timeout(void) {
 void lbm_surrogate_destroy(lbm_surrogate* s) {
     if (!s) return;
     if (s->stream) cudaStreamSynchronize(s->stream);
+    if (s->side) cudaStreamSynchronize(s->side);
+    for (Conv& c : s->convs) {
+        cudaFree(c.g);
+        cudaFree(c.bpart);
+        if (c.ready) cudaEventDestroy(c.ready);
+    }
+    if (s->head_ready) cudaEventDestroy(s->head_ready);
+    if (s->side_done) cudaEventDestroy(s->side_done);
     for (size_t k = 1; k < s->t.size(); ++k) {
         cudaFree(s->t[k].y);
         cudaFree(s->t[k].dy);
@@ -1393,16 +1407,15 @@ void lbm_surrogate_destroy(lbm_surrogate* s) {
     cudaFree(s->wb);
     cudaFree(s->wbd);
     cudaFree(s->col);
-    cudaFree(s->gmask);
-    cudaFree(s->part);
     cudaFree(s->phi);
     cudaFree(s->hpart);
     cudaFree(s->dz);
     cudaFree(s->n_mask);
     if (s->host_loss) cudaFreeHost(s->host_loss);
     cudaFree(s->splitk);
-    cudaFree(s->bpart);
+    cudaFree(s->splitk_side);
     if (s->stream) cudaStreamDestroy(s->stream);
+    if (s->side) cudaStreamDestroy(s->side);
     delete s;
 }
 

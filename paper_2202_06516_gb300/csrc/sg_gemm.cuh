@@ -7,10 +7,38 @@
 #pragma once
 
 #include <cuda_bf16.h>
+#include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace lbm {
 namespace sg {
+
+// Programmatic dependent launch: a kernel launched with the attribute may be placed while the kernel
+// before it in the stream drains, and waits here before it reads or writes anything that kernel
+// or an earlier one touches (each kernel of the network waits, so the order is transitive). A
+// kernel that holds tensor memory lets the next one start only after its own allocation, and
+// allocates only after this wait, so that a kernel never waits for columns of one that waits
+// for it. Data of earlier kernels is read with plain loads (never through the read-only path).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                       A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
 
 // A operand gathered straight from NHWC activations (implicit im2col of a 3 x 3, pad-1
 // convolution): A[p][(ky * 3 + kx) * C + c] = x(n, y + ky - 1, x + kx - 1, c) for output pixel
@@ -91,6 +119,8 @@ namespace sg {
 // sum of the split-K partials in split order (deterministic): out[i] = sum_z part[z * stride + i]
 __global__ void k_splitk_sum(const float* part, int splits, long long stride, long long n,
                              float* out) {
+    pdl_next();
+    pdl_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         float s = 0.f;
@@ -105,6 +135,8 @@ __global__ void k_splitk_sum(const float* part, int splits, long long stride, lo
 // (deterministic: the grouping does not depend on the launch).
 __global__ void k_splitk_sum4(const float* part, int splits, long long stride, long long n,
                               float* out) {
+    pdl_next();
+    pdl_wait();
     __shared__ float4 sm[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long i = blockIdx.x * 32LL + lane, n4 = n / 4;
@@ -138,6 +170,8 @@ __global__ void k_splitk_sum4(const float* part, int splits, long long stride, l
 __global__ void k_splitk_finish(const float* part, int splits, int M, int N, const float* bias,
                                 int relu, __nv_bfloat16* Cb, float* Cf, int ldc, float* Cf2,
                                 int ldc2, int nsplit, int accumulate) {
+    pdl_next();
+    pdl_wait();
     const long long stride = (long long)M * N, n4 = stride / 4;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4;
          i += (long long)gridDim.x * blockDim.x) {

@@ -513,6 +513,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int ke = g.kchunk ? min(g.K, kb + g.kchunk) : g.K;
     const int nk = ke > kb ? (ke - kb + KS - 1) / KS : 0;
 
+    sg::pdl_wait();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                          su32(tmem_slot)),
@@ -528,6 +529,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    sg::pdl_next();
     const uint32_t tmem = *tmem_slot;
     constexpr uint32_t IDESC = idesc_bf16(BM, BN, AMN ? 1 : 0, BMN ? 1 : 0);
 
@@ -819,6 +821,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int kb = blockIdx.x * g.kchunk, ke = min(g.K, kb + g.kchunk);
     const int nk = ke > kb ? (ke - kb) / 64 : 0;
+    sg::pdl_wait();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                          su32(tmem_slot)),
@@ -834,6 +837,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    sg::pdl_next();
     const uint32_t tmem = *tmem_slot;
     constexpr uint32_t IDESC = idesc_bf16(BM, BN, 1, 1);
     const int H = g.conv.H, W = g.conv.W;
@@ -960,6 +964,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __shared__ int s_ok;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    sg::pdl_wait();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                          su32(tmem_slot)),
@@ -976,6 +981,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    sg::pdl_next();
     const uint32_t tmem = *tmem_slot;
     constexpr uint32_t IDESC = idesc_bf16(BM, BN, 0, 0);
     const int H = GD ? g.dg.H : g.conv.H, W = GD ? g.dg.W : g.conv.W;
