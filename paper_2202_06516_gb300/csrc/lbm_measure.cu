@@ -241,21 +241,16 @@ __device__ __forceinline__ double substrate_dist(const Substrate& s, double px, 
     return __dsub_rn(py, -0.5);
 }
 
-// Candidate links of node n (fluid) into the four running bests (side * 2 + target). PRE: points
-// whose FP32 distance is more than a quarter outside the band are dropped before the FP64
-// construction (coordinates and radii up to 10^6: the FP32 distance errs by less than 0.2).
+// Bit sl: the link of fluid node (i, j) along slot sl joins liquid and gas and its point may lie in
+// the measurement's band. PRE: points whose FP32 distance is more than a quarter outside the band
+// are dropped here (coordinates and radii up to 10^6: the FP32 distance errs by less than 0.2).
 template <typename T, bool PRE>
-__device__ __forceinline__ bool scan_node(const T* rho, const uint8_t* flags, int nx, int ny, int P,
-                                          double rho_m, T thr, const Substrate& sub, double qxc,
-                                          double qyc, long long n, Best (&b)[4]) {
-    const int j = (int)n / nx, i = (int)n - j * nx;  // fewer than 2^31 nodes
-    T vb[4];
-    const T va = rho[lidx(P, i, j)];
-    const unsigned ok = link_ends<T>(rho, flags, nx, ny, P, i, j, vb);
-    bool any = false;
+__device__ __forceinline__ unsigned crossing_links(T va, const T (&vb)[4], unsigned ends, double rho_m,
+                                                   T thr, const Substrate& sub, int i, int j) {
+    unsigned m = 0;
 #pragma unroll
     for (int sl = 0; sl < 4; ++sl) {
-        if (!(ok >> sl & 1) || (va > thr) == (vb[sl] > thr)) continue;
+        if (!(ends >> sl & 1) || (va > thr) == (vb[sl] > thr)) continue;
         if (PRE) {
             const float a = (float)va, fr = __fdividef((float)rho_m - a, (float)vb[sl] - a);
             const float x = i + fr * slot_x(sl), y = j + fr * slot_y(sl);
@@ -267,31 +262,39 @@ __device__ __forceinline__ bool scan_node(const T* rho, const uint8_t* flags, in
             }
             if (d < 0.25f || d > 2.75f) continue;
         }
-        double px, py;
-        if (!link_point<T>(va, vb[sl], rho_m, thr, i, j, sl, px, py)) continue;
-        const double d = substrate_dist(sub, px, py);
-        if (!(d >= 0.5 && d <= 2.5)) continue;
-        any = true;
-        int side;
-        if (sub.circle) {
-            const double ax = __dsub_rn(qxc, sub.cx), ay = __dsub_rn(qyc, sub.cy);
-            const double bx = __dsub_rn(px, sub.cx), by = __dsub_rn(py, sub.cy);
-            const double cr = __dsub_rn(__dmul_rn(ax, by), __dmul_rn(ay, bx));
-            // the wall normal into the fluid at the centroid is (ax, ay) on the convex
-            // circle and -(ax, ay) on the concave one
-            side = (sub.concave ? cr < 0.0 : cr > 0.0) ? 0 : 1;
-        } else {
-            side = px < qxc ? 0 : 1;
-        }
-        const long long id = n * 4 + sl;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if ((k >> 1) != side) continue;
-            const double key = fabs(__dsub_rn(d, (double)((k & 1) + 1)));
-            if (better(key, id, b[k].key, b[k].id)) b[k] = Best{key, id, px, py, d};
-        }
+        m |= 1u << sl;
     }
-    return any;
+    return m;
+}
+
+// The link's point, if in the band, into the four running bests (side * 2 + target)
+template <typename T>
+__device__ __forceinline__ bool take_link(long long id, int nx, T va, T vb, double rho_m, T thr,
+                                          const Substrate& sub, double qxc, double qyc, Best (&b)[4]) {
+    const long long n = id >> 2;
+    const int sl = (int)(id & 3), j = (int)(n / nx), i = (int)(n - (long long)j * nx);
+    double px, py;
+    if (!link_point<T>(va, vb, rho_m, thr, i, j, sl, px, py)) return false;
+    const double d = substrate_dist(sub, px, py);
+    if (!(d >= 0.5 && d <= 2.5)) return false;
+    int side;
+    if (sub.circle) {
+        const double ax = __dsub_rn(qxc, sub.cx), ay = __dsub_rn(qyc, sub.cy);
+        const double bx = __dsub_rn(px, sub.cx), by = __dsub_rn(py, sub.cy);
+        const double cr = __dsub_rn(__dmul_rn(ax, by), __dmul_rn(ay, bx));
+        // the wall normal into the fluid at the centroid is (ax, ay) on the convex
+        // circle and -(ax, ay) on the concave one
+        side = (sub.concave ? cr < 0.0 : cr > 0.0) ? 0 : 1;
+    } else {
+        side = px < qxc ? 0 : 1;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if ((k >> 1) != side) continue;
+        const double key = fabs(__dsub_rn(d, (double)((k & 1) + 1)));
+        if (better(key, id, b[k].key, b[k].id)) b[k] = Best{key, id, px, py, d};
+    }
+    return true;
 }
 
 // The line of one side through its two points, its contact point and the wall tangent toward the
@@ -360,9 +363,10 @@ __device__ bool side_line(const Best& b1, const Best& b2, const Substrate& sub, 
 // Both contact angles. The nodes scanned are the listed ones (a few thousand on the wall, against
 // millions in the lattice: the whole-lattice scan it replaces took 152 us on 4096 x 1024 and 18 us on
 // 200 x 120) or, where the list could not be made (band_n negative or above cap), every fluid
-// node. The order of the list does not matter: the winners are minima by (key, link id). The
-// block that finishes last builds the angles, one warp per (side, angle), because chains of
-// dependent FP64 operations are what this part costs.
+// node. The order of the list does not matter: the winners are minima by (key, link id). Chains of
+// dependent FP64 operations are what this kernel costs, so a block first collects its crossing
+// links (FP32 work) and then gives each thread one of them, and the block that finishes last
+// builds the angles with one warp per (side, angle). Four links in turn per thread took 25 us.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
     k_measure(const T* rho, const uint8_t* flags, int nx, int ny, int P, double rho_m, T thr,
@@ -374,16 +378,44 @@ __global__ void __launch_bounds__(kRedThreads)
 #pragma unroll
     for (int k = 0; k < 4; ++k) b[k] = Best{INFINITY, 0x7fffffffffffffffLL, 0, 0, 0};
     bool any = false;
-    const int stride = gridDim.x * kRedThreads, t0 = blockIdx.x * kRedThreads + threadIdx.x;
-    if (nband >= 0 && nband <= cap) {
-        for (int t = t0; t < nband; t += stride)
-            any |= scan_node<T, true>(rho, flags, nx, ny, P, rho_m, thr, sub, qxc, qyc, band[t], b);
-    } else {
-        for (long long n = t0; n < (long long)nx * ny; n += stride) {
-            const int j = (int)(n / nx), i = (int)(n - (long long)j * nx);
-            if (flags[lidx(P, i, j)] == kFluid)
-                any |= scan_node<T, false>(rho, flags, nx, ny, P, rho_m, thr, sub, qxc, qyc, n, b);
+    __shared__ long long s_id[4 * kRedThreads];
+    __shared__ T s_va[4 * kRedThreads], s_vb[4 * kRedThreads];
+    __shared__ int s_n;
+    const bool listed = nband >= 0 && nband <= cap;
+    const long long total = listed ? nband : (long long)nx * ny;
+    const long long stride = (long long)gridDim.x * kRedThreads;
+    for (long long first = (long long)blockIdx.x * kRedThreads; first < total; first += stride) {
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        const long long t = first + threadIdx.x;
+        unsigned m = 0;
+        T va = 0, vb[4];
+        int n = 0;
+        if (t < total) {
+            n = listed ? band[t] : (int)t;  // fewer than 2^31 nodes
+            const int j = n / nx, i = n - j * nx;
+            if (listed || flags[lidx(P, i, j)] == kFluid) {
+                va = rho[lidx(P, i, j)];
+                const unsigned ends = link_ends<T>(rho, flags, nx, ny, P, i, j, vb);
+                m = listed ? crossing_links<T, true>(va, vb, ends, rho_m, thr, sub, i, j)
+                           : crossing_links<T, false>(va, vb, ends, rho_m, thr, sub, i, j);
+            }
         }
+        if (m) {
+            int at = atomicAdd(&s_n, __popc(m));
+#pragma unroll
+            for (int sl = 0; sl < 4; ++sl)
+                if (m >> sl & 1) {
+                    s_id[at] = (long long)n * 4 + sl;
+                    s_va[at] = va;
+                    s_vb[at] = vb[sl];
+                    ++at;
+                }
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < s_n; k += kRedThreads)
+            any |= take_link<T>(s_id[k], nx, s_va[k], s_vb[k], rho_m, thr, sub, qxc, qyc, b);
+        __syncthreads();
     }
     __shared__ Best s[kRedThreads / 32][4];
     __shared__ int s_last;
