@@ -380,6 +380,12 @@ __global__ void k_bf16_copies(const float* w, long long n, bf16* wb, bf16* wd,
 }
 
 
+// how a convolution runs on k_conv_march: cb blocks of kb operand channels, bn output columns per
+// CTA; kb = 0: it does not
+struct March {
+    int kb = 0, cb = 0, bn = 0;
+};
+
 struct Conv {
     int src1, C1, up1;  // source tensor index, channels, stored at half resolution
     int src2, C2;       // second source (-1: none)
@@ -399,12 +405,10 @@ struct Conv {
     // applies (1 or 2), else 0; maps: sources 1 and 2 (32 channels x 72 pixels x 3 rows), dY
     int ww_cb = 0;
     CUtensorMap wwmap[3] = {};
-    // forward (fw) and data gradient (dw) from one staged window per tile of 128 pixels of one
-    // row (k_gemm_fwin): 32-channel blocks of the window operand (1 where it applies, else 0)
-    // and the N tile; maps: source 1 (dY for dw) as boxes of 32 channels x 136 pixels x 3 rows,
-    // source 2 likewise, and the weights as 32 x N-tile blocks
-    int fw_cb = 0, fw_bn = 0, dw_cb = 0, dw_bn = 0;
-    CUtensorMap fwmap[3] = {}, dwmap[3] = {};
+    // forward (fm) and data gradient (dm) on k_conv_march; maps: source 1 (dY for dm) and source 2
+    // as boxes of one row of 136 pixels x kb channels, the weights as kb x bn blocks
+    March fm, dm;
+    CUtensorMap fmmap[3] = {}, dmmap[3] = {};
     // training: gradient with respect to the pre-activation (BF16), the bias gradient's per-block
     // sums, and the event after which the side stream may read them
     bf16* g = nullptr;
@@ -589,8 +593,8 @@ EncodeTiledFn encode_tiled() {
 }
 
 // Map of an NHWC BF16 tensor [N][H][W][C] (C innermost), box ks channels x bw x bh pixels x 1
-// image, ks = 64 with 128-byte or ks = 32 with 64-byte swizzle (the K-major layouts the MMAs
-// read), out-of-range elements zero.
+// image, ks = 64 with 128-byte, 32 with 64-byte or 16 with 32-byte swizzle (the K-major layouts the
+// MMAs read), out-of-range elements zero.
 bool map_nhwc(CUtensorMap* m, const void* base, int C, int W, int H, int N, int bw, int bh,
               int ks, int step = 1) {
     const EncodeTiledFn enc = encode_tiled();
@@ -603,7 +607,9 @@ bool map_nhwc(CUtensorMap* m, const void* base, int C, int W, int H, int N, int 
     const cuuint32_t es[4] = {1, (cuuint32_t)step, (cuuint32_t)step, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dim, stride, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE,
-               ks == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+               ks == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+               : ks == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                          : CU_TENSOR_MAP_SWIZZLE_32B,
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -617,7 +623,9 @@ bool map_rows(CUtensorMap* m, const void* base, int K, int rows, int box_rows, i
     const cuuint32_t es[2] = {1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dim, stride, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE,
-               ks == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+               ks == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+               : ks == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                          : CU_TENSOR_MAP_SWIZZLE_32B,
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -734,38 +742,71 @@ cudaError_t launch_wwin(cudaStream_t st, const GemmArgs& a, int splits, const CU
                       maps[2]);
 }
 
-// Launch of k_gemm_fwin: one CTA per tile of 128 pixels x BN columns.
-template <int BN, int CB, bool GD>
-cudaError_t launch_fwin(cudaStream_t st, const GemmArgs& a, const CUtensorMap* maps) {
-    // 512-byte alignment slack (the 64-byte swizzle repeats every 512 bytes): 45,088 bytes at
-    // BN = 32, five CTAs per SM
-    constexpr int SMEM = 512 + CB * 3 * 136 * 64 + 9 * CB * BN * 64 + 32;
-    auto* kern = lbm::sgtc::k_gemm_fwin<BN, CB, GD>;
+// How a convolution runs on k_conv_march: blocks of kb channels, cb of them, bn output columns per
+// CTA; kb = 0: it does not. Maps: source 1 (dY for the data gradient) and source 2 as boxes of one
+// row of 136 pixels x kb channels, weights as kb x bn blocks.
+template <int KB, int CB, int BN, bool GD, bool UP>
+cudaError_t launch_march(cudaStream_t st, const GemmArgs& a, const CUtensorMap* maps) {
+    using MS = lbm::sgtc::MarchShape<KB, CB, BN, UP>;
+    auto* kern = lbm::sgtc::k_conv_march<KB, CB, BN, GD, UP>;
     static std::atomic<unsigned long long> configured{0};
+    static std::atomic<int> sms{152};
+    // CTAs per SM: two where shared memory allows (232,448 bytes, 1 KB reserved per CTA)
+    constexpr int per_sm = 232448 / (MS::SMEM + 2048) >= 2 ? 2 : 1;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        int n = 152;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, MS::SMEM);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
+        sms.store(n);
         configured.fetch_or(bit);
     }
     int* flag = tc_flag().dev;
     if (!flag) return cudaErrorMemoryAllocation;
-    dim3 grid(a.N / BN, a.M / lbm::sgtc::BM);
-    return launch_pdl(kern, grid, lbm::sgtc::TC_THREADS, SMEM, st, a, flag, maps[0], maps[1],
-                      maps[2]);
+    const int H = GD ? a.dg.H : a.conv.H, W = GD ? a.dg.W : a.conv.W;
+    const int rh = UP ? H / 2 : H, rw = UP ? W / 2 : W, nb = a.N / BN;
+    const int strips = (int)((long long)a.M / ((long long)H * W)) * (rw / 128);
+    // one wave of CTAs: chunks of rows so that strips x chunks x column blocks fill the SMs
+    const int want = std::max(1, per_sm * sms.load() / std::max(1, strips * nb));
+    const int chunk = std::max(1, (rh + want - 1) / want);
+    const dim3 grid((unsigned)strips * ((rh + chunk - 1) / chunk), nb);
+    return launch_pdl(kern, grid, lbm::sgtc::MARCH_THREADS, MS::SMEM, st, a, flag, maps[0], maps[1],
+                      maps[2], chunk);
 }
 
-// The window-fed forward (GD false) or data gradient of a convolution that qualifies (see
-// Conv::fw_cb / dw_cb): a.M a multiple of 128, a.N of bn.
 template <bool GD>
-cudaError_t gemm_fwin(cudaStream_t st, const GemmArgs& a, int cb, int bn, const CUtensorMap* maps) {
-    if (a.M % lbm::sgtc::BM || a.N % bn) return cudaErrorInvalidValue;
-    if (cb == 1 && bn == 32) return launch_fwin<32, 1, GD>(st, a, maps);
-    if (cb == 1 && bn == 64) return launch_fwin<64, 1, GD>(st, a, maps);
-    return cudaErrorInvalidValue;
+cudaError_t conv_march(cudaStream_t st, const GemmArgs& a, const March& m, const CUtensorMap* maps) {
+    const int key = m.kb * 1000 + m.cb * 100 + m.bn;
+    if constexpr (!GD) {
+        if (a.conv.up1) switch (key) {
+                case 32132: return launch_march<32, 1, 32, false, true>(st, a, maps);
+                case 32116: return launch_march<32, 1, 16, false, true>(st, a, maps);
+                case 32232: return launch_march<32, 2, 32, false, true>(st, a, maps);
+                default: return cudaErrorInvalidValue;
+            }
+    }
+    switch (key) {
+        case 16116: return launch_march<16, 1, 16, GD, false>(st, a, maps);
+        case 16132: return launch_march<16, 1, 32, GD, false>(st, a, maps);
+        case 16216: return launch_march<16, 2, 16, GD, false>(st, a, maps);
+        case 32116: return launch_march<32, 1, 16, GD, false>(st, a, maps);
+        case 32132: return launch_march<32, 1, 32, GD, false>(st, a, maps);
+        case 32164: return launch_march<32, 1, 64, GD, false>(st, a, maps);
+        case 32232: return launch_march<32, 2, 32, GD, false>(st, a, maps);
+        case 32264: return launch_march<32, 2, 64, GD, false>(st, a, maps);
+        default: return cudaErrorInvalidValue;
+    }
+}
+// the forms conv_march has
+bool march_form(const March& m, bool up) {
+    const int key = m.kb * 1000 + m.cb * 100 + m.bn;
+    if (up) return key == 32132 || key == 32116 || key == 32232;
+    return key == 16116 || key == 16132 || key == 16216 || key == 32116 || key == 32132 ||
+           key == 32164 || key == 32232 || key == 32264;
 }
 
 // out = the sum of `splits` FP32 partials of `stride` values each, in split order
@@ -960,8 +1001,8 @@ lbm_status forward(lbm_surrogate* s, const bf16* x, int B) {
         g.bias = s->w + c.b_off;
         g.relu = 1;
         if (c.up1 && c.f_ks) g.rperm = std::min(c.W, 128) / 2;
-        if (c.fw_cb)
-            SCUDA(s, gemm_fwin<false>(s->stream, g, c.fw_cb, c.fw_bn, c.fwmap));
+        if (c.fm.kb)
+            SCUDA(s, conv_march<false>(s->stream, g, c.fm, c.fmmap));
         else
             SCUDA(s, (gemm_tc_split<true, false>(s->stream, g, s->splitk, s->splitk_elems, c.fmap,
                                                   c.f_ks)));
@@ -977,6 +1018,40 @@ lbm_status forward(lbm_surrogate* s, const bf16* x, int B) {
     return LBM_OK;
 }
 
+// k_conv_march where it applies: operand rows a multiple of 128 pixels wide (for a forward
+// upsampling convolution the half-resolution source's), 16, 32 or 64 operand channels (input, both
+// sources' blocks aligned; output gradient), 16, 32 or a multiple of 64 output columns. At most
+// 178 KB of shared memory; with 128 operand channels rows and weights would not fit together, so those
+// layers keep the boxes per tap.
+void make_march_maps(lbm_surrogate* s, Conv& c) {
+    auto blocks = [](int c1, int c2, int n) {
+        March m;
+        const int cin = c1 + c2;
+        m.kb = c1 % 32 == 0 && c2 % 32 == 0 ? 32 : c1 % 16 == 0 && c2 % 16 == 0 ? 16 : 0;
+        m.cb = m.kb ? cin / m.kb : 0;
+        m.bn = n % 64 == 0 ? 64 : n % 32 == 0 ? 32 : n % 16 == 0 ? 16 : 0;
+        return m;
+    };
+    if (c.src1 == 0) return;
+    const int cin = c.C1 + c.C2, ow = c.up1 ? c.W / 2 : c.W, oh = c.up1 ? c.H / 2 : c.H;
+    if (ow % 128 == 0 && !(c.up1 && c.C2)) {
+        const March m = blocks(c.C1, c.C2, c.Cout);
+        if (m.kb && m.bn && march_form(m, c.up1) &&
+            map_nhwc(&c.fmmap[0], s->t[c.src1].y, c.C1, ow, oh, s->maxB, 136, 1, m.kb) &&
+            (c.src2 < 0 || map_nhwc(&c.fmmap[1], s->t[c.src2].y, c.C2, ow, oh, s->maxB, 136, 1, m.kb)) &&
+            map_rows(&c.fmmap[2], s->wb + c.w_off, 9 * cin, c.Cout, m.bn, m.kb))
+            c.fm = m;
+    }
+    if (!c.up1 && c.W % 128 == 0) {
+        const March m = blocks(c.Cout, 0, cin);
+        // a column block of eight lies on one side of the split between the sources
+        if (m.kb && m.bn && march_form(m, false) && c.C1 % 8 == 0 &&
+            map_nhwc(&c.dmmap[0], c.g, c.Cout, c.W, c.H, s->maxB, 136, 1, m.kb) &&
+            map_rows(&c.dmmap[2], s->wbd + c.w_off, 9 * c.Cout, cin, m.bn, m.kb))
+            c.dm = m;
+    }
+}
+
 // Tensor maps for the forward and data-gradient GEMMs whose A operand the copy engine can fetch
 // as boxes: no upsampled source, channel counts multiples of 64 (one K-slice of 64 = one tap of
 // one source) or else of 32 (slices of 32), the 128 rows of a tile a whole block of pixels of
@@ -988,6 +1063,7 @@ void make_tensor_maps(lbm_surrogate* s) {
                                          : a % 32 == 0 && b % 32 == 0 ? 32 : 0; };
     for (Conv& c : s->convs) {
         const int W = c.W, H = c.H;
+        make_march_maps(s, c);
         if (c.up1 && c.src1 != 0) {
             // forward of an upsampling convolution: tile rows in runs of even, then odd output
             // columns, each run a box of half a tile row of source pixels
@@ -1025,25 +1101,6 @@ void make_tensor_maps(lbm_surrogate* s) {
             (c.src2 < 0 || map_nhwc(&c.fmap[1], s->t[c.src2].y, c.C2, W, H, s->maxB, bw, bh, fk)) &&
             map_rows(&c.fmap[2], s->wb + c.w_off, 9 * cin, c.Cout, pick_bn(c.Cout), fk))
             c.f_ks = fk;
-        // window-fed forward and data gradient: 128-pixel row segments, a window operand of 32
-        // channels (the input for the forward, dY for the data gradient) and 32 or 64 output
-        // columns (at most 64 KB of shared memory, five or three CTAs per SM). With 64 window
-        // channels (90 KB and two CTAs per SM, each loading, multiplying and storing in turn,
-        // or one CTA per SM at N = 64) the pipelined TMA path is faster, so those keep it.
-        if (W % 128 == 0 && (long long)s->maxB * H * W / 128 <= 65535) {
-            if (cin == 32 && c.C2 == 0 && (c.Cout == 32 || c.Cout == 64) &&
-                map_nhwc(&c.fwmap[0], s->t[c.src1].y, c.C1, W, H, s->maxB, 136, 3, 32) &&
-                map_rows(&c.fwmap[2], s->wb + c.w_off, 9 * cin, c.Cout, c.Cout, 32)) {
-                c.fw_cb = 1;
-                c.fw_bn = c.Cout;
-            }
-            if (c.Cout == 32 && c.C1 % 32 == 0 && c.C2 % 32 == 0 && (cin == 32 || cin == 64) &&
-                map_nhwc(&c.dwmap[0], c.g, c.Cout, W, H, s->maxB, 136, 3, 32) &&
-                map_rows(&c.dwmap[2], s->wbd + c.w_off, 9 * c.Cout, cin, cin, 32)) {
-                c.dw_cb = 1;
-                c.dw_bn = cin;
-            }
-        }
         if (W % 64 == 0 && c.C1 % 32 == 0 && c.C2 % 32 == 0 && (cin == 32 || cin == 64) &&
             (c.Cout == 32 || c.Cout == 64)) {
             const int wc = cin / 32;
@@ -1303,8 +1360,8 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
             gd.ldc2 = c.C2;
             gd.nsplit = c.C1;
         }
-        if (c.dw_cb)
-            SCUDA(s, gemm_fwin<true>(s->stream, gd, c.dw_cb, c.dw_bn, c.dwmap));
+        if (c.dm.kb)
+            SCUDA(s, conv_march<true>(s->stream, gd, c.dm, c.dmmap));
         else
             SCUDA(s, (gemm_tc_split<false, true>(s->stream, gd, s->splitk, s->splitk_elems,
                                                   c.dmap, c.d_ks)));

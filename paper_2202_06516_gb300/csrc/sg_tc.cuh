@@ -14,9 +14,9 @@
 // which frees the slice for the next load. The epilogue reads the accumulator lanes back with
 // tcgen05.ld (warp w owns rows 32 w .. 32 w + 31), adds the bias, applies the leaky ReLU and
 // stores FP32 or BF16. k_gemm_wwin computes the weight gradient of the 32/64-channel levels from
-// one staged input window per slice, and k_gemm_fwin the forward convolution or data gradient of
-// a layer whose window operand has 32 channels from one staged window per 128-pixel tile (the
-// nine taps as operands shifted by whole rows inside the window).
+// one staged input window per slice, and k_conv_march the forward convolutions and data gradients
+// of wide rows with few channels from operand rows staged once (the nine taps as operands shifted
+// by whole pixels inside them).
 //
 // Every wait on an mbarrier is polled by one thread with an iteration limit; on expiry the
 // CTA sets *err, waits (bounded) for the MMAs it issued, frees its tensor memory and returns.
@@ -63,32 +63,22 @@ __device__ __forceinline__ uint32_t su32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// shared-memory matrix descriptor: K-major operand, 128-byte swizzle, 8-row groups 1 KB apart
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) |
-           ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+// Shared-memory matrix descriptors as two words. The high word is a constant of the layout: bytes
+// between 8-row (K-major) or 8-K (MN-major) groups, the fixed version, the swizzle. The low word holds
+// the start address / 16, which advances by bytes / 16, and for MN-major operands the bytes between
+// blocks of the swizzle's width along M or N (1, unused, for K-major ones). Precomputed words
+// matter: one thread issues the MMAs, and building two 64-bit descriptors for each took about as
+// long as the MMA (k_conv_march 57 -> 44 and 34 -> 23 us on the full-resolution layers).
+//   K-major, 128-byte swizzle (64 channels per row): groups 1 KB apart; 64-byte (32): 512 B;
+//   32-byte (16): 256 B. MN-major, 64-byte swizzle: groups 512 B, 32-wide blocks lbo apart;
+//   128-byte swizzle: groups 1 KB, 64-wide blocks 8 KB apart.
+// A start may lie on any whole row of the layout: the swizzle follows the absolute address.
+enum Swizzle { SW128 = 2, SW64 = 4, SW32 = 6 };
+__host__ __device__ constexpr uint32_t desc_hi(int group_bytes, Swizzle sw) {
+    return (uint32_t)(group_bytes >> 4) | (1u << 14) | ((uint32_t)sw << 29);
 }
-
-// the same for 64-byte rows (32 elements of K), 64-byte swizzle, 8-row groups 512 B apart
-__device__ __forceinline__ uint64_t desc_sw64(uint32_t saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) |
-           ((uint64_t)(512 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
-}
-
-// shared-memory descriptor: MN-major operand, 64-byte swizzle; atoms of 32 (M or N) x 8 (K)
-// elements, the 8-row K-groups of one 32-wide block 512 B apart (stride offset), blocks of 64 K
-// rows 4 KB apart along M or N (leading offset)
-__device__ __forceinline__ uint64_t desc_sw64_mn(uint32_t saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(4096 >> 4) << 16) |
-           ((uint64_t)(512 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
-}
-
-// shared-memory descriptor: MN-major operand, 128-byte swizzle; atoms of 64 (M or N) x 8 (K)
-// elements, the 8 K-groups of one 64-wide block 1 KB apart (stride offset), blocks 8 KB apart
-// along M or N (leading offset)
-__device__ __forceinline__ uint64_t desc_sw128_mn(uint32_t saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(8192 >> 4) << 16) |
-           ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes = 16) {
+    return ((saddr & 0x3FFFFu) >> 4) | ((lbo_bytes >> 4) << 16);
 }
 
 // instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, each K-major (0) or
@@ -124,12 +114,13 @@ __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
 
-__device__ __forceinline__ void tc_mma(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                       uint32_t accumulate) {
+__device__ __forceinline__ void tc_mma(uint32_t tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                       uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-        "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate)
+        "{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %6, 0;\n"
+        " mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
@@ -673,19 +664,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     break;
                 }
                 tc_fence_after();
-                const uint32_t a0 = su32(stage_a(st)), b0 = su32(stage_b(st));
+                // K = 16 per MMA: 32 bytes along a K-major row, or two 512-byte K-groups of an
+                // MN-major 64-byte-swizzled block (blocks 4 KB apart)
+                constexpr uint32_t HI = GAM || KS == 32 ? desc_hi(512, SW64) : desc_hi(1024, SW128);
+                constexpr uint32_t STEP = (GAM ? 1024 : 32) >> 4, LBO = GAM ? 4096 : 16;
+                const uint32_t a0 = desc_lo(su32(stage_a(st)), LBO), b0 = desc_lo(su32(stage_b(st)), LBO);
 #pragma unroll
-                for (int j = 0; j < KS / 16; ++j) {
-                    // K = 16 per MMA: 32 bytes along a K-major row, or two 512-byte K-groups of
-                    // an MN-major 64-byte-swizzled block
-                    const uint64_t ad = GAM         ? desc_sw64_mn(a0 + 1024 * j)
-                                        : KS == 64 ? desc_sw128(a0 + 32 * j)
-                                                   : desc_sw64(a0 + 32 * j);
-                    const uint64_t bd = GAM         ? desc_sw64_mn(b0 + 1024 * j)
-                                        : KS == 64 ? desc_sw128(b0 + 32 * j)
-                                                   : desc_sw64(b0 + 32 * j);
-                    tc_mma(tmem, ad, bd, IDESC, (kt > 0 || j > 0) ? 1u : 0u);
-                }
+                for (int j = 0; j < KS / 16; ++j)
+                    tc_mma(tmem, a0 + STEP * j, HI, b0 + STEP * j, HI, IDESC, (kt > 0 || j > 0) ? 1u : 0u);
                 tc_commit(su32(bars + STAGES + st));
                 done_mma = kt + 1;
                 // refill the stage that slice kt - 1 used once its MMAs have read it
@@ -726,15 +712,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         __syncthreads();
         if (tid == 0) {
             tc_fence_after();
-            const uint32_t a0 = su32(stage_a(s)), b0 = su32(stage_b(s));
+            // K = 16 per MMA: 32 bytes along a K-major swizzle row, two 1 KB K-groups of an
+            // MN-major block (blocks 8 KB apart)
+            constexpr uint32_t HI = desc_hi(1024, SW128);
+            const uint32_t a0 = desc_lo(su32(stage_a(s)), AMN ? 8192 : 16);
+            const uint32_t b0 = desc_lo(su32(stage_b(s)), BMN ? 8192 : 16);
 #pragma unroll
-            for (int j = 0; j < BK / 16; ++j) {
-                // K = 16 per MMA: 32 bytes along a K-major swizzle row, two 1 KB K-groups of an
-                // MN-major block
-                const uint64_t ad = AMN ? desc_sw128_mn(a0 + 2048 * j) : desc_sw128(a0 + 32 * j);
-                const uint64_t bd = BMN ? desc_sw128_mn(b0 + 2048 * j) : desc_sw128(b0 + 32 * j);
-                tc_mma(tmem, ad, bd, IDESC, (kt > 0 || j > 0) ? 1u : 0u);
-            }
+            for (int j = 0; j < BK / 16; ++j)
+                tc_mma(tmem, a0 + (AMN ? 128 : 2) * j, HI, b0 + (BMN ? 128 : 2) * j, HI, IDESC,
+                       (kt > 0 || j > 0) ? 1u : 0u);
             tc_commit(su32(bars + s));
         }
         const int nxt = kt + STAGES - 1;
@@ -778,14 +764,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                      "r"(tmem_cols(BN))
                      : "memory");
     }
-}
-
-// shared-memory descriptor of an MN-major, 64-byte-swizzled operand whose 32-wide blocks are
-// lbo bytes apart (K-groups of 8 rows 512 B apart); the start may lie on any 64-byte row, the
-// swizzle follows the absolute shared-memory address
-__device__ __forceinline__ uint64_t desc_sw64_mn_lbo(uint32_t saddr, uint32_t lbo) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) |
-           ((uint64_t)(512 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
 
 __host__ __device__ constexpr uint32_t tmem_pow2(int cols) {
@@ -870,16 +848,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 break;
             }
             tc_fence_after();
+            constexpr uint32_t HI = desc_hi(512, SW64);
+            const uint32_t a0 = desc_lo(win(st, 0), WROW * 64), b0 = desc_lo(dyb(st), 4096);
 #pragma unroll
             for (int t = 0; t < T; ++t) {
                 const int cb = t / 3, dxi = t - 3 * (t / 3);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint64_t ad =
-                        desc_sw64_mn_lbo(win(st, cb) + (uint32_t)((3 + dxi) * 64 + 1024 * j), WROW * 64);
-                    const uint64_t bd = desc_sw64_mn(dyb(st) + 1024 * j);
-                    tc_mma(tmem + (uint32_t)(t * BN), ad, bd, IDESC, (kt > 0 || j > 0) ? 1u : 0u);
-                }
+                for (int j = 0; j < 4; ++j)
+                    tc_mma(tmem + (uint32_t)(t * BN),
+                           a0 + (uint32_t)((cb * WIN + (3 + dxi) * 64 + 1024 * j) >> 4), HI,
+                           b0 + (uint32_t)((1024 * j) >> 4), HI, IDESC, (kt > 0 || j > 0) ? 1u : 0u);
             }
             tc_commit(su32(bars + STAGES + st));
             done_mma = kt + 1;
@@ -937,112 +915,262 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
 }
 
-// Forward convolution (GA) or data gradient (GD) of a 3 x 3 convolution for a tile of 128
-// output pixels of one image row, from one staged window: with C = 32 CB channels of the operand
-// (the input for GA, concatenated sources by channel; the output gradient for GD), thread 0
-// loads with TMA, per 32-channel block, the rows y - 1 .. y + 1 of pixels x - 4 .. x + 131
-// (K-major rows of 32 channels, 64-byte swizzle) and the tile's 32 x BN weight blocks of all
-// nine taps (output columns BN blockIdx.x ..), all on one mbarrier. Each tap (dy, dx) is then a K-major A operand that starts whole rows into
-// the window (GA: row dy + 1, column 4 + dx; GD: the offsets negated), two 16-deep MMAs per
-// (tap, block) into one accumulator. Every operand element is read once per tile instead of once
-// per tap. The epilogue is the GEMM's own (bias and leaky ReLU with BF16 output, or the
-// accumulating, possibly split FP32 output of the data gradient).
-template <int BN, int CB, bool GD>
-__global__ void __launch_bounds__(TC_THREADS, 1)
-    k_gemm_fwin(const sg::GemmArgs g, int* err, const __grid_constant__ CUtensorMap tmA1,
-                const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB) {
-    static_assert((BN == 32 || BN == 64) && (CB == 1 || CB == 2), "32 or 64 columns and channels");
-    constexpr int WROW = 136, WINB = 3 * WROW * 64;  // one 32-channel block of the window
-    constexpr int A_B = CB * WINB, BSUB = BN * 64, B_B = 9 * CB * BSUB;
-    constexpr uint32_t TX = (uint32_t)(A_B + B_B);
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+
+// 32 bytes to a 32-byte-aligned address: a whole sector per lane
+__device__ __forceinline__ void st_global_32B(void* p, const uint32_t (&v)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "r"(v[0]),
+                 "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+
+// a wait for a whole warp: lane 0 polls
+__device__ __forceinline__ bool warp_wait(int lane, uint32_t bar, uint32_t parity) {
+    int ok = 1;
+    if (lane == 0) ok = mbar_wait(bar, parity);
+    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
+// Sizes of k_conv_march: rows of 136 pixels of CB blocks of KB channels in a ring, the nine taps'
+// weight blocks, mbarriers.
+template <int KB, int CB, int BN, bool UP>
+struct MarchShape {
+    static constexpr int R = 6;                        // rows in the ring
+    static constexpr int G = UP ? 4 : 1;               // tiles (accumulators) per operand row
+    static constexpr int ROWB = 136 * KB * 2, SLOT = CB * ROWB;
+    static constexpr int BSUB = BN * KB * 2, WBYTES = 9 * CB * BSUB;
+    static constexpr int NBARS = 2 * R + 6;
+    static constexpr int SMEM = 1024 + WBYTES + R * SLOT + NBARS * 8;
+};
+constexpr int MARCH_THREADS = 192;
+
+// 3 x 3 convolution (GD = false: forward, bias and leaky ReLU, BF16 out) or its data gradient (GD:
+// FP32 out, split at nsplit) along a strip 128 operand pixels wide, marching down the rows: every
+// operand row is copied to shared memory once (not once per tap and tile), the nine taps' weights
+// once per CTA. Each tile of 128 pixels of one row is 9 CB KB / 16 MMAs, whose A operand is a row of
+// the ring starting dx pixels aside; the K order is tap, then channel. UP (forward): the operand
+// has half the output's resolution (nearest upsampling), and each operand row yields four tiles,
+// two output rows of 128 even and 128 odd columns each.
+// Roles: warp 4 copies (TMA), warp 5 issues MMAs, warps 0-3 read the finished accumulator (two in
+// tensor memory, alternating) and store whole 32-byte sectors, so copies, MMAs and stores of
+// neighbouring rows overlap. Bound by the MMAs' shared-memory reads (a 128 x 16 A slice per
+// 16-deep MMA of only BN columns). One 128-pixel tile per CTA with its own window and weights (182 MB
+// through L2 for 32 -> 32 channels at 256 x 256 x 8, against 72 MB here) or one box per tap (750 MB for
+// 64 -> 32) were bound by that traffic and its latency. 256 x 256 x 8: 32 -> 32 channels 34 -> 23 us,
+// 64 -> 32 (concatenated) 69 -> 44, 64 -> 32 (upsampling) 72 -> 35; 128 x 128 x 8, 64 -> 64: 27 -> 18.
+// Waits are polled by one thread each with an iteration limit; a wait that runs out ends its role,
+// the others follow by their own limits, copies and MMAs in flight are waited for (bounded).
+template <int KB, int CB, int BN, bool GD, bool UP>
+__global__ void __launch_bounds__(MARCH_THREADS, 1)
+    k_conv_march(const sg::GemmArgs g, int* err, const __grid_constant__ CUtensorMap tmA1,
+                 const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB,
+                 int chunk) {
+    using S = MarchShape<KB, CB, BN, UP>;
+    static_assert((KB == 16 || KB == 32) && BN % 16 == 0 && BN <= 64 && !(GD && UP), "shape");
+    constexpr int R = S::R, G = S::G;
+    constexpr uint32_t COLS = tmem_pow2(2 * G * BN);
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t raw = su32(smem_raw);
-    // 512-byte-aligned base: the 64-byte swizzle repeats every 512 bytes of shared memory
-    uint8_t* base = smem_raw + ((512u - (raw & 511u)) & 511u);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(base + A_B + B_B);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
+    uint8_t* base = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
+    const uint32_t wgt = su32(base), ring = wgt + S::WBYTES, bars = ring + R * S::SLOT;
+    auto full = [&](int i) { return bars + 8u * i; };
+    auto empty = [&](int i) { return bars + 8u * (R + i); };
+    const uint32_t wfull = bars + 8u * (2 * R), done = wfull + 8u;
+    auto accf = [&](int b) { return done + 8u + 8u * b; };
+    auto acce = [&](int b) { return done + 24u + 8u * b; };
     __shared__ int s_ok;
+    __shared__ uint32_t s_tmem;
+    __shared__ float s_bias[BN];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    sg::pdl_wait();
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                         su32(tmem_slot)),
-                     "r"(tmem_cols(BN))
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-    }
+
+    // the CTA's strip: image, first operand column, operand rows ra .. rb - 1
+    const int H = GD ? g.dg.H : g.conv.H, W = GD ? g.dg.W : g.conv.W;
+    const int RH = UP ? H / 2 : H, RW = UP ? W / 2 : W;
+    const int chunks = (RH + chunk - 1) / chunk, strips = RW / 128;
+    const int ck = blockIdx.x % chunks, st = blockIdx.x / chunks;
+    const int img = st / strips, x0 = (st - img * strips) * 128;
+    const int ra = ck * chunk, rb = min(RH, ra + chunk), n0 = blockIdx.y * BN;
+
     if (tid == 0) {
-        mbar_init(su32(bars), 1);
-        mbar_init(su32(bars + 1), 1);
+        for (int i = 0; i < R; ++i) {
+            mbar_init(full(i), 1);
+            mbar_init(empty(i), 1);
+        }
+        mbar_init(wfull, 1);
+        mbar_init(done, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(accf(b), 1);
+            mbar_init(acce(b), 4);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         s_ok = 1;
     }
+    sg::pdl_wait();
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                         su32(&s_tmem)),
+                     "r"(COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    if (!GD && tid < BN) s_bias[tid] = g.bias ? g.bias[n0 + tid] : 0.f;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     sg::pdl_next();
-    const uint32_t tmem = *tmem_slot;
-    constexpr uint32_t IDESC = idesc_bf16(BM, BN, 0, 0);
-    const int H = GD ? g.dg.H : g.conv.H, W = GD ? g.dg.W : g.conv.W;
-    const int img = m0 / (H * W), rem = m0 - img * (H * W);
-    const int y0 = rem / W, x0 = rem - (rem / W) * W;
-    const uint32_t A = su32(base), B = su32(base + A_B);
-    if (tid == 0) {
+    const uint32_t tmem = s_tmem;
+
+    if (warp == 4 && lane == 0) {
+        // copies: weights, then operand rows ra - 1 .. rb (rows outside the image are zero-filled)
         bool good = true;
-        const uint32_t full = su32(bars);
-        mbar_expect_tx(full, TX);
+        const int rows = rb - ra + 2;
+        int issued = 0;
+        auto load_row = [&](int i) {
+            const int slot = i % R;
+            mbar_expect_tx(full(slot), (uint32_t)S::SLOT);
 #pragma unroll
-        for (int cb = 0; cb < CB; ++cb) {
-            const int ci = 32 * cb;
-            if (GD || ci < g.conv.C1)
-                tma_load_4d(A + cb * WINB, &tmA1, full, ci, x0 - 4, y0 - 1, img);
-            else
-                tma_load_4d(A + cb * WINB, &tmA2, full, ci - g.conv.C1, x0 - 4, y0 - 1, img);
+            for (int cb = 0; cb < CB; ++cb) {
+                const int ci = KB * cb;
+                const uint32_t dst = ring + slot * S::SLOT + cb * S::ROWB;
+                if (GD || ci < g.conv.C1)
+                    tma_load_4d(dst, &tmA1, full(slot), ci, x0 - 4, ra - 1 + i, img);
+                else
+                    tma_load_4d(dst, &tmA2, full(slot), ci - g.conv.C1, x0 - 4, ra - 1 + i, img);
+            }
+        };
+        for (; issued < 3; ++issued) load_row(issued);  // rows >= 3
+        mbar_expect_tx(wfull, (uint32_t)S::WBYTES);
+        for (int t = 0; t < 9 * CB; ++t) tma_load_2d(wgt + t * S::BSUB, &tmB, wfull, t * KB, n0);
+        for (; issued < rows; ++issued) {
+            if (issued >= R && !mbar_wait(empty(issued % R), (issued / R - 1) & 1)) {
+                good = false;
+                break;
+            }
+            load_row(issued);
         }
-        for (int t = 0; t < 9; ++t)
-#pragma unroll
-            for (int cb = 0; cb < CB; ++cb)
-                tma_load_2d(B + (t * CB + cb) * BSUB, &tmB, full, (t * CB + cb) * 32, n0);
-        if (!mbar_wait(full, 0)) {
-            good = false;
-            mbar_wait(full, 0);  // let the copies in flight land before the CTA may leave (bounded)
-        }
-        if (good) {
+        // nothing may still be landing when the CTA leaves
+        for (int i = max(0, issued - R); i < issued; ++i) good &= mbar_wait(full(i % R), (i / R) & 1);
+        good &= mbar_wait(wfull, 0);
+        if (!good) s_ok = 0;
+    } else if (warp == 5 && lane == 0) {
+        constexpr uint32_t IDESC = idesc_bf16(BM, BN, 0, 0);
+        constexpr uint32_t HI = KB == 32 ? desc_hi(512, SW64) : desc_hi(256, SW32);
+        const uint32_t w_lo = desc_lo(wgt);
+        bool good = mbar_wait(wfull, 0);
+        int have = -1;
+        for (int r = ra; r < rb && good; ++r) {
+            const int i0 = r - ra, need = i0 + 2;  // ring indexes of operand rows r - 1 and r + 1
+            while (have < need && good) {
+                ++have;
+                good = mbar_wait(full(have % R), (have / R) & 1);
+            }
+            const int b = i0 & 1;
+            if (good && i0 >= 2) good = mbar_wait(acce(b), ((i0 >> 1) - 1) & 1);
+            if (!good) break;
             tc_fence_after();
+            uint32_t row_lo[3];  // operand rows r - 1, r, r + 1
+#pragma unroll
+            for (int i = 0; i < 3; ++i) row_lo[i] = desc_lo(ring + ((i0 + i) % R) * S::SLOT);
+#pragma unroll
             for (int t = 0; t < 9; ++t) {
                 const int dy = t / 3 - 1, dx = t - (t / 3) * 3 - 1;
-                const int wr = GD ? 1 - dy : 1 + dy, wc = GD ? 4 - dx : 4 + dx;
 #pragma unroll
                 for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        const uint32_t a = A + cb * WINB + (uint32_t)((wr * WROW + wc) * 64 + 32 * j);
-                        const uint32_t b = B + (t * CB + cb) * BSUB + 32 * j;
-                        tc_mma(tmem, desc_sw64(a), desc_sw64(b), IDESC,
-                               (t > 0 || cb > 0 || j > 0) ? 1u : 0u);
-                    }
+                    for (int j = 0; j < KB / 16; ++j)
+#pragma unroll
+                        for (int k = 0; k < G; ++k) {
+                            int wr, wc;  // operand row relative to r - 1, column relative to x0 - 4
+                            if (UP) {
+                                const int yy = (k >> 1) + dy;
+                                wr = yy < 0 ? 0 : yy > 1 ? 2 : 1;
+                                wc = 4 + ((k & 1) ? (dx > 0 ? 1 : 0) : (dx < 0 ? -1 : 0));
+                            } else {
+                                wr = 1 + (GD ? -dy : dy);
+                                wc = GD ? 4 - dx : 4 + dx;
+                            }
+                            tc_mma(tmem + (uint32_t)((b * G + k) * BN),
+                                   row_lo[wr] + ((wc * KB * 2 + cb * S::ROWB + 32 * j) >> 4), HI,
+                                   w_lo + (((t * CB + cb) * S::BSUB + 32 * j) >> 4), HI, IDESC,
+                                   (t > 0 || cb > 0 || j > 0) ? 1u : 0u);
+                        }
             }
-            tc_commit(su32(bars + 1));
-            if (!mbar_wait(su32(bars + 1), 0)) good = false;
+            tc_commit(accf(b));
+            tc_commit(empty(i0 % R));  // operand row r - 1 is not read again
         }
+        tc_commit(done);
+        if (!mbar_wait(done, 0)) good = false;
         if (!good) s_ok = 0;
-    }
-    __syncthreads();
-    if (!s_ok) {
-        if (tid == 0) atomicExch(err, 1);
-    } else {
-        tc_fence_after();
-        // the staging blocks lie in the window, no longer read
-        epilogue_tile<BN>(g, tmem, reinterpret_cast<float*>(base) + warp * (32 * 36), warp, lane,
-                          m0, n0, false, 0);
+    } else if (warp < 4) {
+        // lane: one pixel of the tile
+        for (int r = ra; r < rb; ++r) {
+            const int b = (r - ra) & 1;
+            if (!warp_wait(lane, accf(b), ((r - ra) >> 1) & 1)) {
+                if (lane == 0) s_ok = 0;
+                break;
+            }
+            tc_fence_after();
+            const int px = warp * 32 + lane;
+            for (int k = 0; k < G; ++k) {
+                const size_t m = UP ? ((size_t)img * H + 2 * r + (k >> 1)) * W + 2 * (x0 + px) + (k & 1)
+                                    : ((size_t)img * H + r) * W + x0 + px;
+#pragma unroll
+                for (int c0 = 0; c0 < BN; c0 += 32) {
+                    constexpr int CW = BN < 32 ? BN : 32;
+                    float v[32];
+                    const uint32_t ta =
+                        tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((b * G + k) * BN + c0);
+                    if (CW == 32)
+                        tc_ld32(ta, v);
+                    else
+                        tc_ld16(ta, v);
+                    if (c0 + CW == BN && k == G - 1) {  // the accumulators have been read
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(acce(b));
+                    }
+                    if (!GD) {
+#pragma unroll
+                        for (int c = 0; c < CW; c += 16) {
+                            uint32_t o[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                float a0 = v[c + 2 * i] + s_bias[c0 + c + 2 * i];
+                                float a1 = v[c + 2 * i + 1] + s_bias[c0 + c + 2 * i + 1];
+                                a0 = fmaxf(a0, 0.1f * a0);
+                                a1 = fmaxf(a1, 0.1f * a1);
+                                const __nv_bfloat162 h = __floats2bfloat162_rn(a0, a1);
+                                o[i] = *reinterpret_cast<const uint32_t*>(&h);
+                            }
+                            st_global_32B(g.Cb + m * g.ldc + n0 + c0 + c, o);
+                        }
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < CW; c += 8) {
+                            const int n = n0 + c0 + c;
+                            float* dst = g.Cf2 && n >= g.nsplit ? g.Cf2 + m * g.ldc2 + (n - g.nsplit)
+                                                                : g.Cf + m * g.ldc + n;
+                            uint32_t o[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const float x = g.accumulate ? dst[i] + v[c + i] : v[c + i];
+                                o[i] = __float_as_uint(x);
+                            }
+                            st_global_32B(dst, o);
+                        }
+                    }
+                }
+            }
+        }
     }
     tc_fence_before();
     __syncthreads();
+    if (tid == 0 && !s_ok) atomicExch(err, 1);
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                     "r"(tmem_cols(BN))
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(COLS)
                      : "memory");
     }
 }
