@@ -396,7 +396,7 @@ struct Conv {
     // 2 (concatenation), B; f_ks, d_ks: the K elements per stage of those maps (64 or 32), 0
     // when the shapes do not allow it and the loaders gather with cp.async
     int f_ks = 0, d_ks = 0;
-    CUtensorMap fmap[3] = {}, dmap[3] = {};
+    CUtensorMap fmap[4] = {}, dmap[4] = {};  // [3]: B as 32-row boxes
     // weight gradient (w): A sources 1 and 2 and the output gradient, boxes of 32 channels x 64
     // pixels; w_tma false: gathered with cp.async
     bool w_tma = false;
@@ -593,8 +593,8 @@ EncodeTiledFn encode_tiled() {
 }
 
 // Map of an NHWC BF16 tensor [N][H][W][C] (C innermost), box ks channels x bw x bh pixels x 1
-// image, ks = 64 with 128-byte, 32 with 64-byte or 16 with 32-byte swizzle (the K-major layouts the
-// MMAs read), out-of-range elements zero.
+// image, ks = 64 with 128-byte, 32 with 64-byte, 16 with 32-byte swizzle or 8 without (the K-major
+// layouts the MMAs read), out-of-range elements zero.
 bool map_nhwc(CUtensorMap* m, const void* base, int C, int W, int H, int N, int bw, int bh,
               int ks, int step = 1) {
     const EncodeTiledFn enc = encode_tiled();
@@ -609,7 +609,8 @@ bool map_nhwc(CUtensorMap* m, const void* base, int C, int W, int H, int N, int 
                CU_TENSOR_MAP_INTERLEAVE_NONE,
                ks == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
                : ks == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
-                          : CU_TENSOR_MAP_SWIZZLE_32B,
+               : ks == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
+                          : CU_TENSOR_MAP_SWIZZLE_NONE,
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -625,9 +626,13 @@ bool map_rows(CUtensorMap* m, const void* base, int K, int rows, int box_rows, i
                CU_TENSOR_MAP_INTERLEAVE_NONE,
                ks == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
                : ks == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
-                          : CU_TENSOR_MAP_SWIZZLE_32B,
+               : ks == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
+                          : CU_TENSOR_MAP_SWIZZLE_NONE,
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+
+// CTAs of a launch up to which gemm_tc_tma takes its narrow, deep form.
+constexpr long long kFewTiles = 128;
 
 // The TMA-fed gathering GEMM (GA or GD with tensor maps, see Conv::fmap / dmap), ks elements
 // of K per stage: N tiles of 32, 64, 128 or 256 columns; few stages, so that several CTAs share
@@ -636,6 +641,16 @@ template <bool GA, bool GD>
 cudaError_t gemm_tc_tma(cudaStream_t st, const GemmArgs& a, int splits, const CUtensorMap* maps,
                         int ks) {
     const int bn = pick_bn(a.N);
+    // Few tiles: the launch is one chain of slices per CTA, each waiting for its copies. Then every
+    // tile is cut into columns of 32 (the same products in the same order) until the SMs are
+    // filled, and a CTA keeps eight slices in flight instead of two or three. maps[3]: the weights
+    // as 32-row boxes.
+    const long long ctas = (long long)((a.N + bn - 1) / bn) * ((a.M + lbm::sgtc::BM - 1) / lbm::sgtc::BM) * splits;
+    if (ctas <= kFewTiles && a.N % 32 == 0) {
+        const CUtensorMap m[3] = {maps[0], maps[1], maps[3]};
+        if (ks == 64) return launch_tc<32, 8, false, false, GA, GD, false, 64>(st, a, splits, m);
+        if (ks == 32) return launch_tc<32, 12, false, false, GA, GD, false, 32>(st, a, splits, m);
+    }
     if (ks == 64) switch (bn) {
             case 32: return launch_tc<32, 3, false, false, GA, GD, false, 64>(st, a, splits, maps);
             case 64: return launch_tc<64, 3, false, false, GA, GD, false, 64>(st, a, splits, maps);
@@ -742,6 +757,15 @@ cudaError_t launch_wwin(cudaStream_t st, const GemmArgs& a, int splits, const CU
                       maps[2]);
 }
 
+// out = the sum of `splits` FP32 partials of `stride` values each, in split order
+cudaError_t sum_splits(cudaStream_t st, const float* part, int splits, long long stride, float* out) {
+    if (stride % 4 == 0 && ((uintptr_t)out & 15) == 0)
+        return launch_pdl(k_splitk_sum4, dim3((unsigned)((stride / 4 + 31) / 32)), 256, 0, st, part,
+                          splits, stride, stride, out);
+    return launch_pdl(k_splitk_sum, dim3(blocks_for(stride)), kT, 0, st, part, splits, stride, stride,
+                      out);
+}
+
 // How a convolution runs on k_conv_march: blocks of kb channels, cb of them, bn output columns per
 // CTA; kb = 0: it does not. Maps: source 1 (dY for the data gradient) and source 2 as boxes of one
 // row of 136 pixels x kb channels, weights as kb x bn blocks.
@@ -783,7 +807,6 @@ cudaError_t conv_march(cudaStream_t st, const GemmArgs& a, const March& m, const
     const int key = m.kb * 1000 + m.cb * 100 + m.bn;
     if constexpr (!GD) {
         if (a.conv.up1) switch (key) {
-                case 32132: return launch_march<32, 1, 32, false, true>(st, a, maps);
                 case 32116: return launch_march<32, 1, 16, false, true>(st, a, maps);
                 case 32232: return launch_march<32, 2, 32, false, true>(st, a, maps);
                 default: return cudaErrorInvalidValue;
@@ -804,18 +827,9 @@ cudaError_t conv_march(cudaStream_t st, const GemmArgs& a, const March& m, const
 // the forms conv_march has
 bool march_form(const March& m, bool up) {
     const int key = m.kb * 1000 + m.cb * 100 + m.bn;
-    if (up) return key == 32132 || key == 32116 || key == 32232;
+    if (up) return key == 32116 || key == 32232;
     return key == 16116 || key == 16132 || key == 16216 || key == 32116 || key == 32132 ||
            key == 32164 || key == 32232 || key == 32264;
-}
-
-// out = the sum of `splits` FP32 partials of `stride` values each, in split order
-cudaError_t sum_splits(cudaStream_t st, const float* part, int splits, long long stride, float* out) {
-    if (stride % 4 == 0 && ((uintptr_t)out & 15) == 0)
-        return launch_pdl(k_splitk_sum4, dim3((unsigned)((stride / 4 + 31) / 32)), 256, 0, st, part,
-                          splits, stride, stride, out);
-    return launch_pdl(k_splitk_sum, dim3(blocks_for(stride)), kT, 0, st, part, splits, stride, stride,
-                      out);
 }
 
 // The weight gradient through k_gemm_wwin (a: the transposed, gathered form of gemm_wgrad):
@@ -964,6 +978,12 @@ void build(lbm_surrogate* s) {
     s->nparams += 1;
 }
 
+// the main stream waits for what the side stream holds so far
+cudaError_t join_side(lbm_surrogate* s) {
+    const cudaError_t e = cudaEventRecord(s->side_done, s->side);
+    return e == cudaSuccess ? cudaStreamWaitEvent(s->stream, s->side_done, 0) : e;
+}
+
 // the head on the last activation; with a target (training) also its loss terms and gradients
 cudaError_t launch_head(lbm_surrogate* s, int blocks, float* phi, long long P, const float* target,
                         const uint8_t* mask) {
@@ -1072,7 +1092,8 @@ void make_tensor_maps(lbm_surrogate* s) {
                 c.C2 == 0 && tma_width(pick_bn(c.Cout)) &&
                 map_nhwc(&c.fmap[0], s->t[c.src1].y, c.C1, W / 2, H / 2, s->maxB,
                          std::min(W, 128) / 2, 1, fk) &&
-                map_rows(&c.fmap[2], s->wb + c.w_off, 9 * c.C1, c.Cout, pick_bn(c.Cout), fk))
+                map_rows(&c.fmap[2], s->wb + c.w_off, 9 * c.C1, c.Cout, pick_bn(c.Cout), fk) &&
+                map_rows(&c.fmap[3], s->wb + c.w_off, 9 * c.C1, c.Cout, 32, fk))
                 c.f_ks = fk;
             // data gradient of an upsampling convolution: rows are source pixels (half
             // resolution), the output gradient read every second pixel; B wraps every 9 Cout
@@ -1081,7 +1102,8 @@ void make_tensor_maps(lbm_surrogate* s) {
                 (9 * c.Cout) % dk == 0 && tma_width(pick_bn(cin))) {
                 const int bw = std::min(Ws, 128), bh = 128 / bw;
                 if (map_nhwc(&c.dmap[0], c.g, c.Cout, W, H, s->maxB, bw, bh, dk, 2) &&
-                    map_rows(&c.dmap[2], s->wbd + c.w_off, 9 * c.Cout, cin, pick_bn(cin), dk))
+                    map_rows(&c.dmap[2], s->wbd + c.w_off, 9 * c.Cout, cin, pick_bn(cin), dk) &&
+                    map_rows(&c.dmap[3], s->wbd + c.w_off, 9 * c.Cout, cin, 32, dk))
                     c.d_ks = dk;
             }
             // weight gradient: 32 source pixels x 32 channels per box, and 32 output-gradient
@@ -1099,7 +1121,8 @@ void make_tensor_maps(lbm_surrogate* s) {
         if (fk && tma_width(pick_bn(c.Cout)) &&
             map_nhwc(&c.fmap[0], s->t[c.src1].y, c.C1, W, H, s->maxB, bw, bh, fk) &&
             (c.src2 < 0 || map_nhwc(&c.fmap[1], s->t[c.src2].y, c.C2, W, H, s->maxB, bw, bh, fk)) &&
-            map_rows(&c.fmap[2], s->wb + c.w_off, 9 * cin, c.Cout, pick_bn(c.Cout), fk))
+            map_rows(&c.fmap[2], s->wb + c.w_off, 9 * cin, c.Cout, pick_bn(c.Cout), fk) &&
+            map_rows(&c.fmap[3], s->wb + c.w_off, 9 * cin, c.Cout, 32, fk))
             c.f_ks = fk;
         if (W % 64 == 0 && c.C1 % 32 == 0 && c.C2 % 32 == 0 && (cin == 32 || cin == 64) &&
             (c.Cout == 32 || c.Cout == 64)) {
@@ -1121,7 +1144,8 @@ void make_tensor_maps(lbm_surrogate* s) {
         }
         if (dk && tma_width(pick_bn(cin)) &&
             map_nhwc(&c.dmap[0], c.g, c.Cout, W, H, s->maxB, bw, bh, dk) &&
-            map_rows(&c.dmap[2], s->wbd + c.w_off, 9 * c.Cout, cin, pick_bn(cin), dk))
+            map_rows(&c.dmap[2], s->wbd + c.w_off, 9 * c.Cout, cin, pick_bn(cin), dk) &&
+            map_rows(&c.dmap[3], s->wbd + c.w_off, 9 * c.Cout, cin, 32, dk))
             c.d_ks = dk;
     }
 }
@@ -1297,10 +1321,15 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         else
             SCUDA(s, launch_pdl(dyp ? k_relu_bias<1> : k_relu_bias<0>, dim3(rb), kT, 0, s->stream,
                                 o.dy, dyp, nullptr, o.y, c.g, n_out / 8, c.Cout, c.H, c.W, c.bpart));
-        // the side stream takes the bias and weight gradients from here
-        SCUDA(s, cudaEventRecord(c.ready, s->stream));
-        SCUDA(s, cudaStreamWaitEvent(s->side, c.ready, 0));
-        SCUDA(s, launch_pdl(k_colsum_final, dim3(c.Cout), kT, 0, s->side, c.bpart, rb, c.Cout,
+        // the side stream takes the bias and weight gradients from here; the first convolution's
+        // stay on the main stream, which has nothing left to do by then
+        const bool last = c.src1 == 0;
+        cudaStream_t ws = last ? s->stream : s->side;
+        if (!last) {
+            SCUDA(s, cudaEventRecord(c.ready, s->stream));
+            SCUDA(s, cudaStreamWaitEvent(s->side, c.ready, 0));
+        }
+        SCUDA(s, launch_pdl(k_colsum_final, dim3(c.Cout), kT, 0, ws, c.bpart, rb, c.Cout,
                             s->g + c.b_off, 1, nullptr));
         // weight gradient: dW[co][k] = sum_p g[p][co] col[p][k], the im2col columns gathered by
         // the GEMM's loader when the resolution allows (powers of two), else from a buffer
@@ -1316,7 +1345,9 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         gw.conv.lh = ilog2_exact(c.H);
         gw.conv.lw = ilog2_exact(c.W);
         const bool gather = gw.conv.lh >= 0 && gw.conv.lw >= 0;
-        if (!gather) SCUDA(s, launch_im2col(s, s->side, c, B));
+        if (!gather && last)  // the side stream's last im2col may still be read
+            SCUDA(s, join_side(s));
+        if (!gather) SCUDA(s, launch_im2col(s, ws, c, B));
         gw.A = c.g;
         gw.B = s->col;
         gw.M = c.Cout;
@@ -1325,7 +1356,7 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         gw.lda = c.Cout;
         gw.ldb = 9 * Cin;
         gw.ldc = 9 * Cin;
-        SCUDA(s, gemm_wgrad(s->side, gw, s->splitk_side, s->splitk_elems, s->g + c.w_off, gather,
+        SCUDA(s, gemm_wgrad(ws, gw, last ? s->splitk : s->splitk_side, s->splitk_elems, s->g + c.w_off, gather,
                             gather && c.w_tma ? c.wmap : nullptr, gather ? c.ww_cb : 0, c.wwmap));
         // data gradient (not needed for the input tensor)
         if (c.src1 == 0) continue;
@@ -1366,8 +1397,7 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
             SCUDA(s, (gemm_tc_split<false, true>(s->stream, gd, s->splitk, s->splitk_elems,
                                                   c.dmap, c.d_ks)));
     }
-    SCUDA(s, cudaEventRecord(s->side_done, s->side));
-    SCUDA(s, cudaStreamWaitEvent(s->stream, s->side_done, 0));
+    SCUDA(s, join_side(s));
     if (lr > 0.f) {
         ++s->adam_t;
         const float b1 = 0.9f, b2 = 0.999f;

@@ -323,11 +323,10 @@ __device__ __forceinline__ void epilogue_tile(const sg::GemmArgs& g, uint32_t ta
                                               size_t zoff) {
     // FP32 outputs may accumulate and may be split at column nsplit into two tensors; the
     // vector path then takes a 32-column chunk that lies on one side of the split
-    const bool vec = !g.kchunk &&
-                     (g.Cb ? (!g.accumulate && g.ldc % 8 == 0 && ((uintptr_t)g.Cb & 15) == 0)
-                           : (g.ldc % 4 == 0 && ((uintptr_t)g.Cf & 15) == 0 &&
-                              (!g.Cf2 || (g.ldc2 % 4 == 0 && g.nsplit % 4 == 0 &&
-                                          ((uintptr_t)g.Cf2 & 15) == 0))));
+    const bool vec = g.Cb ? (!g.accumulate && g.ldc % 8 == 0 && ((uintptr_t)g.Cb & 15) == 0)
+                          : (g.ldc % 4 == 0 && zoff % 4 == 0 && ((uintptr_t)g.Cf & 15) == 0 &&
+                             (!g.Cf2 || (g.ldc2 % 4 == 0 && g.nsplit % 4 == 0 &&
+                                         ((uintptr_t)g.Cf2 & 15) == 0)));
 #pragma unroll 1
     for (int c0 = 0; c0 < BN; c0 += 32) {
         if (n0 + c0 >= g.N) break;
@@ -402,7 +401,7 @@ __device__ __forceinline__ void epilogue_tile(const sg::GemmArgs& g, uint32_t ta
                     return (g.Cf2 && n >= g.nsplit)
                                ? reinterpret_cast<float4*>(g.Cf2 + (size_t)m * g.ldc2 +
                                                            (n - g.nsplit))
-                               : reinterpret_cast<float4*>(g.Cf + (size_t)m * g.ldc + n);
+                               : reinterpret_cast<float4*>(g.Cf + (size_t)m * g.ldc + n + zoff);
                 };
                 float4 old[8];
                 if (g.accumulate) {
