@@ -631,7 +631,9 @@ bool map_rows(CUtensorMap* m, const void* base, int K, int rows, int box_rows, i
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// CTAs of a launch up to which gemm_tc_tma takes its narrow, deep form.
+// CTAs of a launch up to which gemm_tc_tma takes its narrow, deep form: with it a forward pass of one
+// 256 x 256 sample (base 32) takes 284 us, without it 304. Launches of more CTAs hide their slices'
+// latency behind one another and would only read the A rows of a tile once per 32 columns.
 constexpr long long kFewTiles = 128;
 
 // The TMA-fed gathering GEMM (GA or GD with tensor maps, see Conv::fmap / dmap), ks elements
@@ -800,6 +802,53 @@ cudaError_t launch_march(cudaStream_t st, const GemmArgs& a, const CUtensorMap* 
     const dim3 grid((unsigned)strips * ((rh + chunk - 1) / chunk), nb);
     return launch_pdl(kern, grid, lbm::sgtc::MARCH_THREADS, MS::SMEM, st, a, flag, maps[0], maps[1],
                       maps[2], chunk);
+}
+
+// The first convolution on k_conv0 / k_wgrad0: rows a multiple of 128 pixels, 16 or 32 outputs and an
+// input the copy engine can address (the maps are made per call, x being the caller's).
+bool conv0_ok(const Conv& c, const void* x) {
+    return c.C1 == 8 && c.C2 == 0 && !c.up1 && c.W % 128 == 0 && (c.Cout == 16 || c.Cout == 32) &&
+           ((uintptr_t)x & 15) == 0;
+}
+
+template <int N>
+cudaError_t launch_conv0(cudaStream_t st, const GemmArgs& a, const CUtensorMap& mx) {
+    int* flag = tc_flag().dev;
+    if (!flag) return cudaErrorMemoryAllocation;
+    const unsigned ctas = (unsigned)(a.M / (128 * lbm::sgtc::C0_ROWS));
+    return launch_pdl(lbm::sgtc::k_conv0<N>, dim3(ctas), lbm::sgtc::TC_THREADS,
+                      lbm::sgtc::Conv0Shape<N>::SMEM, st, a, flag, mx);
+}
+
+template <int N>
+cudaError_t launch_wgrad0(cudaStream_t st, GemmArgs a, float* scratch, float* out, const CUtensorMap& mx,
+                          const CUtensorMap& mdy) {
+    using WS = lbm::sgtc::Wgrad0Shape<N>;
+    static std::atomic<unsigned long long> configured{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(configured.load() & bit)) {
+        e = cudaFuncSetAttribute(lbm::sgtc::k_wgrad0<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 WS::SMEM);
+        if (e != cudaSuccess) return e;
+        configured.fetch_or(bit);
+    }
+    int* flag = tc_flag().dev;
+    if (!flag) return cudaErrorMemoryAllocation;
+    // K ranges of at least four slices, at most two per SM
+    const int slices = a.K / 128;
+    int splits = std::max(1, std::min(304, slices / 4));
+    const int per = (slices + splits - 1) / splits;
+    splits = (slices + per - 1) / per;
+    const long long stride = (long long)N * 72;
+    a.kchunk = per * 128;
+    a.split_stride = splits > 1 ? stride : 0;
+    a.Cf = splits > 1 ? scratch : out;
+    e = launch_pdl(lbm::sgtc::k_wgrad0<N>, dim3(splits), lbm::sgtc::TC_THREADS, WS::SMEM, st, a, flag, mx,
+                   mdy);
+    return e != cudaSuccess || splits == 1 ? e : sum_splits(st, scratch, splits, stride, out);
 }
 
 template <bool GD>
@@ -1021,7 +1070,12 @@ lbm_status forward(lbm_surrogate* s, const bf16* x, int B) {
         g.bias = s->w + c.b_off;
         g.relu = 1;
         if (c.up1 && c.f_ks) g.rperm = std::min(c.W, 128) / 2;
-        if (c.fm.kb)
+        CUtensorMap mx;
+        if (c.src1 == 0 && conv0_ok(c, a.y) &&
+            map_nhwc(&mx, a.y, 8, c.W, c.H, B, lbm::sgtc::C0_PITCH, lbm::sgtc::C0_ROWS + 2, 8))
+            SCUDA(s, c.Cout == 32 ? launch_conv0<32>(s->stream, g, mx)
+                                  : launch_conv0<16>(s->stream, g, mx));
+        else if (c.fm.kb)
             SCUDA(s, conv_march<false>(s->stream, g, c.fm, c.fmmap));
         else
             SCUDA(s, (gemm_tc_split<true, false>(s->stream, g, s->splitk, s->splitk_elems, c.fmap,
@@ -1344,6 +1398,16 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         gw.conv.lc = ilog2_exact(Cin);
         gw.conv.lh = ilog2_exact(c.H);
         gw.conv.lw = ilog2_exact(c.W);
+        CUtensorMap mx, mdy;
+        if (last && conv0_ok(c, gw.conv.x1) && s->splitk_elems >= (size_t)304 * c.Cout * 72 &&
+            map_nhwc(&mx, gw.conv.x1, 8, c.W, c.H, B, lbm::sgtc::C0_PITCH, 3, 8) &&
+            map_nhwc(&mdy, c.g, c.Cout, c.W, c.H, B, 128, 1, c.Cout)) {
+            gw.K = (int)Pc;
+            SCUDA(s, c.Cout == 32
+                         ? launch_wgrad0<32>(ws, gw, s->splitk, s->g + c.w_off, mx, mdy)
+                         : launch_wgrad0<16>(ws, gw, s->splitk, s->g + c.w_off, mx, mdy));
+            continue;  // no data gradient for the input tensor
+        }
         const bool gather = gw.conv.lh >= 0 && gw.conv.lw >= 0;
         if (!gather && last)  // the side stream's last im2col may still be read
             SCUDA(s, join_side(s));

@@ -73,7 +73,10 @@ __device__ __forceinline__ uint32_t su32(const void* p) {
 //   32-byte (16): 256 B. MN-major, 64-byte swizzle: groups 512 B, 32-wide blocks lbo apart;
 //   128-byte swizzle: groups 1 KB, 64-wide blocks 8 KB apart.
 // A start may lie on any whole row of the layout: the swizzle follows the absolute address.
-enum Swizzle { SW128 = 2, SW64 = 4, SW32 = 6 };
+//   Without swizzle the unit is a core matrix of 8 rows x 16 bytes (128 contiguous bytes): K-major,
+//   groups = the next 8 rows and lbo = the next 8 K; MN-major (8 K rows of 8 M or N values),
+//   groups = the next 8 M or N and lbo = the next 8 K.
+enum Swizzle { SW_NONE = 0, SW128 = 2, SW64 = 4, SW32 = 6 };
 __host__ __device__ constexpr uint32_t desc_hi(int group_bytes, Swizzle sw) {
     return (uint32_t)(group_bytes >> 4) | (1u << 14) | ((uint32_t)sw << 29);
 }
@@ -1167,6 +1170,265 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && !s_ok) atomicExch(err, 1);
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(COLS)
+                     : "memory");
+    }
+}
+
+// The network's first convolution: 8 input channels (16 bytes per pixel), N = 16 or 32 outputs. The
+// input window sits in shared memory as it does in memory, one 16-byte row per pixel, which is the
+// unswizzled K-major layout: a tap is a start address, and the second eight K of an MMA is the next
+// tap, whose distance is the descriptor's lbo. Five MMAs (taps 0+1, 2+3, 4+5, 6+7, 8+zeros) per
+// tile of 128 pixels of one row, four rows per CTA from one window of six. Bound by the 64 + 16
+// bytes per pixel it moves; gathering 72 columns per pixel with 16-byte copies (k_gemm_tc, two
+// 64-wide slices) took 63 us at 256 x 256 x 8 and 32 outputs; this takes 15.
+constexpr int C0_ROWS = 4, C0_PITCH = 136;
+template <int N>
+struct Conv0Shape {
+    static constexpr int WIN = (C0_ROWS + 2) * C0_PITCH * 16, ZERO = 128 * 16, WGT = 10 * N * 16;
+    // as much as keeps the CTAs of an SM within the 512 tensor-memory columns
+    static constexpr int RAW = 128 + WIN + ZERO + WGT;
+    static constexpr int MIN_BYTES = 233472 / (512 / (int)tmem_pow2(C0_ROWS * N) + 1) + 1;
+    static constexpr int SMEM = RAW > MIN_BYTES ? RAW : MIN_BYTES;
+};
+
+template <int N>
+__global__ void __launch_bounds__(TC_THREADS)
+    k_conv0(const sg::GemmArgs g, int* err, const __grid_constant__ CUtensorMap tmX) {
+    using S = Conv0Shape<N>;
+    constexpr uint32_t COLS = tmem_pow2(C0_ROWS * N);
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    const uint32_t raw = su32(smem_raw);
+    uint8_t* base = smem_raw + ((128u - (raw & 127u)) & 127u);
+    uint8_t* wgt = base + S::WIN + S::ZERO;
+    __shared__ __align__(8) uint64_t bars[2];
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_ok;
+    __shared__ float s_bias[N];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int H = g.conv.H, W = g.conv.W, strips = W / 128, bands = H / C0_ROWS;
+    const int st = blockIdx.x % strips, q = blockIdx.x / strips, band = q % bands, img = q / bands;
+    const int x0 = st * 128, y0 = band * C0_ROWS;
+    if (tid == 0) {
+        mbar_init(su32(bars), 1);
+        mbar_init(su32(bars + 1), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        s_ok = 1;
+    }
+    // zeros behind the window: the K = 72 .. 79 half of the last MMA
+    for (int i = tid; i < S::ZERO / 16; i += TC_THREADS)
+        reinterpret_cast<uint4*>(base + S::WIN)[i] = make_uint4(0, 0, 0, 0);
+    sg::pdl_wait();
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                         su32(&s_tmem)),
+                     "r"(COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    // weights [n][tap][8] as core matrices of eight n: tap-major, then n / 8; tap 9 is zero
+    for (int i = tid; i < 10 * N; i += TC_THREADS) {
+        const int tap = i / N, n = i - tap * N;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (tap < 9) v = *reinterpret_cast<const uint4*>(g.B + (size_t)n * 72 + tap * 8);
+        *reinterpret_cast<uint4*>(wgt + i * 16) = v;
+    }
+    if (tid < N) s_bias[tid] = g.bias[tid];
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    sg::pdl_next();
+    const uint32_t tmem = s_tmem;
+    if (tid == 0) {
+        const uint32_t full = su32(bars), fin = su32(bars + 1), win = su32(base);
+        mbar_expect_tx(full, (uint32_t)S::WIN);
+        tma_load_4d(win, &tmX, full, 0, x0 - 4, y0 - 1, img);
+        bool good = mbar_wait(full, 0);
+        if (good) {
+            tc_fence_after();
+            constexpr uint32_t HI = desc_hi(128, SW_NONE), IDESC = idesc_bf16(BM, N, 0, 0);
+            const uint32_t zero = win + S::WIN;
+#pragma unroll
+            for (int r = 0; r < C0_ROWS; ++r)
+#pragma unroll
+                for (int p = 0; p < 5; ++p) {
+                    const int t = 2 * p, u = 2 * p + 1;
+                    const uint32_t a = win + ((r + t / 3) * C0_PITCH + 3 + t % 3) * 16;
+                    const uint32_t b = u < 9 ? win + ((r + u / 3) * C0_PITCH + 3 + u % 3) * 16 : zero;
+                    tc_mma(tmem + (uint32_t)(r * N), desc_lo(a, b - a), HI,
+                           desc_lo(su32(wgt) + t * N * 16, N * 16), HI, IDESC, p > 0 ? 1u : 0u);
+                }
+            tc_commit(fin);
+            good = mbar_wait(fin, 0);
+        } else {
+            mbar_wait(full, 0);  // let the copy land (bounded)
+        }
+        if (!good) s_ok = 0;
+    }
+    __syncthreads();
+    if (!s_ok) {
+        if (tid == 0) atomicExch(err, 1);
+    } else {
+        tc_fence_after();
+#pragma unroll
+        for (int r = 0; r < C0_ROWS; ++r) {
+            float v[32];
+            const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(r * N);
+            if (N == 32)
+                tc_ld32(ta, v);
+            else
+                tc_ld16(ta, v);
+            const size_t m = ((size_t)img * H + y0 + r) * W + x0 + warp * 32 + lane;
+#pragma unroll
+            for (int c = 0; c < N; c += 16) {
+                uint32_t o[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    float a0 = v[c + 2 * i] + s_bias[c + 2 * i];
+                    float a1 = v[c + 2 * i + 1] + s_bias[c + 2 * i + 1];
+                    a0 = fmaxf(a0, 0.1f * a0);
+                    a1 = fmaxf(a1, 0.1f * a1);
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(a0, a1);
+                    o[i] = *reinterpret_cast<const uint32_t*>(&h);
+                }
+                st_global_32B(g.Cb + m * N + c, o);
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(COLS)
+                     : "memory");
+    }
+}
+
+// Its weight gradient, dW^T[(tap, ci)][co] = sum over pixels x(p + off(tap))[ci] dY(p)[co], from the
+// same 16-byte pixel rows: as an unswizzled MN-major operand the next eight M are the pixel 16
+// bytes on, i.e. the next dx, so one MMA of M = 128 covers dx = -1, 0, 1 (blocks 0-2; the other
+// blocks read further pixels and their rows are dropped), with one accumulator per dy. Slices of 128
+// pixels of one row (K), each CTA one split-K range of them; the partial is stored as
+// [co][tap][ci]. 256 x 256 x 8, 32 outputs: 98 us with the 72 columns gathered per pixel, 24 here.
+template <int N>
+struct Wgrad0Shape {
+    static constexpr int STAGES = 4, WIN = 3 * C0_PITCH * 16, DY = 128 * N * 2, STAGE = WIN + DY;
+    // window sizes are multiples of 128 bytes, so every dY block stays aligned to its swizzle when
+    // the dY blocks come first; 512 bytes behind the last window for the dropped rows' reads
+    static constexpr int SMEM = 1024 + STAGES * STAGE + 512 + 8 * (2 * STAGES + 1);
+};
+template <int N>
+__global__ void __launch_bounds__(TC_THREADS)
+    k_wgrad0(const sg::GemmArgs g, int* err, const __grid_constant__ CUtensorMap tmX,
+             const __grid_constant__ CUtensorMap tmDY) {
+    using S = Wgrad0Shape<N>;
+    constexpr int STAGES = S::STAGES;
+    constexpr uint32_t COLS = tmem_pow2(3 * N);
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    const uint32_t raw = su32(smem_raw);
+    uint8_t* base = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
+    auto dyb = [&](int st) { return su32(base) + st * S::DY; };
+    auto win = [&](int st) { return su32(base) + STAGES * S::DY + st * S::WIN; };
+    uint64_t* bars = reinterpret_cast<uint64_t*>(base + STAGES * S::STAGE + 512);
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_ok;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int kb = blockIdx.x * g.kchunk, ke = min(g.K, kb + g.kchunk);
+    const int nk = ke > kb ? (ke - kb) / 128 : 0;
+    if (tid == 0) {
+        for (int i = 0; i <= 2 * STAGES; ++i) mbar_init(su32(bars + i), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        s_ok = 1;
+    }
+    sg::pdl_wait();
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                         su32(&s_tmem)),
+                     "r"(COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    sg::pdl_next();
+    const uint32_t tmem = s_tmem;
+    const int H = g.conv.H, W = g.conv.W;
+    auto issue = [&](int st, int k0) {
+        const uint32_t full = su32(bars + st);
+        mbar_expect_tx(full, (uint32_t)S::STAGE);
+        const int pn = k0 / (H * W), pr = k0 - pn * (H * W), py = pr / W, px = pr - py * W;
+        tma_load_4d(win(st), &tmX, full, 0, px - 4, py - 1, pn);
+        tma_load_4d(dyb(st), &tmDY, full, 0, px, py, pn);
+    };
+    if (tid == 0) {
+        constexpr uint32_t IDESC = idesc_bf16(BM, N, 1, 1), AHI = desc_hi(16, SW_NONE);
+        constexpr uint32_t BHI = N == 32 ? desc_hi(512, SW64) : desc_hi(256, SW32);
+        int issued = 0, done_mma = 0;
+        bool good = true;
+        for (; issued < STAGES && issued < nk; ++issued) issue(issued, kb + issued * 128);
+        for (int kt = 0; kt < nk; ++kt) {
+            const int st = kt % STAGES;
+            if (!mbar_wait(su32(bars + st), (kt / STAGES) & 1)) {
+                good = false;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t a0 = desc_lo(win(st) + 3 * 16, 128), b0 = desc_lo(dyb(st), 4096);
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    tc_mma(tmem + (uint32_t)(dy * N), a0 + dy * C0_PITCH + 16 * j, AHI,
+                           b0 + (uint32_t)((j * 16 * N * 2) >> 4), BHI, IDESC, (kt > 0 || j > 0) ? 1u : 0u);
+            tc_commit(su32(bars + STAGES + st));
+            done_mma = kt + 1;
+            if (kt >= 1 && issued < nk) {
+                const int sp = (kt - 1) % STAGES;
+                if (!mbar_wait(su32(bars + STAGES + sp), ((kt - 1) / STAGES) & 1)) {
+                    good = false;
+                    break;
+                }
+                issue(sp, kb + issued * 128);
+                ++issued;
+            }
+        }
+        if (!good)
+            for (int j = done_mma; j < issued; ++j) mbar_wait(su32(bars + j % STAGES), (j / STAGES) & 1);
+        if (nk > 0) {
+            tc_commit(su32(bars + 2 * STAGES));
+            if (!mbar_wait(su32(bars + 2 * STAGES), 0)) good = false;
+        }
+        if (!good) s_ok = 0;
+    }
+    __syncthreads();
+    if (!s_ok) {
+        if (tid == 0) atomicExch(err, 1);
+    } else if (warp == 0) {
+        // lane: block dx = lane / 8 - 1 (the first three), channel lane % 8
+        tc_fence_after();
+        float* out = g.Cf + (size_t)blockIdx.x * g.split_stride;
+#pragma unroll 1
+        for (int dy = 0; dy < 3; ++dy) {
+            float v[32];
+            if (nk == 0) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] = 0.f;
+            } else if (N == 32) {
+                tc_ld32(tmem + (uint32_t)(dy * N), v);
+            } else {
+                tc_ld16(tmem + (uint32_t)(dy * N), v);
+            }
+            if (lane < 24)
+#pragma unroll
+                for (int n = 0; n < N; ++n) out[n * 72 + dy * 24 + lane] = v[n];
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(COLS)
