@@ -28,7 +28,9 @@ namespace {
 using namespace stepdev;
 
 // the interpolated bounce-back kernels exist for the default variant (32 x 16 tiles, 5 CTAs per SM)
-// and its small-lattice forms
+// and its small-lattice forms; the fractions and populations of a node's cut links in flight take
+// registers that five CTAs per SM would spill
+constexpr int kIbbBlocks = 4;
 template <typename T, int TX, int TY, int MINB>
 constexpr bool has_ibb() {
     return TX == 32 && TY == 16 && MINB == 5;
@@ -84,8 +86,8 @@ cudaError_t configure_one() {
     cudaError_t e = allow_smem<T, TX, TY, 256, MINB, false, false>();
     if (e == cudaSuccess) e = allow_smem<T, TX, TY, 256, MINB, true, false>();
     if constexpr (has_ibb<T, TX, TY, MINB>()) {
-        if (e == cudaSuccess) e = allow_smem<T, TX, TY, 256, MINB, false, true>();
-        if (e == cudaSuccess) e = allow_smem<T, TX, TY, 256, MINB, true, true>();
+        if (e == cudaSuccess) e = allow_smem<T, TX, TY, 256, kIbbBlocks, false, true>();
+        if (e == cudaSuccess) e = allow_smem<T, TX, TY, 256, kIbbBlocks, true, true>();
     }
     if constexpr (has_ibb<T, TX, TY, MINB>()) {
 #define X(F, A, B, N, M)                                                       \
@@ -110,8 +112,8 @@ cudaError_t launch_one(lbm_ctx* c, const StepArgs<T>& a, bool macro) {
     }
     if (c->ibb) {
         if constexpr (has_ibb<T, TX, TY, MINB>())
-            return macro ? launch_k<T, TX, TY, 256, MINB, true, true>(c, a)
-                         : launch_k<T, TX, TY, 256, MINB, false, true>(c, a);
+            return macro ? launch_k<T, TX, TY, 256, kIbbBlocks, true, true>(c, a)
+                         : launch_k<T, TX, TY, 256, kIbbBlocks, false, true>(c, a);
         return cudaErrorInvalidValue;
     }
     return macro ? launch_k<T, TX, TY, 256, MINB, true, false>(c, a)

@@ -196,19 +196,24 @@ __device__ __forceinline__ T ibb_return(int q, int o, T rho, T out, T D, T alt, 
     return fma_rn(c, out, mul_rn(sub_rn((T)1, c), alt));  // exactly out at D = 1/2
 }
 
-// The link fractions and the further populations that ibb_return needs, of all cut links of a
-// node: first every fraction is loaded, then every population, so that a node with several cut
+// The link fractions of a node's cut links, and the further population that ibb_return needs of
+// each: first every fraction is loaded, then every population, so that a node with several cut
 // links waits for two memory latencies and not for two per link (that chain was most of the
 // interpolated step's time on small lattices: 17.5 us per step against 8.9 half-way on 520 x 190).
-template <typename T, int RW, bool PP>
-__device__ __forceinline__ void ibb_gather(const StepArgs<T>& a, unsigned us, int o,
-                                           const uint8_t* s_flag, T (&D)[9], T (&alt)[9]) {
-    const unsigned upl = (unsigned)a.plane;
+template <typename T, int RW>
+__device__ __forceinline__ void ibb_fractions(const StepArgs<T>& a, unsigned us, int o,
+                                              const uint8_t* s_flag, T (&D)[9]) {
 #pragma unroll
     for (int q = 1; q < 9; ++q) {
         D[q] = (T)0.5;
-        if (s_flag[o - qy(q) * RW - qx(q)] != kFluid) D[q] = __ldg(a.dlt + (unsigned)(q - 1) * upl + us);
+        if (s_flag[o - qy(q) * RW - qx(q)] != kFluid)
+            D[q] = __ldg(a.dlt + (unsigned)(q - 1) * (unsigned)a.plane + us);
     }
+}
+template <typename T, int RW, bool PP>
+__device__ __forceinline__ void ibb_populations(const StepArgs<T>& a, unsigned us, int o,
+                                                const uint8_t* s_flag, const T (&D)[9], T (&alt)[9]) {
+    const unsigned upl = (unsigned)a.plane;
 #pragma unroll
     for (int q = 1; q < 9; ++q) {
         alt[q] = (T)0;
@@ -216,12 +221,32 @@ __device__ __forceinline__ void ibb_gather(const StepArgs<T>& a, unsigned us, in
         if (D[q] < (T)0.5) {
             if (s_flag[o + qy(q) * RW + qx(q)] == kFluid) {
                 const unsigned ub = us + (unsigned)(qy(q) * a.P + qx(q));
-                alt[q] = PP ? a.hq_in[qopp(q)][ub]
-                            : a.h_in[(unsigned)qopp(q) * upl + ub];
+                alt[q] = PP ? a.hq_in[qopp(q)][ub] : a.h_in[(unsigned)qopp(q) * upl + ub];
             }
         } else {
             alt[q] = PP ? a.hq_in[q][us] : a.h_in[(unsigned)q * upl + us];
         }
+    }
+}
+
+// The nine populations that arrive at a node (Eq. 4): h_q of the source x - e_q, or where that is
+// not fluid the one that left toward it (half-way bounce-back).
+template <typename T, int RW, bool MIXED, bool PP>
+__device__ __forceinline__ void pull(const StepArgs<T>& a, unsigned us, int o, const uint8_t* s_flag,
+                                     T (&h)[9]) {
+    const unsigned upl = (unsigned)a.plane, uP = (unsigned)a.P;
+    // PP: per-plane pointers; else 32-bit element offsets of plane q and of its pulled source (the
+    // same for every thread, so they live in uniform registers)
+    const T* hb = a.h_in + us;
+    const unsigned rdn = us - uP, rup = us + uP;  // rows of the sources with e_q,y = +1, -1
+    h[0] = PP ? a.hq_in[0][us] : *hb;
+#pragma unroll
+    for (int q = 1; q < 9; ++q) {
+        if (!MIXED || s_flag[o - qy(q) * RW - qx(q)] == kFluid)
+            h[q] = PP ? *(a.hq_in[q] + (int)((qy(q) > 0 ? rdn : qy(q) < 0 ? rup : us) - qx(q)))
+                      : *(hb + (int)((unsigned)q * upl - (unsigned)(qy(q) * (int)uP + qx(q))));
+        else
+            h[q] = PP ? a.hq_in[qopp(q)][us] : *(hb + (int)((unsigned)qopp(q) * upl));
     }
 }
 
@@ -298,6 +323,25 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid,
     (void)RH;
     (void)rho_mid;
 
+    // With a thread for every collision node (the small-lattice forms) its populations, and on cut
+    // links what interpolated bounce-back needs, are loaded here and arrive while the layers and the
+    // chemical potential are computed.
+    constexpr bool EARLY = NT >= CW * CH;
+    T eh[9], eD[9], ealt[9];
+    bool mine = false;
+    unsigned eus = 0;
+    int eo = 0;
+    if (EARLY) {
+        const int cy = tid / CW, cx = tid - cy * CW;
+        eo = (cy + 6) * RW + (cx + 7);
+        eus = (unsigned)lidx(a.P, x0 - 1 + cx, y0 - 1 + cy);
+        mine = tid < CW * CH && (!MIXED || s_flag[eo] == kFluid);
+        if (mine) {
+            pull<T, RW, MIXED, PP>(a, eus, eo, s_flag, eh);
+            if (MIXED && IBB) ibb_fractions<T, RW>(a, eus, eo, s_flag, eD);
+        }
+    }
+
     if (MIXED) {
         // (2) first wetting layer (Eq. 14, switch on fluid neighbours)
         for (int idx = tid; idx < (RW - 2) * (RH - 2); idx += NT) {
@@ -316,6 +360,7 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid,
             s_rho[o] = den > (T)0 ? num / den : rho_mid;
         }
         __syncthreads();
+        if (EARLY && IBB && mine) ibb_populations<T, RW, PP>(a, eus, eo, s_flag, eD, ealt);
         // (3) second wetting layer (switch on first-layer neighbours)
         for (int idx = tid; idx < (RW - 4) * (RH - 4); idx += NT) {
             const int ly = 2 + idx / (RW - 4), lx = 2 + idx % (RW - 4);
@@ -356,11 +401,6 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid,
     __syncthreads();
 
     // (5) force and collision on tile + 1
-    // PP = false: 32-bit element offsets of plane q and of the pulled source of direction q
-    // (the same for every thread, so they live in uniform registers)
-    const unsigned upl = (unsigned)a.plane, uP = (unsigned)a.P;
-#define QPL(q) ((unsigned)(q) * upl)
-#define QSRC(q) ((unsigned)(q) * upl - (unsigned)(qy(q) * (int)uP + qx(q)))
     for (int idx = tid; idx < CW * CH; idx += NT) {
         const int cy = idx / CW, cx = idx - cy * CW;
         const int o = (cy + 6) * RW + (cx + 7);
@@ -381,14 +421,25 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid,
                              sub_rn(s_rho[o - 2 * RW], s_rho[o + 2 * RW]));
         const T Fx = fma_rn(rho, fma_rn(Gmx, (T)-1 / (T)12, a.gx), fma_rn(Grx, (T)1 / (T)36, a.gbx));
         const T Fy = fma_rn(rho, fma_rn(Gmy, (T)-1 / (T)12, a.gy), fma_rn(Gry, (T)1 / (T)36, a.gby));
-        // pull the populations of time t (Eq. 4) with half-way bounce-back
+        // the pulled populations of time t as deviations from w_q rho(x)
         const unsigned us = (unsigned)self;
-        const T* hb = a.h_in + us;
-        // PP: rows of the sources with e_q,y = 0, +1, -1
-        const unsigned r0 = us, rdn = us - uP, rup = us + uP;
-        T g[9], D[9], alt[9];
-        if (MIXED && IBB) ibb_gather<T, RW, PP>(a, us, o, s_flag, D, alt);
-        g[0] = PP ? a.hq_in[0][r0] : *hb;
+        T h[9], D[9], alt[9];
+        if (EARLY) {
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                h[q] = eh[q];
+                D[q] = eD[q];
+                alt[q] = ealt[q];
+            }
+        } else {
+            if (MIXED && IBB) {
+                ibb_fractions<T, RW>(a, us, o, s_flag, D);
+                ibb_populations<T, RW, PP>(a, us, o, s_flag, D, alt);
+            }
+            pull<T, RW, MIXED, PP>(a, us, o, s_flag, h);
+        }
+        T g[9];
+        g[0] = h[0];
         T A = mul_rn(qw<T>(0), rho);  // sum_q w_q rho(x - e_q); bounce-back sources take rho(x)
         T dm = (T)0;                  // interpolated bounce-back: mass returned to the rest population
 #pragma unroll
@@ -396,17 +447,13 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid,
             const int os = o - qy(q) * RW - qx(q);
             if (!MIXED || s_flag[os] == kFluid) {
                 const T rs = s_rho[os];
-                const T h = PP ? *(a.hq_in[q] + (int)((qy(q) > 0 ? rdn : qy(q) < 0 ? rup : r0) -
-                                                      qx(q)))
-                               : *(hb + (int)QSRC(q));
-                g[q] = fma_rn(qw<T>(q), sub_rn(rs, rho), h);
+                g[q] = fma_rn(qw<T>(q), sub_rn(rs, rho), h[q]);
                 A = fma_rn(qw<T>(q), rs, A);
             } else {
-                const T out = PP ? a.hq_in[qopp(q)][r0] : *(hb + (int)QPL(qopp(q)));
-                g[q] = out;
+                g[q] = h[q];
                 if (MIXED && IBB) {
-                    g[q] = ibb_return<T, RW>(q, o, rho, out, D[q], alt[q], s_rho, s_flag);
-                    dm = add_rn(dm, sub_rn(out, g[q]));
+                    g[q] = ibb_return<T, RW>(q, o, rho, h[q], D[q], alt[q], s_rho, s_flag);
+                    dm = add_rn(dm, sub_rn(h[q], g[q]));
                 }
                 A = fma_rn(qw<T>(q), rho, A);
             }
@@ -434,8 +481,6 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid,
         stream_out<T, TX, TY, NT, MIXED, true, PP>(a, s_rho, s_g, s_flag, x0, y0);
     else
         stream_out<T, TX, TY, NT, MIXED, false, PP>(a, s_rho, s_g, s_flag, x0, y0);
-#undef QPL
-#undef QSRC
 }
 
 // Programmatic dependent launch (no effect without its launch attribute): the next step's blocks
