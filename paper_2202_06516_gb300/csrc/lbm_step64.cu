@@ -11,8 +11,9 @@
 //   k64_collide   force (Eq. 7), pulled populations (Eq. 4), collision (Eq. 1, 13)
 //   k64_stream    rho(t+1) = sum_q f*_q(x - e_q) and the stored deviations
 // with 32 or 64 nodes per block, so that a 200 x 120 lattice gives every SM about the same work.
-// The launches are plain: placed early by programmatic dependent launch, the next kernel's blocks
-// crowd onto some SMs, and the FP64 pipe of each SM is what the step waits for (44 against 32 us).
+// Only the light k64_stream is placed early (programmatic dependent launch): blocks of the other two
+// placed early crowd onto some SMs, and the FP64 pipe of each SM is what the step waits for (44
+// against 32 us per step; k64_stream alone placed early: 21.2 to 20.6).
 // The operations and their order are those of the fused step; the bulk chemical potential shares one
 // reciprocal between its divisions. 200 x 120 (Carnahan-Starling): 64 us per step fused on 56 CTAs,
 // 21 us here (k64_mu 8.5, k64_collide 12, k64_stream 5 us each alone and cold).
@@ -134,6 +135,7 @@ constexpr int N64 = 32;  // nodes per block of the two per-node kernels
 template <bool MACRO, bool IBB>
 __global__ void __launch_bounds__(N64) k64_collide(const Args64 s) {
     const StepArgs<double>& a = s.a;
+    pdl_launch_next();
     const int n = blockIdx.x * N64 + threadIdx.x;
     const int y = n / a.nx, x = n - y * a.nx, P = a.P;
     const bool in = y < a.ny;
@@ -219,6 +221,7 @@ __global__ void __launch_bounds__(N64) k64_stream(const Args64 s) {
             src[q] = cut ? (unsigned)qopp(q) * upl + us
                          : (unsigned)q * upl + (unsigned)lidx(P, wrap_x(x - qx(q), a.nx), y - qy(q));
         }
+    pdl_wait_previous();
     if (!fluid) return;
     double g[9], t[9];
 #pragma unroll
@@ -259,8 +262,18 @@ cudaError_t launch_step64(lbm_ctx* c, const StepArgs<double>& a, bool macro) {
     auto* collide = macro ? (c->ibb ? k64_collide<true, true> : k64_collide<true, false>)
                           : (c->ibb ? k64_collide<false, true> : k64_collide<false, false>);
     collide<<<gn, N64, 0, c->stream>>>(s);
-    if (!macro) k64_stream<<<gn, N64, 0, c->stream>>>(s);
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    if (macro || e != cudaSuccess) return e;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = gn;
+    cfg.blockDim = dim3(N64);
+    cfg.stream = c->stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k64_stream, s);
 }
 
 }  // namespace lbm
