@@ -401,10 +401,10 @@ struct Conv {
     // pixels; w_tma false: gathered with cp.async
     bool w_tma = false;
     CUtensorMap wmap[3] = {};
-    // weight gradient from one staged input window per slice (k_gemm_wwin): C_in / 32 when it
-    // applies (1 or 2), else 0; maps: sources 1 and 2 (32 channels x 72 pixels x 3 rows), dY
-    int ww_cb = 0;
-    CUtensorMap wwmap[3] = {};
+    // weight gradient from staged rows (k_wgrad_rows): channel blocks of sources 1 and 2 (xb = 0: not
+    // so), cb of them per CTA, blocks yb of the output gradient; maps: source 1, 2, dY
+    int wr_xb = 0, wr_yb = 0, wr_cb = 0;
+    CUtensorMap wrmap[3] = {};
     // forward (fm) and data gradient (dm) on k_conv_march; maps: source 1 (dY for dm) and source 2
     // as boxes of one row of 136 pixels x kb channels, the weights as kb x bn blocks
     March fm, dm;
@@ -596,15 +596,17 @@ EncodeTiledFn encode_tiled() {
 // image, ks = 64 with 128-byte, 32 with 64-byte, 16 with 32-byte swizzle or 8 without (the K-major
 // layouts the MMAs read), out-of-range elements zero.
 bool map_nhwc(CUtensorMap* m, const void* base, int C, int W, int H, int N, int bw, int bh,
-              int ks, int step = 1) {
+              int ks, int step = 1, int ystep = 0) {
     const EncodeTiledFn enc = encode_tiled();
     if (!enc) return false;
     const cuuint64_t dim[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
     const cuuint64_t stride[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2,
                                   (cuuint64_t)H * W * C * 2};
-    // step 2: every second pixel in x and y (the box spans 2 bw x 2 bh pixels, loads bw x bh)
-    const cuuint32_t box[4] = {(cuuint32_t)ks, (cuuint32_t)(bw * step), (cuuint32_t)(bh * step), 1};
-    const cuuint32_t es[4] = {1, (cuuint32_t)step, (cuuint32_t)step, 1};
+    // step 2: every second pixel in x and y (the box spans 2 bw x 2 bh pixels, loads bw x bh); ystep:
+    // another step in y
+    if (!ystep) ystep = step;
+    const cuuint32_t box[4] = {(cuuint32_t)ks, (cuuint32_t)(bw * step), (cuuint32_t)(bh * ystep), 1};
+    const cuuint32_t es[4] = {1, (cuuint32_t)step, (cuuint32_t)ystep, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dim, stride, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE,
                ks == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
@@ -733,30 +735,60 @@ cudaError_t gemm_wgrad_tma(cudaStream_t st, const GemmArgs& a, int splits, const
     }
 }
 
-// Launch of k_gemm_wwin over `splits` K ranges (one CTA each).
-template <int BN, int CB>
-cudaError_t launch_wwin(cudaStream_t st, const GemmArgs& a, int splits, const CUtensorMap* maps) {
-    constexpr int STAGES = 4;
-    constexpr int STAGE = CB * 4 * 72 * 64 + BN * 128;
-    constexpr int RAW = 1024 + STAGES * STAGE + 8 * (2 * STAGES + 1) + 16;
-    constexpr int CTAS = 512 / (int)lbm::sgtc::tmem_pow2(3 * CB * BN);
-    constexpr int MINB = 233472 / (CTAS + 1) + 1;
-    constexpr int SMEM = RAW > MINB ? RAW : MINB;
-    auto* kern = lbm::sgtc::k_gemm_wwin<BN, CB, STAGES>;
+// Launch of k_wgrad_rows: split-K ranges for one wave of CTAs over all column blocks, as far as the
+// partials fit `scratch`; the partials are summed in order. a: M = 9 C_in, N = C_out, K = pixels.
+cudaError_t sum_splits(cudaStream_t st, const float* part, int splits, long long stride, float* out);
+template <int XB, int YB, int CB, bool UP>
+cudaError_t launch_wgrad_rows(cudaStream_t st, GemmArgs a, float* scratch, size_t scratch_elems,
+                              float* out, const CUtensorMap* maps) {
+    using WS = lbm::sgtc::WgradShape<XB, YB, CB, UP>;
+    auto* kern = lbm::sgtc::k_wgrad_rows<XB, YB, CB, UP>;
     static std::atomic<unsigned long long> configured{0};
+    static std::atomic<int> sms{152};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        int n = 152;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, WS::SMEM);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
+        sms.store(n);
         configured.fetch_or(bit);
     }
     int* flag = tc_flag().dev;
     if (!flag) return cudaErrorMemoryAllocation;
-    return launch_pdl(kern, dim3(splits), lbm::sgtc::TC_THREADS, SMEM, st, a, flag, maps[0], maps[1],
-                      maps[2]);
+    const long long stride = (long long)a.N * a.ldc;
+    const int groups = (a.conv.C1 + a.conv.C2) / (XB * CB) * (a.N / YB);
+    a.K /= 64 * WS::RA * (UP ? 2 : 1);  // slices
+    long long splits = std::max(1, std::min(a.K / 2, WS::CTAS * sms.load() / groups));
+    splits = std::max(1ll, std::min(splits, (long long)scratch_elems / stride));
+    a.kchunk = (int)((a.K + splits - 1) / splits);
+    splits = (a.K + a.kchunk - 1) / a.kchunk;
+    a.split_stride = splits > 1 ? stride : 0;
+    a.Cf = splits > 1 ? scratch : out;
+    e = launch_pdl(kern, dim3((unsigned)splits, groups), lbm::sgtc::TC_THREADS, WS::SMEM, st, a, flag,
+                   maps[0], maps[1], maps[2]);
+    return e != cudaSuccess || splits == 1 ? e : sum_splits(st, scratch, (int)splits, stride, out);
+}
+
+cudaError_t gemm_wgrad_rows(cudaStream_t st, const GemmArgs& a, float* scratch, size_t elems, float* out,
+                            int xb, int yb, int cb, const CUtensorMap* maps) {
+    const int key = xb * 1000 + yb * 10 + cb;
+    if (a.conv.up1) switch (key) {
+            case 32161: return launch_wgrad_rows<32, 16, 1, true>(st, a, scratch, elems, out, maps);
+            case 32322: return launch_wgrad_rows<32, 32, 2, true>(st, a, scratch, elems, out, maps);
+            default: return cudaErrorInvalidValue;
+        }
+    switch (key) {
+        case 16161: return launch_wgrad_rows<16, 16, 1, false>(st, a, scratch, elems, out, maps);
+        case 16162: return launch_wgrad_rows<16, 16, 2, false>(st, a, scratch, elems, out, maps);
+        case 16321: return launch_wgrad_rows<16, 32, 1, false>(st, a, scratch, elems, out, maps);
+        case 32321: return launch_wgrad_rows<32, 32, 1, false>(st, a, scratch, elems, out, maps);
+        case 32322: return launch_wgrad_rows<32, 32, 2, false>(st, a, scratch, elems, out, maps);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 // out = the sum of `splits` FP32 partials of `stride` values each, in split order
@@ -881,31 +913,8 @@ bool march_form(const March& m, bool up) {
            key == 32164 || key == 32232 || key == 32264;
 }
 
-// The weight gradient through k_gemm_wwin (a: the transposed, gathered form of gemm_wgrad):
-// K ranges of at least 16 slices, at most two per SM, their partials summed in order.
-cudaError_t gemm_wgrad_window(cudaStream_t st, GemmArgs a, float* scratch, size_t scratch_elems,
-                              float* out, int cb, const CUtensorMap* maps) {
-    const long long stride = (long long)a.N * a.ldc;
-    const int slices = a.K / 64;
-    int splits = std::max(1, std::min(304, slices / 16));
-    while (splits > 1 && (size_t)splits * stride > scratch_elems) splits /= 2;
-    const int chunk = (slices + splits - 1) / splits * 64;
-    splits = (a.K + chunk - 1) / chunk;
-    a.kchunk = chunk;
-    a.split_stride = splits > 1 ? stride : 0;
-    a.Cf = splits > 1 ? scratch : out;
-    cudaError_t e = cudaErrorInvalidValue;
-    if (a.N == 32 && cb == 1) e = launch_wwin<32, 1>(st, a, splits, maps);
-    if (a.N == 32 && cb == 2) e = launch_wwin<32, 2>(st, a, splits, maps);
-    if (a.N == 64 && cb == 1) e = launch_wwin<64, 1>(st, a, splits, maps);
-    if (a.N == 64 && cb == 2) e = launch_wwin<64, 2>(st, a, splits, maps);
-    if (e != cudaSuccess || splits == 1) return e;
-    return sum_splits(st, scratch, splits, stride, out);
-}
-
 cudaError_t gemm_wgrad(cudaStream_t st, GemmArgs a, float* scratch, size_t scratch_elems,
-                       float* out, bool gather, const CUtensorMap* maps = nullptr,
-                       int ww_cb = 0, const CUtensorMap* wwmaps = nullptr) {
+                       float* out, bool gather, const CUtensorMap* maps = nullptr) {
     if (gather) {
         // rows: the 9 C_in im2col columns; columns: C_out; a.ldc (= 9 C_in) stays the row
         // length of dW, written at dW[n * ldc + m]
@@ -916,7 +925,6 @@ cudaError_t gemm_wgrad(cudaStream_t st, GemmArgs a, float* scratch, size_t scrat
         t.ldb = a.lda;
         t.tout = 1;
         a = t;
-        if (ww_cb) return gemm_wgrad_window(st, a, scratch, scratch_elems, out, ww_cb, wwmaps);
     }
     // enough K slices for every SM to hold as many CTAs as fit (three of the narrow tiles, two
     // of the wide ones): each CTA keeps only two K-slices of gathers in flight
@@ -1126,6 +1134,34 @@ void make_march_maps(lbm_surrogate* s, Conv& c) {
     }
 }
 
+// Column blocks (groups of input channels x blocks of output channels) up to which the weight gradient
+// runs on k_wgrad_rows: every block reads the operands again, and with more of them the tiles of
+// k_gemm_tc are wide enough (64 x 64 x 8: 64 -> 128 channels, 4 blocks, 16 us; 128 -> 128, 8 blocks, 24
+// against 21; 256 -> 128, 16 blocks, 40 against 34).
+constexpr int kWgradGroups = 4;
+
+// The weight gradient on k_wgrad_rows: rows of the source a multiple of 64 pixels, whole slices of rows,
+// channels in blocks of 32 or 16.
+void make_wgrad_maps(lbm_surrogate* s, Conv& c) {
+    if (c.src1 == 0 || (c.up1 && c.C2)) return;
+    const int cin = c.C1 + c.C2, ow = c.up1 ? c.W / 2 : c.W, oh = c.up1 ? c.H / 2 : c.H;
+    const int xb = c.C1 % 32 == 0 && c.C2 % 32 == 0 ? 32 : c.C1 % 16 == 0 && c.C2 % 16 == 0 ? 16 : 0;
+    const int yb = c.Cout % 32 == 0 ? 32 : c.Cout == 16 ? 16 : 0;
+    if (!xb || !yb || ow % 64 || c.H % (xb == 32 ? 2 : 4)) return;
+    const int cb = cin / xb % 2 ? 1 : 2, key = xb * 1000 + yb * 10 + cb;
+    const bool form = c.up1 ? key == 32161 || key == 32322
+                            : key == 16161 || key == 16162 || key == 16321 || key == 32321 || key == 32322;
+    if (!form || cin / (xb * cb) * (c.Cout / yb) > kWgradGroups) return;
+    const int ra = xb == 32 ? 2 : 4, rows = c.up1 ? 3 : ra + 2;
+    if (map_nhwc(&c.wrmap[0], s->t[c.src1].y, c.C1, ow, oh, s->maxB, 72, rows, xb) &&
+        (c.src2 < 0 || map_nhwc(&c.wrmap[1], s->t[c.src2].y, c.C2, ow, oh, s->maxB, 72, rows, xb)) &&
+        map_nhwc(&c.wrmap[2], c.g, c.Cout, c.W, c.H, s->maxB, 64, ra, yb, c.up1 ? 2 : 1, 1)) {
+        c.wr_xb = xb;
+        c.wr_yb = yb;
+        c.wr_cb = cb;
+    }
+}
+
 // Tensor maps for the forward and data-gradient GEMMs whose A operand the copy engine can fetch
 // as boxes: no upsampled source, channel counts multiples of 64 (one K-slice of 64 = one tap of
 // one source) or else of 32 (slices of 32), the 128 rows of a tile a whole block of pixels of
@@ -1138,6 +1174,7 @@ void make_tensor_maps(lbm_surrogate* s) {
     for (Conv& c : s->convs) {
         const int W = c.W, H = c.H;
         make_march_maps(s, c);
+        make_wgrad_maps(s, c);
         if (c.up1 && c.src1 != 0) {
             // forward of an upsampling convolution: tile rows in runs of even, then odd output
             // columns, each run a box of half a tile row of source pixels
@@ -1178,15 +1215,6 @@ void make_tensor_maps(lbm_surrogate* s) {
             map_rows(&c.fmap[2], s->wb + c.w_off, 9 * cin, c.Cout, pick_bn(c.Cout), fk) &&
             map_rows(&c.fmap[3], s->wb + c.w_off, 9 * cin, c.Cout, 32, fk))
             c.f_ks = fk;
-        if (W % 64 == 0 && c.C1 % 32 == 0 && c.C2 % 32 == 0 && (cin == 32 || cin == 64) &&
-            (c.Cout == 32 || c.Cout == 64)) {
-            const int wc = cin / 32;
-            if (map_nhwc(&c.wwmap[0], s->t[c.src1].y, c.C1, W, H, s->maxB, 72, 3, 32) &&
-                (c.src2 < 0 ||
-                 map_nhwc(&c.wwmap[1], s->t[c.src2].y, c.C2, W, H, s->maxB, 72, 3, 32)) &&
-                map_nhwc(&c.wwmap[2], c.g, c.Cout, W, H, s->maxB, 64, 1, 32))
-                c.ww_cb = wc;
-        }
         if (W % 64 == 0 || 64 % W == 0) {
             const int ww = std::min(W, 64), wh = 64 / ww;
             c.w_tma = c.C1 % 32 == 0 && c.C2 % 32 == 0 && c.Cout % 32 == 0 &&
@@ -1408,7 +1436,7 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
                          : launch_wgrad0<16>(ws, gw, s->splitk, s->g + c.w_off, mx, mdy));
             continue;  // no data gradient for the input tensor
         }
-        const bool gather = gw.conv.lh >= 0 && gw.conv.lw >= 0;
+        const bool rows = c.wr_xb != 0, gather = rows || (gw.conv.lh >= 0 && gw.conv.lw >= 0);
         if (!gather && last)  // the side stream's last im2col may still be read
             SCUDA(s, join_side(s));
         if (!gather) SCUDA(s, launch_im2col(s, ws, c, B));
@@ -1420,8 +1448,16 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         gw.lda = c.Cout;
         gw.ldb = 9 * Cin;
         gw.ldc = 9 * Cin;
-        SCUDA(s, gemm_wgrad(ws, gw, last ? s->splitk : s->splitk_side, s->splitk_elems, s->g + c.w_off, gather,
-                            gather && c.w_tma ? c.wmap : nullptr, gather ? c.ww_cb : 0, c.wwmap));
+        float* part = last ? s->splitk : s->splitk_side;
+        if (rows) {
+            gw.M = 9 * Cin;
+            gw.N = c.Cout;
+            SCUDA(s, gemm_wgrad_rows(ws, gw, part, s->splitk_elems, s->g + c.w_off, c.wr_xb, c.wr_yb,
+                                     c.wr_cb, c.wrmap));
+        } else {
+            SCUDA(s, gemm_wgrad(ws, gw, part, s->splitk_elems, s->g + c.w_off, gather,
+                                gather && c.w_tma ? c.wmap : nullptr));
+        }
         // data gradient (not needed for the input tensor)
         if (c.src1 == 0) continue;
         // implicit GEMM over the source pixels: dX_src[q][ci] += sum over (sub-pixel, tap, co)

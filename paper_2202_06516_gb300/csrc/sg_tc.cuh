@@ -13,8 +13,8 @@
 // FP32 accumulate into BN tensor-memory columns) and commits them to the slice's mbarrier,
 // which frees the slice for the next load. The epilogue reads the accumulator lanes back with
 // tcgen05.ld (warp w owns rows 32 w .. 32 w + 31), adds the bias, applies the leaky ReLU and
-// stores FP32 or BF16. k_gemm_wwin computes the weight gradient of the 32/64-channel levels from
-// one staged input window per slice, and k_conv_march the forward convolutions and data gradients
+// stores FP32 or BF16. k_wgrad_rows computes weight gradients of rows of 64 pixels and more from
+// staged input rows, and k_conv_march the forward convolutions and data gradients
 // of wide rows with few channels from operand rows staged once (the nine taps as operands shifted
 // by whole pixels inside them).
 //
@@ -772,40 +772,72 @@ __host__ __device__ constexpr uint32_t tmem_pow2(int cols) {
     return cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
 }
 
-// Weight gradient of a 3 x 3 convolution with C_in = 32 CB input channels from one staged input
-// window per K slice: dW^T[(tap, ci)][co] = sum over pixels p of x(p + off(tap))[ci] dY(p)[co]
-// (K = pixels of one image row segment, 64 per slice; each CTA one split-K range, grid = splits).
-// Per slice thread 0 loads with TMA, for each 32-channel block, the input rows y - 1 .. y + 1 of
-// pixels x - 4 .. x + 67 (64-byte-swizzled rows of 32 channels: the MN-major layout with K =
-// pixels), and the 32-channel blocks of dY for the 64 pixels. The nine taps are then MN-major A
-// operands that start a whole number of rows into that window (dx) with the three dy rows as their
-// first three 32-wide M blocks (4,608 B apart; the fourth block reads a row that is not loaded and
-// its outputs are dropped): accumulator tile (block cb, dx) in tensor-memory columns
-// (3 cb + dx + 1) BN. Every input element is read once per slice instead of once per tap. The
-// epilogue writes the split's FP32 partial transposed, dW^T row tap C_in + ci.
-template <int BN, int CB, int STAGES>
+// Sizes of k_wgrad_rows: slices of RA output-gradient rows of 64 pixels (UP: the two row parities, for
+// NP column parities) and the ROWS input rows of 72 pixels around them; an MMA's M blocks are BLK
+// window rows.
+template <int XB, int YB, int CB, bool UP>
+struct WgradShape {
+    static constexpr int RA = XB == 32 ? 2 : 4, NP = UP ? 2 : 1, ROWS = UP ? 3 : RA + 2;
+    static constexpr int BLK = 128 / XB, WROW = 72 * XB * 2, WIN = BLK * WROW, DROW = 64 * YB * 2;
+    static constexpr int A_B = CB * WIN, STAGE = A_B + NP * RA * DROW;
+    static constexpr int STAGES = STAGE <= 36864 ? 4 : 3;
+    static constexpr int N = RA * YB, T = UP ? 4 : 3;  // accumulators per channel block
+    static constexpr uint32_t TX = (uint32_t)(CB * ROWS * WROW + NP * RA * DROW);
+    static constexpr uint32_t COLS = tmem_pow2(CB * T * N);
+    // accumulators the epilogue sums at a time, through the stages' memory
+    static constexpr int D = UP ? T : 1;
+    static constexpr int RAW = 1024 + STAGES * STAGE + 8 * (2 * STAGES + 1) + 16;
+    static constexpr int CTAS = 512 / (int)COLS < 232448 / (RAW + 2048) ? 512 / (int)COLS
+                                                                      : 232448 / (RAW + 2048);
+    // no more CTAs per SM than its tensor memory holds
+    static constexpr int MIN_BYTES = 233472 / (512 / (int)COLS + 1) + 1;
+    static constexpr int SMEM = RAW > MIN_BYTES ? RAW : MIN_BYTES;
+    static_assert(CB * T * N <= 512 && ROWS <= BLK, "accumulators must fit");
+    static_assert(D * N * 128 * 4 <= STAGES * STAGE, "the epilogue's sums must fit the stages");
+};
+
+// Weight gradient of a 3 x 3 convolution from staged rows, for CB blocks of XB (32 or 16) input
+// channels and YB output channels per CTA (blockIdx.y: which), blockIdx.x one split-K range:
+// dW^T[(tap, ci)][co] = sum over pixels p of x(p + off(tap))[ci] dY(p)[co]. Per slice thread 0 loads
+// with TMA the input rows y - 1 .. y + RA of pixels x - 4 .. x + 67 (rows of XB channels, swizzled: the
+// MN-major layout with K = pixels) and the dY rows y .. y + RA - 1 of 64 pixels. An MMA's M is the
+// window's rows (BLK blocks of XB), its N the dY rows (RA blocks of YB), so one MMA per (block, dx, 16
+// pixels) holds every (input row, dY row) pair: those with dy = -1, 0, 1 are the taps, summed over the
+// dY rows at the end, the rest is dropped (as is what M blocks past the loaded rows read). An A operand
+// of 128 x 16 is read from shared memory in 64 cycles, N columns take N / 2: N = 64 or more hides
+// what a single dY row (N = 32, three of four M blocks used) spent on operand reads.
+// UP: the input has half the resolution (nearest upsampling). Output pixel (2 i + a, 2 j + b) of tap
+// (dy, dx) reads input pixel (i + (a + dy) >> 1, j + (b + dx) >> 1), so the products are formed over
+// input pixels for the 2 x 2 parities and the two column offsets each reads, 16 products where the
+// nine taps over output pixels are 36, and summed into the taps at the end. The dY pixels of one
+// column parity come as every second pixel of a box.
+// Bound by the MMAs (about 100 cycles for 128 x 64 x 16). 256 x 256 x 8, input -> output channels, before
+// (one dY row per MMA from a staged window, or im2col columns fetched per tap) and here, us:
+// 32 -> 32 30 / 22, 64 -> 32 82 / 25, 64 -> 32 upsampling 133 / 31; 128 x 128 x 8: 64 -> 64 30 / 24,
+// 128 -> 64 60 / 38, 128 -> 64 upsampling 57 / 30. Relative error against FP64 sums of the same operands
+// 6.4e-6 / 0.9e-6 at worst (shorter FP32 chains per split).
+template <int XB, int YB, int CB, bool UP>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    k_gemm_wwin(const sg::GemmArgs g, int* err, const __grid_constant__ CUtensorMap tmX1,
-                const __grid_constant__ CUtensorMap tmX2, const __grid_constant__ CUtensorMap tmDY) {
-    static_assert(BN % 32 == 0 && 3 * CB * BN <= 512, "accumulators must fit tensor memory");
-    constexpr int T = 3 * CB, WROW = 72, WIN = 4 * WROW * 64;
-    constexpr int A_B = CB * WIN, B_B = BN * 128, STAGE = A_B + B_B;
-    constexpr uint32_t TX = (uint32_t)(CB * 3 * WROW * 64 + B_B);
-    constexpr uint32_t COLS = tmem_pow2(T * BN);
+    k_wgrad_rows(const sg::GemmArgs g, int* err, const __grid_constant__ CUtensorMap tmX1,
+                 const __grid_constant__ CUtensorMap tmX2, const __grid_constant__ CUtensorMap tmDY) {
+    using S = WgradShape<XB, YB, CB, UP>;
+    constexpr int STAGES = S::STAGES, T = S::T, N = S::N, RA = S::RA;
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const uint32_t raw = su32(smem_raw);
     uint8_t* base = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(base + STAGES * STAGE);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(base + STAGES * S::STAGE);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 1);
     __shared__ int s_ok;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int kb = blockIdx.x * g.kchunk, ke = min(g.K, kb + g.kchunk);
-    const int nk = ke > kb ? (ke - kb) / 64 : 0;
+    // kchunk, K: slices
+    const int kb = blockIdx.x * g.kchunk, nk = max(0, min(g.K - kb, g.kchunk));
+    const int cin = g.conv.C1 + g.conv.C2, ny = g.N / YB;
+    const int co0 = (int)(blockIdx.y % ny) * YB, ci0 = (int)(blockIdx.y / ny) * (CB * XB);
     sg::pdl_wait();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                          su32(tmem_slot)),
-                     "r"(COLS)
+                     "r"(S::COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
@@ -819,30 +851,32 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_fence_after();
     sg::pdl_next();
     const uint32_t tmem = *tmem_slot;
-    constexpr uint32_t IDESC = idesc_bf16(BM, BN, 1, 1);
-    const int H = g.conv.H, W = g.conv.W;
-    auto win = [&](int st, int cb) { return su32(base + st * STAGE + cb * WIN); };
-    auto dyb = [&](int st) { return su32(base + st * STAGE + A_B); };
-    auto issue = [&](int st, int k0) {
-        const uint32_t full = su32(bars + st);
-        mbar_expect_tx(full, TX);
-        const int pn = k0 / (H * W), pr = k0 - pn * (H * W);
-        const int py = pr / W, px = pr - (pr / W) * W;
-#pragma unroll
-        for (int cb = 0; cb < CB; ++cb) {
-            const int ci = 32 * cb;
-            if (ci < g.conv.C1)
-                tma_load_4d(win(st, cb), &tmX1, full, ci, px - 4, py - 1, pn);
-            else
-                tma_load_4d(win(st, cb), &tmX2, full, ci - g.conv.C1, px - 4, py - 1, pn);
-        }
-#pragma unroll
-        for (int b = 0; b < BN / 32; ++b) tma_load_4d(dyb(st) + 4096 * b, &tmDY, full, 32 * b, px, py, pn);
-    };
     if (tid == 0) {
+        const int segs = (UP ? g.conv.W / 2 : g.conv.W) / 64, rows = g.conv.H / RA;
+        auto issue = [&](int st, int k) {
+            const uint32_t full = su32(bars + st), a = su32(base + st * S::STAGE);
+            mbar_expect_tx(full, S::TX);
+            const int r = k / segs, px = (k - r * segs) * 64, n = r / rows, row = r - n * rows;
+            const int py = UP ? row : row * RA;
+#pragma unroll
+            for (int cb = 0; cb < CB; ++cb) {
+                const int ci = ci0 + XB * cb;
+                if (ci < g.conv.C1)
+                    tma_load_4d(a + cb * S::WIN, &tmX1, full, ci, px - 4, py - 1, n);
+                else
+                    tma_load_4d(a + cb * S::WIN, &tmX2, full, ci - g.conv.C1, px - 4, py - 1, n);
+            }
+#pragma unroll
+            for (int b = 0; b < S::NP; ++b)
+                tma_load_4d(a + S::A_B + b * RA * S::DROW, &tmDY, full, co0, UP ? 2 * px + b : px,
+                            row * RA, n);
+        };
+        constexpr uint32_t IDESC = idesc_bf16(BM, N, 1, 1);
+        constexpr uint32_t AHI = desc_hi(16 * XB, XB == 32 ? SW64 : SW32);
+        constexpr uint32_t BHI = desc_hi(16 * YB, YB == 32 ? SW64 : SW32);
         int issued = 0, done_mma = 0;
         bool good = true;
-        for (; issued < STAGES && issued < nk; ++issued) issue(issued, kb + issued * 64);
+        for (; issued < STAGES && issued < nk; ++issued) issue(issued, kb + issued);
         for (int kt = 0; kt < nk; ++kt) {
             const int st = kt % STAGES;
             if (!mbar_wait(su32(bars + st), (kt / STAGES) & 1)) {
@@ -850,17 +884,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 break;
             }
             tc_fence_after();
-            constexpr uint32_t HI = desc_hi(512, SW64);
-            const uint32_t a0 = desc_lo(win(st, 0), WROW * 64), b0 = desc_lo(dyb(st), 4096);
+            const uint32_t a = su32(base + st * S::STAGE);
+            const uint32_t a0 = desc_lo(a, S::WROW), b0 = desc_lo(a + S::A_B, S::DROW);
 #pragma unroll
-            for (int t = 0; t < T; ++t) {
-                const int cb = t / 3, dxi = t - 3 * (t / 3);
+            for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    tc_mma(tmem + (uint32_t)(t * BN),
-                           a0 + (uint32_t)((cb * WIN + (3 + dxi) * 64 + 1024 * j) >> 4), HI,
-                           b0 + (uint32_t)((1024 * j) >> 4), HI, IDESC, (kt > 0 || j > 0) ? 1u : 0u);
-            }
+                for (int t = 0; t < T; ++t) {
+                    // accumulator t: dx = t - 1, or (UP) column parity b and its offset e = 0, 1
+                    const int b = UP ? t / 2 : 0, px = UP ? 3 + t / 2 + t % 2 : 3 + t;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        tc_mma(tmem + (uint32_t)((cb * T + t) * N),
+                               a0 + (uint32_t)((cb * S::WIN + (px + 16 * j) * XB * 2) >> 4), AHI,
+                               b0 + (uint32_t)((b * RA * S::DROW + 16 * j * YB * 2) >> 4), BHI, IDESC,
+                               (kt > 0 || j > 0) ? 1u : 0u);
+                }
             tc_commit(su32(bars + STAGES + st));
             done_mma = kt + 1;
             if (kt >= 1 && issued < nk) {
@@ -869,7 +907,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     good = false;
                     break;
                 }
-                issue(sp, kb + issued * 64);
+                issue(sp, kb + issued);
                 ++issued;
             }
         }
@@ -884,35 +922,59 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __syncthreads();
     if (!s_ok) {
         if (tid == 0) atomicExch(err, 1);
-    } else if (warp < 3) {
-        // warp w holds M block w: dy = w - 1, lane = channel within the block
+    } else {
         tc_fence_after();
         const size_t zoff = (size_t)blockIdx.x * g.split_stride;
-        const int cin = 32 * CB;
+        float* sum = reinterpret_cast<float*>(base);  // [D][RA][BLK][YB][XB]
+        constexpr int CELL = YB * XB;
+        const int m = warp * 32 + lane, blk = m / XB, mi = m % XB;
 #pragma unroll 1
-        for (int t = 0; t < T; ++t) {
-            const int cb = t / 3, dxi = t - 3 * (t / 3);
-            const int m = (warp * 3 + dxi) * cin + 32 * cb + lane;
+        for (int cb = 0; cb < CB; ++cb)
 #pragma unroll 1
-            for (int c0 = 0; c0 < BN; c0 += 32) {
-                float v[32];
-                if (nk == 0) {
+            for (int t0 = 0; t0 < T; t0 += S::D) {
+#pragma unroll 1
+                for (int c0 = 0; c0 < S::D * N; c0 += 32) {
+                    float v[32];
+                    if (nk == 0) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = 0.f;
-                } else {
-                    tc_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t * BN + c0), v);
+                        for (int j = 0; j < 32; ++j) v[j] = 0.f;
+                    } else {
+                        tc_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((cb * T + t0) * N + c0), v);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const int da = (c0 + j) / YB, co = (c0 + j) % YB;  // d RA + a
+                        sum[(da * S::BLK + blk) * CELL + co * XB + mi] = v[j];
+                    }
                 }
+                __syncthreads();
+                for (int i = tid; i < (UP ? 9 : 3) * CELL; i += TC_THREADS) {
+                    const int k = i / CELL, cell = i - k * CELL;
+                    const int dyi = UP ? k / 3 : k, dxi = UP ? k - 3 * (k / 3) : t0;
+                    float v = 0.f;
+                    if (UP) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (c0 + j < g.N) g.Cf[(size_t)(c0 + j) * g.ldc + m + zoff] = v[j];
+                        for (int ab = 0; ab < 4; ++ab) {
+                            const int a = ab >> 1, b = ab & 1;
+                            const int br = 1 + ((a + dyi - 1) >> 1);
+                            const int d = 2 * b + ((b + dxi - 1) >> 1) - (b - 1);
+                            v += sum[((d * RA + a) * S::BLK + br) * CELL + cell];
+                        }
+                    } else {
+#pragma unroll
+                        for (int a = 0; a < RA; ++a) v += sum[(a * S::BLK + dyi + a) * CELL + cell];
+                    }
+                    const int co = cell / XB, ci = cell - co * XB;
+                    g.Cf[(size_t)(co0 + co) * g.ldc + (dyi * 3 + dxi) * cin + ci0 + cb * XB + ci + zoff] = v;
+                }
+                __syncthreads();
             }
-        }
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(COLS)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(S::COLS)
                      : "memory");
     }
 }
