@@ -802,9 +802,10 @@ cudaError_t sum_splits(cudaStream_t st, const float* part, int splits, long long
 
 // How a convolution runs on k_conv_march: blocks of kb channels, cb of them, bn output columns per
 // CTA; kb = 0: it does not. Maps: source 1 (dY for the data gradient) and source 2 as boxes of one
-// row of 136 pixels x kb channels, weights as kb x bn blocks.
+// row of 136 pixels x kb channels, weights as kb x bn blocks. parts: how many partial sums per column a
+// fused leaky-ReLU adjoint (GemmArgs::rg) left, 0 when it was not fused.
 template <int KB, int CB, int BN, bool GD, bool UP>
-cudaError_t launch_march(cudaStream_t st, const GemmArgs& a, const CUtensorMap* maps) {
+cudaError_t launch_march(cudaStream_t st, GemmArgs a, const CUtensorMap* maps, int* parts) {
     using MS = lbm::sgtc::MarchShape<KB, CB, BN, UP>;
     auto* kern = lbm::sgtc::k_conv_march<KB, CB, BN, GD, UP>;
     static std::atomic<unsigned long long> configured{0};
@@ -832,6 +833,8 @@ cudaError_t launch_march(cudaStream_t st, const GemmArgs& a, const CUtensorMap* 
     const int want = std::max(1, per_sm * sms.load() / std::max(1, strips * nb));
     const int chunk = std::max(1, (rh + want - 1) / want);
     const dim3 grid((unsigned)strips * ((rh + chunk - 1) / chunk), nb);
+    if (grid.x > (unsigned)kReluBlocks) a.rg = nullptr;  // rpart's columns
+    if (parts) *parts = a.rg ? (int)grid.x : 0;
     return launch_pdl(kern, grid, lbm::sgtc::MARCH_THREADS, MS::SMEM, st, a, flag, maps[0], maps[1],
                       maps[2], chunk);
 }
@@ -884,24 +887,25 @@ cudaError_t launch_wgrad0(cudaStream_t st, GemmArgs a, float* scratch, float* ou
 }
 
 template <bool GD>
-cudaError_t conv_march(cudaStream_t st, const GemmArgs& a, const March& m, const CUtensorMap* maps) {
+cudaError_t conv_march(cudaStream_t st, const GemmArgs& a, const March& m, const CUtensorMap* maps,
+                       int* parts = nullptr) {
     const int key = m.kb * 1000 + m.cb * 100 + m.bn;
     if constexpr (!GD) {
         if (a.conv.up1) switch (key) {
-                case 32116: return launch_march<32, 1, 16, false, true>(st, a, maps);
-                case 32232: return launch_march<32, 2, 32, false, true>(st, a, maps);
+                case 32116: return launch_march<32, 1, 16, false, true>(st, a, maps, parts);
+                case 32232: return launch_march<32, 2, 32, false, true>(st, a, maps, parts);
                 default: return cudaErrorInvalidValue;
             }
     }
     switch (key) {
-        case 16116: return launch_march<16, 1, 16, GD, false>(st, a, maps);
-        case 16132: return launch_march<16, 1, 32, GD, false>(st, a, maps);
-        case 16216: return launch_march<16, 2, 16, GD, false>(st, a, maps);
-        case 32116: return launch_march<32, 1, 16, GD, false>(st, a, maps);
-        case 32132: return launch_march<32, 1, 32, GD, false>(st, a, maps);
-        case 32164: return launch_march<32, 1, 64, GD, false>(st, a, maps);
-        case 32232: return launch_march<32, 2, 32, GD, false>(st, a, maps);
-        case 32264: return launch_march<32, 2, 64, GD, false>(st, a, maps);
+        case 16116: return launch_march<16, 1, 16, GD, false>(st, a, maps, parts);
+        case 16132: return launch_march<16, 1, 32, GD, false>(st, a, maps, parts);
+        case 16216: return launch_march<16, 2, 16, GD, false>(st, a, maps, parts);
+        case 32116: return launch_march<32, 1, 16, GD, false>(st, a, maps, parts);
+        case 32132: return launch_march<32, 1, 32, GD, false>(st, a, maps, parts);
+        case 32164: return launch_march<32, 1, 64, GD, false>(st, a, maps, parts);
+        case 32232: return launch_march<32, 2, 32, GD, false>(st, a, maps, parts);
+        case 32264: return launch_march<32, 2, 64, GD, false>(st, a, maps, parts);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1033,6 +1037,19 @@ void build(lbm_surrogate* s) {
     s->nparams += b;
     s->head_b = s->nparams;
     s->nparams += 1;
+}
+
+// The convolution whose output is c's first source, when c alone reads that output (no pool, no other
+// convolution, not the head) and its channels come in the 16s of k_conv_march's epilogue; else null.
+const Conv* sole_producer(const lbm_surrogate* s, const Conv& c) {
+    const Conv* p = nullptr;
+    int readers = c.src1 == s->head_in;
+    for (const Conv& o : s->convs) {
+        if (o.out == c.src1) p = &o;
+        readers += (o.src1 == c.src1) + (o.src2 == c.src1);
+    }
+    for (const auto& pl : s->pools) readers += pl.first == c.src1;
+    return readers == 1 && c.C1 % 16 == 0 ? p : nullptr;
 }
 
 // the main stream waits for what the side stream holds so far
@@ -1375,6 +1392,8 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
     SCUDA(s, launch_pdl(k_mask_count, dim3((unsigned)std::min<long long>(152, blocks_for(P / 16 + 1))),
                         kT, 0, s->stream, mask, P, s->n_mask));
     std::vector<char> written(s->t.size(), 0);
+    // per tensor: the bias gradient's partial sums when its convolution's g is already there
+    std::vector<int> fused(s->t.size(), 0);
     const int C = s->base;
     const int nb = std::min(s->part_blocks, blocks_for(P));
     SCUDA(s, launch_head(s, nb, s->phi, P, target, mask));
@@ -1396,8 +1415,10 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         const long long Pc = (long long)B * c.H * c.W;
         const long long n_out = Pc * c.Cout;
         // leaky-ReLU adjoint (with the pool's), BF16 copy and the bias gradient's partial sums
-        const int rb = (int)std::min<long long>(kReluBlocks, (n_out / 8 + kT - 1) / kT);
-        if (c.out == s->head_in)
+        const int rb = fused[c.out] ? fused[c.out]
+                                    : (int)std::min<long long>(kReluBlocks, (n_out / 8 + kT - 1) / kT);
+        if (fused[c.out]) {
+        } else if (c.out == s->head_in)
             SCUDA(s, launch_pdl(k_relu_bias<2>, dim3(rb), kT, 0, s->stream, s->dz, nullptr,
                                 s->w + s->head_w, o.y, c.g, n_out / 8, c.Cout, c.H, c.W, c.bpart));
         else
@@ -1483,7 +1504,8 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
             SCUDA(s, cudaMemsetAsync(x.dy, 0, (size_t)B * x.H * x.W * x.C * sizeof(float), s->stream));
             written[fresh] = 1;
         }
-        gd.accumulate = written[c.src1];
+        const bool fresh1 = !written[c.src1];
+        gd.accumulate = !fresh1;
         written[c.src1] = 1;
         if (c.src2 >= 0) written[c.src2] = 1;
         if (c.C2 > 0) {
@@ -1491,11 +1513,18 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
             gd.ldc2 = c.C2;
             gd.nsplit = c.C1;
         }
-        if (c.dm.kb)
-            SCUDA(s, conv_march<true>(s->stream, gd, c.dm, c.dmmap));
-        else
+        if (c.dm.kb) {
+            const Conv* p = fresh1 ? sole_producer(s, c) : nullptr;
+            if (p) {
+                gd.ry = s->t[c.src1].y;
+                gd.rg = p->g;
+                gd.rpart = p->bpart;
+            }
+            SCUDA(s, conv_march<true>(s->stream, gd, c.dm, c.dmmap, &fused[c.src1]));
+        } else {
             SCUDA(s, (gemm_tc_split<false, true>(s->stream, gd, s->splitk, s->splitk_elems,
                                                   c.dmap, c.d_ks)));
+        }
     }
     SCUDA(s, join_side(s));
     if (lr > 0.f) {

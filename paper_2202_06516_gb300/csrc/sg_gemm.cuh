@@ -87,6 +87,12 @@ struct GemmArgs {
     int tout;          // FP32 output stored transposed: Cf[n * ldc + m] (no bias / ReLU)
     int rperm;         // h > 0: the rows of a tile come in runs of 2 h pixels, each run's even
                        // columns first, then its odd columns (row_pixel); 0: in pixel order
+    // k_conv_march's data gradient, columns of the first source (n < nsplit or all): instead of FP32 to
+    // Cf, rg = BF16(result * (ry > 0 ? 1 : 0.1)) [m * ldc + n], the leaky-ReLU adjoint of that source,
+    // and the sums of rg per column and blockIdx.x, rpart[n * gridDim.x + blockIdx.x]
+    const __nv_bfloat16* ry;
+    __nv_bfloat16* rg;
+    float* rpart;
 };
 
 // pixel offset within its tile of tile row r (see GemmArgs::rperm)

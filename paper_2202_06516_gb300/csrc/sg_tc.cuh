@@ -990,6 +990,15 @@ __device__ __forceinline__ void st_global_32B(void* p, const uint32_t (&v)[8]) {
                  : "memory");
 }
 
+// 32 bytes from a 32-byte-aligned address
+__device__ __forceinline__ void ld_global_32B(const void* p, uint32_t (&v)[8]) {
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+                   "=r"(v[7])
+                 : "l"(p)
+                 : "memory");
+}
+
 // a wait for a whole warp: lane 0 polls
 __device__ __forceinline__ bool warp_wait(int lane, uint32_t bar, uint32_t parity) {
     int ok = 1;
@@ -1019,7 +1028,11 @@ constexpr int MARCH_THREADS = 192;
 // two output rows of 128 even and 128 odd columns each.
 // Roles: warp 4 copies (TMA), warp 5 issues MMAs, warps 0-3 read the finished accumulator (two in
 // tensor memory, alternating) and store whole 32-byte sectors, so copies, MMAs and stores of
-// neighbouring rows overlap. Bound by the MMAs' shared-memory reads (a 128 x 16 A slice per
+// neighbouring rows overlap. The data gradient of a source that nothing else reads is not stored in
+// FP32 but as that source's finished pre-activation gradient (GemmArgs::rg), whose activation the
+// epilogue fetches before it waits for the accumulator, with the bias gradient's sums kept per
+// thread until the end: the pass that did this moved 134 MB in 19 us at 256 x 256 x 8, 32 channels.
+// Bound by the MMAs' shared-memory reads (a 128 x 16 A slice per
 // 16-deep MMA of only BN columns). One 128-pixel tile per CTA with its own window and weights (182 MB
 // through L2 for 32 -> 32 channels at 256 x 256 x 8, against 72 MB here) or one box per tap (750 MB for
 // 64 -> 32) were bound by that traffic and its latency. 256 x 256 x 8: 32 -> 32 channels 34 -> 23 us,
@@ -1047,6 +1060,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
     __shared__ int s_ok;
     __shared__ uint32_t s_tmem;
     __shared__ float s_bias[BN];
+    __shared__ float s_col[4][BN];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // the CTA's strip: image, first operand column, operand rows ra .. rb - 1
@@ -1169,8 +1183,17 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
         if (!good) s_ok = 0;
     } else if (warp < 4) {
         // lane: one pixel of the tile
+        const int fuse = GD && g.rg ? min(BN, (g.Cf2 ? g.nsplit : g.N) - n0) : 0;  // columns (may be < 0)
+        float acc[GD ? BN : 1] = {};
+        uint32_t yv[GD ? BN / 16 : 1][8];
         for (int r = ra; r < rb; ++r) {
             const int b = (r - ra) & 1;
+            if (GD) {
+                const size_t m = ((size_t)img * H + r) * W + x0 + warp * 32 + lane;
+#pragma unroll
+                for (int c = 0; c < BN; c += 16)
+                    if (c < fuse) ld_global_32B(g.ry + m * g.ldc + n0 + c, yv[c / 16]);
+            }
             if (!warp_wait(lane, accf(b), ((r - ra) >> 1) & 1)) {
                 if (lane == 0) s_ok = 0;
                 break;
@@ -1212,7 +1235,27 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
                         }
                     } else {
 #pragma unroll
+                        for (int c = 0; c < CW; c += 16) {
+                            if (c0 + c >= fuse) continue;
+                            uint32_t o[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const uint32_t yw = yv[(c0 + c) / 16][i];
+                                const float2 y =
+                                    __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&yw));
+                                const float a0 = v[c + 2 * i], a1 = v[c + 2 * i + 1];
+                                const __nv_bfloat162 h = __floats2bfloat162_rn(
+                                    y.x > 0.f ? a0 : 0.1f * a0, y.y > 0.f ? a1 : 0.1f * a1);
+                                const float2 q = __bfloat1622float2(h);
+                                acc[c0 + c + 2 * i] += q.x;
+                                acc[c0 + c + 2 * i + 1] += q.y;
+                                o[i] = *reinterpret_cast<const uint32_t*>(&h);
+                            }
+                            st_global_32B(g.rg + m * g.ldc + n0 + c0 + c, o);
+                        }
+#pragma unroll
                         for (int c = 0; c < CW; c += 8) {
+                            if (c0 + c < fuse) continue;
                             const int n = n0 + c0 + c;
                             float* dst = g.Cf2 && n >= g.nsplit ? g.Cf2 + m * g.ldc2 + (n - g.nsplit)
                                                                 : g.Cf + m * g.ldc + n;
@@ -1228,10 +1271,30 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
                 }
             }
         }
+        if (GD && fuse > 0) {
+            // the warp's column sums: halves of the columns change places with the lane that sums them
+#pragma unroll
+            for (int c0 = 0; c0 < BN; c0 += 32) {
+                float t[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) t[i] = c0 + i < BN ? acc[(c0 + i) % BN] : 0.f;
+#pragma unroll
+                for (int h = 16; h > 0; h >>= 1)
+#pragma unroll
+                    for (int i = 0; i < h; ++i) {
+                        const float keep = lane & h ? t[i + h] : t[i], give = lane & h ? t[i] : t[i + h];
+                        t[i] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+                    }
+                if (c0 + lane < BN) s_col[warp][c0 + lane] = t[0];
+            }
+        }
     }
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && !s_ok) atomicExch(err, 1);
+    if (GD && g.rg && tid < BN && n0 + tid < (g.Cf2 ? g.nsplit : g.N))
+        g.rpart[(size_t)(n0 + tid) * gridDim.x + blockIdx.x] =
+            (s_col[0][tid] + s_col[1][tid]) + (s_col[2][tid] + s_col[3][tid]);
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(COLS)
