@@ -58,6 +58,8 @@ enum { LBM_BB_HALFWAY = 0, LBM_BB_INTERP = 1 }; /* lbm_geometry.boundary: curved
  *    budget is fitted to (0 = no constraint); all three 0 selects 32x16/5 in FP32 and 32x16/0 in
  *    FP64. Supported (tile/min_blocks):
  *    FP32 32x8/0, 32x8/6, 32x16/0, 32x16/5, 32x16/6, 64x16/0, 32x32/0; FP64 32x8/0, 32x16/0.
+ *    FP64 steps run in untiled kernels, the same for both names; 32x16/5 on an FP32 lattice of few
+ *    tiles runs in a form with smaller tiles or more threads (the same results).
  *    tile_x = LBM_TILE_AUTO: start with the default and let lbm_autotune pick the variant at the
  *    first lbm_step (for lbm_batch_create: lbm_batch_autotune at the first lbm_batch_run).
  *  stream: a cudaStream_t (e.g. torch.cuda.current_stream().cuda_stream) or NULL. */
@@ -185,7 +187,7 @@ lbm_status lbm_measure_contact_angle(lbm_ctx *ctx, lbm_angle out[2]);
 lbm_status lbm_read_fields(lbm_ctx *ctx, uint32_t which, double *rho, double *ux, double *uy,
                            size_t n);
 
-/* FP64 sums over fluid nodes (deterministic two-pass reduction): out[0] total mass, out[1]
+/* Sums over fluid nodes (deterministic; exact for FP32 densities, FP64 for FP64 ones): out[0] total mass, out[1]
  * number of liquid nodes (rho > rho_m), out[2], out[3] their centroid x, y. Returns
  * LBM_ERR_UNSTABLE if a density is non-finite or non-positive. Synchronous. */
 lbm_status lbm_mass(lbm_ctx *ctx, double out[4]);

@@ -806,7 +806,7 @@ cudaError_t sum_splits(cudaStream_t st, const float* part, int splits, long long
 // fused leaky-ReLU adjoint (GemmArgs::rg) left, 0 when it was not fused.
 template <int KB, int CB, int BN, bool GD, bool UP>
 cudaError_t launch_march(cudaStream_t st, GemmArgs a, const CUtensorMap* maps, int* parts) {
-    using MS = lbm::sgtc::MarchShape<KB, CB, BN, UP>;
+    using MS = lbm::sgtc::MarchShape<KB, CB, BN, GD, UP>;
     auto* kern = lbm::sgtc::k_conv_march<KB, CB, BN, GD, UP>;
     static std::atomic<unsigned long long> configured{0};
     static std::atomic<int> sms{152};
@@ -828,7 +828,8 @@ cudaError_t launch_march(cudaStream_t st, GemmArgs a, const CUtensorMap* maps, i
     if (!flag) return cudaErrorMemoryAllocation;
     const int H = GD ? a.dg.H : a.conv.H, W = GD ? a.dg.W : a.conv.W;
     const int rh = UP ? H / 2 : H, rw = UP ? W / 2 : W, nb = a.N / BN;
-    const int strips = (int)((long long)a.M / ((long long)H * W)) * (rw / 128);
+    const long long image = MS::UD ? (long long)rh * rw : (long long)H * W;  // rows of the GEMM
+    const int strips = (int)(a.M / image) * (rw / 128);
     // one wave of CTAs: chunks of rows so that strips x chunks x column blocks fill the SMs
     const int want = std::max(1, per_sm * sms.load() / std::max(1, strips * nb));
     const int chunk = std::max(1, (rh + want - 1) / want);
@@ -896,6 +897,12 @@ cudaError_t conv_march(cudaStream_t st, const GemmArgs& a, const March& m, const
                 case 32232: return launch_march<32, 2, 32, false, true>(st, a, maps, parts);
                 default: return cudaErrorInvalidValue;
             }
+    } else if (a.dg.up1) {
+        switch (key) {
+            case 16132: return launch_march<16, 1, 32, true, true>(st, a, maps, parts);
+            case 32164: return launch_march<32, 1, 64, true, true>(st, a, maps, parts);
+            default: return cudaErrorInvalidValue;
+        }
     }
     switch (key) {
         case 16116: return launch_march<16, 1, 16, GD, false>(st, a, maps, parts);
@@ -910,9 +917,9 @@ cudaError_t conv_march(cudaStream_t st, const GemmArgs& a, const March& m, const
     }
 }
 // the forms conv_march has
-bool march_form(const March& m, bool up) {
+bool march_form(const March& m, bool gd, bool up) {
     const int key = m.kb * 1000 + m.cb * 100 + m.bn;
-    if (up) return key == 32116 || key == 32232;
+    if (up) return gd ? key == 16132 || key == 32164 : key == 32116 || key == 32232;
     return key == 16116 || key == 16132 || key == 16216 || key == 32116 || key == 32132 ||
            key == 32164 || key == 32232 || key == 32264;
 }
@@ -1135,17 +1142,20 @@ void make_march_maps(lbm_surrogate* s, Conv& c) {
     const int cin = c.C1 + c.C2, ow = c.up1 ? c.W / 2 : c.W, oh = c.up1 ? c.H / 2 : c.H;
     if (ow % 128 == 0 && !(c.up1 && c.C2)) {
         const March m = blocks(c.C1, c.C2, c.Cout);
-        if (m.kb && m.bn && march_form(m, c.up1) &&
+        if (m.kb && m.bn && march_form(m, false, c.up1) &&
             map_nhwc(&c.fmmap[0], s->t[c.src1].y, c.C1, ow, oh, s->maxB, 136, 1, m.kb) &&
             (c.src2 < 0 || map_nhwc(&c.fmmap[1], s->t[c.src2].y, c.C2, ow, oh, s->maxB, 136, 1, m.kb)) &&
             map_rows(&c.fmmap[2], s->wb + c.w_off, 9 * cin, c.Cout, m.bn, m.kb))
             c.fm = m;
     }
-    if (!c.up1 && c.W % 128 == 0) {
+    if (ow % 128 == 0 && !(c.up1 && c.C2)) {
         const March m = blocks(c.Cout, 0, cin);
-        // a column block of eight lies on one side of the split between the sources
-        if (m.kb && m.bn && march_form(m, false) && c.C1 % 8 == 0 &&
-            map_nhwc(&c.dmmap[0], c.g, c.Cout, c.W, c.H, s->maxB, 136, 1, m.kb) &&
+        // a column block of eight lies on one side of the split between the sources; upsampling: every
+        // second pixel, in two boxes (a box spans at most 256)
+        if (m.kb && m.bn && march_form(m, true, c.up1) && c.C1 % 8 == 0 &&
+            (c.up1 ? map_nhwc(&c.dmmap[0], c.g, c.Cout, c.W, c.H, s->maxB, 72, 1, m.kb, 2, 1) &&
+                         map_nhwc(&c.dmmap[1], c.g, c.Cout, c.W, c.H, s->maxB, 64, 1, m.kb, 2, 1)
+                   : map_nhwc(&c.dmmap[0], c.g, c.Cout, c.W, c.H, s->maxB, 136, 1, m.kb)) &&
             map_rows(&c.dmmap[2], s->wbd + c.w_off, 9 * c.Cout, cin, m.bn, m.kb))
             c.dm = m;
     }

@@ -1007,12 +1007,13 @@ __device__ __forceinline__ bool warp_wait(int lane, uint32_t bar, uint32_t parit
 }
 
 // Sizes of k_conv_march: rows of 136 pixels of CB blocks of KB channels in a ring, the nine taps'
-// weight blocks, mbarriers.
-template <int KB, int CB, int BN, bool UP>
+// weight blocks, mbarriers. UD (GD and UP): a row is its even and its odd columns.
+template <int KB, int CB, int BN, bool GD, bool UP>
 struct MarchShape {
-    static constexpr int R = 6;                        // rows in the ring
-    static constexpr int G = UP ? 4 : 1;               // tiles (accumulators) per operand row
-    static constexpr int ROWB = 136 * KB * 2, SLOT = CB * ROWB;
+    static constexpr bool UF = UP && !GD, UD = UP && GD;
+    static constexpr int R = UD ? 8 : 6;               // rows in the ring
+    static constexpr int G = UF ? 4 : 1;               // tiles (accumulators) per operand row
+    static constexpr int ROWB = 136 * KB * 2, SLOT = CB * (UD ? 2 : 1) * ROWB;
     static constexpr int BSUB = BN * KB * 2, WBYTES = 9 * CB * BSUB;
     static constexpr int NBARS = 2 * R + 6;
     static constexpr int SMEM = 1024 + WBYTES + R * SLOT + NBARS * 8;
@@ -1025,7 +1026,10 @@ constexpr int MARCH_THREADS = 192;
 // once per CTA. Each tile of 128 pixels of one row is 9 CB KB / 16 MMAs, whose A operand is a row of
 // the ring starting dx pixels aside; the K order is tap, then channel. UP (forward): the operand
 // has half the output's resolution (nearest upsampling), and each operand row yields four tiles,
-// two output rows of 128 even and 128 odd columns each.
+// two output rows of 128 even and 128 odd columns each. UP with GD: a tile is 128 pixels of the
+// half-resolution input's gradient, the sum over the 2 x 2 output pixels and nine taps in which each
+// takes part (K order: output pixel, tap, channel); four operand rows are read per tile and two
+// released, each loaded as its even and its odd columns (every second pixel of a box).
 // Roles: warp 4 copies (TMA), warp 5 issues MMAs, warps 0-3 read the finished accumulator (two in
 // tensor memory, alternating) and store whole 32-byte sectors, so copies, MMAs and stores of
 // neighbouring rows overlap. The data gradient of a source that nothing else reads is not stored in
@@ -1035,7 +1039,8 @@ constexpr int MARCH_THREADS = 192;
 // Bound by the MMAs' shared-memory reads (a 128 x 16 A slice per
 // 16-deep MMA of only BN columns). One 128-pixel tile per CTA with its own window and weights (182 MB
 // through L2 for 32 -> 32 channels at 256 x 256 x 8, against 72 MB here) or one box per tap (750 MB for
-// 64 -> 32) were bound by that traffic and its latency. 256 x 256 x 8: 32 -> 32 channels 34 -> 23 us,
+// 64 -> 32) were bound by that traffic and its latency. 256 x 256 x 8: 32 -> 32 channels 34 -> 23 us, data
+// gradient of 64 -> 32 (upsampling) 58 -> 27 (and the leaky-ReLU pass of 12),
 // 64 -> 32 (concatenated) 69 -> 44, 64 -> 32 (upsampling) 72 -> 35; 128 x 128 x 8, 64 -> 64: 27 -> 18.
 // Waits are polled by one thread each with an iteration limit; a wait that runs out ends its role,
 // the others follow by their own limits, copies and MMAs in flight are waited for (bounded).
@@ -1044,8 +1049,9 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
     k_conv_march(const sg::GemmArgs g, int* err, const __grid_constant__ CUtensorMap tmA1,
                  const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB,
                  int chunk) {
-    using S = MarchShape<KB, CB, BN, UP>;
-    static_assert((KB == 16 || KB == 32) && BN % 16 == 0 && BN <= 64 && !(GD && UP), "shape");
+    using S = MarchShape<KB, CB, BN, GD, UP>;
+    constexpr bool UF = S::UF, UD = S::UD;
+    static_assert((KB == 16 || KB == 32) && BN % 16 == 0 && BN <= 64, "shape");
     constexpr int R = S::R, G = S::G;
     constexpr uint32_t COLS = tmem_pow2(2 * G * BN);
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -1103,7 +1109,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
     if (warp == 4 && lane == 0) {
         // copies: weights, then operand rows ra - 1 .. rb (rows outside the image are zero-filled)
         bool good = true;
-        const int rows = rb - ra + 2;
+        const int rows = (UD ? 2 : 1) * (rb - ra) + 2;
         int issued = 0;
         auto load_row = [&](int i) {
             const int slot = i % R;
@@ -1111,8 +1117,16 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
 #pragma unroll
             for (int cb = 0; cb < CB; ++cb) {
                 const int ci = KB * cb;
-                const uint32_t dst = ring + slot * S::SLOT + cb * S::ROWB;
-                if (GD || ci < g.conv.C1)
+                const uint32_t dst = ring + slot * S::SLOT + cb * (UD ? 2 : 1) * S::ROWB;
+                if (UD) {  // columns x0 - 4 .. x0 + 67 and x0 + 68 .. x0 + 131 of each parity
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        tma_load_4d(dst + q * S::ROWB, &tmA1, full(slot), ci, 2 * (x0 - 4) + q,
+                                    2 * ra - 1 + i, img);
+                        tma_load_4d(dst + q * S::ROWB + 72 * KB * 2, &tmA2, full(slot), ci,
+                                    2 * (x0 + 68) + q, 2 * ra - 1 + i, img);
+                    }
+                } else if (GD || ci < g.conv.C1)
                     tma_load_4d(dst, &tmA1, full(slot), ci, x0 - 4, ra - 1 + i, img);
                 else
                     tma_load_4d(dst, &tmA2, full(slot), ci - g.conv.C1, x0 - 4, ra - 1 + i, img);
@@ -1139,20 +1153,22 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
         bool good = mbar_wait(wfull, 0);
         int have = -1;
         for (int r = ra; r < rb && good; ++r) {
-            const int i0 = r - ra, need = i0 + 2;  // ring indexes of operand rows r - 1 and r + 1
+            // ring indexes of operand rows r - 1 and r + 1 (UD: 2 r - 1 and 2 r + 2)
+            const int it = r - ra, i0 = UD ? 2 * it : it, need = i0 + (UD ? 3 : 2);
             while (have < need && good) {
                 ++have;
                 good = mbar_wait(full(have % R), (have / R) & 1);
             }
-            const int b = i0 & 1;
-            if (good && i0 >= 2) good = mbar_wait(acce(b), ((i0 >> 1) - 1) & 1);
+            const int b = it & 1;
+            if (good && it >= 2) good = mbar_wait(acce(b), ((it >> 1) - 1) & 1);
             if (!good) break;
             tc_fence_after();
-            uint32_t row_lo[3];  // operand rows r - 1, r, r + 1
+            uint32_t row_lo[UD ? 4 : 3];  // operand rows r - 1, r, r + 1 (UD: 2 r - 1 .. 2 r + 2)
 #pragma unroll
-            for (int i = 0; i < 3; ++i) row_lo[i] = desc_lo(ring + ((i0 + i) % R) * S::SLOT);
+            for (int i = 0; i < (UD ? 4 : 3); ++i) row_lo[i] = desc_lo(ring + ((i0 + i) % R) * S::SLOT);
 #pragma unroll
-            for (int t = 0; t < 9; ++t) {
+            for (int st = 0; st < (UD ? 36 : 9); ++st) {
+                const int t = st % 9, sy = st / 18, sx = st / 9 & 1;  // tap and (UD) output pixel
                 const int dy = t / 3 - 1, dx = t - (t / 3) * 3 - 1;
 #pragma unroll
                 for (int cb = 0; cb < CB; ++cb)
@@ -1161,7 +1177,10 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
 #pragma unroll
                         for (int k = 0; k < G; ++k) {
                             int wr, wc;  // operand row relative to r - 1, column relative to x0 - 4
-                            if (UP) {
+                            if (UD) {
+                                wr = 1 + sy - dy;
+                                wc = 4 + ((sx - dx) >> 1) + ((sx - dx) & 1) * 136;  // odd columns follow
+                            } else if (UP) {
                                 const int yy = (k >> 1) + dy;
                                 wr = yy < 0 ? 0 : yy > 1 ? 2 : 1;
                                 wc = 4 + ((k & 1) ? (dx > 0 ? 1 : 0) : (dx < 0 ? -1 : 0));
@@ -1170,13 +1189,14 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
                                 wc = GD ? 4 - dx : 4 + dx;
                             }
                             tc_mma(tmem + (uint32_t)((b * G + k) * BN),
-                                   row_lo[wr] + ((wc * KB * 2 + cb * S::ROWB + 32 * j) >> 4), HI,
+                                   row_lo[wr] + ((wc * KB * 2 + cb * (UD ? 2 : 1) * S::ROWB + 32 * j) >> 4), HI,
                                    w_lo + (((t * CB + cb) * S::BSUB + 32 * j) >> 4), HI, IDESC,
-                                   (t > 0 || cb > 0 || j > 0) ? 1u : 0u);
+                                   (st > 0 || cb > 0 || j > 0) ? 1u : 0u);
                         }
             }
             tc_commit(accf(b));
-            tc_commit(empty(i0 % R));  // operand row r - 1 is not read again
+            tc_commit(empty(i0 % R));  // operand row r - 1 (UD: 2 r - 1 and 2 r) is not read again
+            if (UD) tc_commit(empty((i0 + 1) % R));
         }
         tc_commit(done);
         if (!mbar_wait(done, 0)) good = false;
@@ -1189,7 +1209,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
         for (int r = ra; r < rb; ++r) {
             const int b = (r - ra) & 1;
             if (GD) {
-                const size_t m = ((size_t)img * H + r) * W + x0 + warp * 32 + lane;
+                const size_t m = ((size_t)img * RH + r) * RW + x0 + warp * 32 + lane;
 #pragma unroll
                 for (int c = 0; c < BN; c += 16)
                     if (c < fuse) ld_global_32B(g.ry + m * g.ldc + n0 + c, yv[c / 16]);
@@ -1201,8 +1221,8 @@ __global__ void __launch_bounds__(MARCH_THREADS, 1)
             tc_fence_after();
             const int px = warp * 32 + lane;
             for (int k = 0; k < G; ++k) {
-                const size_t m = UP ? ((size_t)img * H + 2 * r + (k >> 1)) * W + 2 * (x0 + px) + (k & 1)
-                                    : ((size_t)img * H + r) * W + x0 + px;
+                const size_t m = UF ? ((size_t)img * H + 2 * r + (k >> 1)) * W + 2 * (x0 + px) + (k & 1)
+                                    : ((size_t)img * RH + r) * RW + x0 + px;
 #pragma unroll
                 for (int c0 = 0; c0 < BN; c0 += 32) {
                     constexpr int CW = BN < 32 ? BN : 32;

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("base,H,Wd,B", [(8, 16, 128, 2), (16, 8, 128, 1), (16, 16, 128, 2),
-                                         (16, 40, 384, 1), (32, 24, 128, 2), (32, 16, 256, 1),
+                                         (16, 40, 384, 1), (16, 24, 256, 2), (32, 24, 128, 2), (32, 16, 256, 1),
                                          (32, 16, 192, 2)])
 def test_wide_rows_match_oracle(env, base, H, Wd, B):  # noqa: F811
     """Seeded initial weights. Forward and loss within BF16 storage of the oracle. Pre-activations
