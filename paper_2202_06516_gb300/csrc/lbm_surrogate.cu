@@ -330,6 +330,15 @@ struct ConvTable {
     int n;
     long long off[24];
     int cout[24], cin[24];
+    int tile[25];  // first block of each convolution in k_adam
+};
+// Bias gradients to finish: per convolution the partial sums part[c * nb + b], its first column
+// among all of them and where its sums go.
+struct BiasTable {
+    int n;
+    int col[25], nb[24];
+    const float* part[24];
+    float* out[24];
 };
 
 // BF16 copies of parameter t with FP32 value x: wb[t], and for a convolution weight also its
@@ -351,23 +360,84 @@ __device__ __forceinline__ void store_bf16_copies(long long t, float x, bf16* wb
     }
 }
 
-// Adam with bias correction (c1, c2 = 1 / (1 - beta^t)), followed by the BF16 copies of the
-// updated parameter
-__global__ void k_adam(float* w, const float* g, float* m, float* v, long long n, float lr,
-                       float b1, float b2, float eps, float c1, float c2, bf16* wb, bf16* wd,
-                       const ConvTable tab) {
+// The bias gradients of all listed convolutions in one launch, one warp per column (each alone was a
+// launch of 5.6 us on one block per column). Bound by reading the partials, 4 KB per column.
+__global__ void k_bias_final(const BiasTable tab) {
     pdl_next();
     pdl_wait();
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-         t += (long long)gridDim.x * blockDim.x) {
-        const float gi = g[t];
-        const float mi = b1 * m[t] + (1.f - b1) * gi;
-        const float vi = b2 * v[t] + (1.f - b2) * gi * gi;
+    const int col = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x & 31;
+    if (col >= tab.col[tab.n]) return;
+    int k = 0;
+    while (col >= tab.col[k + 1]) ++k;
+    const int c = col - tab.col[k], nb = tab.nb[k];
+    const float* p = tab.part[k] + (size_t)c * nb;
+    float s = 0.f;
+#pragma unroll 8
+    for (int b = lane; b < nb; b += 32) s += p[b];
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) s += __shfl_xor_sync(0xffffffffu, s, h);
+    if (lane == 0) tab.out[k][c] = s;
+}
+
+// Adam with bias correction (c1, c2 = 1 / (1 - beta^t)) and the BF16 copies of the updated
+// parameters. A block takes 32 outputs x 32 inputs (tap, ci) of one convolution and passes the BF16
+// weights through shared memory, so that both copies are written along their rows: writing the
+// data-gradient copy element by element (2 bytes every 18 C_in) took 33 us for 2.1 M parameters,
+// 15 here. The blocks of a convolution's first inputs also take its biases, block 0 the head.
+__global__ void __launch_bounds__(256)
+    k_adam(float* w, const float* g, float* m, float* v, long long n, int nhead, float lr, float b1,
+           float b2, float eps, float c1, float c2, bf16* wb, bf16* wd, const ConvTable tab) {
+    pdl_next();
+    __shared__ bf16 sm[32][34];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int k = 0;
+    while ((int)blockIdx.x >= tab.tile[k + 1]) ++k;
+    const int cin = tab.cin[k], cout = tab.cout[k], K = 9 * cin, kt = (K + 31) / 32;
+    const int tile = blockIdx.x - tab.tile[k], co0 = tile / kt * 32, k0 = tile % kt * 32;
+    pdl_wait();
+    auto step = [&](long long t, float gi, float mo, float vo, float wo) {
+        const float mi = b1 * mo + (1.f - b1) * gi;
+        const float vi = b2 * vo + (1.f - b2) * gi * gi;
         m[t] = mi;
         v[t] = vi;
-        const float wi = w[t] - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+        const float wi = wo - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
         w[t] = wi;
-        store_bf16_copies(t, wi, wb, wd, tab);
+        const bf16 h = __float2bfloat16_rn(wi);
+        wb[t] = h;
+        return h;
+    };
+    float gi[4], mi[4], vi[4], wi[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int co = co0 + warp + 8 * r;
+        if (co >= cout || k0 + lane >= K) continue;
+        const long long t = tab.off[k] + (long long)co * K + k0 + lane;
+        gi[r] = g[t];
+        mi[r] = m[t];
+        vi[r] = v[t];
+        wi[r] = w[t];
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int co = co0 + warp + 8 * r;
+        if (co >= cout || k0 + lane >= K) continue;
+        sm[lane][warp + 8 * r] =
+            step(tab.off[k] + (long long)co * K + k0 + lane, gi[r], mi[r], vi[r], wi[r]);
+    }
+    // biases and head: stored after a convolution's weights, and last
+    if (k0 == 0 && warp == 0 && co0 + lane < cout) {
+        const long long t = tab.off[k] + (long long)cout * K + co0 + lane;
+        step(t, g[t], m[t], v[t], w[t]);
+    }
+    if (blockIdx.x == 0 && warp >= 4)
+        for (long long t = n - nhead + threadIdx.x - 128; t < n; t += 128) step(t, g[t], m[t], v[t], w[t]);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int kk = k0 + warp + 8 * r;
+        if (kk >= K || co0 + lane >= cout) continue;
+        const int tap = kk / cin, ci = kk - tap * cin;
+        wd[tab.off[k] + ((long long)ci * 9 + tap) * cout + co0 + lane] = sm[warp + 8 * r][lane];
     }
 }
 
@@ -794,8 +864,8 @@ cudaError_t gemm_wgrad_rows(cudaStream_t st, const GemmArgs& a, float* scratch, 
 // out = the sum of `splits` FP32 partials of `stride` values each, in split order
 cudaError_t sum_splits(cudaStream_t st, const float* part, int splits, long long stride, float* out) {
     if (stride % 4 == 0 && ((uintptr_t)out & 15) == 0)
-        return launch_pdl(k_splitk_sum4, dim3((unsigned)((stride / 4 + 31) / 32)), 256, 0, st, part,
-                          splits, stride, stride, out);
+        return launch_pdl(k_splitk_sum4, dim3((unsigned)((stride / 4 + 31) / 32)), splits < 64 ? 256 : 1024,
+                          0, st, part, splits, stride, stride, out);
     return launch_pdl(k_splitk_sum, dim3(blocks_for(stride)), kT, 0, st, part, splits, stride, stride,
                       out);
 }
@@ -810,8 +880,6 @@ cudaError_t launch_march(cudaStream_t st, GemmArgs a, const CUtensorMap* maps, i
     auto* kern = lbm::sgtc::k_conv_march<KB, CB, BN, GD, UP>;
     static std::atomic<unsigned long long> configured{0};
     static std::atomic<int> sms{152};
-    // CTAs per SM: two where shared memory allows (232,448 bytes, 1 KB reserved per CTA)
-    constexpr int per_sm = 232448 / (MS::SMEM + 2048) >= 2 ? 2 : 1;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -831,7 +899,7 @@ cudaError_t launch_march(cudaStream_t st, GemmArgs a, const CUtensorMap* maps, i
     const long long image = MS::UD ? (long long)rh * rw : (long long)H * W;  // rows of the GEMM
     const int strips = (int)(a.M / image) * (rw / 128);
     // one wave of CTAs: chunks of rows so that strips x chunks x column blocks fill the SMs
-    const int want = std::max(1, per_sm * sms.load() / std::max(1, strips * nb));
+    const int want = std::max(1, MS::PER_SM * sms.load() / std::max(1, strips * nb));
     const int chunk = std::max(1, (rh + want - 1) / want);
     const dim3 grid((unsigned)strips * ((rh + chunk - 1) / chunk), nb);
     if (grid.x > (unsigned)kReluBlocks) a.rg = nullptr;  // rpart's columns
@@ -1284,6 +1352,8 @@ lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_
     build(s);
     s->tab.n = std::min<int>(24, (int)s->convs.size());  // 17 convolutions
     for (int k = 0; k < s->tab.n; ++k) {
+        const Conv& c = s->convs[k];
+        s->tab.tile[k + 1] = s->tab.tile[k] + (c.Cout + 31) / 32 * ((9 * (c.C1 + c.C2) + 31) / 32);
         s->tab.off[k] = (long long)s->convs[k].w_off;
         s->tab.cout[k] = s->convs[k].Cout;
         s->tab.cin[k] = s->convs[k].C1 + s->convs[k].C2;
@@ -1402,6 +1472,7 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
     SCUDA(s, launch_pdl(k_mask_count, dim3((unsigned)std::min<long long>(152, blocks_for(P / 16 + 1))),
                         kT, 0, s->stream, mask, P, s->n_mask));
     std::vector<char> written(s->t.size(), 0);
+    BiasTable bias{};  // of the layers on the side stream
     // per tensor: the bias gradient's partial sums when its convolution's g is already there
     std::vector<int> fused(s->t.size(), 0);
     const int C = s->base;
@@ -1442,8 +1513,16 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
             SCUDA(s, cudaEventRecord(c.ready, s->stream));
             SCUDA(s, cudaStreamWaitEvent(s->side, c.ready, 0));
         }
-        SCUDA(s, launch_pdl(k_colsum_final, dim3(c.Cout), kT, 0, ws, c.bpart, rb, c.Cout,
-                            s->g + c.b_off, 1, nullptr));
+        if (last) {
+            SCUDA(s, launch_pdl(k_colsum_final, dim3(c.Cout), kT, 0, ws, c.bpart, rb, c.Cout,
+                                s->g + c.b_off, 1, nullptr));
+        } else {
+            bias.part[bias.n] = c.bpart;
+            bias.nb[bias.n] = rb;
+            bias.out[bias.n] = s->g + c.b_off;
+            bias.col[bias.n + 1] = bias.col[bias.n] + c.Cout;
+            ++bias.n;
+        }
         // weight gradient: dW[co][k] = sum_p g[p][co] col[p][k], the im2col columns gathered by
         // the GEMM's loader when the resolution allows (powers of two), else from a buffer
         GemmArgs gw{};
@@ -1536,15 +1615,16 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
                                                   c.dmap, c.d_ks)));
         }
     }
+    SCUDA(s, launch_pdl(k_bias_final, dim3((bias.col[bias.n] + 7) / 8), 256, 0, s->side, bias));
     SCUDA(s, join_side(s));
     if (lr > 0.f) {
         ++s->adam_t;
         const float b1 = 0.9f, b2 = 0.999f;
         const float c1 = 1.f / (1.f - powf(b1, (float)s->adam_t));
         const float c2 = 1.f / (1.f - powf(b2, (float)s->adam_t));
-        SCUDA(s, launch_pdl(k_adam, dim3(blocks_for((long long)s->nparams)), kT, 0, s->stream, s->w,
-                            s->g, s->m, s->v, (long long)s->nparams, lr, b1, b2, 1e-8f, c1, c2, s->wb,
-                            s->wbd, s->tab));
+        SCUDA(s, launch_pdl(k_adam, dim3(s->tab.tile[s->tab.n]), 256, 0, s->stream, s->w, s->g, s->m, s->v,
+                            (long long)s->nparams, s->base + 1, lr, b1, b2, 1e-8f, c1, c2, s->wb, s->wbd,
+                            s->tab));
     }
     SCUDA(s, cudaStreamSynchronize(s->stream));
     if (tc_timed_out())

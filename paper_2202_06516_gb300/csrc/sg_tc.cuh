@@ -1017,6 +1017,9 @@ struct MarchShape {
     static constexpr int BSUB = BN * KB * 2, WBYTES = 9 * CB * BSUB;
     static constexpr int NBARS = 2 * R + 6;
     static constexpr int SMEM = 1024 + WBYTES + R * SLOT + NBARS * 8;
+    // CTAs per SM: two where shared memory allows (232,448 bytes, 1 KB reserved per CTA); registers are
+    // fitted to that (the 32 -> 64 data gradient at 256 x 256 x 8 with one CTA of 182 registers 56 us, 38 so)
+    static constexpr int PER_SM = 232448 / (SMEM + 2048) >= 2 ? 2 : 1;
 };
 constexpr int MARCH_THREADS = 192;
 
@@ -1045,7 +1048,7 @@ constexpr int MARCH_THREADS = 192;
 // Waits are polled by one thread each with an iteration limit; a wait that runs out ends its role,
 // the others follow by their own limits, copies and MMAs in flight are waited for (bounded).
 template <int KB, int CB, int BN, bool GD, bool UP>
-__global__ void __launch_bounds__(MARCH_THREADS, 1)
+__global__ void __launch_bounds__(MARCH_THREADS, MarchShape<KB, CB, BN, GD, UP>::PER_SM)
     k_conv_march(const sg::GemmArgs g, int* err, const __grid_constant__ CUtensorMap tmA1,
                  const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB,
                  int chunk) {
