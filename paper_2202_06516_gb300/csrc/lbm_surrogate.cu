@@ -705,7 +705,8 @@ bool map_rows(CUtensorMap* m, const void* base, int K, int rows, int box_rows, i
 
 // CTAs of a launch up to which gemm_tc_tma takes its narrow, deep form: with it a forward pass of one
 // 256 x 256 sample (base 32) takes 284 us, without it 304. Launches of more CTAs hide their slices'
-// latency behind one another and would only read the A rows of a tile once per 32 columns.
+// latency behind one another and would only read the A rows of a tile once per 32 columns (with 304
+// instead of 128 the forward pass of one sample takes 297 us, of eight 940 instead of 457).
 constexpr long long kFewTiles = 128;
 
 // The TMA-fed gathering GEMM (GA or GD with tensor maps, see Conv::fmap / dmap), ks elements
@@ -1327,142 +1328,10 @@ void make_tensor_maps(lbm_surrogate* s) {
     }
 }
 
-}  // namespace
-
-extern "C" {
-
-lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_batch,
-                                int32_t device, lbm_surrogate** out) {
-    if (!out) return sfail(nullptr, LBM_ERR_ARG, "lbm_surrogate_create: out is NULL");
-    *out = nullptr;
-    if (H <= 0 || W <= 0 || H % 8 || W % 8 || (base != 8 && base != 16 && base != 32) ||
-        max_batch <= 0)
-        return sfail(nullptr, LBM_ERR_ARG,
-                     "lbm_surrogate_create: H, W multiples of 8, base 8, 16 or 32, batch > 0");
-    if (cudaSetDevice(device) != cudaSuccess) {
-        cudaGetLastError();
-        return sfail(nullptr, LBM_ERR_CUDA, "lbm_surrogate_create: cannot select the device");
-    }
-    lbm_surrogate* s = new lbm_surrogate();
-    s->H = H;
-    s->W = W;
-    s->base = base;
-    s->maxB = max_batch;
-    s->device = device;
-    build(s);
-    s->tab.n = std::min<int>(24, (int)s->convs.size());  // 17 convolutions
-    for (int k = 0; k < s->tab.n; ++k) {
-        const Conv& c = s->convs[k];
-        s->tab.tile[k + 1] = s->tab.tile[k] + (c.Cout + 31) / 32 * ((9 * (c.C1 + c.C2) + 31) / 32);
-        s->tab.off[k] = (long long)s->convs[k].w_off;
-        s->tab.cout[k] = s->convs[k].Cout;
-        s->tab.cin[k] = s->convs[k].C1 + s->convs[k].C2;
-    }
-    auto cleanup = [&](const char* e) {
-        lbm_surrogate_destroy(s);
-        return sfail(nullptr, LBM_ERR_CUDA, std::string("lbm_surrogate_create: ") + e);
-    };
-    cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return cleanup(cudaGetErrorString(e));
-    size_t colmax = 0;
-    for (const Conv& c : s->convs)
-        colmax = std::max(colmax, (size_t)max_batch * c.H * c.W * 9 * (c.C1 + c.C2));
-    s->col_elems = colmax;
-    for (size_t k = 1; k < s->t.size() && e == cudaSuccess; ++k) {
-        Tensor& x = s->t[k];
-        const size_t n = (size_t)max_batch * x.H * x.W * x.C;
-        e = cudaMalloc((void**)&x.y, n * sizeof(bf16));
-        if (e == cudaSuccess) e = cudaMalloc((void**)&x.dy, n * sizeof(float));
-    }
-    const size_t np = s->nparams;
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->w, np * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->g, np * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->m, np * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->v, np * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->wb, np * sizeof(bf16));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->wbd, np * sizeof(bf16));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->col, colmax * sizeof(bf16));
-    for (Conv& c : s->convs) {
-        if (e == cudaSuccess)
-            e = cudaMalloc((void**)&c.g, (size_t)max_batch * c.H * c.W * c.Cout * sizeof(bf16));
-        if (e == cudaSuccess)
-            e = cudaMalloc((void**)&c.bpart, (size_t)kReluBlocks * c.Cout * sizeof(float));
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.ready, cudaEventDisableTiming);
-    }
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->head_ready, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->side_done, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->dz, (size_t)max_batch * H * W * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->n_mask, sizeof(int));
-    if (e == cudaSuccess) e = cudaHostAlloc((void**)&s->host_loss, sizeof(float), cudaHostAllocMapped);
-    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&s->host_loss_dev, s->host_loss, 0);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->phi, (size_t)max_batch * H * W * sizeof(float));
-    if (e == cudaSuccess)
-        e = cudaMalloc((void**)&s->hpart, (size_t)s->part_blocks * (base + 2) * sizeof(float));
-    size_t wmax = 0;
-    for (const Conv& c : s->convs) wmax = std::max(wmax, (size_t)c.Cout * 9 * (c.C1 + c.C2));
-    s->splitk_elems = std::min<size_t>(wmax * 128, (size_t)64 << 20);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->splitk, s->splitk_elems * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->splitk_side, s->splitk_elems * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->w, 0, np * sizeof(float), s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->m, 0, np * sizeof(float), s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->v, 0, np * sizeof(float), s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->wb, 0, np * sizeof(bf16), s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->wbd, 0, np * sizeof(bf16), s->stream);
-    if (e != cudaSuccess) return cleanup(cudaGetErrorString(e));
-    make_tensor_maps(s);
-    *out = s;
-    return LBM_OK;
-}
-
-int64_t lbm_surrogate_num_params(const lbm_surrogate* s) { return s ? (int64_t)s->nparams : 0; }
-
-lbm_status lbm_surrogate_set_weights(lbm_surrogate* s, const float* host, int64_t n) {
-    if (!s || !host || n != (int64_t)s->nparams)
-        return sfail(s, LBM_ERR_ARG, "lbm_surrogate_set_weights: need num_params floats");
-    SCUDA(s, cudaSetDevice(s->device));
-    SCUDA(s, cudaMemcpyAsync(s->w, host, n * sizeof(float), cudaMemcpyHostToDevice, s->stream));
-    SCUDA(s, refresh_bf16_weights(s));
-    SCUDA(s, cudaMemsetAsync(s->m, 0, n * sizeof(float), s->stream));
-    SCUDA(s, cudaMemsetAsync(s->v, 0, n * sizeof(float), s->stream));
-    s->adam_t = 0;
-    SCUDA(s, cudaStreamSynchronize(s->stream));
-    return LBM_OK;
-}
-
-lbm_status lbm_surrogate_get_weights(lbm_surrogate* s, float* host, int64_t n, int32_t grads) {
-    if (!s || !host || n != (int64_t)s->nparams)
-        return sfail(s, LBM_ERR_ARG, "lbm_surrogate_get_weights: need num_params floats");
-    SCUDA(s, cudaSetDevice(s->device));
-    SCUDA(s, cudaMemcpyAsync(host, grads ? s->g : s->w, n * sizeof(float), cudaMemcpyDeviceToHost,
-                             s->stream));
-    SCUDA(s, cudaStreamSynchronize(s->stream));
-    return LBM_OK;
-}
-
-lbm_status lbm_surrogate_forward(lbm_surrogate* s, const void* x, int32_t B, float* phi_out) {
-    lbm::NvtxRange nvtx_("lbm_surrogate_forward");
-    if (!s || !x || !phi_out || B <= 0 || B > s->maxB)
-        return sfail(s, LBM_ERR_ARG, "lbm_surrogate_forward: bad arguments");
-    SCUDA(s, cudaSetDevice(s->device));
-    lbm_status st = forward(s, (const bf16*)x, B);
-    if (st != LBM_OK) return st;
-    const long long P = (long long)B * s->H * s->W;
-    const int nb = std::min(s->part_blocks, blocks_for(P));
-    SCUDA(s, launch_head(s, nb, phi_out, P, nullptr, nullptr));
-    SCUDA(s, cudaStreamSynchronize(s->stream));
-    if (tc_timed_out())
-        return sfail(s, LBM_ERR_TIMEOUT, "lbm_surrogate_forward: a tensor-core wait timed out");
-    return LBM_OK;
-}
-
-// Gradients of the masked MSE into s->g; with lr > 0 also an Adam update. *loss gets the loss.
-lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const float* target,
-                                    const uint8_t* mask, int32_t B, float lr, double* loss) {
-    lbm::NvtxRange nvtx_("lbm_surrogate_train_step");
-    if (!s || !xin || !target || !mask || B <= 0 || B > s->maxB)
-        return sfail(s, LBM_ERR_ARG, "lbm_surrogate_train_step: bad arguments");
-    SCUDA(s, cudaSetDevice(s->device));
+// Queues one training step on the two streams: gradients of the masked MSE into s->g, the loss into
+// host_loss; with lr > 0 also an Adam update.
+lbm_status queue_train_step(lbm_surrogate* s, const void* xin, const float* target,
+                            const uint8_t* mask, int32_t B, float lr) {
     lbm_status st = forward(s, (const bf16*)xin, B);
     if (st != LBM_OK) return st;
     const long long P = (long long)B * s->H * s->W;
@@ -1625,6 +1494,151 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
         SCUDA(s, launch_pdl(k_adam, dim3(s->tab.tile[s->tab.n]), 256, 0, s->stream, s->w, s->g, s->m, s->v,
                             (long long)s->nparams, s->base + 1, lr, b1, b2, 1e-8f, c1, c2, s->wb, s->wbd,
                             s->tab));
+    }
+    return LBM_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_batch,
+                                int32_t device, lbm_surrogate** out) {
+    if (!out) return sfail(nullptr, LBM_ERR_ARG, "lbm_surrogate_create: out is NULL");
+    *out = nullptr;
+    if (H <= 0 || W <= 0 || H % 8 || W % 8 || (base != 8 && base != 16 && base != 32) ||
+        max_batch <= 0)
+        return sfail(nullptr, LBM_ERR_ARG,
+                     "lbm_surrogate_create: H, W multiples of 8, base 8, 16 or 32, batch > 0");
+    if (cudaSetDevice(device) != cudaSuccess) {
+        cudaGetLastError();
+        return sfail(nullptr, LBM_ERR_CUDA, "lbm_surrogate_create: cannot select the device");
+    }
+    lbm_surrogate* s = new lbm_surrogate();
+    s->H = H;
+    s->W = W;
+    s->base = base;
+    s->maxB = max_batch;
+    s->device = device;
+    build(s);
+    s->tab.n = std::min<int>(24, (int)s->convs.size());  // 17 convolutions
+    for (int k = 0; k < s->tab.n; ++k) {
+        const Conv& c = s->convs[k];
+        s->tab.tile[k + 1] = s->tab.tile[k] + (c.Cout + 31) / 32 * ((9 * (c.C1 + c.C2) + 31) / 32);
+        s->tab.off[k] = (long long)s->convs[k].w_off;
+        s->tab.cout[k] = s->convs[k].Cout;
+        s->tab.cin[k] = s->convs[k].C1 + s->convs[k].C2;
+    }
+    auto cleanup = [&](const char* e) {
+        lbm_surrogate_destroy(s);
+        return sfail(nullptr, LBM_ERR_CUDA, std::string("lbm_surrogate_create: ") + e);
+    };
+    cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return cleanup(cudaGetErrorString(e));
+    size_t colmax = 0;
+    for (const Conv& c : s->convs)
+        colmax = std::max(colmax, (size_t)max_batch * c.H * c.W * 9 * (c.C1 + c.C2));
+    s->col_elems = colmax;
+    for (size_t k = 1; k < s->t.size() && e == cudaSuccess; ++k) {
+        Tensor& x = s->t[k];
+        const size_t n = (size_t)max_batch * x.H * x.W * x.C;
+        e = cudaMalloc((void**)&x.y, n * sizeof(bf16));
+        if (e == cudaSuccess) e = cudaMalloc((void**)&x.dy, n * sizeof(float));
+    }
+    const size_t np = s->nparams;
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->w, np * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->g, np * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->m, np * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->v, np * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->wb, np * sizeof(bf16));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->wbd, np * sizeof(bf16));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->col, colmax * sizeof(bf16));
+    for (Conv& c : s->convs) {
+        if (e == cudaSuccess)
+            e = cudaMalloc((void**)&c.g, (size_t)max_batch * c.H * c.W * c.Cout * sizeof(bf16));
+        if (e == cudaSuccess)
+            e = cudaMalloc((void**)&c.bpart, (size_t)kReluBlocks * c.Cout * sizeof(float));
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.ready, cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->head_ready, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->side_done, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->dz, (size_t)max_batch * H * W * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->n_mask, sizeof(int));
+    if (e == cudaSuccess) e = cudaHostAlloc((void**)&s->host_loss, sizeof(float), cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&s->host_loss_dev, s->host_loss, 0);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->phi, (size_t)max_batch * H * W * sizeof(float));
+    if (e == cudaSuccess)
+        e = cudaMalloc((void**)&s->hpart, (size_t)s->part_blocks * (base + 2) * sizeof(float));
+    size_t wmax = 0;
+    for (const Conv& c : s->convs) wmax = std::max(wmax, (size_t)c.Cout * 9 * (c.C1 + c.C2));
+    s->splitk_elems = std::min<size_t>(wmax * 128, (size_t)64 << 20);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->splitk, s->splitk_elems * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&s->splitk_side, s->splitk_elems * sizeof(float));
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->w, 0, np * sizeof(float), s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->m, 0, np * sizeof(float), s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->v, 0, np * sizeof(float), s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->wb, 0, np * sizeof(bf16), s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->wbd, 0, np * sizeof(bf16), s->stream);
+    if (e != cudaSuccess) return cleanup(cudaGetErrorString(e));
+    make_tensor_maps(s);
+    *out = s;
+    return LBM_OK;
+}
+
+int64_t lbm_surrogate_num_params(const lbm_surrogate* s) { return s ? (int64_t)s->nparams : 0; }
+
+lbm_status lbm_surrogate_set_weights(lbm_surrogate* s, const float* host, int64_t n) {
+    if (!s || !host || n != (int64_t)s->nparams)
+        return sfail(s, LBM_ERR_ARG, "lbm_surrogate_set_weights: need num_params floats");
+    SCUDA(s, cudaSetDevice(s->device));
+    SCUDA(s, cudaMemcpyAsync(s->w, host, n * sizeof(float), cudaMemcpyHostToDevice, s->stream));
+    SCUDA(s, refresh_bf16_weights(s));
+    SCUDA(s, cudaMemsetAsync(s->m, 0, n * sizeof(float), s->stream));
+    SCUDA(s, cudaMemsetAsync(s->v, 0, n * sizeof(float), s->stream));
+    s->adam_t = 0;
+    SCUDA(s, cudaStreamSynchronize(s->stream));
+    return LBM_OK;
+}
+
+lbm_status lbm_surrogate_get_weights(lbm_surrogate* s, float* host, int64_t n, int32_t grads) {
+    if (!s || !host || n != (int64_t)s->nparams)
+        return sfail(s, LBM_ERR_ARG, "lbm_surrogate_get_weights: need num_params floats");
+    SCUDA(s, cudaSetDevice(s->device));
+    SCUDA(s, cudaMemcpyAsync(host, grads ? s->g : s->w, n * sizeof(float), cudaMemcpyDeviceToHost,
+                             s->stream));
+    SCUDA(s, cudaStreamSynchronize(s->stream));
+    return LBM_OK;
+}
+
+lbm_status lbm_surrogate_forward(lbm_surrogate* s, const void* x, int32_t B, float* phi_out) {
+    lbm::NvtxRange nvtx_("lbm_surrogate_forward");
+    if (!s || !x || !phi_out || B <= 0 || B > s->maxB)
+        return sfail(s, LBM_ERR_ARG, "lbm_surrogate_forward: bad arguments");
+    SCUDA(s, cudaSetDevice(s->device));
+    lbm_status st = forward(s, (const bf16*)x, B);
+    if (st != LBM_OK) return st;
+    const long long P = (long long)B * s->H * s->W;
+    const int nb = std::min(s->part_blocks, blocks_for(P));
+    SCUDA(s, launch_head(s, nb, phi_out, P, nullptr, nullptr));
+    SCUDA(s, cudaStreamSynchronize(s->stream));
+    if (tc_timed_out())
+        return sfail(s, LBM_ERR_TIMEOUT, "lbm_surrogate_forward: a tensor-core wait timed out");
+    return LBM_OK;
+}
+
+// Gradients of the masked MSE into s->g; with lr > 0 also an Adam update. *loss gets the loss.
+lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const float* target,
+                                    const uint8_t* mask, int32_t B, float lr, double* loss) {
+    lbm::NvtxRange nvtx_("lbm_surrogate_train_step");
+    if (!s || !xin || !target || !mask || B <= 0 || B > s->maxB)
+        return sfail(s, LBM_ERR_ARG, "lbm_surrogate_train_step: bad arguments");
+    SCUDA(s, cudaSetDevice(s->device));
+    const lbm_status st = queue_train_step(s, xin, target, mask, B, lr);
+    if (st != LBM_OK) {
+        // the next call's kernels must not overwrite what the side stream still reads
+        cudaStreamSynchronize(s->side);
+        return st;
     }
     SCUDA(s, cudaStreamSynchronize(s->stream));
     if (tc_timed_out())
