@@ -149,6 +149,7 @@ struct lbm_ctx {
     bool graphs_ready = false;
     bool graph_failed = false;
     int tile_x = 32, tile_y = 16, min_blocks = 0;
+    int resident[2] = {0, 0};  // tiles of that variant on the chip at once: half-way, interpolated walls
     bool autotune_pending = false;  // LBM_TILE_AUTO: tune at the first lbm_step
     std::string err;
 };

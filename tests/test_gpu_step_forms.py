@@ -76,3 +76,25 @@ def test_fp64_on_ragged_lattices(lbm, oracle_mod, nx, ny, concave, interp):
                 break  # a start this small can leave the stable range in both
             assert np.abs(a - b).max() <= 1e-9 * cfg.rho_l
         lat.close()
+
+
+def test_tiles_that_fit_at_once_are_spread_over_the_chip(lbm, oracle_mod):
+    """A lattice of 459 tiles against one of 720, both on the chip at once (760 places): three tiles
+    per SM against five. Evenly spread the first takes 0.77 of the second's time, with tiles
+    crowding onto some SMs 0.97; the bound lies between."""
+    import time
+    us = []
+    for nx, ny in ((517, 425), (768, 480)):
+        R = nx // 2 - 10.0
+        w = W.Workload("t", nx, ny, (nx // 2 + 0.0, R + 6.0, R), (nx // 2 + 0.0, 0.2 * ny, 0.15 * ny, 5.6),
+                       concave=True)
+        lat = gpu_lattice(lbm, oracle_config(oracle_mod, w)[0])
+        best = float("inf")
+        for _ in range(15):
+            t = time.perf_counter()
+            lat.step(128)
+            lat.synchronize()
+            best = min(best, time.perf_counter() - t)
+        us.append(best / 128 * 1e6)
+        lat.close()
+    assert us[0] < 0.87 * us[1], us
