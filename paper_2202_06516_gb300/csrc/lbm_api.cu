@@ -446,7 +446,7 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const lbm_geometry* g) {
         LBM_CUDA(c, lbm::launch_geometry(c, a));
     }
     // captured step graphs stay valid across geometries (the kernels read the same buffers);
-    // they hold the boundary scheme and the variant, so a change of either drops them
+    // they hold the boundary scheme, the variant and its form, so a change of one drops them
     const bool ibb = g->boundary == LBM_BB_INTERP;
     if (ibb != c->ibb) destroy_graphs(c);
     c->ibb = ibb;
@@ -478,6 +478,9 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const lbm_geometry* g) {
     }
     c->geom = *g;
     c->geom.rho0 = nullptr;
+    const int form = lbm::step_form(c);
+    if (form != c->form) destroy_graphs(c);
+    c->form = form;
     c->sub.circle = g->has_circle ? 1 : 0;
     c->sub.concave = g->has_circle && g->concave ? 1 : 0;
     c->sub.cx = g->cx;

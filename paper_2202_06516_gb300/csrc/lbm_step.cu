@@ -68,18 +68,16 @@ cudaError_t allow_smem() {
 // recomputed halo and the fewer resident tiles make them slower. Chosen by the number of tiles
 // against the number of SMs. Measured, us per step, 32x16 tiles of 256 threads / forms 1 / 2 / 3:
 // 128x96 7.4 / 4.3 / 5.1 / 4.8; 200x120 8.0 / 4.6 / 5.1 / 5.2; 256x256 8.0 / 6.0 / 5.2 / 5.6;
-// 520x190 10.2 / 6.8 / 7.2 / 6.1; 512x384 11.6 / 10.8 / 10.5 / 8.5; 768x512 12.1 / 17 / 17 / 13.3.
+// 520x190 10.2 / 6.8 / 7.2 / 6.1.
+// Form 3 holds three tiles per SM (456). Up to twice as many run as a second wave, which pays only
+// where the 256-thread form is held up by tiles that a curved wall crosses (its threads take several
+// rounds of wetting layers and cut links), the more the larger the circle; half-way walls, us per step,
+// 256 threads / form 3: 128x1000 (500 tiles) R = 4 7.4 / 7.5, R = 16 8.4 / 7.5; 128x1200 (600) R = 8
+// 7.8 / 7.9, R = 16 8.3 / 8.0, R = 48 9.8 / 7.9; 512x400 (800) R = 16 9.2 / 9.3, R = 32 9.5 / 9.3, R = 64
+// 10.2 / 9.3; 400x560 (910) R = 16 9.5 / 10.5, R = 64 10.0 / 10.5. A cavity leaves most tiles empty:
+// 700x328 (902) 11.4 / 10.3, 1000x224 (896) 11.3 / 9.1. Interpolated walls take longer in the 256-thread
+// form at every size: 128x1200 (600), R = 3, 10.5 / 9.2, 512x456 (912) 15.0 / 11.1.
 #define LBM_SMALL_FORMS(X) X(1, 16, 8, 320, 3) X(2, 32, 16, 640, 1) X(3, 32, 8, 384, 3)
-int small_form(const lbm_ctx* c) {
-    const long long nx = c->nx, ny = c->ny, sms = c->sms;
-    auto tiles = [&](long long tx, long long ty) {
-        return ((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
-    };
-    if (2 * tiles(16, 8) <= 3 * sms) return 1;
-    if (tiles(32, 16) <= sms) return 2;
-    if (tiles(32, 8) <= 6 * sms) return 3;
-    return 0;
-}
 
 // Whether a step of the 256-thread forms is placed early. A grid that fits on the chip at once leaves
 // slots free, and early placement fills those as they are: some SMs get five tiles of the next step,
@@ -128,7 +126,7 @@ cudaError_t configure_one(lbm_ctx* c) {
 template <typename T, int TX, int TY, int MINB>
 cudaError_t launch_one(lbm_ctx* c, const StepArgs<T>& a, bool macro) {
     if constexpr (has_ibb<T, TX, TY, MINB>()) {
-        const int form = macro ? 0 : small_form(c);
+        const int form = macro ? 0 : c->form;
 #define X(F, A, B, N, M)                                                       \
     if (form == F)                                                             \
         return c->ibb ? launch_k<float, A, B, N, M, false, true>(c, a, true)   \
@@ -228,6 +226,21 @@ cudaError_t step_configure(lbm_ctx* c) {
     LBM_STEP_VARIANTS(X)
 #undef X
     return cudaErrorInvalidValue;
+}
+
+int step_form(const lbm_ctx* c) {
+    const long long nx = c->nx, ny = c->ny, sms = c->sms;
+    auto tiles = [&](long long tx, long long ty) {
+        return ((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
+    };
+    if (2 * tiles(16, 8) <= 3 * sms) return 1;
+    if (tiles(32, 16) <= sms) return 2;
+    const lbm_geometry& g = c->geom;
+    const int half_sms = c->ibb || (g.has_circle && g.concave)  ? 12
+                         : g.has_circle && g.R >= 32 ? 11
+                         : g.has_circle && g.R >= 16 ? 10
+                                                     : 6;
+    return 2 * tiles(32, 8) <= half_sms * sms ? 3 : 0;
 }
 
 cudaError_t launch_step(lbm_ctx* c, int src, bool macro) {
