@@ -1,0 +1,48 @@
+"""GPU tests of what a batched step costs beside its tiles: the launch's CTAs past the tile table, and
+how the tiles of a small batch are spread over the chip. Times are the least of several runs; each
+bound lies between two measured behaviours."""
+import time
+
+import pytest
+
+from paper_2202_06516_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    from paper_2202_06516_gb300 import lbm as L
+    L.lib()
+    return L
+
+
+def _batch(lbm, sizes, running=None, **kw):
+    b = lbm.Batch(sizes, **W.MODEL, **kw)
+    mu = W.MODEL["k2"] * lbm.lbm_coexistence(W.MODEL["eos"], W.MODEL["Tr"])["mu_sat"]
+    for i, (nx, ny) in enumerate(sizes[:running]):
+        R = float(max(6, min(nx, ny) // 4))
+        b.set_geometry(i, circle=(nx // 2 + 0.0, 0.0, R), mu_circle=mu, mu_bottom=mu, mu_top=mu,
+                       drop=(nx // 2 + 0.0, R + 0.3 * ny, 0.15 * ny, 5.6))
+    return b
+
+
+def _us_per_step(b, steps=400, runs=8):
+    best = float("inf")
+    for _ in range(runs):
+        t = time.perf_counter()
+        b.run(steps, check_every=steps, tol=0.0)
+        best = min(best, time.perf_counter() - t)
+    return best / steps * 1e6
+
+
+def test_ctas_past_the_tile_table_leave_at_once(lbm):
+    """One running lattice in a batch of 64 (20,480 CTAs per step, 320 with a tile): 13 us per step when
+    the others leave after reading the table's length, 21 us when each first releases the next launch."""
+    b = _batch(lbm, [(512, 320)] * 64, running=1)
+    us = _us_per_step(b)
+    b.close()
+    assert us < 18.0, us
