@@ -294,6 +294,14 @@ lbm_status upload_tiles(lbm_batch* b, int p, int* ntiles, std::vector<int>* act)
     return LBM_OK;
 }
 
+// Early placement (as for k_step) crowds the next step's tiles onto some SMs when a 256-thread form's grid
+// leaves slots free; with four and more tiles per SM the overlap outweighs it. us per step, early / not:
+// 464 tiles 13.7 / 12.0, 531 13.9 / 13.3, 599 13.9 / 13.3, 616 14.4 / 15.0, 687 13.8 / 15.5, 720 13.6 / 15.5. The small
+// forms gain at every size (the 384-thread form, 563 tiles: 8.0 / 9.0).
+bool place_early(const lbm_batch* b, int grid) {
+    return b->variant >= kBatchSmall0 || b->persistent || grid > 4 * b->inst[0]->sms;
+}
+
 cudaError_t launch_batch_step(lbm_batch* b, int parity) {
     int i = 0;
     int grid = b->grid;
@@ -302,9 +310,10 @@ cudaError_t launch_batch_step(lbm_batch* b, int parity) {
         for (const lbm_ctx* c : b->inst) all += tiles_of(b, c);
         grid = (int)std::max<long long>(1, all);
     }
+    const bool early = place_early(b, grid);
 #define X(A, B, M, N)                                                                        \
     if (b->variant == i++) {                                                                 \
-        cudaLaunchAttribute at{};  /* as for k_step: overlap with the previous step's tail */ \
+        cudaLaunchAttribute at{};                                                            \
         at.id = cudaLaunchAttributeProgrammaticStreamSerialization;                          \
         at.val.programmaticStreamSerializationAllowed = 1;                                   \
         cudaLaunchConfig_t cfg{};                                                            \
@@ -313,7 +322,7 @@ cudaError_t launch_batch_step(lbm_batch* b, int parity) {
         cfg.dynamicSmemBytes = Layout<float, A, B>::bytes;                                   \
         cfg.stream = b->stream;                                                              \
         cfg.attrs = &at;                                                                     \
-        cfg.numAttrs = 1;                                                                    \
+        cfg.numAttrs = early ? 1 : 0;                                                        \
         return cudaLaunchKernelEx(&cfg, k_batch_step<A, B, M, N>, (const StepArgs<float>)b->model, \
                                   (const BatchInst*)b->d_desc, (const int2*)b->d_tiles,      \
                                   (const int*)b->d_ntiles, parity);                          \

@@ -46,3 +46,14 @@ def test_ctas_past_the_tile_table_leave_at_once(lbm):
     us = _us_per_step(b)
     b.close()
     assert us < 18.0, us
+
+
+def test_tiles_of_a_small_batch_are_spread_over_the_chip(lbm):
+    """528 tiles of 32x16 against 704: three to four tiles per SM against five. Evenly spread the first
+    take 0.89 of the second's time, crowded 0.98."""
+    us = []
+    for sizes in ([(230, 340)] * 3, [(110, 345)] * 8):
+        b = _batch(lbm, sizes)
+        us.append(_us_per_step(b, steps=1000))
+        b.close()
+    assert us[0] < 0.95 * us[1], us
