@@ -99,9 +99,7 @@ __global__ void __launch_bounds__(NT, MINB)
         const BatchInst& I = inst[e.x];
         StepArgs<float> a = model;
         a.h_in = I.h[parity];
-        a.h_out = I.h[parity ^ 1];
         a.rho_in = I.rho[parity];
-        a.rho_out = I.rho[parity ^ 1];
         a.flags = I.flags;
         a.muw = I.muw;
         a.nx = I.nx;
@@ -110,7 +108,14 @@ __global__ void __launch_bounds__(NT, MINB)
         a.plane = I.plane;
         const int tiles_x = (I.nx + TX - 1) / TX;
         const int ty = e.y / tiles_x, tx = e.y - ty * tiles_x;
-        step_tile<float, TX, TY, NT, false, false>(a, I.rho_mid, smem_raw, tx * TX, ty * TY);
+        // read late where registers are short (48 of the 256-thread forms; held through the collision they
+        // spilled 4 to 12 bytes, 22.4 against 22.1 ms on the 64-instance sweep); the 384-thread form has
+        // room, and waits for no load at its end (563 tiles: 8.0 us per step, 8.6 read late)
+        const StepOut<float> now{I.h[parity ^ 1], I.rho[parity ^ 1]};
+        const auto out = [&] {
+            return NT == 384 ? now : StepOut<float>{I.h[parity ^ 1], I.rho[parity ^ 1]};
+        };
+        step_tile<float, TX, TY, NT, false, false, false>(a, out, I.rho_mid, smem_raw, tx * TX, ty * TY);
         __syncthreads();  // the next tile reuses shared memory
     }
 }

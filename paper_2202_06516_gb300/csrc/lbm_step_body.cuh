@@ -250,14 +250,21 @@ __device__ __forceinline__ void pull(const StepArgs<T>& a, unsigned us, int o, c
     }
 }
 
+// Where a step writes (planes other than StepArgs::hq_out), asked for when the tile gets there: the batched
+// kernel reads these pointers of its instance then and holds no registers for them while it collides.
+template <typename T>
+struct StepOut {
+    T *h, *rho;
+};
+
 // (6) of the step: new density rho(t+1) = sum_q f*_q(x - e_q) (half-way bounce-back where the
 // source is not fluid) and the stored deviations f*_q(x) - w_q rho(t+1)(x). EDGE: the tile lies
 // within kPadX of an x edge and also writes the periodic images into the pads. PP: the planes
 // are addressed through the per-plane pointers of StepArgs (single-lattice kernel), else as
-// h_out + q * plane (batched kernel).
+// StepOut::h + q * plane (batched kernel).
 template <typename T, int TX, int TY, int NT, bool MIXED, bool EDGE, bool PP>
-__device__ __forceinline__ void stream_out(const StepArgs<T>& a, const T* s_rho, const T* s_g,
-                                           const uint8_t* s_flag, int x0, int y0) {
+__device__ __forceinline__ void stream_out(const StepArgs<T>& a, const StepOut<T> to, const T* s_rho,
+                                           const T* s_g, const uint8_t* s_flag, int x0, int y0) {
     using L = Layout<T, TX, TY>;
     constexpr int RW = L::RW, CW = L::CW, CH = L::CH;
     const unsigned upl = (unsigned)a.plane;
@@ -288,23 +295,23 @@ __device__ __forceinline__ void stream_out(const StepArgs<T>& a, const T* s_rho,
             const bool lo = gx < kPadX, hi = gx >= a.nx - kPadX;
 #pragma unroll
             for (int q = 0; q < 9; ++q) {
-                T* ob = (PP ? a.hq_out[q] : a.h_out + (unsigned)q * upl) + us;
+                T* ob = (PP ? a.hq_out[q] : to.h + (unsigned)q * upl) + us;
                 ob[0] = v[q];
                 if (lo) ob[a.nx] = v[q];
                 if (hi) ob[-a.nx] = v[q];
             }
-            a.rho_out[us] = r1;
-            if (lo) a.rho_out[us + a.nx] = r1;
-            if (hi) a.rho_out[us - a.nx] = r1;
+            to.rho[us] = r1;
+            if (lo) to.rho[us + a.nx] = r1;
+            if (hi) to.rho[us - a.nx] = r1;
         } else {
 #pragma unroll
             for (int q = 0; q < 9; ++q) {
                 if (PP)
                     a.hq_out[q][us] = v[q];
                 else
-                    a.h_out[us + (unsigned)q * upl] = v[q];
+                    to.h[us + (unsigned)q * upl] = v[q];
             }
-            a.rho_out[us] = r1;
+            to.rho[us] = r1;
         }
     }
 }
@@ -313,9 +320,9 @@ __device__ __forceinline__ void stream_out(const StepArgs<T>& a, const T* s_rho,
 // wetting layers are rebuilt and every neighbour access checks the node class. Interior tiles
 // take the branch-free path (the choice is uniform per CTA). IBB: interpolated, mass-corrected
 // bounce-back on cut links (a separate kernel, so the default one carries none of its code).
-template <typename T, int TX, int TY, int NT, bool MACRO, bool MIXED, bool PP, bool IBB = false>
-__device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid, T* s_rho,
-                                          T* s_mu, T* s_g, const uint8_t* s_flag, int x0,
+template <typename T, int TX, int TY, int NT, bool MACRO, bool MIXED, bool PP, bool IBB, typename Out>
+__device__ __forceinline__ void step_body(const StepArgs<T>& a, const Out& out, const T rho_mid,
+                                          T* s_rho, T* s_mu, T* s_g, const uint8_t* s_flag, int x0,
                                           int y0) {
     using L = Layout<T, TX, TY>;
     constexpr int RW = L::RW, RH = L::RH, MW = L::MW, MH = L::MH, CW = L::CW, CH = L::CH;
@@ -480,14 +487,15 @@ __device__ __forceinline__ void step_body(const StepArgs<T>& a, const T rho_mid,
         }
     }
     if (MACRO) return;
+    const StepOut<T> to = out();
     __syncthreads();
 
     // (6) streaming into the tile: new density and deviations; tiles within kPadX of the x
     // edges also refresh the periodic images in the pads (a CTA-uniform branch)
     if (x0 < kPadX || x0 + TX > a.nx - kPadX)
-        stream_out<T, TX, TY, NT, MIXED, true, PP>(a, s_rho, s_g, s_flag, x0, y0);
+        stream_out<T, TX, TY, NT, MIXED, true, PP>(a, to, s_rho, s_g, s_flag, x0, y0);
     else
-        stream_out<T, TX, TY, NT, MIXED, false, PP>(a, s_rho, s_g, s_flag, x0, y0);
+        stream_out<T, TX, TY, NT, MIXED, false, PP>(a, to, s_rho, s_g, s_flag, x0, y0);
 }
 
 // Programmatic dependent launch (no effect without its launch attribute): the next step's blocks
@@ -546,8 +554,8 @@ __device__ __forceinline__ int stage_load(const StepArgs<T>& a, T* s_rho, uint8_
 }
 
 // One time step of one TX x TY tile with origin (x0, y0); smem holds Layout<T, TX, TY>::bytes.
-template <typename T, int TX, int TY, int NT, bool MACRO, bool PP, bool IBB = false>
-__device__ __forceinline__ void step_tile(const StepArgs<T>& a, const T rho_mid,
+template <typename T, int TX, int TY, int NT, bool MACRO, bool PP, bool IBB, typename Out>
+__device__ __forceinline__ void step_tile(const StepArgs<T>& a, const Out& out, const T rho_mid,
                                           unsigned char* smem, int x0, int y0) {
     using L = Layout<T, TX, TY>;
     constexpr int RW = L::RW, RH = L::RH, MW = L::MW, MH = L::MH, CW = L::CW, CH = L::CH;
@@ -561,17 +569,19 @@ __device__ __forceinline__ void step_tile(const StepArgs<T>& a, const T rho_mid,
     // (an all-fluid staged region certainly holds fluid nodes: one barrier less for those)
     if (mixed && !__syncthreads_or(any & 2)) return;
     if (mixed)
-        step_body<T, TX, TY, NT, MACRO, true, PP, IBB>(a, rho_mid, s_rho, s_mu, s_g, s_flag, x0,
+        step_body<T, TX, TY, NT, MACRO, true, PP, IBB>(a, out, rho_mid, s_rho, s_mu, s_g, s_flag, x0,
                                                        y0);
     else
-        step_body<T, TX, TY, NT, MACRO, false, PP>(a, rho_mid, s_rho, s_mu, s_g, s_flag, x0, y0);
+        step_body<T, TX, TY, NT, MACRO, false, PP, false>(a, out, rho_mid, s_rho, s_mu, s_g, s_flag, x0,
+                                                          y0);
 }
 
 template <typename T, int TX, int TY, int NT, bool MACRO, int MINB, bool IBB = false>
 __global__ void __launch_bounds__(NT, MINB) k_step(const StepArgs<T> a, const T rho_mid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_launch_next();
-    step_tile<T, TX, TY, NT, MACRO, true, IBB>(a, rho_mid, smem_raw, blockIdx.x * TX,
+    const auto out = [&] { return StepOut<T>{a.h_out, a.rho_out}; };
+    step_tile<T, TX, TY, NT, MACRO, true, IBB>(a, out, rho_mid, smem_raw, blockIdx.x * TX,
                                                blockIdx.y * TY);
 }
 
