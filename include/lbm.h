@@ -290,7 +290,8 @@ lbm_status lbm_batch_run(lbm_batch *b, int64_t max_steps, int32_t check_every, d
  * 32x32, each with its register budget) in both grid modes (one CTA per tile, then persistent;
  * entries in that order, 2 per variant) over trial_steps launches on
  * the tile table of the instances that have geometry (those sharing the parity of the first), and
- * keeps the fastest for later lbm_batch_run calls. As in lbm_autotune the trial launches do not
+ * keeps the fastest for later lbm_batch_run calls. A batch of few tiles also times the form with smaller
+ * tiles that it runs by default; the entries of 32x16 then give the faster of the two. As in lbm_autotune the trial launches do not
  * advance any instance. entries / n_out as in lbm_autotune. LBM_ERR_STATE if no instance has
  * geometry. Synchronous. */
 lbm_status lbm_batch_autotune(lbm_batch *b, int32_t trial_steps, lbm_tune_entry *entries,

@@ -49,6 +49,7 @@ struct lbm_batch {
     int grid = 0;                 // resident slots (persistent grid)
     bool persistent = false;      // grid mode: resident slots, or one CTA per tile
     int variant = 0;              // index into the compiled tile variants
+    int form = 0;                 // what the default stands for here: itself or a small-lattice form
     int tx = 32, ty = 16;         // its tile shape
     bool autotune_pending = false;
     cudaGraphExec_t graph = nullptr;
@@ -68,7 +69,7 @@ constexpr int NTB = 256;
 // Compiled tile variants of the batched kernel: tile (TX, TY), the CTAs per SM its register budget
 // is fitted to, and threads. Variant 1 (32 x 16, 5 CTAs/SM) is the default; the autotuner times
 // the first four on the batch's own tile table. The others are the small-lattice forms of the
-// default (see lbm_step.cu), taken where all instances together have few tiles.
+// default (see lbm_step.cu), taken where all instances together have few tiles, and timed there too.
 #define LBM_BATCH_VARIANTS(X) X(32, 8, 5, 256) X(32, 16, 5, 256) X(64, 16, 3, 256) X(32, 32, 3, 256)
 #define LBM_BATCH_SMALL(X) X(16, 8, 3, 320) X(32, 8, 3, 384)
 constexpr int kBatchDefaultVariant = 1, kBatchSmall0 = 4, kBatchSmall1 = 5;
@@ -460,9 +461,8 @@ lbm_status lbm_batch_create(const lbm_params* model, int32_t n, const int32_t* n
             t32 += tiles_of(c, 32, 8);
         }
         const long long sms = b->inst[0]->sms;
-        e = configure_variant(b, 2 * t16 <= 3 * sms ? kBatchSmall0
-                                 : t32 <= 6 * sms   ? kBatchSmall1
-                                                    : kBatchDefaultVariant);
+        b->form = 2 * t16 <= 3 * sms ? kBatchSmall0 : t32 <= 6 * sms ? kBatchSmall1 : kBatchDefaultVariant;
+        e = configure_variant(b, b->form);
     }
     if (e != cudaSuccess)
         return cleanup(LBM_ERR_CUDA, std::string("lbm_batch_create: ") + cudaGetErrorString(e));
@@ -642,12 +642,18 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int32_t trial_steps, lbm_tune_entry*
     const int keep = b->variant;
     const bool keep_persistent = b->persistent;
     int best = -1;
+    bool best_persistent = false;
     double best_us = 0;
     lbm_status st = LBM_OK;
     std::vector<int> act;
-    // trial k: tile variant k / 2, grid one CTA per tile (k even) or persistent (k odd)
-    for (int k2 = 0; k2 < 2 * num_variants() && err == cudaSuccess && st == LBM_OK; ++k2) {
-        const int v = k2 / 2;
+    // trial k: tile variant k / 2, grid one CTA per tile (k even) or persistent (k odd); last the form that
+    // a batch of few tiles runs by default, which shares the entries of the variant it stands for
+    const int n_entries = 2 * num_variants();
+    const int n_trials = n_entries + (b->form != kBatchDefaultVariant ? 2 : 0);
+    double us_of[2 * 8] = {};
+    for (int k2 = 0; k2 < n_trials && err == cudaSuccess && st == LBM_OK; ++k2) {
+        const int v = k2 < n_entries ? k2 / 2 : b->form;
+        const int at = k2 < n_entries ? k2 : 2 * kBatchDefaultVariant + (k2 & 1);
         b->persistent = (k2 & 1) != 0;
         err = configure_variant(b, v);
         if (err != cudaSuccess) break;
@@ -666,11 +672,13 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int32_t trial_steps, lbm_tune_entry*
         if (err != cudaSuccess) break;
         const double us = 1e3 * (double)ms / trial_steps;
         int vx = 0, vy = 0, vm = 0;
-        variant_shape(v, &vx, &vy, &vm);
-        if (entries && k2 < max_entries)
-            entries[k2] = lbm_tune_entry{vx, vy, vm, us, b->persistent ? 1 : 0};
+        variant_shape(at / 2, &vx, &vy, &vm);
+        us_of[at] = k2 < n_entries ? us : std::min(us, us_of[at]);
+        if (entries && at < max_entries)
+            entries[at] = lbm_tune_entry{vx, vy, vm, us_of[at], b->persistent ? 1 : 0};
         if (best < 0 || us < best_us) {
-            best = k2;
+            best = v;
+            best_persistent = b->persistent;
             best_us = us;
         }
     }
@@ -678,8 +686,8 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int32_t trial_steps, lbm_tune_entry*
     if (e1) cudaEventDestroy(e1);
     b->running = keep_running;
     const bool ok = err == cudaSuccess && st == LBM_OK && best >= 0;
-    b->persistent = ok ? (best & 1) != 0 : keep_persistent;
-    const cudaError_t ce = configure_variant(b, ok ? best / 2 : keep);
+    b->persistent = ok ? best_persistent : keep_persistent;
+    const cudaError_t ce = configure_variant(b, ok ? best : keep);
     if (st != LBM_OK) return st;
     BCUDA(b, err);
     BCUDA(b, ce);
@@ -688,7 +696,7 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int32_t trial_steps, lbm_tune_entry*
     b->graph = nullptr;
     b->graph_chunk = 0;
     b->graph_parity = -1;
-    if (n_out) *n_out = 2 * num_variants();
+    if (n_out) *n_out = n_entries;
     return LBM_OK;
 }
 

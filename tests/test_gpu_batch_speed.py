@@ -57,3 +57,21 @@ def test_tiles_of_a_small_batch_are_spread_over_the_chip(lbm):
         us.append(_us_per_step(b, steps=1000))
         b.close()
     assert us[0] < 0.95 * us[1], us
+
+
+@pytest.mark.parametrize("auto", [False, True])
+def test_autotuning_keeps_the_form_of_small_batches(lbm, auto):
+    """Two 96x64 lattices run in 320-thread tiles of 16x8, which the tuner has to time as well: tuned
+    (by hand or at the first run) the batch is no slower than untuned, where the 256-thread variants
+    take 1.5 times as long. The entries keep their order and number."""
+    sizes = [(96, 64)] * 2
+    plain, tuned = _batch(lbm, sizes), _batch(lbm, sizes, tile_auto=auto)
+    if not auto:
+        res = tuned.autotune(20)
+        tiles = [(32, 8), (32, 16), (64, 16), (32, 32)]
+        assert [(r["tile"], r["persistent"]) for r in res] == [(t, p) for t in tiles for p in (False, True)]
+        assert min(res, key=lambda r: r["us_per_step"])["tile"] == (32, 16)
+    a, b = _us_per_step(plain, steps=1000), _us_per_step(tuned, steps=1000)
+    plain.close()
+    tuned.close()
+    assert b < 1.15 * a, (a, b)
