@@ -243,7 +243,10 @@ __device__ __forceinline__ double substrate_dist(const Substrate& s, double px, 
 
 // Bit sl: the link of fluid node (i, j) along slot sl joins liquid and gas and its point may lie in
 // the measurement's band. PRE: points whose FP32 distance is more than a quarter outside the band
-// are dropped here (coordinates and radii up to 10^6: the FP32 distance errs by less than 0.2).
+// are dropped here. Coordinates and radii up to 10^6 make that distance err by less than 0.2; the
+// point's share of the link errs by up to 4 x 2^-24 rho_m / |vb - va| (the roundings of rho_m and of
+// both ends), so links whose ends differ by less than 1e-4 rho_m stay in, and for the others that is
+// below 0.0025 (0.0036 of distance).
 template <typename T, bool PRE>
 __device__ __forceinline__ unsigned crossing_links(T va, const T (&vb)[4], unsigned ends, double rho_m,
                                                    T thr, const Substrate& sub, int i, int j) {
@@ -252,7 +255,9 @@ __device__ __forceinline__ unsigned crossing_links(T va, const T (&vb)[4], unsig
     for (int sl = 0; sl < 4; ++sl) {
         if (!(ends >> sl & 1) || (va > thr) == (vb[sl] > thr)) continue;
         if (PRE) {
-            const float a = (float)va, fr = __fdividef((float)rho_m - a, (float)vb[sl] - a);
+            const float a = (float)va, w = (float)vb[sl] - a;
+            const bool apart = fabsf(w) >= 1e-4f * (float)rho_m;
+            const float fr = __fdividef((float)rho_m - a, w);
             const float x = i + fr * slot_x(sl), y = j + fr * slot_y(sl);
             float d = y + 0.5f;
             if (sub.circle) {
@@ -260,7 +265,7 @@ __device__ __forceinline__ unsigned crossing_links(T va, const T (&vb)[4], unsig
                 d = sqrtf(dx * dx + dy * dy) - (float)sub.Rs;
                 if (sub.concave) d = -d;
             }
-            if (d < 0.25f || d > 2.75f) continue;
+            if (apart && (d < 0.25f || d > 2.75f)) continue;
         }
         m |= 1u << sl;
     }

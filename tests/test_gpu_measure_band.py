@@ -78,3 +78,32 @@ def test_batch_residual_matches_host_sums(lbm):
         want = math.fsum(np.abs(after - before[i]).ravel().tolist()) / math.fsum(after.ravel().tolist())
         assert res[i] == pytest.approx(want, rel=1e-13, abs=0)
     b.close()
+
+
+@pytest.mark.parametrize("R,lift,r,side", [(20.0, 0.0, 12.0, -1), (20.0, 0.0, 17.3, 1),
+                                           (24.5, 0.5, 10.0, -1), (35.0, 0.0, 14.0, 1),
+                                           (35.0, 0.5, 12.0, -1), (28.0, 0.3, 13.0, 1)])
+def test_links_between_nearly_equal_densities(lbm, oracle_mod, R, lift, r, side):
+    """FP64 lattices almost uniform at rho_m: the two densities are one FP32 spacing apart and rho_m lies
+    0.49 spacings from an FP32 number, so that a point placed with FP32 densities sits at the end of its
+    link (up to 0.9 of a link away). The chosen links, distances and angles equal the oracle's on the
+    identical field; in most of these cases the FP32 point of a chosen link lies outside the band."""
+    O = oracle_mod
+    nx, ny = 120, 90
+    w = W.Workload("flat", nx, ny, (60.0, 0.0, R), (60.0, R + 0.6 * r + lift, r, 5.6))
+    cfg = oracle_config(O, w)[0]
+    mid = np.float32(0.5 * (cfg.rho_g + cfg.rho_l))
+    ulp = float(np.spacing(mid))
+    cfg.rho_l = 2 * (float(mid) + side * 0.49 * ulp) - cfg.rho_g
+    rho_m = 0.5 * (cfg.rho_g + cfg.rho_l)
+    jj, ii = np.mgrid[0:ny, 0:nx]
+    low, high = (0.9, 0.1) if side > 0 else (0.1, 0.9)
+    rho = np.where(np.hypot(ii - w.drop[0], jj - w.drop[1]) < r, rho_m + high * ulp, rho_m - low * ulp)
+    lat = gpu_lattice(lbm, cfg, precision=1, rho0=rho)
+    ol, orr, _ = O.measure(cfg, rho, rho_m)
+    for g, o in zip(lat.measure(), (ol, orr)):
+        assert g.status == 0 and o.status == 0
+        assert (g.link1, g.link2) == (o.link1, o.link2)
+        assert g.d1 == o.d1 and g.d2 == o.d2
+        assert abs(g.theta - o.theta) < 1e-6
+    lat.close()
