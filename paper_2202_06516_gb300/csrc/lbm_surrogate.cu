@@ -1328,6 +1328,25 @@ void make_tensor_maps(lbm_surrogate* s) {
     }
 }
 
+// A call that fails while queuing waits for what it queued before it reports: the caller may free or reuse
+// the input, target and mask, and the next call's kernels the buffers that the side stream reads.
+lbm_status settle(lbm_surrogate* s, lbm_status st) {
+    if (st != LBM_OK) {
+        cudaStreamSynchronize(s->side);
+        cudaStreamSynchronize(s->stream);
+    }
+    return st;
+}
+
+lbm_status queue_forward(lbm_surrogate* s, const bf16* x, int32_t B, float* phi) {
+    lbm_status st = forward(s, x, B);
+    if (st != LBM_OK) return st;
+    const long long P = (long long)B * s->H * s->W;
+    const int nb = std::min(s->part_blocks, blocks_for(P));
+    SCUDA(s, launch_head(s, nb, phi, P, nullptr, nullptr));
+    return LBM_OK;
+}
+
 // Queues one training step on the two streams: gradients of the masked MSE into s->g, the loss into
 // host_loss; with lr > 0 also an Adam update.
 lbm_status queue_train_step(lbm_surrogate* s, const void* xin, const float* target,
@@ -1616,11 +1635,8 @@ lbm_status lbm_surrogate_forward(lbm_surrogate* s, const void* x, int32_t B, flo
     if (!s || !x || !phi_out || B <= 0 || B > s->maxB)
         return sfail(s, LBM_ERR_ARG, "lbm_surrogate_forward: bad arguments");
     SCUDA(s, cudaSetDevice(s->device));
-    lbm_status st = forward(s, (const bf16*)x, B);
+    const lbm_status st = settle(s, queue_forward(s, (const bf16*)x, B, phi_out));
     if (st != LBM_OK) return st;
-    const long long P = (long long)B * s->H * s->W;
-    const int nb = std::min(s->part_blocks, blocks_for(P));
-    SCUDA(s, launch_head(s, nb, phi_out, P, nullptr, nullptr));
     SCUDA(s, cudaStreamSynchronize(s->stream));
     if (tc_timed_out())
         return sfail(s, LBM_ERR_TIMEOUT, "lbm_surrogate_forward: a tensor-core wait timed out");
@@ -1634,12 +1650,8 @@ lbm_status lbm_surrogate_train_step(lbm_surrogate* s, const void* xin, const flo
     if (!s || !xin || !target || !mask || B <= 0 || B > s->maxB)
         return sfail(s, LBM_ERR_ARG, "lbm_surrogate_train_step: bad arguments");
     SCUDA(s, cudaSetDevice(s->device));
-    const lbm_status st = queue_train_step(s, xin, target, mask, B, lr);
-    if (st != LBM_OK) {
-        // the next call's kernels must not overwrite what the side stream still reads
-        cudaStreamSynchronize(s->side);
-        return st;
-    }
+    const lbm_status st = settle(s, queue_train_step(s, xin, target, mask, B, lr));
+    if (st != LBM_OK) return st;
     SCUDA(s, cudaStreamSynchronize(s->stream));
     if (tc_timed_out())
         return sfail(s, LBM_ERR_TIMEOUT, "lbm_surrogate_train_step: a tensor-core wait timed out");
