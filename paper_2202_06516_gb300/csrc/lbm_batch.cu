@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(NT, MINB)
 constexpr int kResSlices = 32;
 __global__ void __launch_bounds__(NTB)
     k_batch_residual(const BatchInst* inst, const int* active, int parity, double* part,
-                     unsigned* tickets, double* res, int refresh) {
+                     unsigned* tickets, double* res) {
     const int id = active[blockIdx.x];
     const BatchInst& I = inst[id];
     const float* rho = I.rho[parity];
@@ -143,10 +143,8 @@ __global__ void __launch_bounds__(NTB)
             load8(rho + o, r);  // columns past nx lie in the row's pad
             load8(I.snap + o, w);
             const uint2 f = __ldg(reinterpret_cast<const uint2*>(I.flags + o));
-            if (refresh) {
-                reinterpret_cast<float4*>(I.snap + o)[0] = make_float4(r[0], r[1], r[2], r[3]);
-                reinterpret_cast<float4*>(I.snap + o)[1] = make_float4(r[4], r[5], r[6], r[7]);
-            }
+            reinterpret_cast<float4*>(I.snap + o)[0] = make_float4(r[0], r[1], r[2], r[3]);
+            reinterpret_cast<float4*>(I.snap + o)[1] = make_float4(r[4], r[5], r[6], r[7]);
             dsum.make_room(16);  // a difference's halves are twice as large
             msum.make_room(8);
 #pragma unroll
@@ -341,7 +339,7 @@ cudaError_t launch_batch_step(lbm_batch* b, int parity) {
 
 cudaError_t launch_residual(lbm_batch* b, int nact, int parity) {
     k_batch_residual<<<dim3(nact, kResSlices), NTB, 0, b->stream>>>(
-        (const BatchInst*)b->d_desc, b->d_active, parity, b->d_part, b->d_ticket, b->d_res, 1);
+        (const BatchInst*)b->d_desc, b->d_active, parity, b->d_part, b->d_ticket, b->d_res);
     return cudaGetLastError();
 }
 

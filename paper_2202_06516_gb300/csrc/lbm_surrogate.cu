@@ -976,8 +976,8 @@ cudaError_t conv_march(cudaStream_t st, const GemmArgs& a, const March& m, const
     switch (key) {
         case 16116: return launch_march<16, 1, 16, GD, false>(st, a, maps, parts);
         case 16132: return launch_march<16, 1, 32, GD, false>(st, a, maps, parts);
-        case 16216: return launch_march<16, 2, 16, GD, false>(st, a, maps, parts);
-        case 32116: return launch_march<32, 1, 16, GD, false>(st, a, maps, parts);
+        // forward only (two sources of 16 channels), data gradient only (32 outputs of 16 inputs)
+        case GD ? 32116 : 16216: return launch_march<GD ? 32 : 16, GD ? 1 : 2, 16, GD, false>(st, a, maps, parts);
         case 32132: return launch_march<32, 1, 32, GD, false>(st, a, maps, parts);
         case 32164: return launch_march<32, 1, 64, GD, false>(st, a, maps, parts);
         case 32232: return launch_march<32, 2, 32, GD, false>(st, a, maps, parts);
@@ -989,8 +989,8 @@ cudaError_t conv_march(cudaStream_t st, const GemmArgs& a, const March& m, const
 bool march_form(const March& m, bool gd, bool up) {
     const int key = m.kb * 1000 + m.cb * 100 + m.bn;
     if (up) return gd ? key == 16132 || key == 32164 : key == 32116 || key == 32232;
-    return key == 16116 || key == 16132 || key == 16216 || key == 32116 || key == 32132 ||
-           key == 32164 || key == 32232 || key == 32264;
+    return key == 16116 || key == 16132 || key == (gd ? 32116 : 16216) || key == 32132 || key == 32164 ||
+           key == 32232 || key == 32264;
 }
 
 cudaError_t gemm_wgrad(cudaStream_t st, GemmArgs a, float* scratch, size_t scratch_elems,
