@@ -489,7 +489,7 @@ struct Conv {
 struct Tensor {
     int H, W, C;
     bf16* y = nullptr;   // activation
-    float* dy = nullptr; // gradient
+    float* dy = nullptr; // gradient (one of lbm_surrogate::dys, shared in turn), where it is stored
 };
 
 }  // namespace
@@ -499,12 +499,13 @@ struct Tensor {
 using namespace lbm::sg;
 
 struct lbm_surrogate {
-    int H = 0, W = 0, base = 0, maxB = 0, device = 0;
+    int H = 0, W = 0, base = 0, maxB = 0, device = 0, sms = 152;
     // main stream, and a side stream for the weight and bias gradients of the backward pass, which
     // nothing in the chain of data gradients waits for
     cudaStream_t stream = nullptr, side = nullptr;
     cudaEvent_t head_ready = nullptr, side_done = nullptr;
     std::vector<Tensor> t;      // 0: input (8 channels)
+    std::vector<float*> dys;    // gradient buffers (gradient_buffers)
     std::vector<Conv> convs;
     std::vector<std::pair<int, int>> pools;  // (from, to)
     int head_in = -1;
@@ -513,8 +514,7 @@ struct lbm_surrogate {
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     bf16* wb = nullptr;
     bf16* wbd = nullptr;        // per convolution [C_in][tap][C_out] (data-gradient operand)
-    bf16* col = nullptr;
-    size_t col_elems = 0;
+    bf16* col = nullptr;      // im2col columns of one layer, where some weight gradient needs them
     float* phi = nullptr;   // head output
     float* hpart = nullptr;
     float* dz = nullptr;      // head: gradient with respect to the pre-sigmoid value, per pixel
@@ -904,6 +904,7 @@ cudaError_t launch_march(cudaStream_t st, GemmArgs a, const CUtensorMap* maps, i
     const int chunk = std::max(1, (rh + want - 1) / want);
     const dim3 grid((unsigned)strips * ((rh + chunk - 1) / chunk), nb);
     if (grid.x > (unsigned)kReluBlocks) a.rg = nullptr;  // rpart's columns
+    if (GD && !a.rg && !a.Cf) return cudaErrorInvalidValue;  // (fused_always rules this out)
     if (parts) *parts = a.rg ? (int)grid.x : 0;
     return launch_pdl(kern, grid, lbm::sgtc::MARCH_THREADS, MS::SMEM, st, a, flag, maps[0], maps[1],
                       maps[2], chunk);
@@ -1126,6 +1127,51 @@ const Conv* sole_producer(const lbm_surrogate* s, const Conv& c) {
     }
     for (const auto& pl : s->pools) readers += pl.first == c.src1;
     return readers == 1 && c.C1 % 16 == 0 ? p : nullptr;
+}
+
+// True when every training step forms the pre-activation gradient of c's first source in the epilogue of c's
+// data gradient (launch_march has at most max(strips, two per SM) CTAs along its rows), so that the
+// source's FP32 gradient is never stored.
+bool fused_always(const lbm_surrogate* s, const Conv& c) {
+    const long long strips = (long long)s->maxB * ((c.up1 ? c.W / 2 : c.W) / 128);
+    return c.dm.kb && sole_producer(s, c) && std::max<long long>(strips, 2 * s->sms) <= kReluBlocks;
+}
+
+// Buffers of the FP32 activation gradients (index per tensor, -1: not stored; sizes for max_batch images).
+// A gradient lives on the main stream from the first data gradient that writes it to the leaky-ReLU pass
+// of its convolution (a pooled map's: of the pool's source), in the order of queue_train_step, so a few
+// buffers serve all of them.
+std::vector<int> gradient_buffers(const lbm_surrogate* s, const std::vector<char>& stored,
+                                  std::vector<size_t>* size) {
+    std::vector<int> buf(s->t.size(), -1), free;
+    auto release = [&](int t) {
+        if (t >= 0 && buf[t] >= 0) free.push_back(buf[t]);
+    };
+    auto take = [&](int t) {
+        if (t < 0 || !stored[t] || buf[t] >= 0) return;
+        const Tensor& x = s->t[t];
+        const size_t n = (size_t)s->maxB * x.H * x.W * x.C;
+        // the largest free buffer (grown if it is too small), else a new one
+        auto big = std::max_element(free.begin(), free.end(),
+                                    [&](int a, int b) { return (*size)[a] < (*size)[b]; });
+        if (big == free.end()) {
+            buf[t] = (int)size->size();
+            size->push_back(n);
+        } else {
+            buf[t] = *big;
+            (*size)[*big] = std::max((*size)[*big], n);
+            free.erase(big);
+        }
+    };
+    for (int ci = (int)s->convs.size() - 1; ci >= 0; --ci) {
+        const Conv& c = s->convs[ci];
+        release(c.out);
+        for (const auto& pl : s->pools)
+            if (pl.first == c.out) release(pl.second);
+        take(c.src1);
+        take(c.src2);
+    }
+    return buf;
 }
 
 // the main stream waits for what the side stream holds so far
@@ -1478,6 +1524,7 @@ lbm_status queue_train_step(lbm_surrogate* s, const void* xin, const float* targ
         if (c.C2 > 0 && written[c.src1] != written[c.src2]) {
             const int fresh = written[c.src1] ? c.src2 : c.src1;
             const Tensor& x = s->t[fresh];
+            if (!x.dy) return sfail(s, LBM_ERR_STATE, "surrogate: missing gradient buffer");
             SCUDA(s, cudaMemsetAsync(x.dy, 0, (size_t)B * x.H * x.W * x.C * sizeof(float), s->stream));
             written[fresh] = 1;
         }
@@ -1555,15 +1602,11 @@ lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_
     cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cleanup(cudaGetErrorString(e));
-    size_t colmax = 0;
-    for (const Conv& c : s->convs)
-        colmax = std::max(colmax, (size_t)max_batch * c.H * c.W * 9 * (c.C1 + c.C2));
-    s->col_elems = colmax;
+    cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, device);
     for (size_t k = 1; k < s->t.size() && e == cudaSuccess; ++k) {
         Tensor& x = s->t[k];
         const size_t n = (size_t)max_batch * x.H * x.W * x.C;
         e = cudaMalloc((void**)&x.y, n * sizeof(bf16));
-        if (e == cudaSuccess) e = cudaMalloc((void**)&x.dy, n * sizeof(float));
     }
     const size_t np = s->nparams;
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->w, np * sizeof(float));
@@ -1572,7 +1615,6 @@ lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->v, np * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->wb, np * sizeof(bf16));
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->wbd, np * sizeof(bf16));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->col, colmax * sizeof(bf16));
     for (Conv& c : s->convs) {
         if (e == cudaSuccess)
             e = cudaMalloc((void**)&c.g, (size_t)max_batch * c.H * c.W * c.Cout * sizeof(bf16));
@@ -1601,6 +1643,25 @@ lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_
     if (e == cudaSuccess) e = cudaMemsetAsync(s->wbd, 0, np * sizeof(bf16), s->stream);
     if (e != cudaSuccess) return cleanup(cudaGetErrorString(e));
     make_tensor_maps(s);
+    // what depends on how the layers run: an im2col buffer for weight gradients that cannot gather, FP32
+    // gradients of the activations that a data gradient stores
+    std::vector<char> stored(s->t.size(), 1);
+    stored[0] = stored[s->head_in] = 0;
+    size_t colmax = 0;
+    for (const Conv& c : s->convs) {
+        if (fused_always(s, c)) stored[c.src1] = 0;
+        if (!c.wr_xb && (ilog2_exact(c.H) < 0 || ilog2_exact(c.W) < 0))
+            colmax = std::max(colmax, (size_t)max_batch * c.H * c.W * 9 * (c.C1 + c.C2));
+    }
+    std::vector<size_t> size;  // of the gradient buffers, in values
+    const std::vector<int> buf = gradient_buffers(s, stored, &size);
+    s->dys.assign(size.size(), nullptr);
+    for (size_t k = 0; k < size.size() && e == cudaSuccess; ++k)
+        e = cudaMalloc((void**)&s->dys[k], size[k] * sizeof(float));
+    for (size_t k = 0; k < s->t.size(); ++k)
+        if (buf[k] >= 0) s->t[k].dy = s->dys[buf[k]];
+    if (e == cudaSuccess && colmax) e = cudaMalloc((void**)&s->col, colmax * sizeof(bf16));
+    if (e != cudaSuccess) return cleanup(cudaGetErrorString(e));
     *out = s;
     return LBM_OK;
 }
@@ -1728,10 +1789,8 @@ void lbm_surrogate_destroy(lbm_surrogate* s) {
     }
     if (s->head_ready) cudaEventDestroy(s->head_ready);
     if (s->side_done) cudaEventDestroy(s->side_done);
-    for (size_t k = 1; k < s->t.size(); ++k) {
-        cudaFree(s->t[k].y);
-        cudaFree(s->t[k].dy);
-    }
+    for (size_t k = 1; k < s->t.size(); ++k) cudaFree(s->t[k].y);
+    for (float* d : s->dys) cudaFree(d);
     cudaFree(s->w);
     cudaFree(s->g);
     cudaFree(s->m);
