@@ -600,13 +600,14 @@ cudaError_t launch_measure(lbm_ctx* c) {
 
 cudaError_t launch_candidates(lbm_ctx* c, uint8_t* d_mark, double* d_pxyd) {
     const double rho_m = 0.5 * (c->rho_g + c->rho_l);
+    const int blocks = 2 * c->sms;  // (not a block per row: wide, flat lattices have few)
     if (c->esz == 4)
-        k_cand_dense<float><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
+        k_cand_dense<float><<<blocks, kRedThreads, 0, c->stream>>>(
             (const float*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m,
             floor_to(rho_m, 0.f), c->sub, d_mark,
             d_pxyd);
     else
-        k_cand_dense<double><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
+        k_cand_dense<double><<<blocks, kRedThreads, 0, c->stream>>>(
             (const double*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, rho_m, rho_m, c->sub, d_mark,
             d_pxyd);
     return cudaGetLastError();
