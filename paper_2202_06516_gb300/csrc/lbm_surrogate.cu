@@ -489,7 +489,7 @@ struct Conv {
 struct Tensor {
     int H, W, C;
     bf16* y = nullptr;   // activation
-    float* dy = nullptr; // gradient (one of lbm_surrogate::dys, shared in turn), where it is stored
+    float* dy = nullptr; // gradient, where it is stored (gradient_buffers: shared in turn)
 };
 
 }  // namespace
@@ -505,7 +505,7 @@ struct lbm_surrogate {
     cudaStream_t stream = nullptr, side = nullptr;
     cudaEvent_t head_ready = nullptr, side_done = nullptr;
     std::vector<Tensor> t;      // 0: input (8 channels)
-    std::vector<float*> dys;    // gradient buffers (gradient_buffers)
+    std::vector<void*> memory;  // the device allocations that everything below points into
     std::vector<Conv> convs;
     std::vector<std::pair<int, int>> pools;  // (from, to)
     int head_in = -1;
@@ -1137,6 +1137,27 @@ bool fused_always(const lbm_surrogate* s, const Conv& c) {
     return c.dm.kb && sole_producer(s, c) && std::max<long long>(strips, 2 * s->sms) <= kReluBlocks;
 }
 
+struct Part {
+    void** p;
+    size_t bytes;
+};
+
+// Sets every pointer to its part of one allocation (each 256-byte aligned). One by one the 80 parts of a
+// small network took longer than everything else in its creation.
+cudaError_t allocate(lbm_surrogate* s, const std::vector<Part>& parts) {
+    size_t total = 0;
+    for (const Part& q : parts) total += (q.bytes + 255) / 256 * 256;
+    char* base = nullptr;
+    const cudaError_t e = total ? cudaMalloc((void**)&base, total) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+    if (base) s->memory.push_back(base);
+    for (const Part& q : parts) {
+        *q.p = base;
+        base += (q.bytes + 255) / 256 * 256;
+    }
+    return cudaSuccess;
+}
+
 // Buffers of the FP32 activation gradients (index per tensor, -1: not stored; sizes for max_batch images).
 // A gradient lives on the main stream from the first data gradient that writes it to the leaky-ReLU pass
 // of its convolution (a pooled map's: of the pool's source), in the order of queue_train_step, so a few
@@ -1603,39 +1624,29 @@ lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cleanup(cudaGetErrorString(e));
     cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, device);
-    for (size_t k = 1; k < s->t.size() && e == cudaSuccess; ++k) {
-        Tensor& x = s->t[k];
-        const size_t n = (size_t)max_batch * x.H * x.W * x.C;
-        e = cudaMalloc((void**)&x.y, n * sizeof(bf16));
-    }
-    const size_t np = s->nparams;
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->w, np * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->g, np * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->m, np * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->v, np * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->wb, np * sizeof(bf16));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->wbd, np * sizeof(bf16));
-    for (Conv& c : s->convs) {
-        if (e == cudaSuccess)
-            e = cudaMalloc((void**)&c.g, (size_t)max_batch * c.H * c.W * c.Cout * sizeof(bf16));
-        if (e == cudaSuccess)
-            e = cudaMalloc((void**)&c.bpart, (size_t)kReluBlocks * c.Cout * sizeof(float));
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.ready, cudaEventDisableTiming);
-    }
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->head_ready, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->side_done, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->dz, (size_t)max_batch * H * W * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->n_mask, sizeof(int));
-    if (e == cudaSuccess) e = cudaHostAlloc((void**)&s->host_loss, sizeof(float), cudaHostAllocMapped);
-    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&s->host_loss_dev, s->host_loss, 0);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->phi, (size_t)max_batch * H * W * sizeof(float));
-    if (e == cudaSuccess)
-        e = cudaMalloc((void**)&s->hpart, (size_t)s->part_blocks * (base + 2) * sizeof(float));
+    const size_t np = s->nparams, px = (size_t)max_batch * H * W;
     size_t wmax = 0;
     for (const Conv& c : s->convs) wmax = std::max(wmax, (size_t)c.Cout * 9 * (c.C1 + c.C2));
     s->splitk_elems = std::min<size_t>(wmax * 128, (size_t)64 << 20);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->splitk, s->splitk_elems * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&s->splitk_side, s->splitk_elems * sizeof(float));
+    std::vector<Part> parts;
+    for (size_t k = 1; k < s->t.size(); ++k)
+        parts.push_back({(void**)&s->t[k].y, (size_t)max_batch * s->t[k].H * s->t[k].W * s->t[k].C * sizeof(bf16)});
+    for (Conv& c : s->convs) {
+        parts.push_back({(void**)&c.g, (size_t)max_batch * c.H * c.W * c.Cout * sizeof(bf16)});
+        parts.push_back({(void**)&c.bpart, (size_t)kReluBlocks * c.Cout * sizeof(float)});
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.ready, cudaEventDisableTiming);
+    }
+    for (float** q : {&s->w, &s->g, &s->m, &s->v}) parts.push_back({(void**)q, np * sizeof(float)});
+    for (bf16** q : {&s->wb, &s->wbd}) parts.push_back({(void**)q, np * sizeof(bf16)});
+    for (float** q : {&s->dz, &s->phi}) parts.push_back({(void**)q, px * sizeof(float)});
+    for (float** q : {&s->splitk, &s->splitk_side}) parts.push_back({(void**)q, s->splitk_elems * sizeof(float)});
+    parts.push_back({(void**)&s->hpart, (size_t)s->part_blocks * (base + 2) * sizeof(float)});
+    parts.push_back({(void**)&s->n_mask, sizeof(int)});
+    if (e == cudaSuccess) e = allocate(s, parts);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->head_ready, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->side_done, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaHostAlloc((void**)&s->host_loss, sizeof(float), cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&s->host_loss_dev, s->host_loss, 0);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->w, 0, np * sizeof(float), s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->m, 0, np * sizeof(float), s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->v, 0, np * sizeof(float), s->stream);
@@ -1655,12 +1666,13 @@ lbm_status lbm_surrogate_create(int32_t H, int32_t W, int32_t base, int32_t max_
     }
     std::vector<size_t> size;  // of the gradient buffers, in values
     const std::vector<int> buf = gradient_buffers(s, stored, &size);
-    s->dys.assign(size.size(), nullptr);
-    for (size_t k = 0; k < size.size() && e == cudaSuccess; ++k)
-        e = cudaMalloc((void**)&s->dys[k], size[k] * sizeof(float));
+    std::vector<float*> dy(size.size(), nullptr);
+    parts.clear();
+    for (size_t k = 0; k < size.size(); ++k) parts.push_back({(void**)&dy[k], size[k] * sizeof(float)});
+    if (colmax) parts.push_back({(void**)&s->col, colmax * sizeof(bf16)});
+    e = allocate(s, parts);
     for (size_t k = 0; k < s->t.size(); ++k)
-        if (buf[k] >= 0) s->t[k].dy = s->dys[buf[k]];
-    if (e == cudaSuccess && colmax) e = cudaMalloc((void**)&s->col, colmax * sizeof(bf16));
+        if (buf[k] >= 0) s->t[k].dy = dy[buf[k]];
     if (e != cudaSuccess) return cleanup(cudaGetErrorString(e));
     *out = s;
     return LBM_OK;
@@ -1782,29 +1794,12 @@ void lbm_surrogate_destroy(lbm_surrogate* s) {
     if (!s) return;
     if (s->stream) cudaStreamSynchronize(s->stream);
     if (s->side) cudaStreamSynchronize(s->side);
-    for (Conv& c : s->convs) {
-        cudaFree(c.g);
-        cudaFree(c.bpart);
+    for (Conv& c : s->convs)
         if (c.ready) cudaEventDestroy(c.ready);
-    }
     if (s->head_ready) cudaEventDestroy(s->head_ready);
     if (s->side_done) cudaEventDestroy(s->side_done);
-    for (size_t k = 1; k < s->t.size(); ++k) cudaFree(s->t[k].y);
-    for (float* d : s->dys) cudaFree(d);
-    cudaFree(s->w);
-    cudaFree(s->g);
-    cudaFree(s->m);
-    cudaFree(s->v);
-    cudaFree(s->wb);
-    cudaFree(s->wbd);
-    cudaFree(s->col);
-    cudaFree(s->phi);
-    cudaFree(s->hpart);
-    cudaFree(s->dz);
-    cudaFree(s->n_mask);
+    for (void* p : s->memory) cudaFree(p);
     if (s->host_loss) cudaFreeHost(s->host_loss);
-    cudaFree(s->splitk);
-    cudaFree(s->splitk_side);
     if (s->stream) cudaStreamDestroy(s->stream);
     if (s->side) cudaStreamDestroy(s->side);
     delete s;
