@@ -18,6 +18,9 @@ namespace {
 thread_local std::string g_last_error;
 
 lbm_status fail(lbm_ctx* c, lbm_status s, const std::string& msg) {
+    // an error is reported once: a refused cudaLaunchKernelEx or cudaMalloc stays with the runtime until it
+    // is asked for, and the next call's cudaGetLastError would find it
+    if (s == LBM_ERR_CUDA) cudaGetLastError();
     if (c)
         c->err = msg;
     else

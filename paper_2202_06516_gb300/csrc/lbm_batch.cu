@@ -183,6 +183,8 @@ __global__ void __launch_bounds__(NTB)
 }
 
 lbm_status bfail(lbm_batch* b, lbm_status st, const std::string& msg) {
+    // reported once (see fail in lbm_api.cu)
+    if (st == LBM_ERR_CUDA) cudaGetLastError();
     if (b)
         b->err = msg;
     else

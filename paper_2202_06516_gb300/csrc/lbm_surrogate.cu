@@ -533,6 +533,8 @@ extern "C" void lbm_surrogate_destroy(lbm_surrogate* s);
 namespace {
 
 lbm_status sfail(lbm_surrogate* s, lbm_status st, const std::string& msg) {
+    // reported once (see fail in lbm_api.cu)
+    if (st == LBM_ERR_CUDA) cudaGetLastError();
     if (s)
         s->err = msg;
     else
