@@ -152,9 +152,10 @@ lbm_status lbm_coexistence(int32_t eos, double Tr, double out[4]);
  * LBM_ERR_ARG for an unknown EOS, Tr outside (0, 1), or rho outside (0, rho_max). */
 lbm_status lbm_eos_eval(int32_t eos, double Tr, double rho, double out[2]);
 
-/* Allocate a lattice on p->device (2 x 9 population planes, 2 density planes, flags, wall
- * chemical potential, reduction and measurement scratch). *out receives the context; on failure
- * *out is NULL and nothing is leaked. */
+/* Allocate a lattice on p->device (2 x 9 population planes, 2 density planes, flags, link masks, wall
+ * chemical potential, the list of nodes near the wall, reduction and measurement scratch; LBM_FP64: 12
+ * more planes of step scratch). *out receives the context; on failure *out is NULL and nothing is
+ * leaked. */
 lbm_status lbm_create(const lbm_params *p, lbm_ctx **out);
 
 /* Build the geometry on the device (classification, wetting layers, wall chemical potential,
@@ -163,8 +164,8 @@ lbm_status lbm_create(const lbm_params *p, lbm_ctx **out);
  * geometry's, the walls already on the device are kept and only the state is set. Synchronous. */
 lbm_status lbm_set_geometry(lbm_ctx *ctx, const lbm_geometry *g);
 
-/* Advance nsteps time steps (Eq. 1-4 with Eq. 7, 12-14): one fused kernel per step, replayed
- * from a CUDA graph in chunks when the stream allows capture. Asynchronous; returns LBM_OK once
+/* Advance nsteps time steps (Eq. 1-4 with Eq. 7, 12-14): one fused kernel per step (LBM_FP64:
+ * three), replayed from a CUDA graph in chunks when the stream allows capture. Asynchronous; returns LBM_OK once
  * the work is queued (LBM_ERR_STATE before lbm_set_geometry, LBM_ERR_ARG for nsteps < 0). */
 lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);
 
@@ -187,8 +188,9 @@ lbm_status lbm_measure_contact_angle(lbm_ctx *ctx, lbm_angle out[2]);
 lbm_status lbm_read_fields(lbm_ctx *ctx, uint32_t which, double *rho, double *ux, double *uy,
                            size_t n);
 
-/* Sums over fluid nodes (deterministic; exact for FP32 densities, FP64 for FP64 ones): out[0] total mass, out[1]
- * number of liquid nodes (rho > rho_m), out[2], out[3] their centroid x, y. Returns
+/* Sums over fluid nodes (deterministic): out[0] total mass, out[1] number of liquid nodes (rho > rho_m),
+ * out[2], out[3] their centroid x, y. FP32 densities in [2^-13, 512) are summed exactly within a block of
+ * the reduction (rows of the lattice), other densities and the blocks' sums in FP64. Returns
  * LBM_ERR_UNSTABLE if a density is non-finite or non-positive. Synchronous. */
 lbm_status lbm_mass(lbm_ctx *ctx, double out[4]);
 
@@ -266,9 +268,9 @@ typedef struct lbm_batch lbm_batch; /* opaque; owns n lattices, their stream and
 /* Create n lattices of sizes nx[i] x ny[i] sharing the model parameters (model->nx, ny, tile_y,
  * min_blocks and stream are ignored; precision must be LBM_FP32; model->tile_x = LBM_TILE_AUTO
  * autotunes the batch kernel at the first lbm_batch_run, any other value starts with the
- * default 32x16 tiles, one CTA per tile). Every instance is an lbm_ctx on the batch's private
- * stream. On failure
- * *out is NULL and nothing is leaked. */
+ * default 32x16 tiles, or a form with smaller tiles where all instances together have few, one CTA
+ * per tile). Every instance is an lbm_ctx on the batch's private stream. On failure *out is NULL and
+ * nothing is leaked. */
 lbm_status lbm_batch_create(const lbm_params *model, int32_t n, const int32_t *nx,
                             const int32_t *ny, lbm_batch **out);
 
@@ -288,11 +290,11 @@ lbm_status lbm_batch_run(lbm_batch *b, int64_t max_steps, int32_t check_every, d
 
 /* Autotuner of the batched kernel: times each compiled tile variant (FP32 32x8, 32x16, 64x16,
  * 32x32, each with its register budget) in both grid modes (one CTA per tile, then persistent;
- * entries in that order, 2 per variant) over trial_steps launches on
- * the tile table of the instances that have geometry (those sharing the parity of the first), and
- * keeps the fastest for later lbm_batch_run calls. A batch of few tiles also times the form with smaller
- * tiles that it runs by default; the entries of 32x16 then give the faster of the two. As in lbm_autotune the trial launches do not
- * advance any instance. entries / n_out as in lbm_autotune. LBM_ERR_STATE if no instance has
+ * entries in that order, 2 per variant) over trial_steps launches on the tile table of the instances
+ * that have geometry (those sharing the parity of the first), and keeps the fastest for later
+ * lbm_batch_run calls. A batch of few tiles also times the form with smaller tiles that it runs by
+ * default; the entries of 32x16 then give the faster of the two. As in lbm_autotune the trial
+ * launches do not advance any instance. entries / n_out as in lbm_autotune. LBM_ERR_STATE if no instance has
  * geometry. Synchronous. */
 lbm_status lbm_batch_autotune(lbm_batch *b, int32_t trial_steps, lbm_tune_entry *entries,
                               int32_t max_entries, int32_t *n_out);

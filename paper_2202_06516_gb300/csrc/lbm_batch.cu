@@ -9,8 +9,8 @@
 // resident slot, looping over the table); the autotuner times both, and one CTA per tile is the
 // default (measured faster: the hardware scheduler interleaves CTAs in different stages of
 // their tiles, while a persistent CTA serialises its tiles' four barriers). A CUDA graph holds
-// `check_every` such launches. After each graph the FP64 residual sum |rho(t) - rho(t - check)| /
-// sum rho of every running instance is computed (one block per instance, fixed order), converged
+// `check_every` such launches. After each graph the residual sum |rho(t) - rho(t - check)| /
+// sum rho of every running instance is computed (32 blocks per instance, fixed order), converged
 // instances leave the table, and the graph is replayed on the shorter table without recapture
 // (the kernels read the table length from device memory).
 #include <stdio.h>

@@ -1,11 +1,10 @@
-// FP64 reductions and the on-device contact-angle measurement (Sec. 3.2, Eq. 15, Fig. 1-2).
+// Reductions and the on-device contact-angle measurement (Sec. 3.2, Eq. 15, Fig. 1-2).
 //
 // Reductions (mass, liquid-node count and centroid): one kernel, deterministic. Every block writes
 // its partial sums to scratch, and the block that finishes last adds them in a fixed order.
 //
 // Measurement: the threads scan the nodes near the wall surface (a list made with the geometry)
-// for liquid/gas links (one end rho > rho_m, the other not)
-// in the four undirected link directions, place the Eq. 15 point on the link, measure its
+// for liquid/gas links (one end rho > rho_m, the other not) in the four undirected link directions, place the Eq. 15 point on the link, measure its
 // distance d to the substrate and keep, per side, the links nearest to d = 1 and d = 2 within
 // the band 0.5 <= d <= 2.5 (ordered by |d - target|, then link id). Blocks reduce with warp
 // shuffles into per-block partials; the last block to finish picks the winners and builds the
@@ -72,8 +71,8 @@ __device__ __forceinline__ void add_node(FixSum& m, unsigned& nbad, double v) {
 
 // Mass, liquid count, liquid centroid and the count of non-finite or non-positive densities over
 // the fluid nodes, one block per row (then striding), eight nodes per thread and access. Bound by
-// the 5 bytes per node it reads and, with few rows, by latency: the mass is summed in exact
-// fixed point (lbm_sum.cuh), counts and coordinate sums are integers (the same values the FP64
+// the 5 bytes per node it reads and, with few rows, by latency: a block's mass is summed in exact
+// fixed point (lbm_sum.cuh) and the blocks' in FP64, counts and coordinate sums are integers (the same values the FP64
 // sums of whole numbers had), and the comparison with rho_m is made against the largest T not
 // above it (the same truth value for every T), so that FP32 lattices use the FP64 pipe only
 // for the blocks' totals. 4096 x 1024: 82 us and 26 us for a serial last pass

@@ -29,8 +29,10 @@ constexpr double kFixUnit = 1.0 / 68719476736.0;  // 2^-36
 // values a thread may add to its 32-bit halves before they move on (255 * 2^22 < 2^30)
 constexpr int kFixMost = 255;
 
-// Sum of one thread: exact part in units of 2^-36 (running 32-bit halves and their 64-bit total,
-// below 2^62 for 2^17 values per thread and 2^13 threads) and FP64 part
+// Sum of one thread: exact part in units of 2^-36 (running 32-bit halves and their 64-bit total) and FP64
+// part. A total passes to the FP64 part once it exceeds 2^52, and at most 255 values of less than 2^45
+// are added between two looks at it, so it stays below 2^54 and the sum over a block of up to 256
+// threads below 2^62. Exact within a block as long as no thread's total has passed on.
 struct FixSum {
     int hi = 0, lo = 0, n = 0;
     long long fix = 0;

@@ -11,12 +11,14 @@
 // Activations BF16 NHWC, weights FP32 masters with BF16 copies, all contractions on the tcgen05
 // tensor cores with FP32 accumulation in tensor memory (sg_tc.cuh), as implicit GEMMs whose
 // operands are the 3 x 3 neighbourhoods of the activations: the forward convolution, the
-// weight gradient (pixels as K; an im2col buffer only when the resolution is not a power of two)
-// and the data gradient (output gradients around each source pixel). Where the shapes allow,
-// the operands arrive as tensor-map (TMA) boxes built once per network (make_tensor_maps): the
-// tap's offset moves the box, the image border is zero-filled, upsampling layers order their
-// rows or K even/odd or read every second pixel; the 32/64-channel levels stage one window per
-// slice or tile and take the nine taps from it; elsewhere the loaders gather with cp.async.
+// weight gradient (pixels as K; an im2col buffer only when the resolution is not a power of two
+// and the rows do not suit k_wgrad_rows) and the data gradient (output gradients around each source
+// pixel). Where the shapes allow, the operands arrive as tensor-map (TMA) boxes built once per
+// network (make_tensor_maps). Levels of 16 to 64 channels with rows of 128 pixels march down a ring of
+// staged rows (k_conv_march), their weight gradients take rows of 64 pixels (k_wgrad_rows), the first
+// convolution reads the input once (k_conv0, k_wgrad0). Other layers fetch a box per tap (k_gemm_tc:
+// the tap's offset moves the box, the image border is zero-filled, upsampling layers order their
+// rows or K even/odd or read every second pixel), or their loaders gather with cp.async.
 // Loss: masked mean squared error on phi. Optimiser: Adam.
 #include <math.h>
 
