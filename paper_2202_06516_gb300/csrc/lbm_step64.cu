@@ -66,7 +66,8 @@ __global__ void __launch_bounds__(MT) k64_mu(const Args64 s) {
     __shared__ double r[H][W];
     __shared__ uint8_t f[H][W];
     const StepArgs<double>& a = s.a;
-    const int x0 = blockIdx.x * MX, y0 = blockIdx.y * MY - 2, tid = threadIdx.x;
+    const int x0 = blockIdx.x * MX, y0 = (int)(blockIdx.z * gridDim.y + blockIdx.y) * MY - 2;
+    const int tid = threadIdx.x;
     int any = 0, e[K];
     uint8_t cl[K];
     double v[K];
@@ -256,7 +257,9 @@ cudaError_t launch_step64(lbm_ctx* c, const StepArgs<double>& a, bool macro) {
     s.ext = (double*)c->scratch64;
     s.mu = s.ext + c->plane;
     s.post = s.mu + c->plane;
-    const dim3 gm((c->nx + MX - 1) / MX, (c->ny + 4 + MY - 1) / MY);
+    // rows of blocks along y and, past the 65535 that y holds (lattices of more than 262136 rows), z
+    const unsigned mrows = (c->ny + 4 + MY - 1) / MY, mz = (mrows + 65534) / 65535;
+    const dim3 gm((c->nx + MX - 1) / MX, (mrows + mz - 1) / mz, mz);
     const dim3 gn((unsigned)(((long long)c->nx * c->ny + N64 - 1) / N64));
     k64_mu<<<gm, MT, 0, c->stream>>>(s);
     auto* collide = macro ? (c->ibb ? k64_collide<true, true> : k64_collide<true, false>)

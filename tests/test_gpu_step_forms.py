@@ -78,6 +78,18 @@ def test_fp64_on_ragged_lattices(lbm, oracle_mod, nx, ny, concave, interp):
         lat.close()
 
 
+def test_fp64_lattice_of_more_block_rows_than_a_grid_dimension_holds(lbm, oracle_mod):
+    """8 x 262200 in FP64: 65551 rows of 16 x 4 blocks, a grid's second dimension holds 65535. The drop lies
+    at the upper end; densities within 1e-9 of rho_l of the oracle (the bound of the parity tests)."""
+    O = oracle_mod
+    cfg = oracle_config(O, W.Workload("t", 8, 262200, None, (4.0, 262160.0, 15.0, 5.6)))[0]
+    lat, ref = gpu_lattice(lbm, cfg, precision=1), O.Sim(cfg)
+    lat.step(3)
+    ref.step(3)
+    assert np.abs(lat.rho() - ref.rho()).max() <= 1e-9 * cfg.rho_l
+    lat.close()
+
+
 def test_tiles_that_fit_at_once_are_spread_over_the_chip(lbm, oracle_mod):
     """A lattice of 459 tiles against one of 720, both on the chip at once (760 places): three tiles
     per SM against five. Evenly spread the first takes 0.77 of the second's time, with tiles
