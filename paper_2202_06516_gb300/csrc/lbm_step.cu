@@ -29,7 +29,9 @@ using namespace stepdev;
 
 // the interpolated bounce-back kernels exist for the default variant (32 x 16 tiles, 5 CTAs per SM)
 // and its small-lattice forms; the fractions and populations of a node's cut links in flight take
-// registers that five CTAs per SM would spill
+// registers that five CTAs per SM would spill. us per step with a cylinder: five CTAs and a chain of two
+// latencies per cut link / four / five that spill 56 bytes: 640x480 19.5 / 16.0 / 16.2, 768x480 20.1 / 16.2 /
+// 18.4, 1024x512 22.3 / 17.9 / 18.9, 1500x701 32.0 / 28.5 / 27.6, 2048x1024 55.7 / 51.6 / 48.5
 constexpr int kIbbBlocks = 4;
 template <typename T, int TX, int TY, int MINB>
 constexpr bool has_ibb() {
