@@ -71,14 +71,20 @@ cudaError_t allow_smem() {
 // against the number of SMs. Measured, us per step, 32x16 tiles of 256 threads / forms 1 / 2 / 3:
 // 128x96 7.4 / 4.3 / 5.1 / 4.8; 200x120 8.0 / 4.6 / 5.1 / 5.2; 256x256 8.0 / 6.0 / 5.2 / 5.6;
 // 520x190 10.2 / 6.8 / 7.2 / 6.1.
-// Form 3 holds three tiles per SM (456). Up to twice as many run as a second wave, which pays only
-// where the 256-thread form is held up by tiles that a curved wall crosses (its threads take several
-// rounds of wetting layers and cut links), the more the larger the circle; half-way walls, us per step,
-// 256 threads / form 3: 128x1000 (500 tiles) R = 4 7.4 / 7.5, R = 16 8.4 / 7.5; 128x1200 (600) R = 8
-// 7.8 / 7.9, R = 16 8.3 / 8.0, R = 48 9.8 / 7.9; 512x400 (800) R = 16 9.2 / 9.3, R = 32 9.5 / 9.3, R = 64
-// 10.2 / 9.3; 400x560 (910) R = 16 9.5 / 10.5, R = 64 10.0 / 10.5. A cavity leaves most tiles empty:
-// 700x328 (902) 11.4 / 10.3, 1000x224 (896) 11.3 / 9.1. Interpolated walls take longer in the 256-thread
-// form at every size: 128x1200 (600), R = 3, 10.5 / 9.2, 512x456 (912) 15.0 / 11.1.
+// Form 3 holds three tiles per SM (456); up to twice as many run as a second wave. It then pays, the more
+// where a curved wall crosses tiles (the 256-thread form's threads take several rounds of wetting layers
+// and cut links there), until the second wave is nearly full; half-way walls, us per step, 256 threads /
+// form 3: flat 700x165 (462 tiles) 8.2 / 6.6, 400x324 (533) 7.4 / 7.3, 700x216 (594) 9.0 / 7.6, 400x397
+// (650) 9.0 / 8.1, 1100x160 (700) 9.2 / 8.3, 700x278 (770) 9.3 / 8.7, 250x835 (840) 9.5 / 9.4, 1100x192 (840) 9.0 /
+// 9.2, 1100x200 (875) 8.5 / 9.5, 400x548 (897) 9.2 / 9.5; R = 24 within 0.2 of flat; R = 48 250x835 9.7 / 9.4,
+// 1100x200 9.9 / 9.6. Where the 256-thread form needs a fourth tile per SM: 700x322 (902) 11.0 / 9.7.
+// Lattices of up to four columns of tiles have few wall tiles but many that write pads, which costs form 3
+// more, and R decides: flat 128x956 (480) 7.0 / 6.9, 128x1197 (600) 7.0 / 7.5, 128x1316 (660) 8.7 / 7.8,
+// 128x1440 (720) 8.6 / 8.0, 128x1560 (780) 7.7 / 8.9, 40x2399 (600) 7.3 / 8.2, 40x2635 (660) 8.7 / 8.8, 40x3119 (780) 8.7 /
+// 9.5 (beyond two tiles of 32x16 per SM, at about 608 of 32x8, the 256-thread form steps up); R = 24 128x1197
+// 8.1 / 7.5, 128x1440 8.9 / 8.1, 128x1806 (904) 8.9 / 9.2; R = 48 128x1560 10.2 / 8.9, 128x1806 10.2 / 9.3. A cavity
+// leaves most tiles empty: 700x328 (902) 11.4 / 10.3, 1000x224 (896) 11.3 / 9.1. Interpolated walls take longer in
+// the 256-thread form at every size: 128x1200 (600), R = 3, 10.5 / 9.2, 512x456 (912) 15.0 / 11.1.
 #define LBM_SMALL_FORMS(X) X(1, 16, 8, 320, 3) X(2, 32, 16, 640, 1) X(3, 32, 8, 384, 3)
 
 // Whether a step of the 256-thread forms is placed early. A grid that fits on the chip at once leaves
@@ -238,11 +244,13 @@ int step_form(const lbm_ctx* c) {
     if (2 * tiles(16, 8) <= 3 * sms) return 1;
     if (tiles(32, 16) <= sms) return 2;
     const lbm_geometry& g = c->geom;
-    const int half_sms = c->ibb || (g.has_circle && g.concave)  ? 12
-                         : g.has_circle && g.R >= 32 ? 11
-                         : g.has_circle && g.R >= 16 ? 10
-                                                     : 6;
-    return 2 * tiles(32, 8) <= half_sms * sms ? 3 : 0;
+    const double R = g.has_circle ? g.R : 0;
+    const long long large = tiles(32, 16);
+    const int quarters = c->ibb || (g.has_circle && g.concave) ? 24  // tiles of 32x8 per SM, times four
+                         : nx <= 4 * 32 ? (R >= 32 ? 24 : R >= 16 ? 20 : large > 2 * sms ? 19 : 14)
+                         : large > 3 * sms ? 24
+                                           : (R >= 32 ? 23 : 22);
+    return 4 * tiles(32, 8) <= quarters * sms ? 3 : 0;
 }
 
 cudaError_t launch_step(lbm_ctx* c, int src, bool macro) {
