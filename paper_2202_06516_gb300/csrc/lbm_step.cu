@@ -247,7 +247,7 @@ int step_form(const lbm_ctx* c) {
     const double R = g.has_circle ? g.R : 0;
     const long long large = tiles(32, 16);
     const int quarters = c->ibb || (g.has_circle && g.concave) ? 24  // tiles of 32x8 per SM, times four
-                         : nx <= 4 * 32 ? (R >= 32 ? 24 : R >= 16 ? 20 : large > 2 * sms ? 19 : 14)
+                         : nx <= 4 * 32 ? (R >= 32 ? 24 : R >= 16 ? 20 : large > 2 * sms ? 19 : 15)
                          : large > 3 * sms ? 24
                                            : (R >= 32 ? 23 : 22);
     return 4 * tiles(32, 8) <= quarters * sms ? 3 : 0;
