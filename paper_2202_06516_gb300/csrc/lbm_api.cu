@@ -449,7 +449,7 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const lbm_geometry* g) {
         LBM_CUDA(c, lbm::launch_geometry(c, a));
     }
     // captured step graphs stay valid across geometries (the kernels read the same buffers);
-    // they hold the boundary scheme, the variant and its form, so a change of one drops them
+    // they hold the boundary scheme, the variant, its form and placement, so a change of one drops them
     const bool ibb = g->boundary == LBM_BB_INTERP;
     if (ibb != c->ibb) destroy_graphs(c);
     c->ibb = ibb;
@@ -481,9 +481,7 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const lbm_geometry* g) {
     }
     c->geom = *g;
     c->geom.rho0 = nullptr;
-    const int form = lbm::step_form(c);
-    if (form != c->form) destroy_graphs(c);
-    c->form = form;
+    if (lbm::step_choose(c)) destroy_graphs(c);
     c->sub.circle = g->has_circle ? 1 : 0;
     c->sub.concave = g->has_circle && g->concave ? 1 : 0;
     c->sub.cx = g->cx;

@@ -149,7 +149,8 @@ struct lbm_ctx {
     bool graphs_ready = false;
     bool graph_failed = false;
     int tile_x = 32, tile_y = 16, min_blocks = 0;
-    int form = 0;  // small-lattice form of the default FP32 variant (step_form), 0: none
+    int form = 0;  // small-lattice form of the default FP32 variant, 0: none
+    bool early = false;  // steps of the other forms are placed before the previous one ends
     int resident[2] = {0, 0};  // tiles of that variant on the chip at once: half-way, interpolated walls
     bool autotune_pending = false;  // LBM_TILE_AUTO: tune at the first lbm_step
     std::string err;
@@ -175,8 +176,9 @@ struct StepVariant {
 };
 // the compiled step-kernel variants for element size esz (4: FP32, 8: FP64)
 void step_variants(size_t esz, std::vector<StepVariant>* out);
-// the form that suits the lattice's size and walls (c->geom, c->ibb)
-int step_form(const lbm_ctx* c);
+// the form and the placement that suit the lattice's size and walls (c->geom, c->ibb) into c->form and
+// c->early; true if one of them changed
+bool step_choose(lbm_ctx* c);
 bool step_has_ibb(size_t esz, int tile_x, int tile_y, int min_blocks);
 cudaError_t step_configure(lbm_ctx* c);
 // sums into aux->red, and into host_out (to_host)

@@ -20,6 +20,8 @@
 // half-way bounce-back on links into the solid) and the new deviations h. Collisions on the
 // one-node ring are recomputed by the neighbouring CTAs; that redundancy buys a single pass over
 // the populations per step (36 B read + 36 B written + 8 B of density per node in FP32).
+#include <algorithm>
+
 #include "lbm_step_body.cuh"
 
 namespace lbm {
@@ -87,15 +89,47 @@ cudaError_t allow_smem() {
 // the 256-thread form at every size: 128x1200 (600), R = 3, 10.5 / 9.2, 512x456 (912) 15.0 / 11.1.
 #define LBM_SMALL_FORMS(X) X(1, 16, 8, 320, 3) X(2, 32, 16, 640, 1) X(3, 32, 8, 384, 3)
 
+// tiles of tx x ty nodes that hold a fluid node (c->geom); the others leave after staging
+long long fluid_tiles(const lbm_ctx* c, int tx, int ty) {
+    const long long cols = (c->nx + tx - 1) / tx, rows = (c->ny + ty - 1) / ty;
+    const lbm_geometry& g = c->geom;
+    if (!g.has_circle) return cols * rows;
+    long long n = 0;
+    for (long long r = 0; r < rows; ++r) {
+        const double y0 = (double)(r * ty), y1 = std::min<double>(y0 + ty, c->ny) - 1;
+        // rows of the tile against the circle: the nearest one (cavity) or the farthest one (cylinder)
+        const double dy = g.concave ? std::max({0.0, y0 - g.cy, g.cy - y1})
+                                    : std::max(fabs(y0 - g.cy), fabs(y1 - g.cy));
+        const double h2 = g.R * g.R - dy * dy;
+        const double lo = h2 >= 0 ? g.cx - sqrt(h2) : 1, hi = h2 >= 0 ? g.cx + sqrt(h2) : 0;
+        if (g.concave) {  // tiles that reach into the cavity
+            const double a = std::max(lo, 0.0), b = std::min(hi, c->nx - 1.0);
+            if (a <= b) n += (long long)(b / tx) - (long long)(a / tx) + 1;
+        } else {  // tiles that do not lie inside the cylinder
+            const double a = std::max(ceil(lo / tx), 0.0);
+            const double b = hi >= c->nx - 1 ? cols - 1.0 : floor((hi + 1) / tx) - 1;
+            n += cols - (lo <= hi && a <= b ? (long long)(b - a) + 1 : 0);
+        }
+    }
+    return n;
+}
+
 // Whether a step of the 256-thread forms is placed early. A grid that fits on the chip at once leaves
 // slots free, and early placement fills those as they are: some SMs get five tiles of the next step,
 // others two, and the step waits for the fullest SM. Placed after the previous step the tiles are
 // spread evenly. us per step, half-way walls, drop on a cylinder / in a cavity, early -> not:
 // 517x425 (459 tiles) 11.8 -> 10.0 / 13.5 -> 11.0; 640x480 (600) 11.9 -> 11.3 / 13.6 -> 12.8; 768x480
 // (720) 12.5 -> 12.3 / 14.0 -> 14.4. Larger grids gain from early placement: 1024x512 (1024 tiles)
-// not 16.2, early 15.6 / 16.5, 16.3; 2048x1024 (4096) 46.4, 45.8.
-bool launch_early(const lbm_ctx* c, int tx, int ty) {
-    return (long long)((c->nx + tx - 1) / tx) * ((c->ny + ty - 1) / ty) > c->resident[c->ibb ? 1 : 0];
+// not 16.2, early 15.6 / 16.5, 16.3; 2048x1024 (4096) 46.4, 45.8. Tiles without fluid nodes leave at once, so a
+// grid that does not fit behaves like one that does when few of its tiles hold fluid. Cavities, fluid
+// tiles / early -> not: 1892x200 271 10.5 -> 9.4; 502x825 405 13.0 -> 10.5; 560x1100 499 13.2 -> 12.2; 620x660 606 13.5 ->
+// 13.1; 640x1000 648 13.7 -> 13.6; 1300x380 660 13.5 -> 13.9; 800x560 753 14.0 -> 14.4. Cylinders, whose empty tiles come
+// first: 900x440 365 11.7 -> 10.9, 768x512 432 12.0 -> 10.8, 800x520 460 11.5 -> 12.0, 640x620 551 11.3 -> 11.7.
+bool launch_early(const lbm_ctx* c) {
+    const int tx = c->tile_x, ty = c->tile_y;
+    const long long grid = (long long)((c->nx + tx - 1) / tx) * ((c->ny + ty - 1) / ty);
+    return grid > c->resident[c->ibb ? 1 : 0] &&
+           fluid_tiles(c, tx, ty) > (c->geom.concave ? 4 : 3) * c->sms;
 }
 
 // CTAs of a kernel that the whole chip holds at once
@@ -142,7 +176,7 @@ cudaError_t launch_one(lbm_ctx* c, const StepArgs<T>& a, bool macro) {
         LBM_SMALL_FORMS(X)
 #undef X
     }
-    const bool early = launch_early(c, TX, TY);
+    const bool early = c->early;
     if (c->ibb) {
         if constexpr (has_ibb<T, TX, TY, MINB>())
             return macro ? launch_k<T, TX, TY, 256, kIbbBlocks, true, true>(c, a, early)
@@ -225,18 +259,7 @@ void step_variants(size_t esz, std::vector<StepVariant>* out) {
 #undef X
 }
 
-cudaError_t step_configure(lbm_ctx* c) {
-#define X(T, A, B, M)                                                                       \
-    if (c->esz == sizeof(T) && c->tile_x == A && c->tile_y == B && minb_of(c) == M) {       \
-        if constexpr (sizeof(T) == 4) return configure_one<T, A, B, M>(c);                   \
-        return cudaSuccess;                                                                 \
-    }
-    LBM_STEP_VARIANTS(X)
-#undef X
-    return cudaErrorInvalidValue;
-}
-
-int step_form(const lbm_ctx* c) {
+static int step_form(const lbm_ctx* c) {
     const long long nx = c->nx, ny = c->ny, sms = c->sms;
     auto tiles = [&](long long tx, long long ty) {
         return ((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
@@ -251,6 +274,27 @@ int step_form(const lbm_ctx* c) {
                          : large > 3 * sms ? 24
                                            : (R >= 32 ? 23 : 22);
     return 4 * tiles(32, 8) <= quarters * sms ? 3 : 0;
+}
+
+bool step_choose(lbm_ctx* c) {
+    const int form = step_form(c);
+    const bool early = launch_early(c), changed = form != c->form || early != c->early;
+    c->form = form;
+    c->early = early;
+    return changed;
+}
+
+cudaError_t step_configure(lbm_ctx* c) {
+    cudaError_t e = cudaErrorInvalidValue;
+#define X(T, A, B, M)                                                                       \
+    if (c->esz == sizeof(T) && c->tile_x == A && c->tile_y == B && minb_of(c) == M) {       \
+        e = cudaSuccess;                                                                    \
+        if constexpr (sizeof(T) == 4) e = configure_one<T, A, B, M>(c);                      \
+    }
+    LBM_STEP_VARIANTS(X)
+#undef X
+    step_choose(c);
+    return e;
 }
 
 cudaError_t launch_step(lbm_ctx* c, int src, bool macro) {

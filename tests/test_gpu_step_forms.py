@@ -156,3 +156,27 @@ def test_flat_lattices_of_few_tiles_past_the_first_wave(lbm, oracle_mod, nx, ny)
     assert a < 0.9 * b, (a, b)
     lat.close()
     fixed.close()
+
+
+def test_grids_of_mostly_empty_tiles_are_spread_over_the_chip(lbm, oracle_mod):
+    """A cavity whose 832 tiles do not fit on the chip at once but whose tiles with fluid (about 380) do, against
+    the same cavity under 480 tiles, which fit: the 352 empty tiles more cost a few percent, fluid tiles
+    crowding onto some SMs a quarter; the bound lies between. Other walls in the same lattice object, placed
+    early and not, give the fields of the fixed 32x32 tiles."""
+    us, lats = [], []
+    for ny in (480, 825):
+        w = W.Workload("t", 502, ny, (251.0, 238.0, 232.0), (251.0, 50.0, 36.0, 5.6), concave=True)
+        lats.append(gpu_lattice(lbm, oracle_config(oracle_mod, w)[0]))
+        us.append(_us_per_step(lats[-1]))
+    assert us[1] < 1.1 * us[0], us
+    lats[0].close()
+    cfg = oracle_config(oracle_mod, W.Workload("t", 502, 825, None, (251.0, 50.0, 36.0, 5.6)))[0]
+    fixed = gpu_lattice(lbm, cfg, tile=(32, 32))
+    for circle in (None, (251.0, 238.0, 232.0), (251.0, 506.0, 500.0)):
+        for o in (lats[1], fixed):
+            o.set_geometry(circle=circle, concave=circle is not None, drop=(251.0, 50.0, 36.0, 5.6),
+                           mu_circle=cfg.mu_bottom, mu_bottom=cfg.mu_bottom, mu_top=cfg.mu_top)
+            o.step(70)
+        assert np.array_equal(lats[1].rho(), fixed.rho(), equal_nan=True)
+    lats[1].close()
+    fixed.close()
