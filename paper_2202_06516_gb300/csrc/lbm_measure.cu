@@ -70,7 +70,9 @@ __device__ __forceinline__ void add_node(FixSum& m, unsigned& nbad, double v) {
 }
 
 // Mass, liquid count, liquid centroid and the count of non-finite or non-positive densities over
-// the fluid nodes, one block per row (then striding), eight nodes per thread and access. Bound by
+// the fluid nodes, eight nodes per thread and access, 2^lt threads per row: one block per row (then
+// striding), or several rows at once where a lattice has more rows than blocks and rows that need few
+// threads (8 x 100000, host to host: 84 us with one row per block, 22 so). Bound by
 // the 5 bytes per node it reads and, with few rows, by latency: a block's mass is summed in exact
 // fixed point (lbm_sum.cuh) and the blocks' in FP64, counts and coordinate sums are integers (the same values the FP64
 // sums of whole numbers had), and the comparison with rho_m is made against the largest T not
@@ -79,16 +81,17 @@ __device__ __forceinline__ void add_node(FixSum& m, unsigned& nbad, double v) {
 // (every operation in FP64) became 20 us; 200 x 120: 7 + 26 us became 8.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
-    k_reduce(const T* rho, const uint8_t* flags, int nx, int ny, int P, T thr, Partials part,
+    k_reduce(const T* rho, const uint8_t* flags, int nx, int ny, int P, int lt, T thr, Partials part,
              unsigned* ticket, ReduceOut* out, ReduceOut* host_out) {
     FixSum mass;
     unsigned long long cnt[4] = {0, 0, 0, 0};  // n_liquid, sx, sy, bad
     const int groups = (nx + 7) / 8;
-    for (int j = blockIdx.x; j < ny; j += gridDim.x) {
+    const int rows = kRedThreads >> lt;
+    for (int j = blockIdx.x * rows + (threadIdx.x >> lt); j < ny; j += gridDim.x * rows) {
         const int row = lidx(P, 0, j);
         unsigned nl = 0, nbad = 0;
         unsigned long long sx = 0;
-        for (int g = threadIdx.x; g < groups; g += kRedThreads) {
+        for (int g = threadIdx.x & ((1 << lt) - 1); g < groups; g += 1 << lt) {
             const int i0 = 8 * g;
             T v[8];
             load8(rho + row + i0, v);  // columns past nx lie in the row's pad
@@ -565,11 +568,14 @@ double floor_to(double x, double) { return x; }
 template <typename T>
 cudaError_t reduce_t(lbm_ctx* c, ReduceOut* host) {
     const double rho_m = 0.5 * (c->rho_g + c->rho_l);
+    int lt = 0;
+    while ((1 << lt) < kRedThreads) ++lt;
+    while (lt > 0 && c->ny > (long long)c->red_blocks * (kRedThreads >> lt) && 8 << (lt - 1) >= c->nx) --lt;
     Partials p;
     p.mass = (double*)c->red_partials;
     p.cnt = (unsigned long long*)(p.mass + c->red_blocks);
     k_reduce<T><<<c->red_blocks, kRedThreads, 0, c->stream>>>(
-        (const T*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, floor_to(rho_m, T()), p,
+        (const T*)c->rho[c->cur], c->flags, c->nx, c->ny, c->P, lt, floor_to(rho_m, T()), p,
         &c->aux->ticket[0], &c->aux->red, host);
     return cudaGetLastError();
 }
