@@ -58,8 +58,11 @@ enum { LBM_BB_HALFWAY = 0, LBM_BB_INTERP = 1 }; /* lbm_geometry.boundary: curved
  *    budget is fitted to (0 = no constraint); all three 0 selects 32x16/5 in FP32 and 32x16/0 in
  *    FP64. Supported (tile/min_blocks):
  *    FP32 32x8/0, 32x8/6, 32x16/0, 32x16/5, 32x16/6, 64x16/0, 32x32/0; FP64 32x8/0, 32x16/0.
- *    FP64 steps run in untiled kernels, the same for both names; 32x16/5 on an FP32 lattice of few
- *    tiles runs in a form with smaller tiles or more threads (the same results).
+ *    FP64 steps run in untiled kernels, the same for both names. The default runs an FP32 lattice of few
+ *    tiles in a form with smaller tiles or more threads (the same results): one lattice alone on the
+ *    GPU takes half the time so, but each step costs the GPU more, and several lattices that step at the
+ *    same time, enough to fill it, take up to 2.3 times as long. For those use a batch, or 32/16/5 given
+ *    explicitly, which runs the 32x16 tiles at every size.
  *    tile_x = LBM_TILE_AUTO: start with the default and let lbm_autotune pick the variant at the
  *    first lbm_step (for lbm_batch_create: lbm_batch_autotune at the first lbm_batch_run).
  *  stream: a cudaStream_t (e.g. torch.cuda.current_stream().cuda_stream) or NULL. */

@@ -343,6 +343,7 @@ lbm_status lbm_create(const lbm_params* p, lbm_ctx** out) {
     c->tile_x = tx;
     c->tile_y = ty;
     c->min_blocks = min_blocks;
+    c->fixed = !tile_default && min_blocks == 5;  // (a variant of 32x16 only)
     c->autotune_pending = tile_auto;
     c->eosc.eos = p->eos;
     c->eosc.RT = he.R * he.T;
@@ -556,6 +557,8 @@ lbm_status lbm_autotune(lbm_ctx* c, int32_t trial_steps, lbm_tune_entry* entries
         LBM_CUDA(c, ce);
     }
     const lbm::StepVariant keep{c->tile_x, c->tile_y, c->min_blocks};
+    const bool keep_fixed = c->fixed;
+    c->fixed = false;  // the tuner's 32x16/5 is the default, with its forms
     int best = -1;
     double best_us = 0;
     cudaError_t err = cudaSuccess;
@@ -585,6 +588,7 @@ lbm_status lbm_autotune(lbm_ctx* c, int32_t trial_steps, lbm_tune_entry* entries
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     const lbm::StepVariant pick = (err == cudaSuccess && best >= 0) ? vs[best] : keep;
+    if (err != cudaSuccess || best < 0) c->fixed = keep_fixed;
     c->tile_x = pick.tile_x;
     c->tile_y = pick.tile_y;
     c->min_blocks = pick.min_blocks;

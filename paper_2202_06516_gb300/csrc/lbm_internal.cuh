@@ -149,6 +149,7 @@ struct lbm_ctx {
     bool graphs_ready = false;
     bool graph_failed = false;
     int tile_x = 32, tile_y = 16, min_blocks = 0;
+    bool fixed = false;  // 32x16/5 was asked for by name: no small-lattice forms
     int form = 0;  // small-lattice form of the default FP32 variant, 0: none
     bool early = false;  // steps of the other forms are placed before the previous one ends
     int resident[2] = {0, 0};  // tiles of that variant on the chip at once: half-way, interpolated walls

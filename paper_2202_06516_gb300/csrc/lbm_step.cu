@@ -70,7 +70,10 @@ cudaError_t allow_smem() {
 // barrier) on a chip that is mostly idle, so these forms give a tile so many threads that
 // every stage is one round, or spread the lattice over more, smaller tiles; on large lattices the
 // recomputed halo and the fewer resident tiles make them slower. Chosen by the number of tiles
-// against the number of SMs. Measured, us per step, 32x16 tiles of 256 threads / forms 1 / 2 / 3:
+// against the number of SMs. They are for one lattice at a time: with the chip full of lattices on streams of
+// their own the recomputed halos count (16 of 200x120 at once 12.5 us per step of all with 256 threads, 18.0
+// with form 1; 256x256 23.6, 53.6; 520x190 36.8, 56.5), which a lattice cannot know: 32x16/5 by name leaves them out.
+// Measured, us per step, 32x16 tiles of 256 threads / forms 1 / 2 / 3:
 // 128x96 7.4 / 4.3 / 5.1 / 4.8; 200x120 8.0 / 4.6 / 5.1 / 5.2; 256x256 8.0 / 6.0 / 5.2 / 5.6;
 // 520x190 10.2 / 6.8 / 7.2 / 6.1.
 // Form 3 holds three tiles per SM (456); up to twice as many run as a second wave. It then pays, the more
@@ -260,6 +263,7 @@ void step_variants(size_t esz, std::vector<StepVariant>* out) {
 }
 
 static int step_form(const lbm_ctx* c) {
+    if (c->fixed) return 0;
     const long long nx = c->nx, ny = c->ny, sms = c->sms;
     auto tiles = [&](long long tx, long long ty) {
         return ((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
